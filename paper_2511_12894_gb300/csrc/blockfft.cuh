@@ -1,160 +1,157 @@
-// Block FFT of B complex64 points held by one thread block: B/16 threads, 16
-// points per thread, Stockham radix-16 stages through shared memory plus one
-// final radix-2/4/8 stage when log2(B) is not a multiple of 4.
+// Block FFT of B complex64 points held by one thread block: B/16 threads, 16 points per
+// thread, decimation in time through shared memory in place: a radix-16 stage on registers, a
+// radix-RM stage (RM = 2, 4 or 8) when log2(B) is not a multiple of 4, then radix-16 stages.
 //
-// Stage with radix R and Ns = product of the earlier radices maps butterfly b
-// (k = b mod Ns) as  a[t] = in[b + t B/R] * w^(t k),  w = exp(sign 2 pi i / (Ns R)),
-// a = DFT_R(a),  out[(b - k) R + k + t Ns] = a[t]  (natural order after the last stage).
+// Locations l hold the input in digit-reversed order.  Stage with radix R and S = product of the
+// earlier radices works on the points l = hi S R + t S + lo (lo < S):
+//   a[t] = w^(t lo) x[l(t)],  w = exp(sign 2 pi i / (S R)),  x[l(t)] = DFT_R(a)[t],
+// and leaves the result in natural order after the last stage.  A butterfly writes the
+// locations it read, so a stage needs no barrier between its reads and its writes: one barrier
+// per exchange (an autosort form needs two), and the warps of a block overlap their loads,
+// butterflies and stores inside a stage.  Measured against the autosort form, with the magnitudes
+// of the window peaks in a region of their own (os_tail.cuh), on one GB300: 256 neighbours at
+// n = 2^20 in two buckets 1690 -> 1637 us, the 32768-point two-phase tails of 96 long kernels at
+// n = 2^23 10.2 -> 9.7 ms with the rest of that call, matched filters 1.5%.  A barrier of only the
+// 256 threads that exchange data between the middle stages was slower (1694 us): the drifted
+// warps spread one block's loads over its neighbour phases.
 //
-// Input: before run(), thread `tid` holds v[t] = x[tid + t B/16] for t < 16.
-// Output: after run(), thread `tid` holds, for q < 16/RL and t < RL,
-//   v[q RL + t] = X[b + t B/RL],  b = tid + q NT   (RL = radix of the last stage).
-// Shared memory: B + B/16 float2 (index p is stored at p + p/16, which makes the
-// stride-16 writes of the first stage bank-conflict free).
+// Input: before the call, thread `tid` holds v[t] = x[tid + t B/16] for t < 16.
+// Output: after it, thread `tid` holds v[t] = X[tid + t B/16].
+// Shared memory: B + 32 float2; location l is stored at l + 2 (l / (B/16)), so that the 16
+// lanes of the first stage's writes, which are B/16 locations apart, fall two bank pairs apart
+// (128-bit stores, eight lanes per wavefront); the later stages touch runs of 16 locations.
 //
-// Twiddles come from per-stage tables laid out in thread order: the stage with
-// radix R and Ns has a table of R*Ns entries, entry t*Ns + k = exp(-2 pi i t k / (R Ns)),
-// so the loads of a warp are contiguous.  A stage reads the rows t = 1, 2, 4 and 8 and forms
-// the other powers by complex products (a last stage of radix 2 or 4 reads only row 1).  The tables of the middle stages and of the
-// last stage follow each other; a block size B needs block_table_size<B>() entries
-// (built on the host by block_fft_tables).
+// Twiddles come from per-stage tables laid out in thread order: the stage with radix R and S has
+// a table of R S entries, entry t S + k = exp(-2 pi i t k / (R S)), so the loads of a warp are
+// contiguous.  A radix-16 stage reads the rows t = 1 and 4 and forms the other powers by complex
+// products.  The tables of the stages after the first follow each other; a block size B needs
+// block_table_size<B>() entries (built on the host by block_fft_tables).
 #pragma once
 
 #include "cplx.cuh"
 
 namespace rf {
 
-__device__ __forceinline__ int bf_pad(int p) { return p + (p >> 4); }
-
-// Multiplies a[t], 0 < t < R (R = 8 or 16), by w^t (conjugated for SIGN = +1) where w^t is
-// table entry t * stride: the entries t = 1 and 4 are loaded and the others formed by complex
-// products (w^2 = w w, w^8 = w^4 w^4, at most three products deep: a few ulp), which keeps 13 of
-// the 15 table loads of a radix-16 stage off the load/store pipe, the scarcer one in the block
-// transforms (loading all 15 made the 2^23-sample step 12% slower, loading 4 was 2% slower).
-template <int R, int SIGN>
-__device__ __forceinline__ void apply_stage_twiddles(float2* a, const float2* __restrict__ tw, int stride) {
-  static_assert(R == 8 || R == 16, "radix");
-  float2 w[R];
+// The powers w[t], 0 < t < R (R = 4, 8 or 16), of which table entry t * stride is w^t: the
+// entries t = 1 and (R >= 8) 4 are loaded and the others formed by complex products (w^2 = w w,
+// w^8 = w^4 w^4, at most three products deep: a few ulp), which keeps 13 of the 15 table loads of
+// a radix-16 stage off the load/store pipe, the scarcer one in the block transforms (loading all
+// 15 made the 2^23-sample step 12% slower, loading 4 was 2% slower).
+template <int R>
+__device__ __forceinline__ void stage_twiddles(float2 (&w)[R], const float2* __restrict__ tw, int stride) {
+  static_assert(R == 2 || R == 4 || R == 8 || R == 16, "radix");
   w[1] = __ldg(tw + stride);
-  w[4] = __ldg(tw + 4 * stride);
-  w[2] = cmul(w[1], w[1]);
-  w[3] = cmul(w[2], w[1]);
-  w[5] = cmul(w[4], w[1]);
-  w[6] = cmul(w[4], w[2]);
-  w[7] = cmul(w[4], w[3]);
+  if constexpr (R >= 4) {
+    w[2] = cmul(w[1], w[1]);
+    w[3] = cmul(w[2], w[1]);
+  }
+  if constexpr (R >= 8) {
+    w[4] = __ldg(tw + 4 * stride);
+    w[5] = cmul(w[4], w[1]);
+    w[6] = cmul(w[4], w[2]);
+    w[7] = cmul(w[4], w[3]);
+  }
   if constexpr (R == 16) {
     w[8] = cmul(w[4], w[4]);
 #pragma unroll
     for (int t = 9; t < 16; ++t) w[t] = cmul(w[8], w[t - 8]);
   }
+}
+
+template <int R, int SIGN>
+__device__ __forceinline__ void apply_twiddles(float2* a, const float2 (&w)[R]) {
 #pragma unroll
   for (int t = 1; t < R; ++t) a[t] = tw_apply<SIGN>(a[t], w[t]);
 }
 
 template <int B>
 struct BlockFFTShape {
-  static constexpr int LOGB = (B == 256) ? 8 : (B == 512) ? 9 : (B == 1024) ? 10 : (B == 2048) ? 11
-                            : (B == 4096) ? 12 : (B == 8192) ? 13 : (B == 16384) ? 14 : -1;
+  static constexpr int LOGB = (B == 512) ? 9 : (B == 1024) ? 10 : (B == 2048) ? 11 : (B == 4096) ? 12
+                            : (B == 8192) ? 13 : (B == 16384) ? 14 : -1;
   static_assert(LOGB > 0, "block size");
   static constexpr int NT = B / 16;
-  static constexpr int N16 = LOGB / 4;                 // radix-16 stages
-  static constexpr int REM = LOGB % 4;
-  static constexpr int RL = REM ? (1 << REM) : 16;     // radix of the last stage
-  static constexpr int SMEM = B + B / 16;              // float2 entries
+  static constexpr int RM = 1 << (LOGB % 4);           // radix of the second stage (1: none)
+  static constexpr int MID16 = LOGB / 4 - 2;           // radix-16 stages between it and the last (0 or 1)
+  static constexpr int SMEM = B + 32;                  // float2 entries
+  static constexpr int NTP = NT + 2;                   // padded stride of NT locations
 };
 
-// Radix-16 stages between the first and the last stage.
-template <int B>
-__host__ __device__ constexpr int block_mid_stages() {
-  return (BlockFFTShape<B>::REM ? BlockFFTShape<B>::N16 : BlockFFTShape<B>::N16 - 1) - 1;
-}
-
-// Entries of the stage twiddle tables of block size B: 16 Ns per middle stage, then B for
-// the last stage.
+// Entries of the stage twiddle tables of block size B.
 template <int B>
 __host__ __device__ constexpr int block_table_size() {
-  int s = 0, ns = 16;
-  for (int st = 0; st < block_mid_stages<B>(); ++st) {
-    s += 16 * ns;
-    ns *= 16;
-  }
-  return s + B;
+  using S = BlockFFTShape<B>;
+  return (S::RM > 1 ? 16 * S::RM : 0) + (S::MID16 ? 256 * S::RM : 0) + B;
 }
 
 // tw: the stage tables of B.  SIGN: -1 forward, +1 inverse (unnormalised).  tid: the
-// thread's index within the transform (0 .. B/16 - 1); several transforms can share a thread
-// block, each with its own shared-memory region, as long as every thread of the block calls
-// block_fft (it synchronises the whole block).
-// Every access of a stage is base + t * stride in the padded index (the strides are
-// multiples of 16, so pad(base + t stride) = pad(base) + t (stride + stride / 16)), which
-// lets the compiler use one base register and immediate offsets.
+// thread's index within the transform (0 .. B/16 - 1); several transforms of B <= 4096 points
+// can share a thread block, each with its own shared-memory region (16-byte aligned), as long as
+// every thread of the block calls block_fft (it synchronises the whole block).  The region may be
+// rewritten by the caller only after a barrier: the last stage reads it without one after it.
 template <int B, int SIGN>
 __device__ __forceinline__ void block_fft(float2 (&v)[16], float2* sm, const float2* __restrict__ tw, int tid) {
   using S = BlockFFTShape<B>;
-  constexpr int NT = S::NT;
-  // first stage: Ns = 1, no twiddles, out[b*16 + t] at padded index 17 b + t
+  constexpr int NT = S::NT, RM = S::RM, NTP = S::NTP;
+  // First stage: no twiddles.  The thread's bins t B/16 + tid sit at locations base + t, with the
+  // digits of tid (t2 of RM, t3 of 16 when there is a middle radix-16 stage, t4 of 16) reversed.
   dft<16, SIGN>(v);
   {
-    float2* o = sm + 17 * tid;
+    constexpr int N3 = S::MID16 ? 16 : 1;
+    const int rest = tid / 16;
+    float2* o = sm + 16 * (rest / N3) + 16 * RM * (rest % N3) + NTP * (tid % 16);
 #pragma unroll
-    for (int t = 0; t < 16; ++t) o[t] = v[t];
+    for (int t = 0; t < 16; t += 2) *reinterpret_cast<float4*>(o + t) = make_float4(v[t].x, v[t].y, v[t + 1].x, v[t + 1].y);
   }
   __syncthreads();
-  int Ns = 16;
-  // middle radix-16 stages (all but the last stage)
-  constexpr int MID = block_mid_stages<B>();
-  constexpr int RSTR = B / 16 + B / 256;  // padded stride of the stage reads
+  if constexpr (RM > 1) {
+    // second stage, S = 16: butterflies tid + q NT, q < 16 / RM; all have lo = tid mod 16
+    const int lo = tid % 16;
+    float2 w[RM];
+    stage_twiddles<RM>(w, tw + lo, 16);
+    const int l0 = (tid / 16) * 16 * RM + lo;
+    float2* p = sm + l0 + 2 * (l0 / NT);
 #pragma unroll
-  for (int st = 0; st < MID; ++st) {
-    {
-      const float2* in = sm + bf_pad(tid);
+    for (int q = 0; q < 16 / RM; ++q) {
+      float2 a[RM];
+      float2* pq = p + q * RM * NTP;
 #pragma unroll
-      for (int t = 0; t < 16; ++t) v[t] = in[t * RSTR];
+      for (int t = 0; t < RM; ++t) a[t] = pq[16 * t];
+      apply_twiddles<RM, SIGN>(a, w);
+      dft<RM, SIGN>(a);
+#pragma unroll
+      for (int t = 0; t < RM; ++t) pq[16 * t] = a[t];
     }
+    tw += 16 * RM;
     __syncthreads();
-    const int k = tid & (Ns - 1);
-    apply_stage_twiddles<16, SIGN>(v, tw + k, Ns);
-    dft<16, SIGN>(v);
-    {
-      float2* o = sm + bf_pad((tid - k) * 16 + k);
-      const int wstr = Ns + Ns / 16;
-#pragma unroll
-      for (int t = 0; t < 16; ++t) o[t * wstr] = v[t];
-    }
-    __syncthreads();
-    tw += 16 * Ns;
-    Ns *= 16;
   }
-  // last stage: radix RL, Ns = B / RL, every butterfly index b < Ns so k = b
-  constexpr int RL = S::RL;
-  constexpr int LSTR = B / RL + B / (16 * RL);
-  // for RL <= 4, w^1 of butterfly b = tid + q NT is that of tid times exp(-2 pi i q / 16)
-  // (NT / B = 1/16): one table load for the thread, exact-constant rotations for the others
-  [[maybe_unused]] const float2 w1t = RL <= 4 ? __ldg(tw + (B / RL) + tid) : make_float2(1.f, 0.f);
-  static_for<0, 16 / RL>([&](auto qc) {
-    constexpr int q = decltype(qc)::value;
-    const int b = tid + q * NT;
-    float2 a[RL];
-    const float2* in = sm + bf_pad(b);
+  if constexpr (S::MID16) {
+    // middle radix-16 stage, S = 16 RM: group hi of NT = 16 S locations
+    constexpr int ST = 16 * RM;
+    const int lo = tid % ST;
+    float2* p = sm + (tid / ST) * NTP + lo;
 #pragma unroll
-    for (int t = 0; t < RL; ++t) a[t] = in[t * LSTR];
-    if constexpr (RL <= 4) {
-      // w^t for t < RL from w^1 (the table's t = 1 row): the square (and cube) cost a complex
-      // product each (about 1 ulp more error)
-      const float2 w1 = rot16<q, -1>(w1t);
-      a[1] = tw_apply<SIGN>(a[1], w1);
-      if constexpr (RL == 4) {
-        const float2 w2 = cmul(w1, w1);
-        a[2] = tw_apply<SIGN>(a[2], w2);
-        a[3] = tw_apply<SIGN>(a[3], cmul(w2, w1));
-      }
-    } else {
-      apply_stage_twiddles<RL, SIGN>(a, tw + b, B / RL);
+    for (int t = 0; t < 16; ++t) v[t] = p[t * ST];
+    {
+      float2 w[16];
+      stage_twiddles<16>(w, tw + lo, ST);
+      apply_twiddles<16, SIGN>(v, w);
     }
-    dft<RL, SIGN>(a);
+    dft<16, SIGN>(v);
 #pragma unroll
-    for (int t = 0; t < RL; ++t) v[q * RL + t] = a[t];
-  });
+    for (int t = 0; t < 16; ++t) p[t * ST] = v[t];
+    tw += 16 * ST;
+    __syncthreads();
+  }
+  // last stage, S = NT: butterfly lo = tid
+  {
+    const float2* p = sm + tid;
+#pragma unroll
+    for (int t = 0; t < 16; ++t) v[t] = p[t * NTP];
+    float2 w[16];
+    stage_twiddles<16>(w, tw + tid, NT);
+    apply_twiddles<16, SIGN>(v, w);
+  }
+  dft<16, SIGN>(v);
 }
 
 // One transform per thread block (tid = threadIdx.x).

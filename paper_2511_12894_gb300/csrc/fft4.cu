@@ -34,7 +34,7 @@ constexpr int kF4Product = 2;
 // float2 entries of one line's shared-memory region in a tile of G lines.
 template <int L, int G>
 __host__ __device__ constexpr int f4_line() {
-  return L + L / 16 + 16 / G;
+  return BlockFFTShape<L>::SMEM + 16 / G;
 }
 
 template <int L, int G>
@@ -50,8 +50,7 @@ __global__ void __launch_bounds__(G * L / 16) k_fft4_cols(const void* __restrict
                                                           const float2* __restrict__ tw4, int lo_bits) {
   using S = BlockFFTShape<L>;
   constexpr int NT = S::NT;
-  constexpr int RL = S::RL;
-  extern __shared__ float2 f4_sm[];
+  extern __shared__ __align__(16) float2 f4_sm[];
   const int c = (int)threadIdx.x % G;
   const int ltid = (int)threadIdx.x / G;
   const int64_t N2 = (int64_t)1 << n2log;
@@ -81,7 +80,7 @@ __global__ void __launch_bounds__(G * L / 16) k_fft4_cols(const void* __restrict
       v[t] = t * tstep <= lim ? cmul(px[t * tstep], pf[t * tstep]) : make_float2(0.f, 0.f);
   }
   block_fft<L, SIGN>(v, f4_sm + c * f4_line<L, G>(), twb, ltid);
-  // v[q RL + t] holds the column's bin k1 = ltid + NT u, u = q + t 16/RL (every u < 16 once).
+  // v[u] holds the column's bin k1 = ltid + NT u, u < 16.
   // Twiddle w_n^(col k1) = w_n^(col ltid) e^u with e = w_n^(col NT): e, e^2, e^4 and e^8 come
   // from the tables (a product of two entries each, m = col NT 2^i < n), e^3, e^5 .. e^7 by at
   // most two more products, and e^(u + 8) = e^u e^8 (a few ulp in all).
@@ -105,11 +104,8 @@ __global__ void __launch_bounds__(G * L / 16) k_fft4_cols(const void* __restrict
     else eu = cmul(e4, cmul(e2, e1));
     const float2 w = u == 0 ? b0 : cmul(b0, eu);
     const float2 w8 = cmul(w, e8);
-    constexpr int QN = 16 / RL;
-    const int r0 = (u % QN) * RL + u / QN;              // register of bin ltid + NT u
-    const int r8 = ((u + 8) % QN) * RL + (u + 8) / QN;  // register of bin ltid + NT (u + 8)
-    o[(int64_t)(u * NT) * N2] = tw_apply<SIGN>(v[r0], w);
-    o[(int64_t)((u + 8) * NT) * N2] = tw_apply<SIGN>(v[r8], w8);
+    o[(int64_t)(u * NT) * N2] = tw_apply<SIGN>(v[u], w);
+    o[(int64_t)((u + 8) * NT) * N2] = tw_apply<SIGN>(v[u + 8], w8);
   }
 }
 
@@ -119,9 +115,8 @@ __global__ void __launch_bounds__(R * L / 16) k_fft4_rows(const float2* __restri
                                                           int n1log, const float2* __restrict__ twb) {
   using S = BlockFFTShape<L>;
   constexpr int NT = S::NT;
-  constexpr int RL = S::RL;
   constexpr int SL = f4_line<L, R>();
-  extern __shared__ float2 f4_sm[];
+  extern __shared__ __align__(16) float2 f4_sm[];
   const int g = (int)threadIdx.x / NT;
   const int ltid = (int)threadIdx.x % NT;
   const int64_t N1 = (int64_t)1 << n1log;
@@ -135,9 +130,7 @@ __global__ void __launch_bounds__(R * L / 16) k_fft4_rows(const float2* __restri
   block_fft<L, SIGN>(v, sm, twb, ltid);
   __syncthreads();  // the last stage has read its inputs from shared memory
 #pragma unroll
-  for (int q = 0; q < 16 / RL; ++q)
-#pragma unroll
-    for (int t = 0; t < RL; ++t) sm[ltid + q * NT + t * (L / RL)] = v[q * RL + t];
+  for (int t = 0; t < 16; ++t) sm[ltid + t * NT] = v[t];
   __syncthreads();
   float2* dst = out + (int64_t)blockIdx.y * n + row0;
 #pragma unroll

@@ -117,7 +117,6 @@ __device__ __forceinline__ void os_block_tail(float2 (&v)[16], int s, int64_t m0
   constexpr int NT = S::NT;
   constexpr int LP = B / Q;
   constexpr int H = B - LP;
-  constexpr int RL = S::RL;
   constexpr int CH = H / NT;
   const int tid = threadIdx.x;
   const int64_t mask = n - 1;
@@ -127,26 +126,19 @@ __device__ __forceinline__ void os_block_tail(float2 (&v)[16], int s, int64_t m0
   const int64_t lim = n - o0;                       // block positions LP + t with t < lim exist
   if (!WINMAX) {
 #pragma unroll
-    for (int q = 0; q < 16 / RL; ++q)
-#pragma unroll
-      for (int t = 0; t < RL; ++t) {
-        const int idx = tid + q * NT + t * (B / RL);
-        if (idx >= LP && idx - LP < lim) zrow[(base + idx - LP) & mask] = v[q * RL + t];
-      }
+    for (int t = 16 / Q; t < 16; ++t) {
+      const int idx = tid + t * NT - LP;
+      if (idx < lim) zrow[(base + idx) & mask] = v[t];
+    }
     __syncthreads();  // the next block's FFT overwrites the shared memory read above
   } else {
-    __syncthreads();  // the last FFT stage has finished reading shared memory
-    float* mag = reinterpret_cast<float*>(sm);
+    // |y|^2 into its own region, so that no barrier is needed before these writes (the last stage
+    // of slower warps still reads the transform's region); the barrier after them also frees the
+    // transform's region for the next block, whose own barriers come before the region of the
+    // magnitudes is written again
+    float* mag = reinterpret_cast<float*>(sm + S::SMEM);
 #pragma unroll
-    for (int q = 0; q < 16 / RL; ++q)
-#pragma unroll
-      for (int t = 0; t < RL; ++t) {
-        const int idx = tid + q * NT + t * (B / RL);
-        if (idx >= LP) {
-          const float2 y = v[q * RL + t];
-          mag[idx - LP] = y.x * y.x + y.y * y.y;
-        }
-      }
+    for (int t = 16 / Q; t < 16; ++t) mag[tid + t * NT - LP] = v[t].x * v[t].x + v[t].y * v[t].y;
     __syncthreads();
     const int qbase = tid * CH;
     float mv[CH];
@@ -163,8 +155,13 @@ __device__ __forceinline__ void os_block_tail(float2 (&v)[16], int s, int64_t m0
     const int64_t avail = lim - qbase;
     const int cnt = avail <= 0 ? 0 : (avail >= CH ? CH : (int)avail);
     window_keys<CH>(mv, cnt, (int)((base + qbase) & mask), n, W, nw, fastwin, kj);
-    __syncthreads();  // mag (shared memory) is reused by the next block's FFT
   }
+}
+
+// Shared memory of a CTA that runs os_block_tail: the transform's region, then the magnitudes.
+template <int B, int Q, bool WINMAX>
+constexpr size_t os_tail_smem() {
+  return sizeof(float2) * BlockFFTShape<B>::SMEM + (WINMAX ? sizeof(float) * (B - B / Q) : 0);
 }
 
 // ------------------------------------------------------- 32768-point blocks on CTA pairs
@@ -216,7 +213,6 @@ __device__ __forceinline__ void os2_block_tail(float2 (&v)[16], int s, int64_t m
                                                const float2* __restrict__ twc, float2* sm, unsigned r, uint32_t peer) {
   using S = BlockFFTShape<kBH>;
   constexpr int NT = S::NT;
-  constexpr int RL = S::RL;
   constexpr int LP = kB2 / Q;  // outputs start at block position LP (<= BH)
   constexpr int H = kB2 - LP;
   static_assert(Q == 2 || Q == 4, "partition ratio");
@@ -228,9 +224,7 @@ __device__ __forceinline__ void os2_block_tail(float2 (&v)[16], int s, int64_t m
   block_fft<kBH, +1>(v, sm, tw);
   __syncthreads();  // the last stage has read shared memory
 #pragma unroll
-  for (int qq = 0; qq < 16 / RL; ++qq)
-#pragma unroll
-    for (int t = 0; t < RL; ++t) sm[tid + qq * NT + t * (kBH / RL)] = v[qq * RL + t];
+  for (int t = 0; t < 16; ++t) sm[tid + t * NT] = v[t];
   cluster_sync_all();  // both halves in shared memory
   // combine: this CTA takes t = r BH/2 + e NT + tid, e < 8 (consecutive lanes, consecutive t)
   const int64_t o0 = (int64_t)s * H;  // pre-relabel index of block position LP
@@ -286,7 +280,6 @@ __device__ __forceinline__ void pair1_halves(Load&& load, float2* __restrict__ e
                                              float2* sm) {
   using S = BlockFFTShape<kBH>;
   constexpr int NT = S::NT;
-  constexpr int RL = S::RL;
   const int tid = threadIdx.x;
   // one loop body, so that the code holds one transform
 #pragma unroll 1
@@ -296,15 +289,13 @@ __device__ __forceinline__ void pair1_halves(Load&& load, float2* __restrict__ e
     block_fft<kBH, +1>(v, sm, tw);
     __syncthreads();  // the last stage has read shared memory
 #pragma unroll
-    for (int q = 0; q < 16 / RL; ++q)
-#pragma unroll
-      for (int t = 0; t < RL; ++t) {
-        const int idx = tid + q * NT + t * (kBH / RL);
-        if (h == 0)
-          __stcg(e0 + idx, v[q * RL + t]);
-        else
-          sm[idx] = v[q * RL + t];
-      }
+    for (int t = 0; t < 16; ++t) {
+      const int idx = tid + t * NT;
+      if (h == 0)
+        __stcg(e0 + idx, v[t]);
+      else
+        sm[idx] = v[t];
+    }
   }
   __syncthreads();  // E_1 staged; E_0 of every thread written to the scratch row
 }

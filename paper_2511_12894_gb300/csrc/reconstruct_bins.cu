@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(B / 16, 16384 / B)
     k_bins_tail(const OsItem* __restrict__ items, const float2* __restrict__ Y, int s0, int ns,
                 const float2* __restrict__ tw, int64_t n, float2* __restrict__ z_out,
                 unsigned long long* __restrict__ keys, int64_t W, int64_t nw, int fastwin) {
-  extern __shared__ float2 sm[];
+  extern __shared__ __align__(16) float2 sm[];
   const int si = blockIdx.x, ii = blockIdx.y;
   const OsItem it = items[ii];
   const float2* y = Y + ((int64_t)ii * ns + si) * B + threadIdx.x;
@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(kBH / 16, 1)
                      const float2* __restrict__ tw, const float2* __restrict__ twc, int64_t n,
                      float2* __restrict__ z_out, unsigned long long* __restrict__ keys, int64_t W, int64_t nw,
                      int fastwin, float2* __restrict__ e0_all) {
-  extern __shared__ float2 sm[];
+  extern __shared__ __align__(16) float2 sm[];
   constexpr int NT = kBH / 16;
   const int tid = threadIdx.x;
   float2* e0 = e0_all + (int64_t)blockIdx.x * kBH;
@@ -253,7 +253,7 @@ void products_pm(int pm, const OsItem* items, const float2* zs_one, int B, int N
 template <int B, int Q, bool WINMAX>
 void launch_tail(const OsItem* items, const float2* Y, int s0, int ns, int nitems, const float2* tw, int64_t n,
                  float2* z_out, unsigned long long* keys, int64_t W, int64_t nw, int fastwin, cudaStream_t s) {
-  const size_t smem = sizeof(float2) * BlockFFTShape<B>::SMEM;
+  constexpr size_t smem = os_tail_smem<B, Q, WINMAX>();
   auto fn = k_bins_tail<B, Q, WINMAX>;
   RF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   fn<<<dim3((unsigned)ns, (unsigned)nitems), B / 16, smem, s>>>(items, Y, s0, ns, tw, n, z_out, keys, W, nw,

@@ -34,7 +34,7 @@ template <int B>
 __global__ void __launch_bounds__(B / 16) k_os_segments(const float2* __restrict__ z_ref, int64_t n, int Lp,
                                                         const float2* __restrict__ tw, float2* __restrict__ Zs) {
   using S = BlockFFTShape<B>;
-  extern __shared__ float2 sm[];
+  extern __shared__ __align__(16) float2 sm[];
   const int64_t s = blockIdx.x;
   const int tid = threadIdx.x;
   const int64_t mask = n - 1;
@@ -44,9 +44,7 @@ __global__ void __launch_bounds__(B / 16) k_os_segments(const float2* __restrict
   block_fft<B, -1>(v, sm, tw);
   float2* out = Zs + s * B;
 #pragma unroll
-  for (int q = 0; q < 16 / S::RL; ++q)
-#pragma unroll
-    for (int t = 0; t < S::RL; ++t) out[tid + q * S::NT + t * (B / S::RL)] = v[q * S::RL + t];
+  for (int t = 0; t < 16; ++t) out[tid + t * S::NT] = v[t];
 }
 
 // Segment spectra of several references: block (s, g) transforms segment s of z_refs[g].
@@ -55,7 +53,7 @@ __global__ void __launch_bounds__(B / 16) k_os_segments_batched(const float2* co
                                                                 int Lp, const float2* __restrict__ tw,
                                                                 float2* __restrict__ Zs_all) {
   using S = BlockFFTShape<B>;
-  extern __shared__ float2 sm[];
+  extern __shared__ __align__(16) float2 sm[];
   const int64_t s = blockIdx.x;
   const int64_t g = blockIdx.y;
   const int64_t NQ = n / Lp;
@@ -68,9 +66,7 @@ __global__ void __launch_bounds__(B / 16) k_os_segments_batched(const float2* co
   block_fft<B, -1>(v, sm, tw);
   float2* out = Zs_all + (g * NQ + s) * B;
 #pragma unroll
-  for (int q = 0; q < 16 / S::RL; ++q)
-#pragma unroll
-    for (int t = 0; t < S::RL; ++t) out[tid + q * S::NT + t * (B / S::RL)] = v[q * S::RL + t];
+  for (int t = 0; t < 16; ++t) out[tid + t * S::NT] = v[t];
 }
 
 // One neighbour's output blocks [s0, s1): spectral products, then the block tail (inverse block
@@ -132,7 +128,7 @@ __global__ void __launch_bounds__(B / 16, 16384 / B) k_os(const float2* __restri
                                               int NQ, int NB, int SC, float2* __restrict__ z_out,
                                               unsigned long long* __restrict__ keys, int64_t W, int64_t nw,
                                               int fastwin, int herm) {
-  extern __shared__ float2 sm[];
+  extern __shared__ __align__(16) float2 sm[];
   const int j = idx[y0 + blockIdx.y];
   const int s0 = blockIdx.x * SC;
   const int s1 = min(NB, s0 + SC);
@@ -158,7 +154,7 @@ __global__ void __launch_bounds__(B / 16, 16384 / B) k_os_batched(const OsItem* 
                                                                  unsigned long long* __restrict__ keys,
                                                                  int64_t W, int64_t nw, int fastwin, int herm,
                                                                  unsigned long long* __restrict__ counter) {
-  extern __shared__ float2 sm[];
+  extern __shared__ __align__(16) float2 sm[];
   __shared__ long long s_unit;
   for (;;) {
     if (threadIdx.x == 0) s_unit = (long long)atomicAdd(counter, 1ull);
@@ -240,7 +236,7 @@ __global__ void __launch_bounds__(kBH / 16) k_os2_segments(const float2* __restr
                                                           int NQ, const float2* __restrict__ tw,
                                                           const float2* __restrict__ twc, float2* __restrict__ Zs_all) {
   using S = BlockFFTShape<kBH>;
-  extern __shared__ float2 sm[];
+  extern __shared__ __align__(16) float2 sm[];
   const int64_t q = blockIdx.x;
   const int r = blockIdx.y;
   const int64_t g = blockIdx.z;
@@ -258,9 +254,7 @@ __global__ void __launch_bounds__(kBH / 16) k_os2_segments(const float2* __restr
   block_fft<kBH, -1>(v, sm, tw);
   float2* out = Zs_all + ((int64_t)g * NQ + q) * kB2 + (int64_t)r * kBH;
 #pragma unroll
-  for (int qq = 0; qq < 16 / S::RL; ++qq)
-#pragma unroll
-    for (int t = 0; t < S::RL; ++t) out[tid + qq * S::NT + t * (kBH / S::RL)] = v[qq * S::RL + t];
+  for (int t = 0; t < 16; ++t) out[tid + t * S::NT] = v[t];
 }
 
 // Spectral products of one output block for the bins of parity r (as os_blocks, on the
@@ -320,7 +314,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kBH / 16, 1)
           const int* __restrict__ parts, const int* __restrict__ lag0, const int* __restrict__ idx, int y0,
           const float2* __restrict__ tw, const float2* __restrict__ twc, int64_t n, int NQ, int NB, int SC,
           float2* __restrict__ z_out, unsigned long long* __restrict__ keys, int64_t W, int64_t nw, int fastwin) {
-  extern __shared__ float2 sm[];
+  extern __shared__ __align__(16) float2 sm[];
   const int j = idx[y0 + blockIdx.y];
   const int s0 = (int)(blockIdx.x >> 1) * SC;
   const int s1 = min(NB, s0 + SC);
@@ -335,7 +329,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kBH / 16, 1)
     k_os2_batched(const OsItem* __restrict__ items, int nchunk, const float2* __restrict__ tw,
                   const float2* __restrict__ twc, int64_t n, int NQ, int NB, int SC,
                   unsigned long long* __restrict__ keys, int64_t W, int64_t nw, int fastwin) {
-  extern __shared__ float2 sm[];
+  extern __shared__ __align__(16) float2 sm[];
   const OsItem it = items[blockIdx.y];
   const int s0 = (int)(blockIdx.x >> 1) * SC;
   const int s1 = min(NB, s0 + SC);
@@ -388,11 +382,12 @@ void launch_os(rf_ctx* c, const rf_kernels* kern, const OsBucket& bk, const floa
   const int nchunk = (NB + SC - 1) / SC;
   const int fastwin = (WINMAX && W >= os_warp_span<B, Q>()) ? 1 : 0;  // a warp's outputs span <= 2 windows
   auto fn = k_os<B, Q, WINMAX>;
-  RF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)os_smem<B>()));
+  constexpr size_t smem = os_tail_smem<B, Q, WINMAX>();
+  RF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   for (int done = 0; done < count; done += 65535) {
     const int cnt = std::min(65535, count - done);
     dim3 grid((unsigned)nchunk, (unsigned)cnt);
-    fn<<<grid, B / 16, os_smem<B>(), s>>>(Zs, kern->os_spec.as<float2>(), kern->os_off_d.as<int64_t>(),
+    fn<<<grid, B / 16, smem, s>>>(Zs, kern->os_spec.as<float2>(), kern->os_off_d.as<int64_t>(),
                                           kern->os_parts_d.as<int>(), kern->lag0_d.as<int>(), bk.idx_d.as<int>(), done,
                                           tw, c->n, NQ, NB, SC, z_out, keys, W, nw, fastwin, kern->real ? 1 : 0);
     RF_LAUNCHED();
@@ -473,27 +468,25 @@ void dispatch_bq(int B, int Q, F&& f) {
 
 namespace {
 
-// Stage tables of one block size, in the order block_fft reads them.
+// Stage tables of one block size, in the order block_fft reads them: the stages after the first,
+// radix R after S points, entry t S + k = exp(-2 pi i t k / (R S)).
 template <int B>
 void append_tables(std::vector<float2>& out) {
   using S = BlockFFTShape<B>;
   const size_t start = out.size();
-  int Ns = 16;
-  for (int st = 0; st < block_mid_stages<B>(); ++st) {
-    const std::vector<double2> w = host_twiddles(16 * (int64_t)Ns);  // exp(-2 pi i m / (16 Ns))
-    for (int t = 0; t < 16; ++t)
-      for (int k = 0; k < Ns; ++k) {
+  int st = 16;
+  auto stage = [&](int radix) {
+    const std::vector<double2> w = host_twiddles((int64_t)radix * st);
+    for (int t = 0; t < radix; ++t)
+      for (int k = 0; k < st; ++k) {
         const double2 v = w[(size_t)t * k];
         out.push_back(make_float2((float)v.x, (float)v.y));
       }
-    Ns *= 16;
-  }
-  const std::vector<double2> w = host_twiddles(B);  // last stage: exp(-2 pi i t b / B)
-  for (int t = 0; t < S::RL; ++t)
-    for (int b = 0; b < B / S::RL; ++b) {
-      const double2 v = w[(size_t)t * b];
-      out.push_back(make_float2((float)v.x, (float)v.y));
-    }
+    st *= radix;
+  };
+  if (S::RM > 1) stage(S::RM);
+  if (S::MID16) stage(16);
+  stage(16);
   if (out.size() - start != (size_t)block_table_size<B>()) throw Fail{RF_EINVAL};
 }
 
@@ -1135,11 +1128,12 @@ void reconstruct_batched(rf_ctx* c, int32_t G, const void* const* z_refs, rf_ker
                                                                          tw, c->batch_zs.as<float2>());
       RF_LAUNCHED();
       auto fn = k_os_batched<BB, QQ>;
-      RF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)os_smem<BB>()));
+      constexpr size_t smem = os_tail_smem<BB, QQ, true>();
+      RF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
       int per_sm = 0;
-      RF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, BB / 16, os_smem<BB>()));
+      RF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, BB / 16, smem));
       const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((int64_t)per_sm * c->nsm, units));
-      fn<<<(unsigned)grid, BB / 16, os_smem<BB>(), s>>>(c->batch_items.as<OsItem>() + first,
+      fn<<<(unsigned)grid, BB / 16, smem, s>>>(c->batch_items.as<OsItem>() + first,
                                                         c->batch_order.as<long long>() + c->batch_unit_off[b], units,
                                                         nchunk, tw, n, NQ, NB, SC, keys, W, nw, fastwin, herm,
                                                         counter);
