@@ -11,6 +11,8 @@
 // broadcast tap load per E complex multiply-adds.  Real-form kernels (real taps T = R) take
 // complex x real products: two multiply-adds per tap and output instead of four.
 #include <cfloat>
+#include <cstddef>
+#include <cstdint>
 #include <type_traits>
 
 #include "cplx.cuh"
@@ -217,30 +219,115 @@ void launch_direct(rf_ctx* c, const rf_kernels* kern, const V* z_ref, V* z_out, 
   }
 }
 
-// Window peaks of series already in memory: one block per (window, series).
+// Window peaks of series already in memory: CS blocks per (window, series), one cluster.  Block c
+// reads the c-th part of the window with 16-byte loads and the cluster's first block takes the
+// best of the parts through distributed shared memory, so no workspace is needed (calls on
+// several streams stay independent).  Bound by HBM.  One block per window left most SMs idle when
+// windows are long: 6 series of 2^23 samples in 2^20-sample windows took 464 us on 48 blocks of
+// 256 threads (24 series of 2^20 in 2^17-sample windows: 65 us).
 template <typename V, int NT>
 __global__ void __launch_bounds__(NT) k_winmax_series(const V* __restrict__ z, int64_t n, int64_t W, int64_t nw,
-                                                      float* __restrict__ max_out, int* __restrict__ arg_out) {
+                                                      int CS, float* __restrict__ max_out,
+                                                      int* __restrict__ arg_out) {
   using R = typename real_of<V>::type;
-  const int64_t w = blockIdx.x;
+  constexpr int E = 16 / (int)sizeof(V);  // samples per 16-byte load
+  const int64_t w = blockIdx.x / (unsigned)CS;
+  const int part = (int)(blockIdx.x % (unsigned)CS);
   const int64_t row = blockIdx.y;
   const V* zr = z + row * n;
-  const int64_t lo = w * W, hi = min(n, (w + 1) * W);
+  const int64_t wlo = w * W, whi = min(n, wlo + W);
+  const int64_t per = ((whi - wlo + CS - 1) / CS + E - 1) / E * E;
+  const int64_t lo = min(whi, wlo + part * per), hi = min(whi, lo + per);
   R bv = (R)-1;
   long long bi = 0;
-  for (int64_t i = lo + threadIdx.x; i < hi; i += NT) {
-    const V a = zr[i];
+  auto take = [&](V a, int64_t i) {
     const R v = a.x * a.x + a.y * a.y;
     if (v > bv) {
       bv = v;
       bi = i;
     }
+  };
+  if constexpr (E == 1) {
+    int64_t i = lo + threadIdx.x;
+    for (; i + 3 * NT < hi; i += 4 * NT) {
+      V a[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) a[u] = __ldg(zr + i + u * NT);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) take(a[u], i + u * NT);
+    }
+    for (; i < hi; i += NT) take(zr[i], i);
+  } else {
+    // rows start 16-byte aligned (n even): pairs [2p, 2p + 1] inside [lo, hi), and up to one
+    // sample at each end; every thread meets its samples in increasing order
+    const int64_t p0 = (lo + 1) / 2, p1 = hi / 2;
+    if (threadIdx.x == 0 && (lo & 1) && lo < hi) take(zr[lo], lo);
+    const float4* z4 = reinterpret_cast<const float4*>(zr);
+    auto pair = [&](float4 q, int64_t p) {
+      take(cmake<V>(q.x, q.y), 2 * p);
+      take(cmake<V>(q.z, q.w), 2 * p + 1);
+    };
+    int64_t p = p0 + threadIdx.x;
+    for (; p + 3 * NT < p1; p += 4 * NT) {
+      float4 a[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) a[u] = __ldg(z4 + p + u * NT);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) pair(a[u], p + u * NT);
+    }
+    for (; p < p1; p += NT) pair(__ldg(z4 + p), p);
+    if (threadIdx.x == 0 && (hi & 1) && hi - 1 >= 2 * p0 && lo < hi) take(zr[hi - 1], hi - 1);
   }
-  const Best<R> b = block_best<R, NT>(bv, bi);
-  if (threadIdx.x == 0) {
+  Best<R> b = block_best<R, NT>(bv, bi);
+  if (CS > 1) {
+    __shared__ Best<R> best;
+    if (threadIdx.x == 0) best = b;
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (part == 0 && threadIdx.x == 0) {
+      const uint32_t own = (uint32_t)__cvta_generic_to_shared(&best);
+      for (int c = 1; c < CS; ++c) {
+        uint32_t at;
+        Best<R> o;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(own), "r"(c));
+        if constexpr (sizeof(R) == 8)
+          asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(o.v) : "r"(at) : "memory");
+        else
+          asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(o.v) : "r"(at) : "memory");
+        asm volatile("ld.shared::cluster.s64 %0, [%1];" : "=l"(o.i) : "r"(at + (uint32_t)offsetof(Best<R>, i)) : "memory");
+        if (better(o.v, o.i, b.v, b.i)) b = o;
+      }
+    }
+    // the other blocks' shared memory stays until it has been read
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
+  if (part == 0 && threadIdx.x == 0) {
     max_out[row * nw + w] = (float)b.v;
     arg_out[row * nw + w] = (int)b.i;
   }
+}
+
+template <typename V, int NT>
+void launch_winmax_series(rf_ctx* c, const void* z, int32_t count, int64_t W, int64_t nw, float* max_out,
+                          int32_t* argmax_out, cudaStream_t s) {
+  // Blocks per window (clusters of at most 8): doubled while the launch has fewer than four
+  // blocks per SM and a part keeps 4096 samples (a shorter part's loads no longer cover its
+  // start-up).
+  int CS = 1;
+  while (CS < 8 && nw * count * CS < 4LL * c->nsm && W / (2 * CS) >= 4096) CS *= 2;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(nw * CS), (unsigned)count);
+  cfg.blockDim = dim3(NT);
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)CS;
+  at.val.clusterDim.y = 1;
+  at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = CS > 1 ? 1 : 0;
+  RF_CUDA(cudaLaunchKernelEx(&cfg, k_winmax_series<V, NT>, static_cast<const V*>(z), c->n, W, nw, CS, max_out,
+                             (int*)argmax_out));
+  RF_LAUNCHED();
 }
 
 }  // namespace
@@ -274,12 +361,12 @@ void winmax_series(rf_ctx* c, const void* z, int32_t count, int64_t W, float* ma
   const int64_t n = c->n;
   const int64_t nw = (n + W - 1) / W;
   RF_REQUIRE(nw <= 0x7fffffff && count <= 65535, "winmax: too many windows or series");
-  dim3 grid((unsigned)nw, (unsigned)count);
   if (c->g.dtype == RF_F64)
-    k_winmax_series<double2, 256><<<grid, 256, 0, s>>>(static_cast<const double2*>(z), n, W, nw, max_out, argmax_out);
+    launch_winmax_series<double2, 512>(c, z, count, W, nw, max_out, argmax_out, s);
+  else if (W >= 8192)  // enough samples for 512 threads with four 16-byte loads each in flight
+    launch_winmax_series<float2, 512>(c, z, count, W, nw, max_out, argmax_out, s);
   else
-    k_winmax_series<float2, 256><<<grid, 256, 0, s>>>(static_cast<const float2*>(z), n, W, nw, max_out, argmax_out);
-  RF_LAUNCHED();
+    launch_winmax_series<float2, 256>(c, z, count, W, nw, max_out, argmax_out, s);
 }
 
 }  // namespace rf
