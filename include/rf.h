@@ -124,8 +124,9 @@ uint64_t rf_launch_count(void);
 /* Message of the last failing call on this host thread ("" if none). Borrowed. */
 const char* rf_last_error(void);
 
-/* Create a context for one grid on the current device.  Allocates the FFT twiddle
- * tables and workspaces (about 40 n bytes).  Caller frees with rf_destroy. */
+/* Create a context for one grid on the current device.  Allocates the FFT twiddle and
+ * bin-power tables and workspaces (about 56 n bytes, and up to 100 MB for batches of reference
+ * templates).  Caller frees with rf_destroy. */
 rf_status rf_create(const rf_grid* grid, rf_ctx** out);
 
 /* Release a context and everything it owns.  Waits for the device.  NULL is a no-op. */

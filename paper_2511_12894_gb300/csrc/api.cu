@@ -157,6 +157,7 @@ rf_status rf_create(const rf_grid* grid, rf_ctx** out) {
     c->fa.ensure(esz * n);
     c->fb.ensure(esz * n);
     c->red.ensure(sizeof(double) * 1024);
+    mf_create(c.get());
     c->status.ensure(sizeof(int) * 4);
     RF_CUDA(cudaMemset(c->status.p, 0, sizeof(int) * 4));
     *out = c.release();

@@ -99,33 +99,31 @@ __global__ void k_real_form(double2* __restrict__ rho, int64_t count) {
     rho[i] = make_double2(2.0 * rho[i].x, 0.0);
 }
 
-__global__ void __launch_bounds__(256) k_ref_phase(Tf2 ref, int64_t nbins, double df, double* __restrict__ psi) {
-  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= nbins) return;
-  psi[k] = (k > 0) ? tf2_phase(ref, (double)k * df) : 0.0;
-}
-
-// One row per template (grid.y): K~ over the full length-n buffer.
-__global__ void __launch_bounds__(256) k_kernel_spectrum(const Tf2* __restrict__ tg, const double* __restrict__ dfl,
-                                                         const double* __restrict__ psi_ref, int64_t n, double df,
-                                                         double f_low, double f_high, double df_high,
-                                                         double2* __restrict__ K) {
+// One row per template (grid.y): K~ over the full length-n buffer.  dq: the template's phase minus
+// the reference's (tf2.cuh); [k0, k1]: the bins inside [f_low, f_high], where W = 1.  Bound by the
+// FP64 pipe (two lanes per SM): the phase from the tables of bin powers is about ten multiply-adds
+// a bin.
+//
+// K~ = (N_ref / N_j) W conj(h~_j / h~_ref) (Eq. 5 normalised as in Eq. 3).  Every template of the
+// stationary-phase family has the amplitude law A f^-7/6 on the same band, so h~_j / h~_ref =
+// (A_j / A_ref) e^{-i dPsi} and N_j / N_ref = A_j / A_ref: the two amplitude factors cancel exactly
+// for any scales A, and |K~| = W.
+__global__ void __launch_bounds__(256) k_kernel_spectrum(const Tf2Bins* __restrict__ dq,
+                                                         const double* __restrict__ dfl, int64_t n, double df,
+                                                         int64_t k0, int64_t k1, double f_low, double f_high,
+                                                         double df_high, const double* __restrict__ pw,
+                                                         int64_t stride, double2* __restrict__ K) {
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
   const int j = blockIdx.y;
   double2 out = make_double2(0.0, 0.0);
   if (k > 0 && k <= n / 2) {
-    const double f = (double)k * df;
-    const double w = window_w(f, f_low, f_high, dfl[j], df_high);
-    if (w > 0.0) {
-      const double dpsi = tf2_phase(tg[j], f) - psi_ref[k];
-      // K~ = (N_ref / N_j) W conj(h~_j / h~_ref) (Eq. 5 normalised as in Eq. 3).  Every
-      // template of the stationary-phase family has the amplitude law A f^-7/6 on the same
-      // band, so h~_j / h~_ref = (A_j / A_ref) e^{-i dPsi} and N_j / N_ref = A_j / A_ref: the
-      // two amplitude factors cancel exactly for any scales A, and |K~| = W.
+    const double inv_n = 1.0 / (double)n;  // n a power of two: exact
+    const double a =
+        k >= k0 && k <= k1 ? inv_n : inv_n * window_w((double)k * df, f_low, f_high, dfl[j], df_high);
+    if (a > 0.0) {
       double s, c;
-      sincos(dpsi, &s, &c);
-      const double a = w / (double)n;
+      sincospi(2.0 * tf2_turn(dq[j], k, pw[k], pw[stride + k], pw[2 * stride + k]), &s, &c);
       out = make_double2(a * c, a * s);
     }
   }
@@ -268,13 +266,12 @@ rf_kernels* build_impl(rf_ctx* c, const rf_template& ref, const rf_template* nbr
     return owner.release();
   }
 
-  // device scratch: [Tf2 k][dfl k][extent k][Tf2 k, grid order][dfl k, grid order][psi_ref]
-  // [amax2][m0][len]
-  const int64_t nbins = n / 2 + 1;
+  // device scratch: [Tf2 k][dfl k][extent k][Tf2 k, grid order][dfl k, grid order]
+  // [phase differences][amax2][m0][len]
   const int64_t kmax_chunk = std::min<int64_t>(k, 4096);
   DevBuf meta;
-  const size_t meta_bytes = 2 * sizeof(Tf2) * (size_t)k + sizeof(double) * (3 * (size_t)k + nbins + 8 + kmax_chunk) +
-                            2 * sizeof(int) * (size_t)kmax_chunk + 8192;
+  const size_t meta_bytes = 2 * sizeof(Tf2) * (size_t)k + sizeof(double) * (3 * (size_t)k + 8 + kmax_chunk) +
+                            (sizeof(Tf2Bins) + 2 * sizeof(int)) * (size_t)kmax_chunk + 8192;
   meta.ensure(meta_bytes);
   char* mp = static_cast<char*>(meta.p);
   auto carve = [&](size_t bytes) {
@@ -287,7 +284,7 @@ rf_kernels* build_impl(rf_ctx* c, const rf_template& ref, const rf_template* nbr
   double* d_ext = reinterpret_cast<double*>(carve(sizeof(double) * k));
   Tf2* d_tgs = reinterpret_cast<Tf2*>(carve(sizeof(Tf2) * k));
   double* d_dfls = reinterpret_cast<double*>(carve(sizeof(double) * k));
-  double* d_psi = reinterpret_cast<double*>(carve(sizeof(double) * nbins));
+  Tf2Bins* d_dq = reinterpret_cast<Tf2Bins*>(carve(sizeof(Tf2Bins) * kmax_chunk));
   double* d_amax = reinterpret_cast<double*>(carve(sizeof(double) * kmax_chunk));
   int* d_m0 = reinterpret_cast<int*>(carve(sizeof(int) * kmax_chunk));
   int* d_len = reinterpret_cast<int*>(carve(sizeof(int) * kmax_chunk));
@@ -339,7 +336,7 @@ rf_kernels* build_impl(rf_ctx* c, const rf_template& ref, const rf_template* nbr
   std::vector<int64_t> at_in_part(k);
   std::vector<int> hm0(kmax_chunk), hlen(kmax_chunk);
   DevBuf rows;
-  int64_t psi_grid = 0;
+  std::vector<Tf2Bins> dq;
   for (int q0 = 0; q0 < k;) {
     const int64_t nb = kern->grid[order[q0]];
     // templates per chunk: three complex128 rows of nb per template, about 1.5 GB in total
@@ -349,18 +346,21 @@ rf_kernels* build_impl(rf_ctx* c, const rf_template& ref, const rf_template* nbr
     int cnt = 0;
     while (q0 + cnt < k && cnt < chunk && kern->grid[order[q0 + cnt]] == nb) ++cnt;
     const double dfb = c->g.fs / (double)nb;
-    if (psi_grid != nb) {
-      k_ref_phase<<<(unsigned)((nb / 2 + 1 + 255) / 256), 256, 0, s>>>(pr, nb / 2 + 1, dfb, d_psi);
-      RF_LAUNCHED();
-      psi_grid = nb;
-    }
+    rf_grid gb = c->g;
+    gb.n = nb;
+    int64_t k0, k1;
+    band_bins(gb, &k0, &k1);
+    const Tf2Bins qr = make_tf2_bins(pr, dfb);
+    dq.resize(cnt);  // read by the copy until the chunk's synchronisation below
+    for (int q = 0; q < cnt; ++q) dq[q] = tf2_bins_minus(make_tf2_bins(tg[order[q0 + q]], dfb), qr);
+    RF_CUDA(cudaMemcpyAsync(d_dq, dq.data(), sizeof(Tf2Bins) * cnt, cudaMemcpyHostToDevice, s));
     rows.ensure((size_t)3 * cnt * nb * sizeof(double2));
     double2* bufK = rows.as<double2>();
     double2* bufR = bufK + cnt * nb;
     double2* bufT = bufR + cnt * nb;
     dim3 g1((unsigned)((nb + 255) / 256), (unsigned)cnt);
-    k_kernel_spectrum<<<g1, 256, 0, s>>>(d_tgs + q0, d_dfls + q0, d_psi, nb, dfb, c->g.f_low,
-                                         c->g.f_high, c->g.df_high, bufK);
+    k_kernel_spectrum<<<g1, 256, 0, s>>>(d_dq, d_dfls + q0, nb, dfb, k0, k1, c->g.f_low, c->g.f_high, c->g.df_high,
+                                         c->pw.as<double>(), c->pw_stride, bufK);
     RF_LAUNCHED();
     fft_c2c_f64(bufK, bufR, bufT, nb, cnt, +1, c->tw64.as<double2>(), n, s);
     if (relative & RF_KERNEL_REAL) {

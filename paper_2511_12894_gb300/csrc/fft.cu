@@ -80,6 +80,21 @@ int pass_threads(int64_t work) {
   return nt;
 }
 
+// First pass of a forward transform of real data.
+template <typename V, int R>
+__global__ void __launch_bounds__(256) k_stockham_first_real(const typename real_of<V>::type* __restrict__ x,
+                                                             V* __restrict__ out, int64_t n) {
+  const int64_t nb = n / R;
+  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= nb) return;
+  V a[R];
+#pragma unroll
+  for (int t = 0; t < R; ++t) a[t] = cmake<V>(x[j + t * nb], 0);
+  dft<R, -1>(a);
+#pragma unroll
+  for (int t = 0; t < R; ++t) out[j * R + t] = a[t];
+}
+
 template <typename V, int R>
 void launch_pass(const V* in, V* out, int64_t n, int64_t Ns, int batch, int sign, const V* tw,
                  int64_t tw_stride, cudaStream_t s) {
@@ -96,11 +111,12 @@ void launch_pass(const V* in, V* out, int64_t n, int64_t Ns, int batch, int sign
 
 template <typename V>
 void fft_c2c(const V* in, V* out, V* tmp, int64_t n, int batch, int sign, const V* tw,
-             int64_t table_n, cudaStream_t s, const V* mulF = nullptr, int64_t fstride = 0) {
+             int64_t table_n, cudaStream_t s, const V* mulF = nullptr, int64_t fstride = 0,
+             const typename real_of<V>::type* real_in = nullptr) {
   RF_REQUIRE(n >= 2 && (n & (n - 1)) == 0, "fft: n=%lld is not a power of two", (long long)n);
   RF_REQUIRE(table_n % n == 0, "fft: twiddle table too small");
   RF_REQUIRE(batch >= 1 && batch <= 65535, "fft: batch %d out of range", batch);
-  RF_REQUIRE(in != out && in != tmp && out != tmp, "fft: buffers must be distinct");
+  RF_REQUIRE(((in || real_in) && in != out && in != tmp) && out != tmp, "fft: buffers must be distinct");
   int bits = 0;
   while ((int64_t(1) << bits) < n) ++bits;
   // pass radices in a fixed array (no host allocation per call): n < 2^40 needs at most 10
@@ -117,6 +133,15 @@ void fft_c2c(const V* in, V* out, V* tmp, int64_t n, int batch, int sign, const 
   int64_t Ns = 1;
   for (int p = 0; p < P; ++p) {
     V* dst = ((P - 1 - p) % 2 == 0) ? out : tmp;
+    if (p == 0 && real_in) {
+      RF_REQUIRE(radix[0] == 16 && sign < 0 && batch == 1, "fft: the real pass needs n >= 16, one forward transform");
+      const int nt = pass_threads(n / 16);
+      k_stockham_first_real<V, 16><<<(unsigned)((n / 16 + nt - 1) / nt), nt, 0, s>>>(real_in, dst, n);
+      RF_LAUNCHED();
+      Ns *= radix[p];
+      src = dst;
+      continue;
+    }
     if (p == 0 && mulF) {
       RF_REQUIRE(radix[0] == 16 && sign > 0, "fft: the product pass needs n >= 16 and an inverse transform");
       const int nt = pass_threads(n / 16 * batch);
@@ -136,12 +161,6 @@ void fft_c2c(const V* in, V* out, V* tmp, int64_t n, int batch, int sign, const 
     Ns *= radix[p];
     src = dst;
   }
-}
-
-template <typename T, typename V>
-__global__ void k_real_to_complex(const T* __restrict__ x, V* __restrict__ out, int64_t n) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) out[i] = cmake<V>(x[i], (T)0);
 }
 
 }  // namespace
@@ -166,14 +185,14 @@ void ifft_product_f32(const float2* X, const float2* F, int64_t fstride, float2*
   fft_c2c<float2>(X, out, tmp, n, batch, +1, tw, table_n, s, F, fstride);
 }
 
-void real_to_complex_f64(const double* x, double2* out, int64_t n, cudaStream_t s) {
-  k_real_to_complex<double, double2><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(x, out, n);
-  RF_LAUNCHED();
+void fft_r2c_f64(const double* x, double2* out, double2* tmp, int64_t n, const double2* tw, int64_t table_n,
+                 cudaStream_t s) {
+  fft_c2c<double2>(nullptr, out, tmp, n, 1, -1, tw, table_n, s, nullptr, 0, x);
 }
 
-void real_to_complex_f32(const float* x, float2* out, int64_t n, cudaStream_t s) {
-  k_real_to_complex<float, float2><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(x, out, n);
-  RF_LAUNCHED();
+void fft_r2c_f32(const float* x, float2* out, float2* tmp, int64_t n, const float2* tw, int64_t table_n,
+                 cudaStream_t s) {
+  fft_c2c<float2>(nullptr, out, tmp, n, 1, -1, tw, table_n, s, nullptr, 0, x);
 }
 
 std::vector<double2> host_twiddles(int64_t n) {

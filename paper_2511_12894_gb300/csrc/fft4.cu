@@ -18,8 +18,8 @@
 // w_n^(2^s floor(m / 2^s)), with 2^s = 2^ceil(log2(n) / 2); the tables (about 2 sqrt(n)
 // entries) stay in cache.
 //
-// Modes of pass 1: real input (the data transform), complex input, and the one-sided product
-// X[k] F[k] for k <= n/2, zero above (the matched-filter integrand, formed on load).
+// Modes of pass 1: real input (the data transform) and the one-sided product X[k] F[k] for
+// k <= n/2, zero above (the matched-filter integrand, formed on load).
 #include "blockfft.cuh"
 #include "rf_internal.h"
 
@@ -28,8 +28,7 @@ namespace rf {
 namespace {
 
 constexpr int kF4Real = 0;
-constexpr int kF4Complex = 1;
-constexpr int kF4Product = 2;
+constexpr int kF4Product = 1;
 
 // float2 entries of one line's shared-memory region in a tile of G lines.
 template <int L, int G>
@@ -65,10 +64,6 @@ __global__ void __launch_bounds__(G * L / 16) k_fft4_cols(const void* __restrict
     const float* p = static_cast<const float*>(in) + boff + j0;
 #pragma unroll
     for (int t = 0; t < 16; ++t) v[t] = make_float2(p[t * tstep], 0.f);
-  } else if constexpr (MODE == kF4Complex) {
-    const float2* p = static_cast<const float2*>(in) + boff + j0;
-#pragma unroll
-    for (int t = 0; t < 16; ++t) v[t] = p[t * tstep];
   } else {
     // X is one spectrum shared by the batch; F holds one filter of n/2 + 1 values per row.
     // Rows a > N1/2 lie above n/2 (zero); row N1/2 holds only column 0.
@@ -233,14 +228,6 @@ void fft4_forward_real(const rf_ctx* c, const float* x, float2* out, float2* tmp
   split(c->n, n1log, n2log);
   cols_dispatch<kF4Real, -1>(n1log, x, nullptr, 0, tmp, n2log, 1, c, s);
   rows_dispatch<-1>(n2log, tmp, out, n1log, 1, c, s);
-}
-
-void fft4_inverse(const rf_ctx* c, const float2* in, float2* out, float2* tmp, int batch, cudaStream_t s) {
-  check(c, in, out, tmp, batch);
-  int n1log, n2log;
-  split(c->n, n1log, n2log);
-  cols_dispatch<kF4Complex, +1>(n1log, in, nullptr, 0, tmp, n2log, batch, c, s);
-  rows_dispatch<+1>(n2log, tmp, out, n1log, batch, c, s);
 }
 
 void fft4_inverse_product(const rf_ctx* c, const float2* X, const float2* F, int64_t fstride, float2* out,

@@ -45,12 +45,339 @@ Tf2 make_tf2(const rf_template& t, int pn_order) {
   return p;
 }
 
+// The bins of the band: the k with f_low <= k df <= f_high, as compared in FP64 (k >= 1).
+void band_bins(const rf_grid& g, int64_t* k0, int64_t* k1) {
+  const double df = g.fs / (double)g.n;
+  int64_t a = (int64_t)std::ceil(g.f_low / df), b = (int64_t)std::floor(g.f_high / df);
+  while (a > 1 && (double)(a - 1) * df >= g.f_low) --a;
+  while ((double)a * df < g.f_low) ++a;
+  while ((double)(b + 1) * df <= g.f_high) ++b;
+  while (b > 0 && (double)b * df > g.f_high) --b;
+  *k0 = std::max<int64_t>(1, a);
+  *k1 = std::min<int64_t>(g.n / 2, b);
+}
+
 namespace {
 
 constexpr int kRedThreads = 256;
 constexpr int kRedBlocks = 512;
 // complex values of the four-step inverse transforms launched together (their intermediate)
 constexpr int64_t kF4Chunk = int64_t(1) << 23;
+
+// Tables of powers of the bin index k = 0..n/2 (rows of `stride`): k^(1/3), k^(-5/3), ln(k)/3 and
+// k^(-7/6), 0 at k = 0.  The cube root is corrected by its exact residual, so the first two are good
+// to about half an ulp.
+__global__ void __launch_bounds__(256) k_bin_powers(int64_t nbins, int64_t stride, double* __restrict__ pw) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= nbins) return;
+  double u = 0.0, u5 = 0.0, lu = 0.0, ua = 0.0;
+  if (i > 0) {
+    const double k = (double)i;
+    const double r = rcbrt(k);
+    // e = 1 - k r^3 from r^2 = r2 + r2l and r^3 = r3 + r3l (exact products): k^(-1/3) = r (1 + e / 3)
+    const double r2 = r * r, r2l = fma(r, r, -r2);
+    const double r3 = r2 * r, r3l = fma(r2, r, -r3) + r2l * r;
+    const double kr = k * r3;
+    const double e = (1.0 - kr) - (fma(k, r3, -kr) + k * r3l);
+    const double c2 = r2l + r2 * (2.0 / 3.0) * e;  // k^(-2/3) = r2 + c2
+    u = k * r2;
+    u += fma(k, r2, -u) + k * c2;
+    u5 = r2 / k;
+    u5 += (fma(-u5, k, r2) + c2) / k;
+    lu = log(k) / 3.0;
+    ua = rsqrt(k) * (r2 + c2);
+  }
+  pw[i] = u;
+  pw[stride + i] = u5;
+  pw[2 * stride + i] = lu;
+  pw[3 * stride + i] = ua;
+}
+
+// Partial sums of 4 df B(f_k)^2 inv_psd[k] over the bins k0..k1 of the band, one partial per
+// block; ua[k] = k^(-7/6), amp2 = 4 df df^(-7/3).
+__global__ void __launch_bounds__(kRedThreads) k_sigma2_bins(const double* __restrict__ ip,
+                                                             const double* __restrict__ ua, int64_t k0, int64_t k1,
+                                                             double amp2, double* __restrict__ part) {
+  double acc = 0.0;
+  for (int64_t k = k0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k <= k1;
+       k += (int64_t)gridDim.x * blockDim.x)
+    acc = fma(ua[k] * ua[k], ip[k], acc);
+  __shared__ double sh[kRedThreads];
+  sh[threadIdx.x] = acc;
+  __syncthreads();
+  for (int s = kRedThreads / 2; s > 0; s >>= 1) {
+    if ((int)threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) part[blockIdx.x] = amp2 * sh[0];
+}
+
+// out[0] = sigma^2, out[1] = the filter scale 4 / (n sqrt(sigma^2)) df^(-7/6); sigma to `nref`
+// places of sigma_out (every template of the unit-amplitude family has the same N).
+__global__ void k_sigma2_finish(const double* __restrict__ part, int count, double n, double amp,
+                                double* __restrict__ out, double* __restrict__ sigma_out, int nref) {
+  __shared__ double sh[kRedThreads];
+  double acc = 0.0;
+  for (int i = threadIdx.x; i < count; i += blockDim.x) acc += part[i];
+  sh[threadIdx.x] = acc;
+  __syncthreads();
+  for (int s = kRedThreads / 2; s > 0; s >>= 1) {
+    if ((int)threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
+    __syncthreads();
+  }
+  const double sg = sqrt(sh[0]);
+  if (threadIdx.x == 0) {
+    out[0] = sh[0];
+    out[1] = 4.0 / (n * sg) * amp;
+  }
+  if (sigma_out)
+    for (int r = threadIdx.x; r < nref; r += blockDim.x) sigma_out[r] = sg;
+}
+
+constexpr int kFiltRefs = 8;  // references of one filter launch (their coefficients are arguments)
+struct FiltRefs {
+  Tf2Bins q[kFiltRefs];
+};
+
+// Filters F_r[k] = (4 / (n N)) conj(h~_r,k) inv_psd[k], k = 0..n/2, of `cnt` references; 0 outside
+// the bins k0..k1 of the band.  With X the unnormalised DFT of the data, X[k] F_r[k] is the
+// integrand of Eq. 2 (4 df dt = 4 / n).  One thread per bin: the tables and inv_psd are read once
+// for all references.  PREC: phase, amplitude and product in FP64, rounded once (stored filters);
+// else (FP32 grids, filters made and used within one call) the FP64 phase is reduced to a
+// fraction of a turn before the FP32 sine and cosine.
+template <typename V, bool PREC>
+__global__ void __launch_bounds__(256) k_ref_filters(const double* __restrict__ ip, const double* __restrict__ pw,
+                                                     int64_t stride, const double* __restrict__ sig, FiltRefs refs,
+                                                     int cnt, int64_t nbins, int64_t k0, int64_t k1,
+                                                     V* __restrict__ F, int64_t fstride) {
+  using R = typename real_of<V>::type;
+  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= nbins) return;
+  if (k < k0 || k > k1) {
+    for (int r = 0; r < cnt; ++r) F[r * fstride + k] = cmake<V>((R)0, (R)0);
+    return;
+  }
+  const double u = pw[k], u5 = pw[stride + k], lu = pw[2 * stride + k];
+  const double a = sig[1] * pw[3 * stride + k] * ip[k];
+  for (int r = 0; r < cnt; ++r) {
+    const double t = tf2_turn(refs.q[r], k, u, u5, lu);
+    if constexpr (PREC) {
+      double s, c;
+      sincospi(2.0 * t, &s, &c);
+      F[r * fstride + k] = cmake<V>((R)(a * c), (R)(a * s));  // conj(h~) = B exp(+i Psi)
+    } else {
+      float s, c;
+      sincospif(2.0f * (float)t, &s, &c);
+      F[r * fstride + k] = cmake<V>((R)a * c, (R)a * s);
+    }
+  }
+}
+
+template <typename V>
+__global__ void __launch_bounds__(256) k_template_fd(Tf2Bins q, const double* __restrict__ pw, int64_t stride,
+                                                     double amp, int64_t nbins, V* __restrict__ h) {
+  using R = typename real_of<V>::type;
+  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= nbins) return;
+  V out = cmake<V>((R)0, (R)0);
+  if (k > 0) {
+    double s, c;
+    sincospi(2.0 * tf2_turn(q, k, pw[k], pw[stride + k], pw[2 * stride + k]), &s, &c);
+    const double a = amp * pw[3 * stride + k];
+    out = cmake<V>((R)(a * c), (R)(-a * s));
+  }
+  h[k] = out;
+}
+
+// df^(-7/6)
+double amp_scale(double df) { return 1.0 / (df * std::cbrt(std::sqrt(df))); }
+
+// sigma^2 and the filter scale into c->red (after the partials), sigma to sigma_out[nref] (or null)
+double* launch_sigma2(rf_ctx* c, const double* inv_psd, double* sigma_out, int nref, cudaStream_t s) {
+  const double df = c->g.fs / (double)c->n;
+  int64_t k0, k1;
+  band_bins(c->g, &k0, &k1);
+  const double amp = amp_scale(df);
+  double* part = c->red.as<double>();
+  double* sig = part + kRedBlocks;
+  const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(kRedBlocks, (k1 - k0 + 1) / (2 * kRedThreads)));
+  k_sigma2_bins<<<blocks, kRedThreads, 0, s>>>(inv_psd, c->pw.as<double>() + 3 * c->pw_stride, k0, k1,
+                                               4.0 * df * amp * amp, part);
+  RF_LAUNCHED();
+  k_sigma2_finish<<<1, kRedThreads, 0, s>>>(part, blocks, (double)c->n, amp, sig, sigma_out, nref);
+  RF_LAUNCHED();
+  return sig;
+}
+
+template <typename V, bool PREC>
+void launch_filters(rf_ctx* c, const double* inv_psd, const double* sig, int cnt, const rf_template* refs, V* F,
+                    int64_t fstride, cudaStream_t s) {
+  const int64_t nbins = c->n / 2 + 1;
+  const double df = c->g.fs / (double)c->n;
+  int64_t k0, k1;
+  band_bins(c->g, &k0, &k1);
+  for (int r0 = 0; r0 < cnt; r0 += kFiltRefs) {
+    const int m = std::min(kFiltRefs, cnt - r0);
+    FiltRefs fr{};
+    for (int r = 0; r < m; ++r) fr.q[r] = make_tf2_bins(make_tf2(refs[r0 + r], c->g.pn_order), df);
+    k_ref_filters<V, PREC><<<(unsigned)((nbins + 255) / 256), 256, 0, s>>>(
+        inv_psd, c->pw.as<double>(), c->pw_stride, sig, fr, m, nbins, k0, k1, F + (int64_t)r0 * fstride, fstride);
+    RF_LAUNCHED();
+  }
+}
+
+}  // namespace
+
+void mf_create(rf_ctx* c) {
+  const int64_t nbins = c->n / 2 + 1;
+  c->pw_stride = (nbins + 15) & ~(int64_t)15;
+  c->pw.ensure(sizeof(double) * 4 * (size_t)c->pw_stride);
+  k_bin_powers<<<(unsigned)((nbins + 255) / 256), 256>>>(nbins, c->pw_stride, c->pw.as<double>());
+  RF_LAUNCHED();
+  RF_CUDA(cudaStreamSynchronize(nullptr));
+  // up to 8 references, 2^22 intermediate values in all (above that one reference fills the GPU)
+  c->mf_batch = (int)std::max<int64_t>(1, std::min<int64_t>(8, ((int64_t)1 << 22) / c->n));
+  const size_t esz = c->g.dtype == RF_F64 ? sizeof(double2) : sizeof(float2);
+  if (c->mf_batch > 1) c->mf_ref.ensure(esz * (size_t)c->mf_batch * (size_t)(c->n + nbins + 15));
+}
+
+namespace {
+
+// Filters of a batch, then one product inverse for the batch.
+template <typename V, typename Inverse>
+void mf_batches(rf_ctx* c, const double* inv_psd, const double* sig, int32_t nref, const rf_template* refs,
+                V* z_out, Inverse&& inverse, cudaStream_t s) {
+  constexpr bool PREC = sizeof(V) == sizeof(double2);
+  const int64_t n = c->n, nbins = n / 2 + 1;
+  const int64_t fstride = (nbins + 1) & ~(int64_t)1;
+  const int batch = std::min<int>(c->mf_batch, nref);
+  V* tmp = batch > 1 ? c->mf_ref.as<V>() : c->fb.as<V>();
+  V* F = batch > 1 ? tmp + (int64_t)c->mf_batch * n : c->fa.as<V>();
+  for (int r0 = 0; r0 < nref; r0 += batch) {
+    const int cnt = std::min(batch, nref - r0);
+    launch_filters<V, PREC>(c, inv_psd, sig, cnt, refs + r0, F, fstride, s);
+    inverse(F, fstride, z_out + (int64_t)r0 * n, tmp, cnt);
+  }
+}
+
+}  // namespace
+
+void mf_reference_impl(rf_ctx* c, const void* x, const double* inv_psd, int32_t nref, const rf_template* refs,
+                       void* z_out, double* sigma_out, cudaStream_t s) {
+  const int64_t n = c->n;
+  const double* sig = launch_sigma2(c, inv_psd, sigma_out, nref, s);
+  if (c->g.dtype == RF_F64) {
+    const double2* tw = c->tw64.as<double2>();
+    fft_r2c_f64(static_cast<const double*>(x), c->xf.as<double2>(), c->fb.as<double2>(), n, tw, n, s);
+    mf_batches(c, inv_psd, sig, nref, refs, static_cast<double2*>(z_out),
+               [&](const double2* F, int64_t fs, double2* z, double2* tmp, int cnt) {
+                 ifft_product_f64(c->xf.as<double2>(), F, fs, z, tmp, n, cnt, tw, n, s);
+               }, s);
+  } else if (fft4_supported(n)) {  // two-pass four-step transforms, else radix passes
+    fft4_forward_real(c, static_cast<const float*>(x), c->xf.as<float2>(), c->fb.as<float2>(), s);
+    mf_batches(c, inv_psd, sig, nref, refs, static_cast<float2*>(z_out),
+               [&](const float2* F, int64_t fs, float2* z, float2* tmp, int cnt) {
+                 fft4_inverse_product(c, c->xf.as<float2>(), F, fs, z, tmp, cnt, s);
+               }, s);
+  } else {
+    const float2* tw = c->tw32.as<float2>();
+    fft_r2c_f32(static_cast<const float*>(x), c->xf.as<float2>(), c->fb.as<float2>(), n, tw, n, s);
+    mf_batches(c, inv_psd, sig, nref, refs, static_cast<float2*>(z_out),
+               [&](const float2* F, int64_t fs, float2* z, float2* tmp, int cnt) {
+                 ifft_product_f32(c->xf.as<float2>(), F, fs, z, tmp, n, cnt, tw, n, s);
+               }, s);
+  }
+}
+
+void reference_filters_impl(rf_ctx* c, const double* inv_psd, int32_t nref, const rf_template* refs, void* filt,
+                            double* sigma_out, cudaStream_t s) {
+  const int64_t nb = c->n / 2 + 1;
+  const double* sig = launch_sigma2(c, inv_psd, sigma_out, nref, s);
+  if (c->g.dtype == RF_F64)
+    launch_filters<double2, true>(c, inv_psd, sig, nref, refs, static_cast<double2*>(filt), nb, s);
+  else
+    launch_filters<float2, true>(c, inv_psd, sig, nref, refs, static_cast<float2*>(filt), nb, s);
+}
+
+void mf_filtered_impl(rf_ctx* c, const void* x, int32_t nref, const void* filt, void* z_out, cudaStream_t s) {
+  const int64_t n = c->n;
+  const int64_t nb = n / 2 + 1;
+  // references per batched inverse transform, bounded by the temporary buffer
+  const int chunk = (int)std::max<int64_t>(1, std::min<int64_t>(nref, std::min<int64_t>(65535, (int64_t)(1 << 27) / n)));
+  if (c->g.dtype == RF_F64) {
+    c->mf_tmp.ensure(sizeof(double2) * (size_t)chunk * n);
+    fft_r2c_f64(static_cast<const double*>(x), c->xf.as<double2>(), c->fb.as<double2>(), n, c->tw64.as<double2>(), n,
+                s);
+    for (int r0 = 0; r0 < nref; r0 += chunk) {
+      const int cnt = std::min(chunk, nref - r0);
+      ifft_product_f64(c->xf.as<double2>(), static_cast<const double2*>(filt) + (int64_t)r0 * nb, nb,
+                       static_cast<double2*>(z_out) + (int64_t)r0 * n, c->mf_tmp.as<double2>(), n, cnt,
+                       c->tw64.as<double2>(), n, s);
+    }
+  } else if (fft4_supported(n)) {
+    // two-pass four-step transforms; the inverses of kF4Chunk references share one launch pair,
+    // whose intermediate (kF4Chunk n complex values) is meant to stay in L2
+    const int c4 = (int)std::min<int64_t>(nref, std::max<int64_t>(1, kF4Chunk / n));
+    c->mf_tmp.ensure(sizeof(float2) * (size_t)c4 * n);
+    fft4_forward_real(c, static_cast<const float*>(x), c->xf.as<float2>(), c->mf_tmp.as<float2>(), s);
+    for (int r0 = 0; r0 < nref; r0 += c4) {
+      const int cnt = std::min(c4, nref - r0);
+      fft4_inverse_product(c, c->xf.as<float2>(), static_cast<const float2*>(filt) + (int64_t)r0 * nb, nb,
+                           static_cast<float2*>(z_out) + (int64_t)r0 * n, c->mf_tmp.as<float2>(), cnt, s);
+    }
+  } else {
+    c->mf_tmp.ensure(sizeof(float2) * (size_t)chunk * n);
+    fft_r2c_f32(static_cast<const float*>(x), c->xf.as<float2>(), c->fb.as<float2>(), n, c->tw32.as<float2>(), n, s);
+    for (int r0 = 0; r0 < nref; r0 += chunk) {
+      const int cnt = std::min(chunk, nref - r0);
+      ifft_product_f32(c->xf.as<float2>(), static_cast<const float2*>(filt) + (int64_t)r0 * nb, nb,
+                       static_cast<float2*>(z_out) + (int64_t)r0 * n, c->mf_tmp.as<float2>(), n, cnt,
+                       c->tw32.as<float2>(), n, s);
+    }
+  }
+}
+
+void template_fd_impl(rf_ctx* c, const rf_template& t, void* h_out, cudaStream_t s) {
+  const int64_t nbins = c->n / 2 + 1;
+  const double df = c->g.fs / (double)c->n;
+  const Tf2Bins q = make_tf2_bins(make_tf2(t, c->g.pn_order), df);
+  const unsigned grid = (unsigned)((nbins + 255) / 256);
+  if (c->g.dtype == RF_F64)
+    k_template_fd<double2><<<grid, 256, 0, s>>>(q, c->pw.as<double>(), c->pw_stride, amp_scale(df), nbins,
+                                                static_cast<double2*>(h_out));
+  else
+    k_template_fd<float2><<<grid, 256, 0, s>>>(q, c->pw.as<double>(), c->pw_stride, amp_scale(df), nbins,
+                                               static_cast<float2*>(h_out));
+  RF_LAUNCHED();
+}
+
+// ---------------------------------------------------------------- allocation-free variant
+// rf_mf_reference_noalloc: the reference matched filter for callers that may not
+// allocate device memory.  Its workspace is the file-scope array below (about
+// 4 MiB, reserved in every GPU that loads the library, until the process exits).
+
+namespace {
+
+constexpr int64_t kNoAllocMaxN = int64_t(1) << 16;
+constexpr size_t kNoAllocSlot = (size_t)kNoAllocMaxN * sizeof(double2);  // one complex128 row of kNoAllocMaxN
+constexpr size_t kNoAllocRed = 8192;                                      // FP64 partial sums + sigma^2
+constexpr size_t kNoAllocBytes = 4 * kNoAllocSlot + kNoAllocRed;
+// The array has its own device address in every CUDA context that loads the module (the
+// runtime's primary context of each device, or a context a host application created with
+// the driver API), so the addresses are remembered per context, keyed by the context's
+// process-unique ID (a handle value can be reused by a later context; the ID is not).
+constexpr int kNoAllocCacheSlots = 64;
+struct NoAllocSlot {
+  unsigned long long ctx_id;
+  void* addr;
+};
+std::mutex g_noalloc_mu;
+NoAllocSlot g_noalloc_cache[kNoAllocCacheSlots] = {};
+int g_noalloc_used = 0;
+int g_noalloc_next = 0;
+
+// The allocation-free form has no room for tables of bin powers and evaluates the template at
+// every bin.
 
 // Partial sums of 4 df B(f_k)^2 inv_psd[k] over the band, one partial per block.
 __global__ void __launch_bounds__(kRedThreads) k_sigma2_partial(const double* __restrict__ ip, int64_t nbins,
@@ -118,214 +445,6 @@ __global__ void __launch_bounds__(256) k_mf_pointwise(const V* __restrict__ X, c
   }
   Z[k] = out;
 }
-
-// Stored reference filter: F[k] = (4 / (n N)) conj(h~_k) inv_psd[k] on the band, 0 elsewhere,
-// k = 0..n/2, phase and scale in FP64 and rounded once.  With X the unnormalised DFT of the
-// data, X[k] F[k] is the integrand of Eq. 2 (4 df dt = 4 / n).
-template <typename V>
-__global__ void __launch_bounds__(256) k_ref_filter(const double* __restrict__ ip, const double* __restrict__ sigma2,
-                                                    Tf2 p, int64_t n, double df, double f_low, double f_high,
-                                                    V* __restrict__ F, double* __restrict__ sigma_out) {
-  using R = typename real_of<V>::type;
-  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k == 0 && sigma_out) sigma_out[0] = sqrt(sigma2[0]);
-  if (k > n / 2) return;
-  const double f = (double)k * df;
-  V out = cmake<V>((R)0, (R)0);
-  if (k > 0 && f >= f_low && f <= f_high) {
-    double sn, cs;
-    sincos(tf2_phase(p, f), &sn, &cs);
-    const double a = 4.0 / ((double)n * sqrt(sigma2[0])) * tf2_amp(f) * ip[k];
-    out = cmake<V>((R)(a * cs), (R)(a * sn));  // conj(h~) = B exp(+i Psi)
-  }
-  F[k] = out;
-}
-
-template <typename V>
-__global__ void __launch_bounds__(256) k_template_fd(Tf2 p, int64_t nbins, double df, V* __restrict__ h) {
-  using R = typename real_of<V>::type;
-  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= nbins) return;
-  V out = cmake<V>((R)0, (R)0);
-  if (k > 0) {
-    const double f = (double)k * df;
-    const double psi = tf2_phase(p, f);
-    double s, c;
-    sincos(psi, &s, &c);
-    const double a = tf2_amp(f);
-    out = cmake<V>((R)(a * c), (R)(-a * s));
-  }
-  h[k] = out;
-}
-
-}  // namespace
-
-void sigma2_impl(rf_ctx* c, const double* inv_psd, int count, double* out, cudaStream_t s) {
-  const int64_t nbins = c->n / 2 + 1;
-  c->red.ensure(sizeof(double) * kRedBlocks);
-  double* part = c->red.as<double>();
-  const double df = c->g.fs / (double)c->n;
-  k_sigma2_partial<<<kRedBlocks, kRedThreads, 0, s>>>(inv_psd, nbins, df, c->g.f_low, c->g.f_high, part);
-  RF_LAUNCHED();
-  for (int i = 0; i < count; ++i) {
-    k_sum_partials<<<1, kRedThreads, 0, s>>>(part, kRedBlocks, out + i);
-    RF_LAUNCHED();
-  }
-}
-
-void mf_reference_impl(rf_ctx* c, const void* x, const double* inv_psd, int32_t nref, const rf_template* refs,
-                       void* z_out, double* sigma_out, cudaStream_t s) {
-  const int64_t n = c->n;
-  const double df = c->g.fs / (double)n;
-  // sigma^2 is the same for every template of the unit-amplitude family (B = f^-7/6);
-  // it is computed once per call in FP64 (Eq. 3) and kept after the partials.
-  c->red.ensure(sizeof(double) * (kRedBlocks + 8));
-  double* sig2 = c->red.as<double>() + kRedBlocks;
-  {
-    const int64_t nbins = n / 2 + 1;
-    k_sigma2_partial<<<kRedBlocks, kRedThreads, 0, s>>>(inv_psd, nbins, df, c->g.f_low, c->g.f_high,
-                                                       c->red.as<double>());
-    RF_LAUNCHED();
-    k_sum_partials<<<1, kRedThreads, 0, s>>>(c->red.as<double>(), kRedBlocks, sig2);
-    RF_LAUNCHED();
-  }
-  const unsigned grid = (unsigned)((n + 255) / 256);
-  if (c->g.dtype == RF_F64) {
-    real_to_complex_f64(static_cast<const double*>(x), c->fa.as<double2>(), n, s);
-    fft_c2c_f64(c->fa.as<double2>(), c->xf.as<double2>(), c->fb.as<double2>(), n, 1, -1, c->tw64.as<double2>(), n,
-                s);
-    for (int r = 0; r < nref; ++r) {
-      const Tf2 p = make_tf2(refs[r], c->g.pn_order);
-      k_mf_pointwise<double2><<<grid, 256, 0, s>>>(c->xf.as<double2>(), inv_psd, sig2, p, n, df, c->g.f_low,
-                                                   c->g.f_high, c->fa.as<double2>(), sigma_out ? sigma_out + r : nullptr);
-      RF_LAUNCHED();
-      fft_c2c_f64(c->fa.as<double2>(), static_cast<double2*>(z_out) + (int64_t)r * n, c->fb.as<double2>(), n, 1,
-                  +1, c->tw64.as<double2>(), n, s);
-    }
-  } else {
-    const bool four = fft4_supported(n);  // two-pass four-step transforms, else radix passes
-    if (four) {
-      fft4_forward_real(c, static_cast<const float*>(x), c->xf.as<float2>(), c->fb.as<float2>(), s);
-    } else {
-      real_to_complex_f32(static_cast<const float*>(x), c->fa.as<float2>(), n, s);
-      fft_c2c_f32(c->fa.as<float2>(), c->xf.as<float2>(), c->fb.as<float2>(), n, 1, -1, c->tw32.as<float2>(), n,
-                  s);
-    }
-    for (int r = 0; r < nref; ++r) {
-      const Tf2 p = make_tf2(refs[r], c->g.pn_order);
-      k_mf_pointwise<float2><<<grid, 256, 0, s>>>(c->xf.as<float2>(), inv_psd, sig2, p, n, df, c->g.f_low,
-                                                  c->g.f_high, c->fa.as<float2>(), sigma_out ? sigma_out + r : nullptr);
-      RF_LAUNCHED();
-      float2* zr = static_cast<float2*>(z_out) + (int64_t)r * n;
-      if (four)
-        fft4_inverse(c, c->fa.as<float2>(), zr, c->fb.as<float2>(), 1, s);
-      else
-        fft_c2c_f32(c->fa.as<float2>(), zr, c->fb.as<float2>(), n, 1, +1, c->tw32.as<float2>(), n, s);
-    }
-  }
-}
-
-void reference_filters_impl(rf_ctx* c, const double* inv_psd, int32_t nref, const rf_template* refs, void* filt,
-                            double* sigma_out, cudaStream_t s) {
-  const int64_t n = c->n;
-  const int64_t nb = n / 2 + 1;
-  const double df = c->g.fs / (double)n;
-  c->red.ensure(sizeof(double) * (kRedBlocks + 8));
-  double* sig2 = c->red.as<double>() + kRedBlocks;
-  k_sigma2_partial<<<kRedBlocks, kRedThreads, 0, s>>>(inv_psd, nb, df, c->g.f_low, c->g.f_high, c->red.as<double>());
-  RF_LAUNCHED();
-  k_sum_partials<<<1, kRedThreads, 0, s>>>(c->red.as<double>(), kRedBlocks, sig2);
-  RF_LAUNCHED();
-  const unsigned grid = (unsigned)((nb + 255) / 256);
-  for (int r = 0; r < nref; ++r) {
-    const Tf2 p = make_tf2(refs[r], c->g.pn_order);
-    double* so = sigma_out ? sigma_out + r : nullptr;
-    if (c->g.dtype == RF_F64)
-      k_ref_filter<double2><<<grid, 256, 0, s>>>(inv_psd, sig2, p, n, df, c->g.f_low, c->g.f_high,
-                                                 static_cast<double2*>(filt) + (int64_t)r * nb, so);
-    else
-      k_ref_filter<float2><<<grid, 256, 0, s>>>(inv_psd, sig2, p, n, df, c->g.f_low, c->g.f_high,
-                                                static_cast<float2*>(filt) + (int64_t)r * nb, so);
-    RF_LAUNCHED();
-  }
-}
-
-void mf_filtered_impl(rf_ctx* c, const void* x, int32_t nref, const void* filt, void* z_out, cudaStream_t s) {
-  const int64_t n = c->n;
-  const int64_t nb = n / 2 + 1;
-  // references per batched inverse transform, bounded by the temporary buffer
-  const int chunk = (int)std::max<int64_t>(1, std::min<int64_t>(nref, std::min<int64_t>(65535, (int64_t)(1 << 27) / n)));
-  if (c->g.dtype == RF_F64) {
-    c->mf_tmp.ensure(sizeof(double2) * (size_t)chunk * n);
-    real_to_complex_f64(static_cast<const double*>(x), c->fa.as<double2>(), n, s);
-    fft_c2c_f64(c->fa.as<double2>(), c->xf.as<double2>(), c->fb.as<double2>(), n, 1, -1, c->tw64.as<double2>(), n,
-                s);
-    for (int r0 = 0; r0 < nref; r0 += chunk) {
-      const int cnt = std::min(chunk, nref - r0);
-      ifft_product_f64(c->xf.as<double2>(), static_cast<const double2*>(filt) + (int64_t)r0 * nb, nb,
-                       static_cast<double2*>(z_out) + (int64_t)r0 * n, c->mf_tmp.as<double2>(), n, cnt,
-                       c->tw64.as<double2>(), n, s);
-    }
-  } else if (fft4_supported(n)) {
-    // two-pass four-step transforms; the inverses of kF4Chunk references share one launch pair,
-    // whose intermediate (kF4Chunk n complex values) is meant to stay in L2
-    const int c4 = (int)std::min<int64_t>(nref, std::max<int64_t>(1, kF4Chunk / n));
-    c->mf_tmp.ensure(sizeof(float2) * (size_t)c4 * n);
-    fft4_forward_real(c, static_cast<const float*>(x), c->xf.as<float2>(), c->mf_tmp.as<float2>(), s);
-    for (int r0 = 0; r0 < nref; r0 += c4) {
-      const int cnt = std::min(c4, nref - r0);
-      fft4_inverse_product(c, c->xf.as<float2>(), static_cast<const float2*>(filt) + (int64_t)r0 * nb, nb,
-                           static_cast<float2*>(z_out) + (int64_t)r0 * n, c->mf_tmp.as<float2>(), cnt, s);
-    }
-  } else {
-    c->mf_tmp.ensure(sizeof(float2) * (size_t)chunk * n);
-    real_to_complex_f32(static_cast<const float*>(x), c->fa.as<float2>(), n, s);
-    fft_c2c_f32(c->fa.as<float2>(), c->xf.as<float2>(), c->fb.as<float2>(), n, 1, -1, c->tw32.as<float2>(), n, s);
-    for (int r0 = 0; r0 < nref; r0 += chunk) {
-      const int cnt = std::min(chunk, nref - r0);
-      ifft_product_f32(c->xf.as<float2>(), static_cast<const float2*>(filt) + (int64_t)r0 * nb, nb,
-                       static_cast<float2*>(z_out) + (int64_t)r0 * n, c->mf_tmp.as<float2>(), n, cnt,
-                       c->tw32.as<float2>(), n, s);
-    }
-  }
-}
-
-void template_fd_impl(rf_ctx* c, const rf_template& t, void* h_out, cudaStream_t s) {
-  const int64_t nbins = c->n / 2 + 1;
-  const double df = c->g.fs / (double)c->n;
-  const Tf2 p = make_tf2(t, c->g.pn_order);
-  const unsigned grid = (unsigned)((nbins + 255) / 256);
-  if (c->g.dtype == RF_F64)
-    k_template_fd<double2><<<grid, 256, 0, s>>>(p, nbins, df, static_cast<double2*>(h_out));
-  else
-    k_template_fd<float2><<<grid, 256, 0, s>>>(p, nbins, df, static_cast<float2*>(h_out));
-  RF_LAUNCHED();
-}
-
-// ---------------------------------------------------------------- allocation-free variant
-// rf_mf_reference_noalloc: the reference matched filter for callers that may not
-// allocate device memory.  Its workspace is the file-scope array below (about
-// 4 MiB, reserved in every GPU that loads the library, until the process exits).
-
-namespace {
-
-constexpr int64_t kNoAllocMaxN = int64_t(1) << 16;
-constexpr size_t kNoAllocSlot = (size_t)kNoAllocMaxN * sizeof(double2);  // one complex128 row of kNoAllocMaxN
-constexpr size_t kNoAllocRed = 8192;                                      // FP64 partial sums + sigma^2
-constexpr size_t kNoAllocBytes = 4 * kNoAllocSlot + kNoAllocRed;
-// The array has its own device address in every CUDA context that loads the module (the
-// runtime's primary context of each device, or a context a host application created with
-// the driver API), so the addresses are remembered per context, keyed by the context's
-// process-unique ID (a handle value can be reused by a later context; the ID is not).
-constexpr int kNoAllocCacheSlots = 64;
-struct NoAllocSlot {
-  unsigned long long ctx_id;
-  void* addr;
-};
-std::mutex g_noalloc_mu;
-NoAllocSlot g_noalloc_cache[kNoAllocCacheSlots] = {};
-int g_noalloc_used = 0;
-int g_noalloc_next = 0;
 
 // exp(-2 pi i m / n), m < n, into the workspace (rebuilt on every call).
 template <typename V>
@@ -483,8 +602,7 @@ void mf_reference_noalloc_impl(const rf_grid& g, const void* x, const double* in
   if (g.dtype == RF_F64) {
     k_noalloc_twiddles<double2><<<grid, 256, 0, s>>>(static_cast<double2*>(tw), n);
     RF_LAUNCHED();
-    real_to_complex_f64(static_cast<const double*>(x), static_cast<double2*>(fa), n, s);
-    fft_c2c_f64(static_cast<double2*>(fa), static_cast<double2*>(xf), static_cast<double2*>(fb), n, 1, -1,
+    fft_r2c_f64(static_cast<const double*>(x), static_cast<double2*>(xf), static_cast<double2*>(fb), n,
                 static_cast<double2*>(tw), n, s);
     k_mf_pointwise<double2><<<grid, 256, 0, s>>>(static_cast<double2*>(xf), inv_psd, sig2, p, n, df, g.f_low,
                                                  g.f_high, static_cast<double2*>(fa), sigma_out);
@@ -494,8 +612,7 @@ void mf_reference_noalloc_impl(const rf_grid& g, const void* x, const double* in
   } else {
     k_noalloc_twiddles<float2><<<grid, 256, 0, s>>>(static_cast<float2*>(tw), n);
     RF_LAUNCHED();
-    real_to_complex_f32(static_cast<const float*>(x), static_cast<float2*>(fa), n, s);
-    fft_c2c_f32(static_cast<float2*>(fa), static_cast<float2*>(xf), static_cast<float2*>(fb), n, 1, -1,
+    fft_r2c_f32(static_cast<const float*>(x), static_cast<float2*>(xf), static_cast<float2*>(fb), n,
                 static_cast<float2*>(tw), n, s);
     k_mf_pointwise<float2><<<grid, 256, 0, s>>>(static_cast<float2*>(xf), inv_psd, sig2, p, n, df, g.f_low,
                                                 g.f_high, static_cast<float2*>(fa), sigma_out);

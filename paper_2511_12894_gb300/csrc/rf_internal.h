@@ -151,6 +151,14 @@ struct rf_ctx {
   // w[2^tw4_lo_bits m] for m < n / 2^tw4_lo_bits; empty where the four-step FFT does not apply.
   rf::DevBuf tw4;
   int tw4_lo_bits = 0;
+  // Powers of the bin index k = 0..n/2 in FP64, rows of pw_stride: k^(1/3), k^(-5/3), ln(k)/3 and
+  // k^(-7/6) (0 at k = 0): the template phase and amplitude on any grid f_k = k df (tf2.cuh).
+  rf::DevBuf pw;
+  int64_t pw_stride = 0;
+  // Filters and intermediates of a batch of mf_batch references of rf_mf_reference, sized when the
+  // context is made, so that the call never allocates (mf_batch = 1: fa and fb serve).
+  rf::DevBuf mf_ref;
+  int mf_batch = 1;
   // Workspaces (grid dtype complex unless stated).
   rf::DevBuf xf;       // data spectrum, complex[n]
   rf::DevBuf fa, fb;   // FFT ping-pong, complex[n]
@@ -278,17 +286,18 @@ void ifft_product_f32(const float2* X, const float2* F, int64_t fstride, float2*
 void fft_c2c_f32(const float2* in, float2* out, float2* tmp, int64_t n, int batch, int sign,
                  const float2* tw_table, int64_t table_n, cudaStream_t s);
 // Four-step FP32 transforms of the context's n (fft4.cu), for n = 2^18 .. 2^24: two passes
-// through HBM.  Forward of real data (natural order out), the unnormalised inverse of batch
-// complex rows, and the inverse of the one-sided product X[k] F_r[k] (k <= n/2, zero above;
+// through HBM.  Forward of real data (natural order out) and the inverse of the one-sided product X[k] F_r[k] (k <= n/2, zero above;
 // row r of F at r fstride).  tmp holds batch n complex values.
 bool fft4_supported(int64_t n);
 int fft4_lo_bits(int64_t n);
 void fft4_forward_real(const rf_ctx* c, const float* x, float2* out, float2* tmp, cudaStream_t s);
-void fft4_inverse(const rf_ctx* c, const float2* in, float2* out, float2* tmp, int batch, cudaStream_t s);
 void fft4_inverse_product(const rf_ctx* c, const float2* X, const float2* F, int64_t fstride, float2* out,
                           float2* tmp, int batch, cudaStream_t s);
-void real_to_complex_f64(const double* x, double2* out, int64_t n, cudaStream_t s);
-void real_to_complex_f32(const float* x, float2* out, int64_t n, cudaStream_t s);
+// Forward transform of real data (natural order, unnormalised).
+void fft_r2c_f64(const double* x, double2* out, double2* tmp, int64_t n, const double2* tw, int64_t table_n,
+                 cudaStream_t s);
+void fft_r2c_f32(const float* x, float2* out, float2* tmp, int64_t n, const float2* tw, int64_t table_n,
+                 cudaStream_t s);
 // Host-side FP64 twiddle table exp(-2 pi i m / n), m < n (octant symmetric, accurate).
 std::vector<double2> host_twiddles(int64_t n);
 // Stage twiddle tables of the block FFTs for B = 2^9 .. 2^14 (float2, concatenated), with
@@ -302,8 +311,10 @@ void mf_filtered_impl(rf_ctx* c, const void* x, int32_t nref, const void* filt, 
 void mf_reference_impl(rf_ctx* c, const void* x, const double* inv_psd, int32_t nref,
                        const rf_template* refs, void* z_out, double* sigma_out, cudaStream_t s);
 void template_fd_impl(rf_ctx* c, const rf_template& t, void* h_out, cudaStream_t s);
-// sigma^2 = 4 df sum_band B(f)^2 inv_psd for `count` templates -> out[count] (device, FP64)
-void sigma2_impl(rf_ctx* c, const double* inv_psd, int count, double* out, cudaStream_t s);
+// the bins k0..k1 of [f_low, f_high] on a grid
+void band_bins(const rf_grid& g, int64_t* k0, int64_t* k1);
+// tables of powers of the bin index and the batch workspace of a new context
+void mf_create(rf_ctx* c);
 
 // ---------------------------------------------------------------- builder (builder.cu)
 rf_kernels* build_impl(rf_ctx* c, const rf_template& ref, const rf_template* nbrs, int32_t k,

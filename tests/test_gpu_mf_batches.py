@@ -1,0 +1,33 @@
+"""Reference templates generated in batches: every row equals the call with that reference alone,
+at the edges of a batch, and the matched filter of its stored filter."""
+import numpy as np
+import pytest
+
+import workload
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("n,nref", [(1 << 9, 1), (1 << 12, 8), (1 << 12, 9), (1 << 13, 17), (1 << 20, 5),
+                                    (1 << 22, 2)])
+def test_rows_equal_single_calls(dtype, n, nref):
+    torch = pytest.importorskip("torch")
+    from paper_2511_12894_gb300 import RatioFilter
+    if dtype == "f64" and n > 1 << 20:
+        pytest.skip("the FP64 passes are the same code at every batch of one")
+    rf = RatioFilter(n, 2048.0, 20.0, 971.0, 7, dtype)
+    rng = np.random.default_rng(nref)
+    x = torch.tensor(rng.standard_normal(n), dtype=rf.rdtype, device="cuda")
+    ip = torch.tensor(rng.uniform(0.5, 2.0, n // 2 + 1), device="cuda")
+    refs = [workload.Template(float(m), 1.2, tc=float(t), phic=0.3)
+            for m, t in zip(rng.uniform(1.2, 2.4, nref), rng.uniform(0.0, 0.1, nref))]
+    z, sg = rf.mf_reference(x, ip, refs)
+    for r, t in enumerate(refs):
+        z1, s1 = rf.mf_reference(x, ip, [t])
+        assert torch.equal(z[r], z1[0]) and torch.equal(sg[r], s1[0])
+    filt, sf = rf.reference_filters(ip, refs)
+    zf = rf.mf_filtered(x, filt)
+    assert torch.equal(sf, sg)
+    tol = 1e-12 if dtype == "f64" else 2e-6
+    assert (zf - z).abs().max().item() <= tol * z.abs().max().item()
