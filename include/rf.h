@@ -360,8 +360,12 @@ void rf_kernels_free(rf_kernels* kern);
 /* Neighbour SNR series (Eq. 8, circular):  z_j[i] = sum_{l<L_j} c_j[l] z_ref[(i - m0_j - l) mod n].
  * z_ref: complex[n]; z_out: complex[k][n] (grid dtype).  algo: rf_algo.  RF_ALGO_OS needs an
  * RF_F32 grid with n >= 512 (else RF_EUNSUPPORTED) and evaluates the same sum through the
- * frequency form (Eq. 7) in overlap-save blocks; RF_ALGO_AUTO takes OS on RF_F32 grids and the
- * direct sum on RF_F64 grids.  The context's workspace grows on first use ((B / Lp) n
+ * frequency form (Eq. 7) in overlap-save blocks; RF_ALGO_AUTO takes OS on RF_F32 grids and, on
+ * RF_F64 grids, whichever is modelled cheaper of the direct sum and a double-precision overlap-save
+ * (the first such call prepares the kernel set and SYNCHRONISES `stream`; while a set is not prepared
+ * a call under stream capture runs the direct sum; the workspace comes in stream order from a pool of
+ * the context).  In the overlap-save forms a non-finite sample of z_ref reaches every output of the
+ * blocks that hold it.  The context's workspace grows on first use ((B / Lp) n
  * complex64 for OS; see rf_reserve).  Async on stream, except that an OS call on a kernel set that was not
  * prepared prepares it first (see rf_kernels_prepare). */
 rf_status rf_reconstruct(rf_ctx* ctx, const void* z_ref, const rf_kernels* kern, int32_t algo,

@@ -158,6 +158,7 @@ rf_status rf_create(const rf_grid* grid, rf_ctx** out) {
     c->fb.ensure(esz * n);
     c->red.ensure(sizeof(double) * 1024);
     mf_create(c.get());
+    if (g.dtype == RF_F64) os64_create(c.get());
     c->status.ensure(sizeof(int) * 4);
     RF_CUDA(cudaMemset(c->status.p, 0, sizeof(int) * 4));
     *out = c.release();
@@ -494,8 +495,11 @@ void rf_kernels_free(rf_kernels* kern) {
 }
 
 // Validates a reconstruction call and resolves RF_ALGO_AUTO: the autotuned form of the kernel
-// set (with its precision) when there is one, else overlap-save on FP32 grids with n >= 512 and
-// the direct sum otherwise.
+// set (with its precision) when there is one, else overlap-save on FP32 grids with n >= 512,
+// kAuto64 on FP64 grids (FP64 overlap-save or the direct sum, run_direct) and the direct sum
+// otherwise.
+static constexpr int kAuto64 = 64;
+
 static int check_recon(rf_ctx* ctx, const void* z_ref, const rf_kernels* kern, int32_t algo, int32_t& prec) {
   check_ctx(ctx);
   RF_REQUIRE(kern != nullptr, "kern is NULL");
@@ -522,8 +526,16 @@ static int check_recon(rf_ctx* ctx, const void* z_ref, const rf_kernels* kern, i
     set_error("overlap-save needs an RF_F32 grid with n >= 512");
     throw Fail{RF_EUNSUPPORTED};
   }
-  if (algo == RF_ALGO_AUTO) algo = os_ok ? RF_ALGO_OS : RF_ALGO_DIRECT;
+  if (algo == RF_ALGO_AUTO) algo = os_ok ? RF_ALGO_OS : (ctx->g.dtype == RF_F64 ? kAuto64 : RF_ALGO_DIRECT);
   return algo;
+}
+
+// The forms that are neither single-precision overlap-save nor tensor-core.
+static void run_direct(int a, rf_ctx* ctx, const void* z_ref, const rf_kernels* kern, void* z_out, int64_t W,
+                       float* max_out, int32_t* argmax_out, cudaStream_t s) {
+  if (a == kAuto64 && reconstruct_os64(ctx, z_ref, const_cast<rf_kernels*>(kern), z_out, W, max_out, argmax_out, s))
+    return;
+  reconstruct_direct(ctx, z_ref, kern, z_out, W, max_out, argmax_out, s);
 }
 
 rf_status rf_reconstruct(rf_ctx* ctx, const void* z_ref, const rf_kernels* kern, int32_t algo, int32_t prec,
@@ -537,7 +549,7 @@ rf_status rf_reconstruct(rf_ctx* ctx, const void* z_ref, const rf_kernels* kern,
       reconstruct_gemm(ctx, z_ref, const_cast<rf_kernels*>(kern), prec, z_out, 0, nullptr, nullptr,
                        (cudaStream_t)stream);
     else
-      reconstruct_direct(ctx, z_ref, kern, z_out, 0, nullptr, nullptr, (cudaStream_t)stream);
+      run_direct(a, ctx, z_ref, kern, z_out, 0, nullptr, nullptr, (cudaStream_t)stream);
   });
 }
 
@@ -557,7 +569,7 @@ rf_status rf_reconstruct_winmax(rf_ctx* ctx, const void* z_ref, const rf_kernels
       reconstruct_gemm(ctx, z_ref, const_cast<rf_kernels*>(kern), prec, nullptr, W, max_out, argmax_out,
                        (cudaStream_t)stream);
     else
-      reconstruct_direct(ctx, z_ref, kern, nullptr, W, max_out, argmax_out, (cudaStream_t)stream);
+      run_direct(a, ctx, z_ref, kern, nullptr, W, max_out, argmax_out, (cudaStream_t)stream);
   });
 }
 
@@ -598,8 +610,8 @@ rf_status rf_reconstruct_batched(rf_ctx* ctx, int32_t G, const void* const* z_re
           reconstruct_gemm(ctx, z_refs[g], ks[g], prec, nullptr, W, max_out + row * nw, argmax_out + row * nw,
                            (cudaStream_t)stream);
         else
-          reconstruct_direct(ctx, z_refs[g], ks[g], nullptr, W, max_out + row * nw, argmax_out + row * nw,
-                             (cudaStream_t)stream);
+          run_direct(a, ctx, z_refs[g], ks[g], nullptr, W, max_out + row * nw, argmax_out + row * nw,
+                     (cudaStream_t)stream);
       }
       row += ks[g]->k;
     }

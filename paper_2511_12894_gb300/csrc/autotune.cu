@@ -229,7 +229,8 @@ void autotune_impl(rf_ctx* c, int32_t G, const void* const* z_refs, rf_kernels* 
   for (int g = 0; g < G; ++g) {
     // bucketed preparations (overlap-save, two-phase or mixed) run through the overlap-save entry
     const bool bucketed = w.cut || w.algo == RF_ALGO_OS_BINS;
-    ks[g]->tuned_algo = bucketed ? RF_ALGO_OS : w.algo;
+    // (on FP64 grids the direct sum is the only form timed, and AUTO keeps its own rule)
+    ks[g]->tuned_algo = bucketed ? RF_ALGO_OS : (f32 ? w.algo : RF_ALGO_AUTO);
     ks[g]->tuned_prec = bucketed ? RF_PREC_NATIVE : w.prec;
   }
   RF_CUDA(cudaStreamSynchronize(s));

@@ -1,4 +1,4 @@
-// Block FFT of B complex64 points held by one thread block: B/16 threads, 16 points per
+// Block FFT of B complex points (complex64 or complex128) held by one thread block: B/16 threads, 16 points per
 // thread, decimation in time through shared memory in place: a radix-16 stage on registers, a
 // radix-RM stage (RM = 2, 4 or 8) when log2(B) is not a multiple of 4, then radix-16 stages.
 //
@@ -17,14 +17,15 @@
 //
 // Input: before the call, thread `tid` holds v[t] = x[tid + t B/16] for t < 16.
 // Output: after it, thread `tid` holds v[t] = X[tid + t B/16].
-// Shared memory: B + 32 float2; location l is stored at l + 2 (l / (B/16)), so that the 16
-// lanes of the first stage's writes, which are B/16 locations apart, fall two bank pairs apart
-// (128-bit stores, eight lanes per wavefront); the later stages touch runs of 16 locations.
+// Shared memory: location l is stored at l + PAD (l / (B/16)), B + 16 PAD values.  The 16 lanes of
+// the first stage's writes are B/16 locations apart; PAD keeps them 16 bytes apart modulo the
+// banks (PAD = 2 for complex64, written two at a time, 1 for complex128), so that eight lanes of
+// 128-bit stores fill a wavefront.  The later stages touch runs of 16 locations.
 //
 // Twiddles come from per-stage tables laid out in thread order: the stage with radix R and S has
 // a table of R S entries, entry t S + k = exp(-2 pi i t k / (R S)), so the loads of a warp are
-// contiguous.  A radix-16 stage reads the rows t = 1 and 4 and forms the other powers by complex
-// products.  The tables of the stages after the first follow each other; a block size B needs
+// contiguous.  In FP32 a radix-16 stage reads the rows t = 1 and 4 and forms the other powers by
+// complex products; in FP64, whose pipe is the scarce one, it reads every row.  The tables of the stages after the first follow each other; a block size B needs
 // block_table_size<B>() entries (built on the host by block_fft_tables).
 #pragma once
 
@@ -37,9 +38,14 @@ namespace rf {
 // w^8 = w^4 w^4, at most three products deep: a few ulp), which keeps 13 of the 15 table loads of
 // a radix-16 stage off the load/store pipe, the scarcer one in the block transforms (loading all
 // 15 made the 2^23-sample step 12% slower, loading 4 was 2% slower).
-template <int R>
-__device__ __forceinline__ void stage_twiddles(float2 (&w)[R], const float2* __restrict__ tw, int stride) {
+template <int R, typename V>
+__device__ __forceinline__ void stage_twiddles(V (&w)[R], const V* __restrict__ tw, int stride) {
   static_assert(R == 2 || R == 4 || R == 8 || R == 16, "radix");
+  if constexpr (sizeof(V) == sizeof(double2)) {
+#pragma unroll
+    for (int t = 1; t < R; ++t) w[t] = __ldg(tw + t * stride);
+    return;
+  }
   w[1] = __ldg(tw + stride);
   if constexpr (R >= 4) {
     w[2] = cmul(w[1], w[1]);
@@ -58,13 +64,13 @@ __device__ __forceinline__ void stage_twiddles(float2 (&w)[R], const float2* __r
   }
 }
 
-template <int R, int SIGN>
-__device__ __forceinline__ void apply_twiddles(float2* a, const float2 (&w)[R]) {
+template <int R, int SIGN, typename V>
+__device__ __forceinline__ void apply_twiddles(V* a, const V (&w)[R]) {
 #pragma unroll
   for (int t = 1; t < R; ++t) a[t] = tw_apply<SIGN>(a[t], w[t]);
 }
 
-template <int B>
+template <int B, int PAD = 2>
 struct BlockFFTShape {
   static constexpr int LOGB = (B == 512) ? 9 : (B == 1024) ? 10 : (B == 2048) ? 11 : (B == 4096) ? 12
                             : (B == 8192) ? 13 : (B == 16384) ? 14 : -1;
@@ -72,8 +78,8 @@ struct BlockFFTShape {
   static constexpr int NT = B / 16;
   static constexpr int RM = 1 << (LOGB % 4);           // radix of the second stage (1: none)
   static constexpr int MID16 = LOGB / 4 - 2;           // radix-16 stages between it and the last (0 or 1)
-  static constexpr int SMEM = B + 32;                  // float2 entries
-  static constexpr int NTP = NT + 2;                   // padded stride of NT locations
+  static constexpr int SMEM = B + 16 * PAD;            // shared-memory values
+  static constexpr int NTP = NT + PAD;                 // padded stride of NT locations
 };
 
 // Entries of the stage twiddle tables of block size B.
@@ -88,9 +94,10 @@ __host__ __device__ constexpr int block_table_size() {
 // can share a thread block, each with its own shared-memory region (16-byte aligned), as long as
 // every thread of the block calls block_fft (it synchronises the whole block).  The region may be
 // rewritten by the caller only after a barrier: the last stage reads it without one after it.
-template <int B, int SIGN>
-__device__ __forceinline__ void block_fft(float2 (&v)[16], float2* sm, const float2* __restrict__ tw, int tid) {
-  using S = BlockFFTShape<B>;
+template <int B, int SIGN, typename V>
+__device__ __forceinline__ void block_fft(V (&v)[16], V* sm, const V* __restrict__ tw, int tid) {
+  constexpr int PAD = sizeof(V) == sizeof(double2) ? 1 : 2;
+  using S = BlockFFTShape<B, PAD>;
   constexpr int NT = S::NT, RM = S::RM, NTP = S::NTP;
   // First stage: no twiddles.  The thread's bins t B/16 + tid sit at locations base + t, with the
   // digits of tid (t2 of RM, t3 of 16 when there is a middle radix-16 stage, t4 of 16) reversed.
@@ -98,22 +105,28 @@ __device__ __forceinline__ void block_fft(float2 (&v)[16], float2* sm, const flo
   {
     constexpr int N3 = S::MID16 ? 16 : 1;
     const int rest = tid / 16;
-    float2* o = sm + 16 * (rest / N3) + 16 * RM * (rest % N3) + NTP * (tid % 16);
+    V* o = sm + 16 * (rest / N3) + 16 * RM * (rest % N3) + NTP * (tid % 16);
+    if constexpr (PAD == 1) {
 #pragma unroll
-    for (int t = 0; t < 16; t += 2) *reinterpret_cast<float4*>(o + t) = make_float4(v[t].x, v[t].y, v[t + 1].x, v[t + 1].y);
+      for (int t = 0; t < 16; ++t) o[t] = v[t];
+    } else {
+#pragma unroll
+      for (int t = 0; t < 16; t += 2)
+        *reinterpret_cast<float4*>(o + t) = make_float4(v[t].x, v[t].y, v[t + 1].x, v[t + 1].y);
+    }
   }
   __syncthreads();
   if constexpr (RM > 1) {
     // second stage, S = 16: butterflies tid + q NT, q < 16 / RM; all have lo = tid mod 16
     const int lo = tid % 16;
-    float2 w[RM];
+    V w[RM];
     stage_twiddles<RM>(w, tw + lo, 16);
     const int l0 = (tid / 16) * 16 * RM + lo;
-    float2* p = sm + l0 + 2 * (l0 / NT);
+    V* p = sm + l0 + PAD * (l0 / NT);
 #pragma unroll
     for (int q = 0; q < 16 / RM; ++q) {
-      float2 a[RM];
-      float2* pq = p + q * RM * NTP;
+      V a[RM];
+      V* pq = p + q * RM * NTP;
 #pragma unroll
       for (int t = 0; t < RM; ++t) a[t] = pq[16 * t];
       apply_twiddles<RM, SIGN>(a, w);
@@ -128,11 +141,11 @@ __device__ __forceinline__ void block_fft(float2 (&v)[16], float2* sm, const flo
     // middle radix-16 stage, S = 16 RM: group hi of NT = 16 S locations
     constexpr int ST = 16 * RM;
     const int lo = tid % ST;
-    float2* p = sm + (tid / ST) * NTP + lo;
+    V* p = sm + (tid / ST) * NTP + lo;
 #pragma unroll
     for (int t = 0; t < 16; ++t) v[t] = p[t * ST];
     {
-      float2 w[16];
+      V w[16];
       stage_twiddles<16>(w, tw + lo, ST);
       apply_twiddles<16, SIGN>(v, w);
     }
@@ -144,10 +157,10 @@ __device__ __forceinline__ void block_fft(float2 (&v)[16], float2* sm, const flo
   }
   // last stage, S = NT: butterfly lo = tid
   {
-    const float2* p = sm + tid;
+    const V* p = sm + tid;
 #pragma unroll
     for (int t = 0; t < 16; ++t) v[t] = p[t * NTP];
-    float2 w[16];
+    V w[16];
     stage_twiddles<16>(w, tw + tid, NT);
     apply_twiddles<16, SIGN>(v, w);
   }
@@ -155,8 +168,8 @@ __device__ __forceinline__ void block_fft(float2 (&v)[16], float2* sm, const flo
 }
 
 // One transform per thread block (tid = threadIdx.x).
-template <int B, int SIGN>
-__device__ __forceinline__ void block_fft(float2 (&v)[16], float2* sm, const float2* __restrict__ tw) {
+template <int B, int SIGN, typename V>
+__device__ __forceinline__ void block_fft(V (&v)[16], V* sm, const V* __restrict__ tw) {
   block_fft<B, SIGN>(v, sm, tw, (int)threadIdx.x);
 }
 

@@ -195,6 +195,11 @@ void fft_r2c_f32(const float* x, float2* out, float2* tmp, int64_t n, const floa
   fft_c2c<float2>(nullptr, out, tmp, n, 1, -1, tw, table_n, s, nullptr, 0, x);
 }
 
+const std::vector<double2>& block_twiddles() {
+  static const std::vector<double2> w = host_twiddles(kBlockTwiddles);
+  return w;
+}
+
 std::vector<double2> host_twiddles(int64_t n) {
   // exp(-2 pi i m / n) for m < n.  Angles are reduced to the first octant, where
   // cos and sin are evaluated directly; the other octants follow by exact symmetry.

@@ -392,9 +392,10 @@ void bins_run(rf_ctx* c, const BinsPlan& pl, const OsItem* items_dev, const floa
 
 }  // namespace rf
 
-// the two-phase side stream and events (created by rf::bins_prepare_scratch)
+// the two-phase side stream and events (created by rf::bins_prepare_scratch) and the FP64 pool
 rf_ctx::~rf_ctx() {
   for (cudaEvent_t e : bins_ev)
     if (e) cudaEventDestroy(e);
   if (bins_side) cudaStreamDestroy(bins_side);
+  if (pool) cudaMemPoolDestroy(pool);
 }

@@ -476,10 +476,11 @@ void append_tables(std::vector<float2>& out) {
   const size_t start = out.size();
   int st = 16;
   auto stage = [&](int radix) {
-    const std::vector<double2> w = host_twiddles((int64_t)radix * st);
+    const std::vector<double2>& w = block_twiddles();
+    const size_t step = (size_t)(kBlockTwiddles / ((int64_t)radix * st));
     for (int t = 0; t < radix; ++t)
       for (int k = 0; k < st; ++k) {
-        const double2 v = w[(size_t)t * k];
+        const double2 v = w[(size_t)t * k * step];
         out.push_back(make_float2((float)v.x, (float)v.y));
       }
     st *= radix;
@@ -510,7 +511,8 @@ std::vector<float2> block_fft_tables(int64_t off[16]) {
   // the pair layout's twiddles exp(-2 pi i m / 32768), m < 16384 (segment split and combine)
   off[15] = (int64_t)out.size();
   {
-    const std::vector<double2> w = host_twiddles(kB2);
+    static_assert(kBlockTwiddles == kB2, "pair twiddles");
+    const std::vector<double2>& w = block_twiddles();
     for (int m = 0; m < kBH; ++m) out.push_back(make_float2((float)w[(size_t)m].x, (float)w[(size_t)m].y));
   }
   return out;

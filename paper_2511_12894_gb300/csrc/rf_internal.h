@@ -147,6 +147,11 @@ struct rf_ctx {
   // block size 2^b start at entry twb_off[b].
   rf::DevBuf twb32;
   int64_t twb_off[16] = {0};
+  // FP64 grids: stage twiddle tables of the FP64 block FFTs (B = 1024, 2048, 4096) and the pool of
+  // the FP64 overlap-save calls' workspaces.
+  rf::DevBuf twb64;
+  int64_t twb64_off[3] = {0};
+  cudaMemPool_t pool = nullptr;
   // Four-step FFT twiddles (float2): w[m] = exp(-2 pi i m / n) for m < 2^tw4_lo_bits, then
   // w[2^tw4_lo_bits m] for m < n / 2^tw4_lo_bits; empty where the four-step FFT does not apply.
   rf::DevBuf tw4;
@@ -251,6 +256,10 @@ struct rf_kernels {
   rf::DevBuf os_spec;      // float2, sum_j P_j B_j values
   rf::DevBuf os_off_d;     // int64 [k]: element offset of kernel j's first partition spectrum
   rf::DevBuf os_parts_d;   // int32 [k]
+  // FP64 overlap-save (reconstruct_os64.cu): layout (os64_B = 0: not prepared, -1: the direct sum)
+  // and partition spectra, double2.
+  int os64_B = 0, os64_Q = 0;
+  rf::DevBuf os64_spec, os64_off_d, os64_parts_d;
   // Tensor-core direct form: split-BF16 (or TF32) tap operands per group of gemm_NJ neighbours and
   // gemm_S output shifts, taps padded to gemm_LP and extended to gemm_NCK chunks of gemm_KC
   // (see reconstruct_gemm.cu).
@@ -300,6 +309,10 @@ void fft_r2c_f32(const float* x, float2* out, float2* tmp, int64_t n, const floa
                  cudaStream_t s);
 // Host-side FP64 twiddle table exp(-2 pi i m / n), m < n (octant symmetric, accurate).
 std::vector<double2> host_twiddles(int64_t n);
+// exp(-2 pi i m / kBlockTwiddles), from which the block FFT tables are taken (constant; made by the
+// first context of the process)
+constexpr int64_t kBlockTwiddles = 32768;
+const std::vector<double2>& block_twiddles();
 // Stage twiddle tables of the block FFTs for B = 2^9 .. 2^14 (float2, concatenated), with
 // the entry offset of each block size in off[log2 B].
 std::vector<float2> block_fft_tables(int64_t off[16]);
@@ -325,6 +338,11 @@ rf_kernels* import_impl(rf_ctx* c, int32_t k, const int32_t* lag0, const int32_t
 // ---------------------------------------------------------------- reconstruct
 void reconstruct_direct(rf_ctx* c, const void* z_ref, const rf_kernels* kern, void* z_out,
                         int64_t W, float* max_out, int32_t* argmax_out, cudaStream_t s);
+// FP64 overlap-save (reconstruct_os64.cu): tables and pool of an RF_F64 context; a reconstruction,
+// false when the direct sum is to run instead
+void os64_create(rf_ctx* c);
+bool reconstruct_os64(rf_ctx* c, const void* z_ref, rf_kernels* kern, void* z_out, int64_t W, float* max_out,
+                      int32_t* argmax_out, cudaStream_t s);
 void winmax_series(rf_ctx* c, const void* z, int32_t count, int64_t W, float* max_out,
                    int32_t* argmax_out, cudaStream_t s);
 // overlap-save (reconstruct_os.cu); FP32 grids, block sizes 512..16384
