@@ -1,6 +1,7 @@
 // Block FFT of B complex points (complex64 or complex128) held by one thread block: B/16 threads, 16 points per
 // thread, decimation in time through shared memory in place: a radix-16 stage on registers, a
-// radix-RM stage (RM = 2, 4 or 8) when log2(B) is not a multiple of 4, then radix-16 stages.
+// radix-RM stage (RM = 2, 4 or 8) when log2(B) is not a multiple of 4, then radix-16 stages
+// (B = 128: no more).
 //
 // Locations l hold the input in digit-reversed order.  Stage with radix R and S = product of the
 // earlier radices works on the points l = hi S R + t S + lo (lo < S):
@@ -72,12 +73,13 @@ __device__ __forceinline__ void apply_twiddles(V* a, const V (&w)[R]) {
 
 template <int B, int PAD = 2>
 struct BlockFFTShape {
-  static constexpr int LOGB = (B == 512) ? 9 : (B == 1024) ? 10 : (B == 2048) ? 11 : (B == 4096) ? 12
+  static constexpr int LOGB = (B == 128) ? 7 : (B == 256) ? 8 : (B == 512) ? 9 : (B == 1024) ? 10 : (B == 2048) ? 11 : (B == 4096) ? 12
                             : (B == 8192) ? 13 : (B == 16384) ? 14 : -1;
   static_assert(LOGB > 0, "block size");
   static constexpr int NT = B / 16;
   static constexpr int RM = 1 << (LOGB % 4);           // radix of the second stage (1: none)
-  static constexpr int MID16 = LOGB / 4 - 2;           // radix-16 stages between it and the last (0 or 1)
+  static constexpr int MID16 = LOGB >= 8 ? LOGB / 4 - 2 : 0;  // radix-16 stages between it and the last (0 or 1)
+  static constexpr bool LAST16 = LOGB >= 8;            // the last stage is radix 16 (else the second one is)
   static constexpr int SMEM = B + 16 * PAD;            // shared-memory values
   static constexpr int NTP = NT + PAD;                 // padded stride of NT locations
 };
@@ -86,7 +88,7 @@ struct BlockFFTShape {
 template <int B>
 __host__ __device__ constexpr int block_table_size() {
   using S = BlockFFTShape<B>;
-  return (S::RM > 1 ? 16 * S::RM : 0) + (S::MID16 ? 256 * S::RM : 0) + B;
+  return (S::RM > 1 ? 16 * S::RM : 0) + (S::MID16 ? 256 * S::RM : 0) + (S::LAST16 ? B : 0);
 }
 
 // tw: the stage tables of B.  SIGN: -1 forward, +1 inverse (unnormalised).  tid: the
@@ -105,7 +107,7 @@ __device__ __forceinline__ void block_fft(V (&v)[16], V* sm, const V* __restrict
   {
     constexpr int N3 = S::MID16 ? 16 : 1;
     const int rest = tid / 16;
-    V* o = sm + 16 * (rest / N3) + 16 * RM * (rest % N3) + NTP * (tid % 16);
+    V* o = S::LAST16 ? sm + 16 * (rest / N3) + 16 * RM * (rest % N3) + NTP * (tid % 16) : sm + (16 + PAD) * tid;
     if constexpr (PAD == 1) {
 #pragma unroll
       for (int t = 0; t < 16; ++t) o[t] = v[t];
@@ -116,7 +118,25 @@ __device__ __forceinline__ void block_fft(V (&v)[16], V* sm, const V* __restrict
     }
   }
   __syncthreads();
-  if constexpr (RM > 1) {
+  if constexpr (!S::LAST16) {
+    // B = 128: 16 points, then the radix-8 stage, whose butterflies lo = tid + q NT leave
+    // X[lo + 16 t] = X[tid + (q + 2 t) NT]
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int lo = tid + q * NT;
+      V a[8];
+#pragma unroll
+      for (int t = 0; t < 8; ++t) a[t] = sm[lo + t * (16 + PAD)];  // padded per 16 locations
+      V w[8];
+      stage_twiddles<8>(w, tw + lo, 16);
+      apply_twiddles<8, SIGN>(a, w);
+      dft<8, SIGN>(a);
+#pragma unroll
+      for (int t = 0; t < 8; ++t) v[q + 2 * t] = a[t];
+    }
+    return;
+  }
+  if constexpr (RM > 1 && S::LAST16) {
     // second stage, S = 16: butterflies tid + q NT, q < 16 / RM; all have lo = tid mod 16
     const int lo = tid % 16;
     V w[RM];
@@ -156,15 +176,15 @@ __device__ __forceinline__ void block_fft(V (&v)[16], V* sm, const V* __restrict
     __syncthreads();
   }
   // last stage, S = NT: butterfly lo = tid
-  {
+  if constexpr (S::LAST16) {
     const V* p = sm + tid;
 #pragma unroll
     for (int t = 0; t < 16; ++t) v[t] = p[t * NTP];
     V w[16];
     stage_twiddles<16>(w, tw + tid, NT);
     apply_twiddles<16, SIGN>(v, w);
+    dft<16, SIGN>(v);
   }
-  dft<16, SIGN>(v);
 }
 
 // One transform per thread block (tid = threadIdx.x).

@@ -1,5 +1,5 @@
-// Four-step FP32 FFT of n = N1 N2 points in two passes through HBM (the matched filter of
-// Eq. 2 at large n: the data transform and the per-template inverse transforms).
+// Four-step FFT of n = N1 N2 points in two passes through HBM, FP32 and FP64 (the matched filter of
+// Eq. 2: the data transform and the per-template inverse transforms).
 //
 // With the input index j = N2 a + b (a < N1, b < N2) and the output index k = k1 + N1 k2,
 //   X[k1 + N1 k2] = sum_b w_N2^(b k2) [ w_n^(b k1) sum_a x[N2 a + b] w_N1^(a k1) ],
@@ -10,16 +10,22 @@
 // Both passes run the shared-memory block FFT (blockfft.cuh) on several lines per thread
 // block: pass 1 on G adjacent columns, whose lanes interleave so that every load and store of
 // a warp covers runs of G consecutive elements; pass 2 on R adjacent rows, staged through
-// shared memory for the transposed store (runs of R elements).  Lines of a tile start at
-// offsets 16/G float2 apart modulo 16 bank pairs, which keeps the half-warp accesses of every
-// stage conflict free.
+// shared memory for the transposed store (runs of R elements).  Lines of a tile start 128 / G bytes
+// apart modulo the 128 bytes of the banks, which keeps the accesses of every stage conflict free.
 //
-// The twiddle w_n^m (m = b k1 < n) is the product of two table entries: w_n^(m mod 2^s) and
+// FP32: the twiddle w_n^m (m = b k1 < n) is the product of two table entries: w_n^(m mod 2^s) and
 // w_n^(2^s floor(m / 2^s)), with 2^s = 2^ceil(log2(n) / 2); the tables (about 2 sqrt(n)
-// entries) stay in cache.
+// entries) stay in cache.  FP64 reads w_n^m from the context's n-entry table: products would
+// cost the FP64 pipe, which has two lanes per SM, more than the gathers cost.
 //
 // Modes of pass 1: real input (the data transform) and the one-sided product X[k] F[k] for
 // k <= n/2, zero above (the matched-filter integrand, formed on load).
+//
+// FP32 grids of at most 16384 points fit one thread block: block_mf forms the spectrum of the data,
+// the product with a filter and the inverse transform in one launch, a block per reference (each
+// forms the spectrum anew: the copies run at the same time on other SMs).
+#include <type_traits>
+
 #include "blockfft.cuh"
 #include "rf_internal.h"
 
@@ -30,26 +36,28 @@ namespace {
 constexpr int kF4Real = 0;
 constexpr int kF4Product = 1;
 
-// float2 entries of one line's shared-memory region in a tile of G lines.
-template <int L, int G>
+// Values of one line's shared-memory region in a tile of G lines.
+template <typename V, int L, int G>
 __host__ __device__ constexpr int f4_line() {
-  return BlockFFTShape<L>::SMEM + 16 / G;
+  return BlockFFTShape<L, 16 / (int)sizeof(V)>::SMEM + 128 / (int)sizeof(V) / G;
 }
 
-template <int L, int G>
+template <typename V, int L, int G>
 constexpr size_t f4_smem() {
-  return sizeof(float2) * (size_t)G * (size_t)f4_line<L, G>();
+  return sizeof(V) * (size_t)G * (size_t)f4_line<V, L, G>();
 }
+
+extern __shared__ __align__(16) unsigned char f4_raw[];
 
 // Pass 1: columns col0 .. col0 + G - 1 of batch row blockIdx.y; L = N1.
-template <int L, int G, int MODE, int SIGN>
-__global__ void __launch_bounds__(G * L / 16) k_fft4_cols(const void* __restrict__ in, const float2* __restrict__ F,
-                                                          int64_t fstride, float2* __restrict__ out, int n2log,
-                                                          const float2* __restrict__ twb,
-                                                          const float2* __restrict__ tw4, int lo_bits) {
-  using S = BlockFFTShape<L>;
-  constexpr int NT = S::NT;
-  extern __shared__ __align__(16) float2 f4_sm[];
+template <typename V, int L, int G, int MODE, int SIGN>
+__global__ void __launch_bounds__(G * L / 16) k_fft4_cols(const void* __restrict__ in, const V* __restrict__ F,
+                                                          int64_t fstride, V* __restrict__ out, int n2log,
+                                                          const V* __restrict__ twb, const V* __restrict__ tw4,
+                                                          int lo_bits) {
+  using T = typename real_of<V>::type;
+  constexpr int NT = L / 16;
+  V* f4_sm = reinterpret_cast<V*>(f4_raw);
   const int c = (int)threadIdx.x % G;
   const int ltid = (int)threadIdx.x / G;
   const int64_t N2 = (int64_t)1 << n2log;
@@ -59,23 +67,31 @@ __global__ void __launch_bounds__(G * L / 16) k_fft4_cols(const void* __restrict
   // element (a = ltid + t NT, col) sits at j0 + t NT N2
   const int64_t j0 = (int64_t)ltid * N2 + col;
   const int64_t tstep = (int64_t)NT * N2;
-  float2 v[16];
+  V v[16];
   if constexpr (MODE == kF4Real) {
-    const float* p = static_cast<const float*>(in) + boff + j0;
+    const T* p = static_cast<const T*>(in) + boff + j0;
 #pragma unroll
-    for (int t = 0; t < 16; ++t) v[t] = make_float2(p[t * tstep], 0.f);
+    for (int t = 0; t < 16; ++t) v[t] = cmake<V>(p[t * tstep], (T)0);
   } else {
     // X is one spectrum shared by the batch; F holds one filter of n/2 + 1 values per row.
     // Rows a > N1/2 lie above n/2 (zero); row N1/2 holds only column 0.
-    const float2* px = static_cast<const float2*>(in) + j0;
-    const float2* pf = F + (int64_t)blockIdx.y * fstride + j0;
+    const V* px = static_cast<const V*>(in) + j0;
+    const V* pf = F + (int64_t)blockIdx.y * fstride + j0;
     const int64_t lim = n / 2 - j0;
 #pragma unroll
     for (int t = 0; t < 16; ++t)
-      v[t] = t * tstep <= lim ? cmul(px[t * tstep], pf[t * tstep]) : make_float2(0.f, 0.f);
+      v[t] = t * tstep <= lim ? cmul(px[t * tstep], pf[t * tstep]) : cmake<V>((T)0, (T)0);
   }
-  block_fft<L, SIGN>(v, f4_sm + c * f4_line<L, G>(), twb, ltid);
-  // v[u] holds the column's bin k1 = ltid + NT u, u < 16.
+  block_fft<L, SIGN>(v, f4_sm + c * f4_line<V, L, G>(), twb, ltid);
+  // v[u] holds the column's bin k1 = ltid + NT u, u < 16, which goes to row k1: o + NT u N2.
+  V* o = out + boff + j0;
+  if constexpr (sizeof(T) == 8) {
+    const V* w = tw4 + col * ltid;
+    const int64_t step = col * NT;
+#pragma unroll
+    for (int u = 0; u < 16; ++u) o[(int64_t)(u * NT) * N2] = tw_apply<SIGN>(v[u], __ldg(w + u * step));
+    return;
+  } else {
   // Twiddle w_n^(col k1) = w_n^(col ltid) e^u with e = w_n^(col NT): e, e^2, e^4 and e^8 come
   // from the tables (a product of two entries each, m = col NT 2^i < n), e^3, e^5 .. e^7 by at
   // most two more products, and e^(u + 8) = e^u e^8 (a few ulp in all).
@@ -85,7 +101,6 @@ __global__ void __launch_bounds__(G * L / 16) k_fft4_cols(const void* __restrict
   const unsigned cu = (unsigned)col;  // col k1 < n <= 2^24
   const float2 b0 = table(cu * (unsigned)ltid);
   const float2 e1 = table(cu * NT), e2 = table(cu * 2u * NT), e4 = table(cu * 4u * NT), e8 = table(cu * 8u * NT);
-  float2* o = out + boff + j0;  // bin k1 goes to row k1: o + NT u N2
 #pragma unroll
   for (int u = 0; u < 8; ++u) {
     float2 eu;
@@ -102,32 +117,32 @@ __global__ void __launch_bounds__(G * L / 16) k_fft4_cols(const void* __restrict
     o[(int64_t)(u * NT) * N2] = tw_apply<SIGN>(v[u], w);
     o[(int64_t)((u + 8) * NT) * N2] = tw_apply<SIGN>(v[u + 8], w8);
   }
+  }
 }
 
 // Pass 2: rows row0 .. row0 + R - 1 of batch row blockIdx.y; L = N2.  Output k1 + N1 k2.
-template <int L, int R, int SIGN>
-__global__ void __launch_bounds__(R * L / 16) k_fft4_rows(const float2* __restrict__ in, float2* __restrict__ out,
-                                                          int n1log, const float2* __restrict__ twb) {
-  using S = BlockFFTShape<L>;
-  constexpr int NT = S::NT;
-  constexpr int SL = f4_line<L, R>();
-  extern __shared__ __align__(16) float2 f4_sm[];
+template <typename V, int L, int R, int SIGN>
+__global__ void __launch_bounds__(R * L / 16) k_fft4_rows(const V* __restrict__ in, V* __restrict__ out, int n1log,
+                                                          const V* __restrict__ twb) {
+  constexpr int NT = L / 16;
+  constexpr int SL = f4_line<V, L, R>();
+  V* f4_sm = reinterpret_cast<V*>(f4_raw);
   const int g = (int)threadIdx.x / NT;
   const int ltid = (int)threadIdx.x % NT;
   const int64_t N1 = (int64_t)1 << n1log;
   const int64_t n = N1 * L;
   const int64_t row0 = (int64_t)blockIdx.x * R;
-  const float2* src = in + (int64_t)blockIdx.y * n + (row0 + g) * L;
-  float2 v[16];
+  const V* src = in + (int64_t)blockIdx.y * n + (row0 + g) * L;
+  V v[16];
 #pragma unroll
   for (int t = 0; t < 16; ++t) v[t] = src[ltid + t * NT];
-  float2* sm = f4_sm + g * SL;
+  V* sm = f4_sm + g * SL;
   block_fft<L, SIGN>(v, sm, twb, ltid);
   __syncthreads();  // the last stage has read its inputs from shared memory
 #pragma unroll
   for (int t = 0; t < 16; ++t) sm[ltid + t * NT] = v[t];
   __syncthreads();
-  float2* dst = out + (int64_t)blockIdx.y * n + row0;
+  V* dst = out + (int64_t)blockIdx.y * n + row0;
 #pragma unroll
   for (int i = 0; i < 16; ++i) {
     const int f = (int)threadIdx.x + i * (R * NT);
@@ -137,36 +152,75 @@ __global__ void __launch_bounds__(R * L / 16) k_fft4_rows(const float2* __restri
   }
 }
 
-constexpr int kF4MinLog = 18;  // N1, N2 >= 512: the block FFT tables start at 2^9
-constexpr int kF4MaxLog = 24;  // N1, N2 <= 4096
+// One reference per block: spectrum of the data, product with the filter, inverse transform, all
+// in registers and shared memory.
+template <int B>
+__global__ void __launch_bounds__(B / 16) k_block_mf(const float* __restrict__ x, const float2* __restrict__ F,
+                                                     int64_t fstride, float2* __restrict__ out,
+                                                     const float2* __restrict__ twb) {
+  constexpr int NT = B / 16;
+  float2* sm = reinterpret_cast<float2*>(f4_raw);
+  const int tid = threadIdx.x;
+  F += blockIdx.x * fstride + tid;
+  out += (int64_t)blockIdx.x * B + tid;
+  float2 v[16];
+#pragma unroll
+  for (int t = 0; t < 16; ++t) v[t] = make_float2(__ldg(x + tid + t * NT), 0.f);
+  block_fft<B, -1>(v, sm, twb, tid);
+  // bins tid + t NT: those below n/2 are t < 8, n/2 itself is t = 8 of thread 0
+#pragma unroll
+  for (int t = 0; t < 8; ++t) v[t] = cmul(v[t], __ldg(F + t * NT));
+  v[8] = tid == 0 ? cmul(v[8], __ldg(F + 8 * NT)) : make_float2(0.f, 0.f);
+#pragma unroll
+  for (int t = 9; t < 16; ++t) v[t] = make_float2(0.f, 0.f);
+  __syncthreads();  // the forward transform's last stage has read shared memory
+  block_fft<B, +1>(v, sm, twb, tid);
+#pragma unroll
+  for (int t = 0; t < 16; ++t) out[t * NT] = v[t];
+}
 
-// Tile widths: G columns of N1 points (G N1 / 16 <= 1024 threads), R rows of N2 points.
-template <int L> constexpr int f4_cols_g() { return L >= 4096 ? 4 : 8; }
-template <int L> constexpr int f4_rows_r() { return 4; }
+constexpr int kF4MinLog = 15;    // FP32: below, one block does it (block_mf)
+constexpr int kF4MinLog64 = 14;  // N1, N2 >= 128
+constexpr int kF4MaxLog = 24;    // N1, N2 <= 4096
 
-template <int L, int MODE, int SIGN>
-void launch_cols(const void* in, const float2* F, int64_t fstride, float2* out, int n2log, int batch,
-                 const rf_ctx* c, cudaStream_t s) {
-  constexpr int G = f4_cols_g<L>();
-  const auto fn = k_fft4_cols<L, G, MODE, SIGN>;
-  constexpr size_t smem = f4_smem<L, G>();
+// Tile widths: G columns of N1 points, R rows of N2 points, at most 1024 (FP32) or 512 (FP64) threads
+// of 16 points; lines of up to 512 points take narrower tiles, so that the few blocks of a small
+// transform spread over more SMs.
+template <typename V, int L> constexpr int f4_cols_g() {
+  return sizeof(V) == 8 ? (L >= 4096 ? 4 : (L >= 512 ? 8 : 4)) : (L >= 4096 ? 2 : 4);
+}
+template <typename V, int L> constexpr int f4_rows_r() { return sizeof(V) == 16 && L >= 4096 ? 2 : 4; }
+
+template <typename V>
+const V* block_tables(const rf_ctx* c, int logb) {
+  if constexpr (sizeof(V) == 8) return c->twb32.as<float2>() + c->twb_off[logb];
+  else return c->twb64.as<double2>() + c->twb64_off[logb];
+}
+
+template <typename V, int L, int MODE, int SIGN>
+void launch_cols(const void* in, const V* F, int64_t fstride, V* out, int n2log, int batch, const rf_ctx* c,
+                 cudaStream_t s) {
+  constexpr int G = f4_cols_g<V, L>();
+  const auto fn = k_fft4_cols<V, L, G, MODE, SIGN>;
+  constexpr size_t smem = f4_smem<V, L, G>();
   RF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  const int lb = BlockFFTShape<L>::LOGB;
+  const V* tw;
+  if constexpr (sizeof(V) == 8) tw = c->tw4.as<float2>();
+  else tw = c->tw64.as<double2>();
   dim3 grid((unsigned)(((int64_t)1 << n2log) / G), (unsigned)batch);
-  fn<<<grid, G * L / 16, smem, s>>>(in, F, fstride, out, n2log, c->twb32.as<float2>() + c->twb_off[lb],
-                                     c->tw4.as<float2>(), c->tw4_lo_bits);
+  fn<<<grid, G * L / 16, smem, s>>>(in, F, fstride, out, n2log, block_tables<V>(c, BlockFFTShape<L>::LOGB), tw,
+                                     c->tw4_lo_bits);
   RF_LAUNCHED();
 }
 
-template <int L, int SIGN>
-void launch_rows(const float2* in, float2* out, int n1log, int batch, const rf_ctx* c, cudaStream_t s) {
-  constexpr int R = f4_rows_r<L>();
-  const auto fn = k_fft4_rows<L, R, SIGN>;
-  constexpr size_t smem = f4_smem<L, R>();
+template <typename V, int L, int SIGN>
+void launch_rows(const V* in, V* out, int n1log, int batch, const rf_ctx* c, cudaStream_t s) {
+  constexpr int R = f4_rows_r<V, L>();
+  const auto fn = k_fft4_rows<V, L, R, SIGN>;
+  constexpr size_t smem = f4_smem<V, L, R>();
   RF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  const int lb = BlockFFTShape<L>::LOGB;
   dim3 grid((unsigned)(((int64_t)1 << n1log) / R), (unsigned)batch);
-  fn<<<grid, R * L / 16, smem, s>>>(in, out, n1log, c->twb32.as<float2>() + c->twb_off[lb]);
+  fn<<<grid, R * L / 16, smem, s>>>(in, out, n1log, block_tables<V>(c, BlockFFTShape<L>::LOGB));
   RF_LAUNCHED();
 }
 
@@ -176,25 +230,15 @@ int ilog2(int64_t n) {
   return b;
 }
 
-template <int MODE, int SIGN>
-void cols_dispatch(int n1log, const void* in, const float2* F, int64_t fstride, float2* out, int n2log, int batch,
-                   const rf_ctx* c, cudaStream_t s) {
-  switch (n1log) {
-    case 9: launch_cols<512, MODE, SIGN>(in, F, fstride, out, n2log, batch, c, s); break;
-    case 10: launch_cols<1024, MODE, SIGN>(in, F, fstride, out, n2log, batch, c, s); break;
-    case 11: launch_cols<2048, MODE, SIGN>(in, F, fstride, out, n2log, batch, c, s); break;
-    default: launch_cols<4096, MODE, SIGN>(in, F, fstride, out, n2log, batch, c, s); break;
-  }
-}
-
-template <int SIGN>
-void rows_dispatch(int n2log, const float2* in, float2* out, int n1log, int batch, const rf_ctx* c,
-                   cudaStream_t s) {
-  switch (n2log) {
-    case 9: launch_rows<512, SIGN>(in, out, n1log, batch, c, s); break;
-    case 10: launch_rows<1024, SIGN>(in, out, n1log, batch, c, s); break;
-    case 11: launch_rows<2048, SIGN>(in, out, n1log, batch, c, s); break;
-    default: launch_rows<4096, SIGN>(in, out, n1log, batch, c, s); break;
+template <typename F>
+void dispatch_line(int log, F&& f) {
+  switch (log) {
+    case 7: f(std::integral_constant<int, 128>{}); break;
+    case 8: f(std::integral_constant<int, 256>{}); break;
+    case 9: f(std::integral_constant<int, 512>{}); break;
+    case 10: f(std::integral_constant<int, 1024>{}); break;
+    case 11: f(std::integral_constant<int, 2048>{}); break;
+    default: f(std::integral_constant<int, 4096>{}); break;
   }
 }
 
@@ -205,39 +249,72 @@ void split(int64_t n, int& n1log, int& n2log) {
   n2log = b - n1log;
 }
 
-void check(const rf_ctx* c, const void* in, const void* out, const void* tmp, int batch) {
-  RF_REQUIRE(fft4_supported(c->n), "fft4: n=%lld is outside 2^%d .. 2^%d", (long long)c->n, kF4MinLog, kF4MaxLog);
-  RF_REQUIRE(c->tw4.p != nullptr, "fft4: twiddle tables missing");
+// The two passes: columns from `in` (and F) into tmp, rows from tmp into out.
+template <typename V, int MODE, int SIGN>
+void two_passes(const rf_ctx* c, const void* in, const V* F, int64_t fstride, V* out, V* tmp, int batch,
+                cudaStream_t s) {
+  RF_REQUIRE(fft4_supported(c->n, sizeof(V) == 16), "fft4: n=%lld is not supported", (long long)c->n);
+  RF_REQUIRE(sizeof(V) == 16 || c->tw4.p != nullptr, "fft4: twiddle tables missing");
   RF_REQUIRE(batch >= 1 && batch <= 65535, "fft4: batch %d out of range", batch);
   RF_REQUIRE(in != out && in != tmp && out != tmp, "fft4: buffers must be distinct");
+  int n1log, n2log;
+  split(c->n, n1log, n2log);
+  dispatch_line(n1log, [&](auto l) {
+    launch_cols<V, decltype(l)::value, MODE, SIGN>(in, F, fstride, tmp, n2log, batch, c, s);
+  });
+  dispatch_line(n2log, [&](auto l) { launch_rows<V, decltype(l)::value, SIGN>(tmp, out, n1log, batch, c, s); });
 }
 
 }  // namespace
 
-bool fft4_supported(int64_t n) {
+bool fft4_supported(int64_t n, bool f64) {
   if (n <= 0 || (n & (n - 1)) != 0) return false;
   const int b = ilog2(n);
-  return b >= kF4MinLog && b <= kF4MaxLog;
+  return b >= (f64 ? kF4MinLog64 : kF4MinLog) && b <= kF4MaxLog;
 }
 
 int fft4_lo_bits(int64_t n) { return (ilog2(n) + 1) / 2; }
 
 void fft4_forward_real(const rf_ctx* c, const float* x, float2* out, float2* tmp, cudaStream_t s) {
-  check(c, x, out, tmp, 1);
-  int n1log, n2log;
-  split(c->n, n1log, n2log);
-  cols_dispatch<kF4Real, -1>(n1log, x, nullptr, 0, tmp, n2log, 1, c, s);
-  rows_dispatch<-1>(n2log, tmp, out, n1log, 1, c, s);
+  two_passes<float2, kF4Real, -1>(c, x, nullptr, 0, out, tmp, 1, s);
+}
+
+void fft4_forward_real(const rf_ctx* c, const double* x, double2* out, double2* tmp, cudaStream_t s) {
+  two_passes<double2, kF4Real, -1>(c, x, nullptr, 0, out, tmp, 1, s);
 }
 
 void fft4_inverse_product(const rf_ctx* c, const float2* X, const float2* F, int64_t fstride, float2* out,
                           float2* tmp, int batch, cudaStream_t s) {
-  check(c, X, out, tmp, batch);
   RF_REQUIRE(fstride >= c->n / 2 + 1, "fft4: filter stride %lld below n/2 + 1", (long long)fstride);
-  int n1log, n2log;
-  split(c->n, n1log, n2log);
-  cols_dispatch<kF4Product, +1>(n1log, X, F, fstride, tmp, n2log, batch, c, s);
-  rows_dispatch<+1>(n2log, tmp, out, n1log, batch, c, s);
+  two_passes<float2, kF4Product, +1>(c, X, F, fstride, out, tmp, batch, s);
+}
+
+void fft4_inverse_product(const rf_ctx* c, const double2* X, const double2* F, int64_t fstride, double2* out,
+                          double2* tmp, int batch, cudaStream_t s) {
+  RF_REQUIRE(fstride >= c->n / 2 + 1, "fft4: filter stride %lld below n/2 + 1", (long long)fstride);
+  two_passes<double2, kF4Product, +1>(c, X, F, fstride, out, tmp, batch, s);
+}
+
+bool block_mf_supported(const rf_ctx* c) { return c->g.dtype == RF_F32 && c->n >= 512 && c->n <= 16384; }
+
+void block_mf(const rf_ctx* c, const float* x, const float2* F, int64_t fstride, float2* out, int nref,
+              cudaStream_t s) {
+  auto run = [&](auto bc) {
+    constexpr int B = decltype(bc)::value;
+    constexpr size_t smem = sizeof(float2) * BlockFFTShape<B>::SMEM;
+    RF_CUDA(cudaFuncSetAttribute(k_block_mf<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    k_block_mf<B><<<(unsigned)nref, B / 16, smem, s>>>(x, F, fstride, out,
+                                                       block_tables<float2>(c, BlockFFTShape<B>::LOGB));
+    RF_LAUNCHED();
+  };
+  switch (ilog2(c->n)) {
+    case 9: run(std::integral_constant<int, 512>{}); break;
+    case 10: run(std::integral_constant<int, 1024>{}); break;
+    case 11: run(std::integral_constant<int, 2048>{}); break;
+    case 12: run(std::integral_constant<int, 4096>{}); break;
+    case 13: run(std::integral_constant<int, 8192>{}); break;
+    default: run(std::integral_constant<int, 16384>{}); break;
+  }
 }
 
 }  // namespace rf

@@ -243,6 +243,26 @@ void mf_create(rf_ctx* c) {
 
 namespace {
 
+// The context's transforms: two-pass four-step where n allows, else radix passes.
+void forward_real(rf_ctx* c, const float* x, float2* X, float2* tmp, cudaStream_t s) {
+  if (fft4_supported(c->n, false)) fft4_forward_real(c, x, X, tmp, s);
+  else fft_r2c_f32(x, X, tmp, c->n, c->tw32.as<float2>(), c->n, s);
+}
+void forward_real(rf_ctx* c, const double* x, double2* X, double2* tmp, cudaStream_t s) {
+  if (fft4_supported(c->n, true)) fft4_forward_real(c, x, X, tmp, s);
+  else fft_r2c_f64(x, X, tmp, c->n, c->tw64.as<double2>(), c->n, s);
+}
+void inverse_product(rf_ctx* c, const float2* X, const float2* F, int64_t fstride, float2* z, float2* tmp, int cnt,
+                     cudaStream_t s) {
+  if (fft4_supported(c->n, false)) fft4_inverse_product(c, X, F, fstride, z, tmp, cnt, s);
+  else ifft_product_f32(X, F, fstride, z, tmp, c->n, cnt, c->tw32.as<float2>(), c->n, s);
+}
+void inverse_product(rf_ctx* c, const double2* X, const double2* F, int64_t fstride, double2* z, double2* tmp, int cnt,
+                     cudaStream_t s) {
+  if (fft4_supported(c->n, true)) fft4_inverse_product(c, X, F, fstride, z, tmp, cnt, s);
+  else ifft_product_f64(X, F, fstride, z, tmp, c->n, cnt, c->tw64.as<double2>(), c->n, s);
+}
+
 // Filters of a batch, then one product inverse for the batch.
 template <typename V, typename Inverse>
 void mf_batches(rf_ctx* c, const double* inv_psd, const double* sig, int32_t nref, const rf_template* refs,
@@ -264,27 +284,23 @@ void mf_batches(rf_ctx* c, const double* inv_psd, const double* sig, int32_t nre
 
 void mf_reference_impl(rf_ctx* c, const void* x, const double* inv_psd, int32_t nref, const rf_template* refs,
                        void* z_out, double* sigma_out, cudaStream_t s) {
-  const int64_t n = c->n;
   const double* sig = launch_sigma2(c, inv_psd, sigma_out, nref, s);
   if (c->g.dtype == RF_F64) {
-    const double2* tw = c->tw64.as<double2>();
-    fft_r2c_f64(static_cast<const double*>(x), c->xf.as<double2>(), c->fb.as<double2>(), n, tw, n, s);
+    forward_real(c, static_cast<const double*>(x), c->xf.as<double2>(), c->fb.as<double2>(), s);
     mf_batches(c, inv_psd, sig, nref, refs, static_cast<double2*>(z_out),
                [&](const double2* F, int64_t fs, double2* z, double2* tmp, int cnt) {
-                 ifft_product_f64(c->xf.as<double2>(), F, fs, z, tmp, n, cnt, tw, n, s);
+                 inverse_product(c, c->xf.as<double2>(), F, fs, z, tmp, cnt, s);
                }, s);
-  } else if (fft4_supported(n)) {  // two-pass four-step transforms, else radix passes
-    fft4_forward_real(c, static_cast<const float*>(x), c->xf.as<float2>(), c->fb.as<float2>(), s);
+  } else if (block_mf_supported(c)) {
     mf_batches(c, inv_psd, sig, nref, refs, static_cast<float2*>(z_out),
-               [&](const float2* F, int64_t fs, float2* z, float2* tmp, int cnt) {
-                 fft4_inverse_product(c, c->xf.as<float2>(), F, fs, z, tmp, cnt, s);
+               [&](const float2* F, int64_t fs, float2* z, float2*, int cnt) {
+                 block_mf(c, static_cast<const float*>(x), F, fs, z, cnt, s);
                }, s);
   } else {
-    const float2* tw = c->tw32.as<float2>();
-    fft_r2c_f32(static_cast<const float*>(x), c->xf.as<float2>(), c->fb.as<float2>(), n, tw, n, s);
+    forward_real(c, static_cast<const float*>(x), c->xf.as<float2>(), c->fb.as<float2>(), s);
     mf_batches(c, inv_psd, sig, nref, refs, static_cast<float2*>(z_out),
                [&](const float2* F, int64_t fs, float2* z, float2* tmp, int cnt) {
-                 ifft_product_f32(c->xf.as<float2>(), F, fs, z, tmp, n, cnt, tw, n, s);
+                 inverse_product(c, c->xf.as<float2>(), F, fs, z, tmp, cnt, s);
                }, s);
   }
 }
@@ -302,39 +318,29 @@ void reference_filters_impl(rf_ctx* c, const double* inv_psd, int32_t nref, cons
 void mf_filtered_impl(rf_ctx* c, const void* x, int32_t nref, const void* filt, void* z_out, cudaStream_t s) {
   const int64_t n = c->n;
   const int64_t nb = n / 2 + 1;
-  // references per batched inverse transform, bounded by the temporary buffer
-  const int chunk = (int)std::max<int64_t>(1, std::min<int64_t>(nref, std::min<int64_t>(65535, (int64_t)(1 << 27) / n)));
-  if (c->g.dtype == RF_F64) {
-    c->mf_tmp.ensure(sizeof(double2) * (size_t)chunk * n);
-    fft_r2c_f64(static_cast<const double*>(x), c->xf.as<double2>(), c->fb.as<double2>(), n, c->tw64.as<double2>(), n,
-                s);
-    for (int r0 = 0; r0 < nref; r0 += chunk) {
-      const int cnt = std::min(chunk, nref - r0);
-      ifft_product_f64(c->xf.as<double2>(), static_cast<const double2*>(filt) + (int64_t)r0 * nb, nb,
-                       static_cast<double2*>(z_out) + (int64_t)r0 * n, c->mf_tmp.as<double2>(), n, cnt,
-                       c->tw64.as<double2>(), n, s);
-    }
-  } else if (fft4_supported(n)) {
-    // two-pass four-step transforms; the inverses of kF4Chunk references share one launch pair,
-    // whose intermediate (kF4Chunk n complex values) is meant to stay in L2
-    const int c4 = (int)std::min<int64_t>(nref, std::max<int64_t>(1, kF4Chunk / n));
-    c->mf_tmp.ensure(sizeof(float2) * (size_t)c4 * n);
-    fft4_forward_real(c, static_cast<const float*>(x), c->xf.as<float2>(), c->mf_tmp.as<float2>(), s);
-    for (int r0 = 0; r0 < nref; r0 += c4) {
-      const int cnt = std::min(c4, nref - r0);
-      fft4_inverse_product(c, c->xf.as<float2>(), static_cast<const float2*>(filt) + (int64_t)r0 * nb, nb,
-                           static_cast<float2*>(z_out) + (int64_t)r0 * n, c->mf_tmp.as<float2>(), cnt, s);
-    }
-  } else {
-    c->mf_tmp.ensure(sizeof(float2) * (size_t)chunk * n);
-    fft_r2c_f32(static_cast<const float*>(x), c->xf.as<float2>(), c->fb.as<float2>(), n, c->tw32.as<float2>(), n, s);
-    for (int r0 = 0; r0 < nref; r0 += chunk) {
-      const int cnt = std::min(chunk, nref - r0);
-      ifft_product_f32(c->xf.as<float2>(), static_cast<const float2*>(filt) + (int64_t)r0 * nb, nb,
-                       static_cast<float2*>(z_out) + (int64_t)r0 * n, c->mf_tmp.as<float2>(), n, cnt,
-                       c->tw32.as<float2>(), n, s);
-    }
+  if (block_mf_supported(c)) {
+    block_mf(c, static_cast<const float*>(x), static_cast<const float2*>(filt), nb, static_cast<float2*>(z_out), nref,
+             s);
+    return;
   }
+  auto run = [&](auto vtag) {
+    using V = decltype(vtag);
+    using T = typename real_of<V>::type;
+    // references per launch: bounded by the temporary buffer, and for the two-pass four-step
+    // transforms by kF4Chunk values, whose intermediate is meant to stay in L2
+    const int64_t most = fft4_supported(n, sizeof(T) == 8) ? std::max<int64_t>(1, kF4Chunk / n)
+                                                           : std::min<int64_t>(65535, ((int64_t)1 << 27) / n);
+    const int chunk = (int)std::max<int64_t>(1, std::min<int64_t>(nref, most));
+    c->mf_tmp.ensure(sizeof(V) * (size_t)chunk * n);
+    forward_real(c, static_cast<const T*>(x), c->xf.as<V>(), c->mf_tmp.as<V>(), s);
+    for (int r0 = 0; r0 < nref; r0 += chunk) {
+      const int cnt = std::min(chunk, nref - r0);
+      inverse_product(c, c->xf.as<V>(), static_cast<const V*>(filt) + (int64_t)r0 * nb, nb,
+                      static_cast<V*>(z_out) + (int64_t)r0 * n, c->mf_tmp.as<V>(), cnt, s);
+    }
+  };
+  if (c->g.dtype == RF_F64) run(double2{});
+  else run(float2{});
 }
 
 void template_fd_impl(rf_ctx* c, const rf_template& t, void* h_out, cudaStream_t s) {

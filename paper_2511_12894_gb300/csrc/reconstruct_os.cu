@@ -487,7 +487,7 @@ void append_tables(std::vector<float2>& out) {
   };
   if (S::RM > 1) stage(S::RM);
   if (S::MID16) stage(16);
-  stage(16);
+  if (S::LAST16) stage(16);
   if (out.size() - start != (size_t)block_table_size<B>()) throw Fail{RF_EINVAL};
 }
 
@@ -496,6 +496,10 @@ void append_tables(std::vector<float2>& out) {
 std::vector<float2> block_fft_tables(int64_t off[16]) {
   std::vector<float2> out;
   for (int b = 0; b < 16; ++b) off[b] = 0;
+  off[7] = (int64_t)out.size();
+  append_tables<128>(out);
+  off[8] = (int64_t)out.size();
+  append_tables<256>(out);
   off[9] = (int64_t)out.size();
   append_tables<512>(out);
   off[10] = (int64_t)out.size();

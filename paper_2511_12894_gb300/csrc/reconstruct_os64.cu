@@ -255,7 +255,7 @@ constexpr size_t smem64(int H) {
   return sizeof(double2) * BlockFFTShape<B, 1>::SMEM + sizeof(long long) * (size_t)H;
 }
 
-int table64(int B) { return B == 1024 ? 0 : (B == 2048 ? 1 : 2); }
+int table64(int B) { return B == 1024 ? 10 : (B == 2048 ? 11 : 12); }
 
 // Cheapest (B, Q) for the kernel lengths by modelled SM cycles, or B = 0 for the direct sum.  The
 // FP64 pipe runs 1.6 instructions per clock; blocks are spread whole over the SMs, the direct
@@ -365,11 +365,14 @@ void os64_create(rf_ctx* c) {
     };
     if (S::RM > 1) stage(S::RM);
     if (S::MID16) stage(16);
-    stage(16);
+    if (S::LAST16) stage(16);
   };
-  tables(std::integral_constant<int, 1024>{}, 0);
-  tables(std::integral_constant<int, 2048>{}, 1);
-  tables(std::integral_constant<int, 4096>{}, 2);
+  tables(std::integral_constant<int, 128>{}, 7);
+  tables(std::integral_constant<int, 256>{}, 8);
+  tables(std::integral_constant<int, 512>{}, 9);
+  tables(std::integral_constant<int, 1024>{}, 10);
+  tables(std::integral_constant<int, 2048>{}, 11);
+  tables(std::integral_constant<int, 4096>{}, 12);
   c->twb64.ensure(sizeof(double2) * tw.size());
   RF_CUDA(cudaMemcpy(c->twb64.p, tw.data(), sizeof(double2) * tw.size(), cudaMemcpyHostToDevice));
   cudaMemPoolProps props{};

@@ -143,14 +143,14 @@ struct rf_ctx {
   int nsm = 0;
   // Twiddle tables w[m] = exp(-2 pi i m / n), m < n: FP64 and FP32 copies.
   rf::DevBuf tw64, tw32;
-  // Stage twiddle tables of the block FFTs (float2), B = 2^9 .. 2^14; the tables of
+  // Stage twiddle tables of the block FFTs (float2), B = 2^7 .. 2^14; the tables of
   // block size 2^b start at entry twb_off[b].
   rf::DevBuf twb32;
   int64_t twb_off[16] = {0};
-  // FP64 grids: stage twiddle tables of the FP64 block FFTs (B = 1024, 2048, 4096) and the pool of
-  // the FP64 overlap-save calls' workspaces.
+  // FP64 grids: stage twiddle tables of the FP64 block FFTs (B = 2^7 .. 2^12, as twb32) and the pool
+  // of the FP64 overlap-save calls' workspaces.
   rf::DevBuf twb64;
-  int64_t twb64_off[3] = {0};
+  int64_t twb64_off[16] = {0};
   cudaMemPool_t pool = nullptr;
   // Four-step FFT twiddles (float2): w[m] = exp(-2 pi i m / n) for m < 2^tw4_lo_bits, then
   // w[2^tw4_lo_bits m] for m < n / 2^tw4_lo_bits; empty where the four-step FFT does not apply.
@@ -294,14 +294,23 @@ void ifft_product_f32(const float2* X, const float2* F, int64_t fstride, float2*
                       int batch, const float2* tw, int64_t table_n, cudaStream_t s);
 void fft_c2c_f32(const float2* in, float2* out, float2* tmp, int64_t n, int batch, int sign,
                  const float2* tw_table, int64_t table_n, cudaStream_t s);
-// Four-step FP32 transforms of the context's n (fft4.cu), for n = 2^18 .. 2^24: two passes
-// through HBM.  Forward of real data (natural order out) and the inverse of the one-sided product X[k] F_r[k] (k <= n/2, zero above;
-// row r of F at r fstride).  tmp holds batch n complex values.
-bool fft4_supported(int64_t n);
+// Four-step transforms of the context's n (fft4.cu) in two passes through HBM, and for FP32 up to
+// 2^14 points a whole matched filter per thread block.  Forward of real data (natural order out) and
+// the inverse of the one-sided product X[k] F_r[k] (k <= n/2, zero above; row r of F at r fstride).
+// tmp holds batch n complex values.
+bool fft4_supported(int64_t n, bool f64);
 int fft4_lo_bits(int64_t n);
 void fft4_forward_real(const rf_ctx* c, const float* x, float2* out, float2* tmp, cudaStream_t s);
+void fft4_forward_real(const rf_ctx* c, const double* x, double2* out, double2* tmp, cudaStream_t s);
 void fft4_inverse_product(const rf_ctx* c, const float2* X, const float2* F, int64_t fstride, float2* out,
                           float2* tmp, int batch, cudaStream_t s);
+void fft4_inverse_product(const rf_ctx* c, const double2* X, const double2* F, int64_t fstride, double2* out,
+                          double2* tmp, int batch, cudaStream_t s);
+// FP32, n = 512 .. 16384: the spectrum of x and the inverse transforms of its products with `nref`
+// filters (rows of fstride >= n/2 + 1) in one launch.
+bool block_mf_supported(const rf_ctx* c);
+void block_mf(const rf_ctx* c, const float* x, const float2* F, int64_t fstride, float2* out, int nref,
+              cudaStream_t s);
 // Forward transform of real data (natural order, unnormalised).
 void fft_r2c_f64(const double* x, double2* out, double2* tmp, int64_t n, const double2* tw, int64_t table_n,
                  cudaStream_t s);
@@ -313,7 +322,7 @@ std::vector<double2> host_twiddles(int64_t n);
 // first context of the process)
 constexpr int64_t kBlockTwiddles = 32768;
 const std::vector<double2>& block_twiddles();
-// Stage twiddle tables of the block FFTs for B = 2^9 .. 2^14 (float2, concatenated), with
+// Stage twiddle tables of the block FFTs for B = 2^7 .. 2^14 (float2, concatenated), with
 // the entry offset of each block size in off[log2 B].
 std::vector<float2> block_fft_tables(int64_t off[16]);
 

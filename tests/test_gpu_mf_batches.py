@@ -31,3 +31,25 @@ def test_rows_equal_single_calls(dtype, n, nref):
     assert torch.equal(sf, sg)
     tol = 1e-12 if dtype == "f64" else 2e-6
     assert (zf - z).abs().max().item() <= tol * z.abs().max().item()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("log2n", list(range(8, 19)) + [20])
+def test_every_size_against_a_64_bit_transform(dtype, log2n):
+    """One-block, four-step (every line length) and radix-pass transforms of the stored-filter
+    matched filter; an odd number of references."""
+    torch = pytest.importorskip("torch")
+    from paper_2511_12894_gb300 import RatioFilter
+    n, nref = 1 << log2n, 3
+    rf = RatioFilter(n, 2048.0, 20.0, 971.0, 7, dtype)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(log2n)
+    x = torch.randn(n, dtype=torch.float64, device="cuda", generator=g).to(rf.rdtype)
+    f = torch.randn((nref, n // 2 + 1, 2), dtype=torch.float64, device="cuda", generator=g)
+    filt = torch.view_as_complex(f).to(rf.cdtype)
+    z = rf.mf_filtered(x, filt)
+    full = torch.zeros((nref, n), dtype=torch.complex128, device="cuda")
+    full[:, : n // 2 + 1] = torch.fft.rfft(x.double()) * filt.to(torch.complex128)
+    want = torch.fft.ifft(full) * n
+    tol = 1e-12 if dtype == "f64" else 2e-6
+    assert (z - want).abs().max().item() <= tol * want.abs().max().item()
