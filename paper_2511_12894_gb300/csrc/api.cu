@@ -43,6 +43,16 @@ void DevBuf::ensure(size_t b) {
   bytes = b;
 }
 
+void pool_create(rf_ctx* c) {
+  cudaMemPoolProps props{};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = c->device;
+  RF_CUDA(cudaMemPoolCreate(&c->pool, &props));
+  unsigned long long keep = 2ull << 30;  // what is above goes back to the device at a synchronisation
+  RF_CUDA(cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep));
+}
+
 namespace {
 
 bool is_pow2(int64_t n) { return n > 0 && (n & (n - 1)) == 0; }
@@ -157,6 +167,7 @@ rf_status rf_create(const rf_grid* grid, rf_ctx** out) {
     c->fa.ensure(esz * n);
     c->fb.ensure(esz * n);
     c->red.ensure(sizeof(double) * 1024);
+    pool_create(c.get());
     mf_create(c.get());
     if (g.dtype == RF_F64) os64_create(c.get());
     c->status.ensure(sizeof(int) * 4);

@@ -132,18 +132,37 @@ __global__ void __launch_bounds__(256) k_kernel_spectrum(const Tf2Bins* __restri
 
 __device__ __forceinline__ double mag2_rn(double2 v) { return __dadd_rn(__dmul_rn(v.x, v.x), __dmul_rn(v.y, v.y)); }
 
-__global__ void __launch_bounds__(1024) k_row_max2(const double2* __restrict__ rho, int64_t n, double* __restrict__ out) {
-  const double2* r = rho + (int64_t)blockIdx.x * n;
-  double m = 0.0;
-  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) m = fmax(m, mag2_rn(r[i]));
-  __shared__ double sh[1024];
-  sh[threadIdx.x] = m;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) sh[threadIdx.x] = fmax(sh[threadIdx.x], sh[threadIdx.x + s]);
-    __syncthreads();
+// The magnitudes are compared as integers (non-negative doubles order as their bits) and formed only
+// where they can matter: a value whose parts are both below `floor_hi` (high words) has
+// x^2 + y^2 below the bound that gave floor_hi, so the FP64 pipe (two lanes per SM) is left out of
+// most of the rows.
+__device__ __forceinline__ unsigned part_hi(double2 v) {
+  return max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu);
+}
+// High word below which both parts of a value with x^2 + y^2 >= m2 cannot lie: of sqrt(m2 / 2) (1 - 2^-19).
+__device__ __forceinline__ unsigned floor_hi(double m2) {
+  return (unsigned)__double2hiint(sqrt(0.5 * m2) * (1.0 - 1.9073486328125e-06));
+}
+
+// max |rho|^2 of a row's part (blockIdx.x of gridDim.x, row blockIdx.y) into amax2 (bits; 0 before).
+// One block per row left most SMs idle: 612 us for 48 rows of 2^19 values.
+__global__ void __launch_bounds__(256) k_row_max2(const double2* __restrict__ rho, int64_t n,
+                                                  unsigned long long* __restrict__ amax2) {
+  const double2* r = rho + (int64_t)blockIdx.y * n;
+  unsigned long long m = 0;
+  unsigned lim = 0;
+  for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
+    const double2 v = r[i];
+    if (part_hi(v) < lim) continue;
+    const double a = mag2_rn(v);
+    if (a > __longlong_as_double((long long)m)) {  // NaN never counts
+      m = (unsigned long long)__double_as_longlong(a);
+      lim = floor_hi(a);
+    }
   }
-  if (threadIdx.x == 0) out[blockIdx.x] = sh[0];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0 && m) atomicMax(amax2 + blockIdx.y, m);
 }
 
 struct ArcBest {
@@ -159,54 +178,90 @@ __device__ __forceinline__ void arc_take(ArcBest& b, long long gap, long long m,
   }
 }
 
-// Shortest covering arc of {m : |rho[m]|^2 >= cut2}, one block per template.
-// Each thread summarises a contiguous range (first kept, last kept, best internal gap);
-// thread 0 joins the summaries in order and closes the circle.
-__global__ void __launch_bounds__(1024) k_arc(const double2* __restrict__ rho, int64_t n,
-                                              const double* __restrict__ amax2, double thr, int relative,
-                                              int* __restrict__ m0_out, int* __restrict__ len_out) {
-  const int j = blockIdx.x;
+// Kept lags of a contiguous range: first and last (-1: none) and the widest gap between two
+// consecutive ones with the lag after it.
+struct ArcPart {
+  long long first, last;
+  ArcBest best;
+};
+
+// b followed by a later range c
+__device__ __forceinline__ void arc_join(ArcPart& b, const ArcPart& c, long long n) {
+  if (c.first < 0) return;
+  if (b.last >= 0) arc_take(b.best, c.first - b.last - 1, c.first, n);
+  if (c.best.gap >= 0) arc_take(b.best, c.best.gap, c.best.m0, n);
+  if (b.first < 0) b.first = c.first;
+  b.last = c.last;
+}
+
+// Shortest covering arc of {m : |rho[m]|^2 >= cut2}, first step: a warp summarises `per` consecutive
+// lags, 32 at a time by ballot.  (One block per row with a range per thread read its 2^19 values at a
+// stride: 676 us for 48 rows.)
+__global__ void __launch_bounds__(256) k_arc_parts(const double2* __restrict__ rho, int64_t n, int per, int nparts,
+                                                   const double* __restrict__ amax2, double thr, int relative,
+                                                   ArcPart* __restrict__ parts) {
+  const int j = blockIdx.y;
+  const int part = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (part >= nparts) return;
+  const int lane = threadIdx.x & 31;
   const double2* r = rho + (int64_t)j * n;
   const double cut2 = __dmul_rn(__dmul_rn(thr, thr), relative ? amax2[j] : 1.0);
-  const int nt = blockDim.x;
-  const int64_t ch = n / nt;
-  const int t = threadIdx.x;
-  long long first = -1, last = -1;
-  ArcBest b{-1, 0};
-  const bool any = relative ? (amax2[j] > 0.0) : true;
-  if (any) {
-    for (int64_t m = (int64_t)t * ch; m < (int64_t)(t + 1) * ch; ++m) {
-      if (mag2_rn(r[m]) >= cut2) {
-        if (last >= 0) arc_take(b, m - last - 1, m, n);
-        if (first < 0) first = m;
-        last = m;
+  const unsigned lim = floor_hi(cut2);
+  ArcPart b{-1, -1, {-1, 0}};
+  if (!relative || amax2[j] > 0.0) {
+    const int64_t lo = (int64_t)part * per, hi = min(n, lo + per);
+    for (int64_t base = lo; base < hi; base += 32) {
+      const int64_t m = base + lane;
+      bool keep = false;
+      if (m < hi) {
+        const double2 v = r[m];
+        if (part_hi(v) >= lim) keep = mag2_rn(v) >= cut2;
       }
+      const unsigned mask = __ballot_sync(0xffffffffu, keep);
+      if (!mask) continue;
+      const int f = __ffs(mask) - 1;
+      if (b.last >= 0) arc_take(b.best, base + f - b.last - 1, base + f, n);
+      if (b.first < 0) b.first = base + f;
+      // the lags after the first of the group: all of them while no gap is known, else only those
+      // that follow a gap
+      unsigned rest = mask & (mask - 1);
+      if (b.best.gap > 0) rest &= ~(mask << 1);
+      while (rest) {
+        const int q = __ffs(rest) - 1;
+        rest &= rest - 1;
+        const int before = 31 - __clz(mask & ((1u << q) - 1u));
+        arc_take(b.best, q - before - 1, base + q, n);
+      }
+      b.last = base + 31 - __clz(mask);
     }
   }
-  __shared__ long long s_first[1024], s_last[1024], s_gap[1024], s_m0[1024];
-  s_first[t] = first;
-  s_last[t] = last;
-  s_gap[t] = b.gap;
-  s_m0[t] = b.m0;
-  __syncthreads();
-  if (t == 0) {
-    long long gfirst = -1, glast = -1;
-    ArcBest g{-1, 0};
-    for (int q = 0; q < nt; ++q) {
-      if (s_first[q] < 0) continue;
-      if (glast >= 0) arc_take(g, s_first[q] - glast - 1, s_first[q], n);
-      if (s_gap[q] >= 0) arc_take(g, s_gap[q], s_m0[q], n);
-      if (gfirst < 0) gfirst = s_first[q];
-      glast = s_last[q];
-    }
-    if (gfirst < 0) {
-      m0_out[j] = 0;
-      len_out[j] = 0;
-    } else {
-      arc_take(g, gfirst + n - glast - 1, gfirst, n);
-      m0_out[j] = (int)arc_key(g.m0, n);
-      len_out[j] = (int)(n - g.gap);
-    }
+  if (lane == 0) parts[(int64_t)j * nparts + part] = b;
+}
+
+// Second step, a warp per row: the ranges joined in order, then the circle closed.
+__global__ void __launch_bounds__(32) k_arc_join(const ArcPart* __restrict__ parts, int nparts, int64_t n,
+                                                 int* __restrict__ m0_out, int* __restrict__ len_out) {
+  const int j = blockIdx.x, lane = threadIdx.x;
+  const int ch = (nparts + 31) / 32;
+  ArcPart b{-1, -1, {-1, 0}};
+  for (int q = lane * ch; q < min(nparts, (lane + 1) * ch); ++q) arc_join(b, parts[(int64_t)j * nparts + q], n);
+  ArcPart g{-1, -1, {-1, 0}};
+  for (int l = 0; l < 32; ++l) {
+    ArcPart c;
+    c.first = __shfl_sync(0xffffffffu, b.first, l);
+    c.last = __shfl_sync(0xffffffffu, b.last, l);
+    c.best.gap = __shfl_sync(0xffffffffu, b.best.gap, l);
+    c.best.m0 = __shfl_sync(0xffffffffu, b.best.m0, l);
+    arc_join(g, c, n);
+  }
+  if (lane) return;
+  if (g.first < 0) {
+    m0_out[j] = 0;
+    len_out[j] = 0;
+  } else {
+    arc_take(g.best, g.first + n - g.last - 1, g.first, n);
+    m0_out[j] = (int)arc_key(g.best.m0, n);
+    len_out[j] = (int)(n - g.best.gap);
   }
 }
 
@@ -269,11 +324,10 @@ rf_kernels* build_impl(rf_ctx* c, const rf_template& ref, const rf_template* nbr
   // device scratch: [Tf2 k][dfl k][extent k][Tf2 k, grid order][dfl k, grid order]
   // [phase differences][amax2][m0][len]
   const int64_t kmax_chunk = std::min<int64_t>(k, 4096);
-  DevBuf meta;
   const size_t meta_bytes = 2 * sizeof(Tf2) * (size_t)k + sizeof(double) * (3 * (size_t)k + 8 + kmax_chunk) +
                             (sizeof(Tf2Bins) + 2 * sizeof(int)) * (size_t)kmax_chunk + 8192;
-  meta.ensure(meta_bytes);
-  char* mp = static_cast<char*>(meta.p);
+  StreamBuf meta(c, meta_bytes, s);
+  char* mp = meta.need().as<char>();
   auto carve = [&](size_t bytes) {
     char* r = mp;
     mp += (bytes + 255) & ~(size_t)255;
@@ -288,7 +342,7 @@ rf_kernels* build_impl(rf_ctx* c, const rf_template& ref, const rf_template* nbr
   double* d_amax = reinterpret_cast<double*>(carve(sizeof(double) * kmax_chunk));
   int* d_m0 = reinterpret_cast<int*>(carve(sizeof(int) * kmax_chunk));
   int* d_len = reinterpret_cast<int*>(carve(sizeof(int) * kmax_chunk));
-  RF_REQUIRE((size_t)(mp - static_cast<char*>(meta.p)) <= meta_bytes, "builder: scratch layout");
+  RF_REQUIRE((size_t)(mp - meta.as<char>()) <= meta_bytes, "builder: scratch layout");
 
   std::vector<Tf2> tg(k);
   for (int j = 0; j < k; ++j) tg[j] = make_tf2(nbrs[j], c->g.pn_order);
@@ -318,7 +372,12 @@ rf_kernels* build_impl(rf_ctx* c, const rf_template& ref, const rf_template* nbr
   std::vector<int> order(k);
   for (int j = 0; j < k; ++j) order[j] = j;
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return kern->grid[a] < kern->grid[b]; });
-  {
+  bool identity = true;
+  for (int q = 0; q < k && identity; ++q) identity = order[q] == q;
+  if (identity) {
+    d_tgs = d_tg;
+    d_dfls = d_dfl;
+  } else {
     std::vector<Tf2> tgs(k);
     std::vector<double> dfls(k);
     for (int q = 0; q < k; ++q) {
@@ -330,21 +389,38 @@ rf_kernels* build_impl(rf_ctx* c, const rf_template& ref, const rf_template* nbr
     RF_CUDA(cudaStreamSynchronize(s));  // the host vectors go out of scope
   }
 
-  // per kernel: its taps in a part buffer (one per chunk) and its place there
-  std::vector<std::unique_ptr<DevBuf>> parts;
+  // per kernel: its taps in a part buffer (one per chunk) and its place there; a build of a single
+  // chunk packs straight into the kernel set
+  std::vector<std::unique_ptr<StreamBuf>> parts;
   std::vector<int> part_of(k);
   std::vector<int64_t> at_in_part(k);
   std::vector<int> hm0(kmax_chunk), hlen(kmax_chunk);
-  DevBuf rows;
   std::vector<Tf2Bins> dq;
+  std::vector<std::vector<int64_t>> off_host;
+  // templates per chunk: three complex128 rows of nb per template, about 1.5 GB in total
+  auto chunk_at = [&](int q0) {
+    const int64_t nb = kern->grid[order[q0]];
+    const int64_t per = 3 * nb * (int64_t)sizeof(double2);
+    const int64_t most = std::min<int64_t>(kmax_chunk, std::max<int64_t>(1, ((int64_t)1536 << 20) / per));
+    int cnt = 0;
+    while (q0 + cnt < k && cnt < most && kern->grid[order[q0 + cnt]] == nb) ++cnt;
+    return cnt;
+  };
+  size_t rows_bytes = 0;
+  for (int q0 = 0; q0 < k;) {
+    const int cnt = chunk_at(q0);
+    rows_bytes = std::max(rows_bytes, (size_t)3 * cnt * kern->grid[order[q0]] * sizeof(double2));
+    q0 += cnt;
+  }
+  StreamBuf rows(c, rows_bytes, s);
+  rows.need();
+  constexpr int kArcParts = 256;  // warps per row at most
+  StreamBuf arcs(c, sizeof(ArcPart) * kArcParts * (size_t)kmax_chunk, s);
+  arcs.need();
+  const bool one_chunk = identity && chunk_at(0) == k;
   for (int q0 = 0; q0 < k;) {
     const int64_t nb = kern->grid[order[q0]];
-    // templates per chunk: three complex128 rows of nb per template, about 1.5 GB in total
-    const int64_t per = 3 * nb * (int64_t)sizeof(double2);
-    int64_t chunk = std::max<int64_t>(1, ((int64_t)1536 << 20) / per);
-    chunk = std::min<int64_t>(chunk, kmax_chunk);
-    int cnt = 0;
-    while (q0 + cnt < k && cnt < chunk && kern->grid[order[q0 + cnt]] == nb) ++cnt;
+    const int cnt = chunk_at(q0);
     const double dfb = c->g.fs / (double)nb;
     rf_grid gb = c->g;
     gb.n = nb;
@@ -354,7 +430,6 @@ rf_kernels* build_impl(rf_ctx* c, const rf_template& ref, const rf_template* nbr
     dq.resize(cnt);  // read by the copy until the chunk's synchronisation below
     for (int q = 0; q < cnt; ++q) dq[q] = tf2_bins_minus(make_tf2_bins(tg[order[q0 + q]], dfb), qr);
     RF_CUDA(cudaMemcpyAsync(d_dq, dq.data(), sizeof(Tf2Bins) * cnt, cudaMemcpyHostToDevice, s));
-    rows.ensure((size_t)3 * cnt * nb * sizeof(double2));
     double2* bufK = rows.as<double2>();
     double2* bufR = bufK + cnt * nb;
     double2* bufT = bufR + cnt * nb;
@@ -367,7 +442,9 @@ rf_kernels* build_impl(rf_ctx* c, const rf_template& ref, const rf_template* nbr
       k_real_form<<<(unsigned)std::min<int64_t>(4096, (cnt * nb + 255) / 256), 256, 0, s>>>(bufR, cnt * nb);
       RF_LAUNCHED();
     }
-    k_row_max2<<<cnt, 1024, 0, s>>>(bufR, nb, d_amax);
+    RF_CUDA(cudaMemsetAsync(d_amax, 0, sizeof(double) * cnt, s));
+    const unsigned mx = (unsigned)std::max<int64_t>(1, std::min<int64_t>(nb / 2048, (8LL * c->nsm + cnt - 1) / cnt));
+    k_row_max2<<<dim3(mx, (unsigned)cnt), 256, 0, s>>>(bufR, nb, reinterpret_cast<unsigned long long*>(d_amax));
     RF_LAUNCHED();
     if (relative & RF_TRUNC_ANALYTIC) {
       k_analytic_span<<<(cnt + 63) / 64, 64, 0, s>>>(pr, d_tgs + q0, d_dfls + q0, d_amax, cnt, thr,
@@ -375,8 +452,12 @@ rf_kernels* build_impl(rf_ctx* c, const rf_template& ref, const rf_template* nbr
                                                      (relative & RF_KERNEL_REAL) ? 1.0 : 2.0, nb, c->g.fs,
                                                      c->g.f_low, c->g.f_high, c->g.df_high, d_m0, d_len);
     } else {
-      const int nt = (int)std::min<int64_t>(1024, nb);
-      k_arc<<<cnt, nt, 0, s>>>(bufR, nb, d_amax, thr, relative & RF_TRUNC_RELATIVE, d_m0, d_len);
+      const int per = (int)std::max<int64_t>(32, nb / kArcParts);
+      const int np = (int)((nb + per - 1) / per);
+      k_arc_parts<<<dim3((unsigned)((np + 7) / 8), (unsigned)cnt), 256, 0, s>>>(
+          bufR, nb, per, np, d_amax, thr, relative & RF_TRUNC_RELATIVE, arcs.as<ArcPart>());
+      RF_LAUNCHED();
+      k_arc_join<<<cnt, 32, 0, s>>>(arcs.as<ArcPart>(), np, nb, d_m0, d_len);
     }
     RF_LAUNCHED();
     RF_CUDA(cudaMemcpyAsync(hm0.data(), d_m0, sizeof(int) * cnt, cudaMemcpyDeviceToHost, s));
@@ -391,32 +472,34 @@ rf_kernels* build_impl(rf_ctx* c, const rf_template& ref, const rf_template* nbr
       at_in_part[j] = off[q];
       off[q + 1] = off[q] + hlen[q];
     }
-    std::unique_ptr<DevBuf> part(new DevBuf());
-    part->ensure(std::max<size_t>(16, (size_t)off[cnt] * esz));
-    DevBuf offd;
-    offd.ensure(sizeof(int64_t) * (cnt + 1));
-    RF_CUDA(cudaMemcpyAsync(offd.p, off.data(), sizeof(int64_t) * (cnt + 1), cudaMemcpyHostToDevice, s));
+    void* dst;
+    if (one_chunk) {
+      kern->taps.ensure(std::max<size_t>(16, (size_t)off[cnt] * esz));
+      dst = kern->taps.p;
+    } else {
+      parts.emplace_back(new StreamBuf(c, (size_t)off[cnt] * esz, s));
+      dst = parts.back()->need().p;
+    }
+    StreamBuf offd(c, sizeof(int64_t) * (cnt + 1), s);
+    RF_CUDA(cudaMemcpyAsync(offd.need().p, off.data(), sizeof(int64_t) * (cnt + 1), cudaMemcpyHostToDevice, s));
     dim3 g2(64, (unsigned)cnt);
     if (real_form && f64)
-      k_pack_real<double><<<g2, 256, 0, s>>>(bufR, nb, d_m0, d_len, offd.as<int64_t>(), part->as<double>());
+      k_pack_real<double><<<g2, 256, 0, s>>>(bufR, nb, d_m0, d_len, offd.as<int64_t>(), static_cast<double*>(dst));
     else if (real_form)
-      k_pack_real<float><<<g2, 256, 0, s>>>(bufR, nb, d_m0, d_len, offd.as<int64_t>(), part->as<float>());
+      k_pack_real<float><<<g2, 256, 0, s>>>(bufR, nb, d_m0, d_len, offd.as<int64_t>(), static_cast<float*>(dst));
     else if (f64)
-      k_pack<double2><<<g2, 256, 0, s>>>(bufR, nb, d_m0, d_len, offd.as<int64_t>(), part->as<double2>());
+      k_pack<double2><<<g2, 256, 0, s>>>(bufR, nb, d_m0, d_len, offd.as<int64_t>(), static_cast<double2*>(dst));
     else
-      k_pack<float2><<<g2, 256, 0, s>>>(bufR, nb, d_m0, d_len, offd.as<int64_t>(), part->as<float2>());
+      k_pack<float2><<<g2, 256, 0, s>>>(bufR, nb, d_m0, d_len, offd.as<int64_t>(), static_cast<float2*>(dst));
     RF_LAUNCHED();
-    RF_CUDA(cudaStreamSynchronize(s));  // offd and the rows are reused
-    parts.push_back(std::move(part));
+    off_host.push_back(std::move(off));  // read by the copy above
     q0 += cnt;
   }
   for (int j = 0; j < k; ++j) kern->offset[j + 1] = kern->offset[j] + kern->len[j];
   const int64_t total = kern->offset[k];
-  kern->taps.ensure(std::max<size_t>(16, (size_t)total * esz));
   // taps in neighbour order: one copy per part when the order is unchanged, else one per kernel
-  bool identity = true;
-  for (int q = 0; q < k && identity; ++q) identity = order[q] == q;
-  if (identity) {
+  if (one_chunk) {
+  } else if (kern->taps.ensure(std::max<size_t>(16, (size_t)total * esz)), identity) {
     int64_t at = 0;
     for (size_t pi = 0; pi < parts.size(); ++pi) {
       int64_t elems = 0;

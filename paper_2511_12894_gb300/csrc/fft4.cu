@@ -33,13 +33,93 @@ namespace rf {
 
 namespace {
 
+// FP64 lines of up to 1024 points: four points per thread, radix-4 stages in place (with one radix-2
+// stage when log2(L) is odd), the same digit-reversed scheme as blockfft.cuh.  The FP64 pipe gives
+// each of an SM's four partitions half a lane, so a warp alone on a partition takes 64 clocks per
+// FP64 instruction and a pass wants a warp on every partition: with 16 points per thread the 128 warps
+// of a 2^16-point pass took 16 to 25 us, whatever the tile.  A radix-4 stage costs 28 FP64 instructions for
+// four points and two levels, 3.5 per point and level; radix 16 costs 3.7.
+// Thread tid holds x[tid + t L/4] before and X[tid + t L/4] after; w: exp(-2 pi i m / 4096).
+// Shared memory: L + L/8 values.
+constexpr int kRoots64 = 4096;
+__device__ __forceinline__ int quad_pad(int l) { return l + (l >> 3); }
+
+template <int L, int SIGN>
+__device__ __forceinline__ void quad_fft(double2 (&v)[4], double2* sm, const double2* __restrict__ w, int tid) {
+  constexpr int NT = L / 4;
+  constexpr int LOG = L == 128 ? 7 : L == 256 ? 8 : L == 512 ? 9 : 10;
+  static_assert(L <= 1024 && (1 << LOG) == L, "line length");
+  constexpr int RM = 1 << (LOG & 1);
+  dft<4, SIGN>(v);
+  {
+    // location of digit t: 4 r + t, r = the digits of tid (RM first, then fours) reversed
+    int rest = tid, r = 0, place = 1;
+    if (RM > 1) {
+      r = rest / (NT / RM);
+      rest %= NT / RM;
+      place = RM;
+    }
+#pragma unroll
+    for (int m = NT / RM / 4; m >= 1; m /= 4) {
+      r += place * (rest / m);
+      rest %= m;
+      place *= 4;
+    }
+#pragma unroll
+    for (int t = 0; t < 4; ++t) sm[quad_pad(4 * r + t)] = v[t];
+  }
+  __syncthreads();
+  int S = 4;
+  if constexpr (RM > 1) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int b = tid + q * NT, lo = b & 3, l = (b >> 2) * 8 + lo;
+      double2 a[2] = {sm[quad_pad(l)], sm[quad_pad(l + 4)]};
+      a[1] = tw_apply<SIGN>(a[1], __ldg(w + lo * (kRoots64 / 8)));
+      dft<2, SIGN>(a);
+      sm[quad_pad(l)] = a[0];
+      sm[quad_pad(l + 4)] = a[1];
+    }
+    __syncthreads();
+    S = 8;
+  }
+#pragma unroll
+  for (; S < L; S *= 4) {
+    const int lo = tid & (S - 1), l = (tid - lo) * 4 + lo;
+    const int step = kRoots64 / (4 * S);
+#pragma unroll
+    for (int t = 0; t < 4; ++t) v[t] = sm[quad_pad(l + t * S)];
+#pragma unroll
+    for (int t = 1; t < 4; ++t) v[t] = tw_apply<SIGN>(v[t], __ldg(w + t * lo * step));
+    dft<4, SIGN>(v);
+    if (4 * S < L) {
+#pragma unroll
+      for (int t = 0; t < 4; ++t) sm[quad_pad(l + t * S)] = v[t];
+      __syncthreads();
+    }
+  }
+}
+
+// Points per thread and the transform of a line.
+template <typename V, int L>
+constexpr int f4_points() {
+  return sizeof(V) == 16 && L <= 1024 ? 4 : 16;
+}
+
+template <int L, int SIGN, typename V, int N>
+__device__ __forceinline__ void line_fft(V (&v)[N], V* sm, const V* __restrict__ tw, int tid) {
+  if constexpr (N == 4) quad_fft<L, SIGN>(v, sm, tw, tid);
+  else block_fft<L, SIGN>(v, sm, tw, tid);
+}
+
 constexpr int kF4Real = 0;
 constexpr int kF4Product = 1;
 
 // Values of one line's shared-memory region in a tile of G lines.
 template <typename V, int L, int G>
 __host__ __device__ constexpr int f4_line() {
-  return BlockFFTShape<L, 16 / (int)sizeof(V)>::SMEM + 128 / (int)sizeof(V) / G;
+  return (f4_points<V, L>() == 4 ? L + L / 8 : BlockFFTShape<L, 16 / (int)sizeof(V)>::SMEM) +
+         128 / (int)sizeof(V) / G;
 }
 
 template <typename V, int L, int G>
@@ -51,12 +131,13 @@ extern __shared__ __align__(16) unsigned char f4_raw[];
 
 // Pass 1: columns col0 .. col0 + G - 1 of batch row blockIdx.y; L = N1.
 template <typename V, int L, int G, int MODE, int SIGN>
-__global__ void __launch_bounds__(G * L / 16) k_fft4_cols(const void* __restrict__ in, const V* __restrict__ F,
+__global__ void __launch_bounds__(G * L / f4_points<V, L>()) k_fft4_cols(const void* __restrict__ in, const V* __restrict__ F,
                                                           int64_t fstride, V* __restrict__ out, int n2log,
                                                           const V* __restrict__ twb, const V* __restrict__ tw4,
                                                           int lo_bits) {
   using T = typename real_of<V>::type;
-  constexpr int NT = L / 16;
+  constexpr int NP = f4_points<V, L>();
+  constexpr int NT = L / NP;
   V* f4_sm = reinterpret_cast<V*>(f4_raw);
   const int c = (int)threadIdx.x % G;
   const int ltid = (int)threadIdx.x / G;
@@ -67,11 +148,11 @@ __global__ void __launch_bounds__(G * L / 16) k_fft4_cols(const void* __restrict
   // element (a = ltid + t NT, col) sits at j0 + t NT N2
   const int64_t j0 = (int64_t)ltid * N2 + col;
   const int64_t tstep = (int64_t)NT * N2;
-  V v[16];
+  V v[NP];
   if constexpr (MODE == kF4Real) {
     const T* p = static_cast<const T*>(in) + boff + j0;
 #pragma unroll
-    for (int t = 0; t < 16; ++t) v[t] = cmake<V>(p[t * tstep], (T)0);
+    for (int t = 0; t < NP; ++t) v[t] = cmake<V>(p[t * tstep], (T)0);
   } else {
     // X is one spectrum shared by the batch; F holds one filter of n/2 + 1 values per row.
     // Rows a > N1/2 lie above n/2 (zero); row N1/2 holds only column 0.
@@ -79,17 +160,17 @@ __global__ void __launch_bounds__(G * L / 16) k_fft4_cols(const void* __restrict
     const V* pf = F + (int64_t)blockIdx.y * fstride + j0;
     const int64_t lim = n / 2 - j0;
 #pragma unroll
-    for (int t = 0; t < 16; ++t)
+    for (int t = 0; t < NP; ++t)
       v[t] = t * tstep <= lim ? cmul(px[t * tstep], pf[t * tstep]) : cmake<V>((T)0, (T)0);
   }
-  block_fft<L, SIGN>(v, f4_sm + c * f4_line<V, L, G>(), twb, ltid);
-  // v[u] holds the column's bin k1 = ltid + NT u, u < 16, which goes to row k1: o + NT u N2.
+  line_fft<L, SIGN>(v, f4_sm + c * f4_line<V, L, G>(), twb, ltid);
+  // v[u] holds the column's bin k1 = ltid + NT u, u < NP, which goes to row k1: o + NT u N2.
   V* o = out + boff + j0;
   if constexpr (sizeof(T) == 8) {
     const V* w = tw4 + col * ltid;
     const int64_t step = col * NT;
 #pragma unroll
-    for (int u = 0; u < 16; ++u) o[(int64_t)(u * NT) * N2] = tw_apply<SIGN>(v[u], __ldg(w + u * step));
+    for (int u = 0; u < NP; ++u) o[(int64_t)(u * NT) * N2] = tw_apply<SIGN>(v[u], __ldg(w + u * step));
     return;
   } else {
   // Twiddle w_n^(col k1) = w_n^(col ltid) e^u with e = w_n^(col NT): e, e^2, e^4 and e^8 come
@@ -122,9 +203,10 @@ __global__ void __launch_bounds__(G * L / 16) k_fft4_cols(const void* __restrict
 
 // Pass 2: rows row0 .. row0 + R - 1 of batch row blockIdx.y; L = N2.  Output k1 + N1 k2.
 template <typename V, int L, int R, int SIGN>
-__global__ void __launch_bounds__(R * L / 16) k_fft4_rows(const V* __restrict__ in, V* __restrict__ out, int n1log,
+__global__ void __launch_bounds__(R * L / f4_points<V, L>()) k_fft4_rows(const V* __restrict__ in, V* __restrict__ out, int n1log,
                                                           const V* __restrict__ twb) {
-  constexpr int NT = L / 16;
+  constexpr int NP = f4_points<V, L>();
+  constexpr int NT = L / NP;
   constexpr int SL = f4_line<V, L, R>();
   V* f4_sm = reinterpret_cast<V*>(f4_raw);
   const int g = (int)threadIdx.x / NT;
@@ -133,18 +215,18 @@ __global__ void __launch_bounds__(R * L / 16) k_fft4_rows(const V* __restrict__ 
   const int64_t n = N1 * L;
   const int64_t row0 = (int64_t)blockIdx.x * R;
   const V* src = in + (int64_t)blockIdx.y * n + (row0 + g) * L;
-  V v[16];
+  V v[NP];
 #pragma unroll
-  for (int t = 0; t < 16; ++t) v[t] = src[ltid + t * NT];
+  for (int t = 0; t < NP; ++t) v[t] = src[ltid + t * NT];
   V* sm = f4_sm + g * SL;
-  block_fft<L, SIGN>(v, sm, twb, ltid);
+  line_fft<L, SIGN>(v, sm, twb, ltid);
   __syncthreads();  // the last stage has read its inputs from shared memory
 #pragma unroll
-  for (int t = 0; t < 16; ++t) sm[ltid + t * NT] = v[t];
+  for (int t = 0; t < NP; ++t) sm[ltid + t * NT] = v[t];
   __syncthreads();
   V* dst = out + (int64_t)blockIdx.y * n + row0;
 #pragma unroll
-  for (int i = 0; i < 16; ++i) {
+  for (int i = 0; i < NP; ++i) {
     const int f = (int)threadIdx.x + i * (R * NT);
     const int gg = f % R;
     const int k2 = f / R;
@@ -183,18 +265,20 @@ constexpr int kF4MinLog = 15;    // FP32: below, one block does it (block_mf)
 constexpr int kF4MinLog64 = 14;  // N1, N2 >= 128
 constexpr int kF4MaxLog = 24;    // N1, N2 <= 4096
 
-// Tile widths: G columns of N1 points, R rows of N2 points, at most 1024 (FP32) or 512 (FP64) threads
-// of 16 points; lines of up to 512 points take narrower tiles, so that the few blocks of a small
-// transform spread over more SMs.
+// Tile widths: G columns of N1 points, R rows of N2 points.  FP32: lines of 512 and 1024 points in
+// tiles of 8 columns, longer ones in tiles of 4, so that two blocks share an SM up to 2048 points
+// (8 columns of 2048 points, one block per SM: 640 us against 624 for 6 references of 2^23 samples); shorter
+// lines, of small transforms, in tiles of 4 for more blocks.  FP64: at most 1024 threads.
 template <typename V, int L> constexpr int f4_cols_g() {
-  return sizeof(V) == 8 ? (L >= 4096 ? 4 : (L >= 512 ? 8 : 4)) : (L >= 4096 ? 2 : 4);
+  return sizeof(V) == 8 ? (L == 512 || L == 1024 ? 8 : 4) : (L >= 4096 ? 2 : 4);
 }
-template <typename V, int L> constexpr int f4_rows_r() { return sizeof(V) == 16 && L >= 4096 ? 2 : 4; }
+template <typename V, int L> constexpr int f4_rows_r() { return sizeof(V) == 16 && (L <= 256 || L >= 4096) ? 2 : 4; }
 
-template <typename V>
-const V* block_tables(const rf_ctx* c, int logb) {
-  if constexpr (sizeof(V) == 8) return c->twb32.as<float2>() + c->twb_off[logb];
-  else return c->twb64.as<double2>() + c->twb64_off[logb];
+template <typename V, int L>
+const V* line_tables(const rf_ctx* c) {
+  constexpr int LOGB = BlockFFTShape<L>::LOGB;
+  if constexpr (sizeof(V) == 8) return c->twb32.as<float2>() + c->twb_off[LOGB];
+  else return c->twb64.as<double2>() + c->twb64_off[f4_points<V, L>() == 4 ? 0 : LOGB];
 }
 
 template <typename V, int L, int MODE, int SIGN>
@@ -208,7 +292,7 @@ void launch_cols(const void* in, const V* F, int64_t fstride, V* out, int n2log,
   if constexpr (sizeof(V) == 8) tw = c->tw4.as<float2>();
   else tw = c->tw64.as<double2>();
   dim3 grid((unsigned)(((int64_t)1 << n2log) / G), (unsigned)batch);
-  fn<<<grid, G * L / 16, smem, s>>>(in, F, fstride, out, n2log, block_tables<V>(c, BlockFFTShape<L>::LOGB), tw,
+  fn<<<grid, G * L / f4_points<V, L>(), smem, s>>>(in, F, fstride, out, n2log, line_tables<V, L>(c), tw,
                                      c->tw4_lo_bits);
   RF_LAUNCHED();
 }
@@ -220,7 +304,7 @@ void launch_rows(const V* in, V* out, int n1log, int batch, const rf_ctx* c, cud
   constexpr size_t smem = f4_smem<V, L, R>();
   RF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   dim3 grid((unsigned)(((int64_t)1 << n1log) / R), (unsigned)batch);
-  fn<<<grid, R * L / 16, smem, s>>>(in, out, n1log, block_tables<V>(c, BlockFFTShape<L>::LOGB));
+  fn<<<grid, R * L / f4_points<V, L>(), smem, s>>>(in, out, n1log, line_tables<V, L>(c));
   RF_LAUNCHED();
 }
 
@@ -304,7 +388,7 @@ void block_mf(const rf_ctx* c, const float* x, const float2* F, int64_t fstride,
     constexpr size_t smem = sizeof(float2) * BlockFFTShape<B>::SMEM;
     RF_CUDA(cudaFuncSetAttribute(k_block_mf<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     k_block_mf<B><<<(unsigned)nref, B / 16, smem, s>>>(x, F, fstride, out,
-                                                       block_tables<float2>(c, BlockFFTShape<B>::LOGB));
+                                                       line_tables<float2, B>(c));
     RF_LAUNCHED();
   };
   switch (ilog2(c->n)) {

@@ -61,8 +61,12 @@ namespace {
 
 constexpr int kRedThreads = 256;
 constexpr int kRedBlocks = 512;
-// complex values of the four-step inverse transforms launched together (their intermediate)
-constexpr int64_t kF4Chunk = int64_t(1) << 23;
+// Complex values of the four-step inverse transforms launched together (their intermediate).  Larger
+// launches leave a smaller share of their last wave of blocks empty, which is worth more than an
+// intermediate that fits L2 (the passes reach 20-40% of the HBM rate): 2^23, 2^24 and 2^25 values
+// take 251, 243 and 232 us for 24 references of 2^20 samples, 694, 640 and 624 us for 6 of 2^23
+// (with their window peaks).
+constexpr int64_t kF4Chunk = int64_t(1) << 25;
 
 // Tables of powers of the bin index k = 0..n/2 (rows of `stride`): k^(1/3), k^(-5/3), ln(k)/3 and
 // k^(-7/6), 0 at k = 0.  The cube root is corrected by its exact residual, so the first two are good
@@ -113,25 +117,21 @@ __global__ void __launch_bounds__(kRedThreads) k_sigma2_bins(const double* __res
 }
 
 // out[0] = sigma^2, out[1] = the filter scale 4 / (n sqrt(sigma^2)) df^(-7/6); sigma to `nref`
-// places of sigma_out (every template of the unit-amplitude family has the same N).
-__global__ void k_sigma2_finish(const double* __restrict__ part, int count, double n, double amp,
-                                double* __restrict__ out, double* __restrict__ sigma_out, int nref) {
-  __shared__ double sh[kRedThreads];
+// places of sigma_out (every template of the unit-amplitude family has the same N).  One warp.
+__global__ void __launch_bounds__(32) k_sigma2_finish(const double* __restrict__ part, int count, double n,
+                                                      double amp, double* __restrict__ out,
+                                                      double* __restrict__ sigma_out, int nref) {
   double acc = 0.0;
-  for (int i = threadIdx.x; i < count; i += blockDim.x) acc += part[i];
-  sh[threadIdx.x] = acc;
-  __syncthreads();
-  for (int s = kRedThreads / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
-    __syncthreads();
-  }
-  const double sg = sqrt(sh[0]);
+  for (int i = threadIdx.x; i < count; i += 32) acc += part[i];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  const double sg = sqrt(acc);
   if (threadIdx.x == 0) {
-    out[0] = sh[0];
+    out[0] = acc;
     out[1] = 4.0 / (n * sg) * amp;
   }
   if (sigma_out)
-    for (int r = threadIdx.x; r < nref; r += blockDim.x) sigma_out[r] = sg;
+    for (int r = threadIdx.x; r < nref; r += 32) sigma_out[r] = sg;
 }
 
 constexpr int kFiltRefs = 8;  // references of one filter launch (their coefficients are arguments)
@@ -200,11 +200,12 @@ double* launch_sigma2(rf_ctx* c, const double* inv_psd, double* sigma_out, int n
   const double amp = amp_scale(df);
   double* part = c->red.as<double>();
   double* sig = part + kRedBlocks;
-  const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(kRedBlocks, (k1 - k0 + 1) / (2 * kRedThreads)));
+  // two blocks per SM at most, so that the one-warp sum of the partials stays short
+  const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(kRedBlocks, 2 * c->nsm), (k1 - k0 + 1) / (2 * kRedThreads)));
   k_sigma2_bins<<<blocks, kRedThreads, 0, s>>>(inv_psd, c->pw.as<double>() + 3 * c->pw_stride, k0, k1,
                                                4.0 * df * amp * amp, part);
   RF_LAUNCHED();
-  k_sigma2_finish<<<1, kRedThreads, 0, s>>>(part, blocks, (double)c->n, amp, sig, sigma_out, nref);
+  k_sigma2_finish<<<1, 32, 0, s>>>(part, blocks, (double)c->n, amp, sig, sigma_out, nref);
   RF_LAUNCHED();
   return sig;
 }
@@ -326,8 +327,7 @@ void mf_filtered_impl(rf_ctx* c, const void* x, int32_t nref, const void* filt, 
   auto run = [&](auto vtag) {
     using V = decltype(vtag);
     using T = typename real_of<V>::type;
-    // references per launch: bounded by the temporary buffer, and for the two-pass four-step
-    // transforms by kF4Chunk values, whose intermediate is meant to stay in L2
+    // references per launch, bounded by the temporary buffer
     const int64_t most = fft4_supported(n, sizeof(T) == 8) ? std::max<int64_t>(1, kF4Chunk / n)
                                                            : std::min<int64_t>(65535, ((int64_t)1 << 27) / n);
     const int chunk = (int)std::max<int64_t>(1, std::min<int64_t>(nref, most));

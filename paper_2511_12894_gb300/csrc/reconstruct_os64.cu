@@ -321,23 +321,6 @@ void prepare64(rf_ctx* c, rf_kernels* kern, int B, int Q, cudaStream_t s) {
   kern->os64_Q = Q;
 }
 
-// A stream-ordered allocation from the context's pool, given back in stream order.
-struct StreamBuf {
-  void* p = nullptr;
-  cudaStream_t s;
-  StreamBuf(rf_ctx* c, size_t bytes, cudaStream_t st) : s(st) {
-    if (cudaMallocFromPoolAsync(&p, bytes, c->pool, s) != cudaSuccess) {
-      (void)cudaGetLastError();
-      p = nullptr;
-    }
-  }
-  ~StreamBuf() {
-    if (p) cudaFreeAsync(p, s);
-  }
-  StreamBuf(const StreamBuf&) = delete;
-  StreamBuf& operator=(const StreamBuf&) = delete;
-};
-
 bool capturing(cudaStream_t s) {
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
@@ -367,22 +350,13 @@ void os64_create(rf_ctx* c) {
     if (S::MID16) stage(16);
     if (S::LAST16) stage(16);
   };
-  tables(std::integral_constant<int, 128>{}, 7);
-  tables(std::integral_constant<int, 256>{}, 8);
-  tables(std::integral_constant<int, 512>{}, 9);
+  // slot 0: the 4096th roots of unity, for the lines of four points per thread (fft4.cu)
+  for (int m = 0; m < 4096; ++m) tw.push_back(block_twiddles()[(size_t)m * (kBlockTwiddles / 4096)]);
   tables(std::integral_constant<int, 1024>{}, 10);
   tables(std::integral_constant<int, 2048>{}, 11);
   tables(std::integral_constant<int, 4096>{}, 12);
   c->twb64.ensure(sizeof(double2) * tw.size());
   RF_CUDA(cudaMemcpy(c->twb64.p, tw.data(), sizeof(double2) * tw.size(), cudaMemcpyHostToDevice));
-  cudaMemPoolProps props{};
-  props.allocType = cudaMemAllocationTypePinned;
-  props.location.type = cudaMemLocationTypeDevice;
-  props.location.id = c->device;
-  RF_CUDA(cudaMemPoolCreate(&c->pool, &props));
-  // keep up to 1 GB between calls; more goes back to the device at the next synchronisation
-  unsigned long long keep = 1ull << 30;
-  RF_CUDA(cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep));
 }
 
 // False where the direct sum should run instead: it is modelled cheaper, the kernel set cannot be

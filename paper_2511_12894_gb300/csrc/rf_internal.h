@@ -147,10 +147,12 @@ struct rf_ctx {
   // block size 2^b start at entry twb_off[b].
   rf::DevBuf twb32;
   int64_t twb_off[16] = {0};
-  // FP64 grids: stage twiddle tables of the FP64 block FFTs (B = 2^7 .. 2^12, as twb32) and the pool
-  // of the FP64 overlap-save calls' workspaces.
+  // FP64 grids: exp(-2 pi i m / 4096) (slot 0), the stage twiddle tables of the FP64 block FFTs (B =
+  // 2^10 .. 2^12, as twb32).
   rf::DevBuf twb64;
   int64_t twb64_off[16] = {0};
+  // Pool of stream-ordered temporaries (kernel building, FP64 overlap-save); it keeps at most 2 GB
+  // between calls and goes with the context.
   cudaMemPool_t pool = nullptr;
   // Four-step FFT twiddles (float2): w[m] = exp(-2 pi i m / n) for m < 2^tw4_lo_bits, then
   // w[2^tw4_lo_bits m] for m < n / 2^tw4_lo_bits; empty where the four-step FFT does not apply.
@@ -279,6 +281,36 @@ inline size_t tap_bytes(const rf_kernels* k) {
   const size_t r = k->dtype == RF_F64 ? sizeof(double) : sizeof(float);
   return k->real ? r : 2 * r;
 }
+
+// A stream-ordered allocation from the context's pool, given back in stream order; p is null when
+// there is no memory (StreamBuf::need throws then).
+struct StreamBuf {
+  void* p = nullptr;
+  cudaStream_t s;
+  StreamBuf(rf_ctx* c, size_t bytes, cudaStream_t st) : s(st) {
+    if (cudaMallocFromPoolAsync(&p, bytes ? bytes : 16, c->pool, s) != cudaSuccess) {
+      (void)cudaGetLastError();
+      p = nullptr;
+    }
+  }
+  ~StreamBuf() {
+    if (p) cudaFreeAsync(p, s);
+  }
+  StreamBuf(const StreamBuf&) = delete;
+  StreamBuf& operator=(const StreamBuf&) = delete;
+  StreamBuf& need() {
+    if (!p) {
+      set_error("out of device memory for a temporary");
+      throw Fail{RF_ENOMEM};
+    }
+    return *this;
+  }
+  template <typename T>
+  T* as() const {
+    return static_cast<T*>(p);
+  }
+};
+void pool_create(rf_ctx* c);
 
 // ---------------------------------------------------------------- FFT (fft.cu)
 // Batched out-of-place Stockham FFT of length n (power of two) over `batch`
