@@ -1,4 +1,5 @@
-// Ratio-kernel builder (Sec. II.B-II.D; Eqs. 5, 7, 9, 10), FP64 throughout.
+// Ratio-kernel builder (Sec. II.B-II.D; Eqs. 5, 7, 9, 10), FP64 (on FP32 grids the transforms in FP32
+// pairs, below).
 //
 // Per neighbour j of the reference, on its build grid of n_b bins (f_k = k fs / n_b; n_b = n
 // unless a coarser grid is asked for, Sec. II.D):
@@ -18,7 +19,10 @@
 #include <climits>
 #include <cmath>
 #include <memory>
+#include <type_traits>
+#include <utility>
 
+#include "cdf.cuh"
 #include "cplx.cuh"
 #include "rf_internal.h"
 #include "tf2.cuh"
@@ -99,6 +103,11 @@ __global__ void k_real_form(double2* __restrict__ rho, int64_t count) {
     rho[i] = make_double2(2.0 * rho[i].x, 0.0);
 }
 
+__global__ void k_real_form(cdf* __restrict__ rho, int64_t count) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x)
+    rho[i] = cdf{make_float2(2.f * rho[i].h.x, 0.f), make_float2(2.f * rho[i].l.x, 0.f)};
+}
+
 // One row per template (grid.y): K~ over the full length-n buffer.  dq: the template's phase minus
 // the reference's (tf2.cuh); [k0, k1]: the bins inside [f_low, f_high], where W = 1.  Bound by the
 // FP64 pipe (two lanes per SM): the phase from the tables of bin powers is about ten multiply-adds
@@ -130,6 +139,133 @@ __global__ void __launch_bounds__(256) k_kernel_spectrum(const Tf2Bins* __restri
   K[(int64_t)j * n + k] = out;
 }
 
+// ---------------------------------------------------------------- FP32 grids: transforms in pairs
+// The taps of an FP32 grid are rounded to FP32, and the transform that makes them cost 2.9 of the 7 ms
+// of building 48 kernels on 2^19 bins, all of it on the FP64 pipe.  The same radix passes in FP32
+// pairs (cdf.cuh) are bound by HBM; the phase stays FP64.  A pair carries about 46 bits of the row's
+// largest value, so the kept span, decided at thr times that value, is the FP64 one wherever thr is
+// far above 2^-46: pairs are used from thr = 1e-7 on (and for analytic spans, which only take the
+// largest value), FP64 below it, for absolute thresholds and for grids below 4096 bins.
+constexpr double kPairMinThr = 1e-7;
+constexpr int64_t kPairMinGrid = 4096;
+
+// exp(-2 pi i m / nb) as pairs, from the FP64 table of n entries
+__global__ void __launch_bounds__(256) k_split_roots(const double2* __restrict__ tw, int64_t stride, int64_t nb,
+                                                     cdf* __restrict__ out) {
+  const int64_t m = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (m >= nb) return;
+  const double2 w = tw[m * stride];
+  const float x = (float)w.x, y = (float)w.y;
+  out[m] = cdf{make_float2(x, y), make_float2((float)(w.x - (double)x), (float)(w.y - (double)y))};
+}
+
+// exp(2 pi i t), t in [-1/2, 1/2]: the nearest 4096th root of unity and the series of the rest, whose
+// angle is below 7.7e-4 (relative errors of FP32 in its square and cube: 2e-14 and less).
+__device__ __forceinline__ cdf expi_turn(double t, const cdf* __restrict__ roots, int64_t root_step) {
+  const double big = 6755399441055744.0;
+  const double r = fma(t, 4096.0, big);
+  const double d = fma(-(r - big), 1.0 / 4096.0, t);
+  const float dh = (float)d, dl = (float)(d - (double)dh);
+  constexpr double two_pi = 6.28318530717958647692528676655900577;
+  constexpr float ph = (float)two_pi, pl = (float)(two_pi - (double)ph);
+  const float ah = __fmul_rn(dh, ph);
+  const float al = __fmaf_rn(dh, ph, -ah) + (dh * pl + dl * ph);
+  const float q = __fmaf_rn(ah, ah, 2.f * ah * al);
+  const float c1 = q * __fmaf_rn(q, 1.f / 24.f, -0.5f);
+  const float ch = __fadd_rn(1.f, c1);
+  const cdf e{make_float2(ch, ah),
+              make_float2(__fadd_rn(c1, -__fadd_rn(ch, -1.f)), al + ah * q * __fmaf_rn(q, 1.f / 120.f, -1.f / 6.f))};
+  return cmul(e, cconj_pair(roots[(int64_t)(__double2loint(r) & 4095) * root_step]));
+}
+
+// First radix-16 pass of row blockIdx.y with K~ (as k_kernel_spectrum) formed on load: its bins above
+// n/2 are zero, so half of the inputs are never formed and the spectrum never reaches memory.
+__global__ void __launch_bounds__(128) k_pair_first(const Tf2Bins* __restrict__ dq, const double* __restrict__ dfl,
+                                                    int64_t n, double df, int64_t k0, int64_t k1, double f_low,
+                                                    double f_high, double df_high, const double* __restrict__ pw,
+                                                    int64_t stride, const cdf* __restrict__ roots,
+                                                    cdf* __restrict__ out) {
+  const int64_t nq = n / 16;
+  const int64_t i = (int64_t)blockIdx.x * 128 + threadIdx.x;
+  if (i >= nq) return;
+  const int j = blockIdx.y;
+  const Tf2Bins q = dq[j];
+  const float inv_n = 1.f / (float)n;  // n a power of two: exact
+  const int64_t root_step = n / 4096;
+  auto spectrum = [&](int64_t k) {
+    cdf v{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+    const bool in = k >= k0 && k <= k1;
+    const double w = in ? 1.0 : (k > 0 ? window_w((double)k * df, f_low, f_high, dfl[j], df_high) : 0.0);
+    if (w > 0.0) {
+      v = expi_turn(tf2_turn(q, k, pw[k], pw[stride + k], pw[2 * stride + k]), roots, root_step);
+      if (!in) {
+        const float wh = (float)w, wl = (float)(w - (double)wh);
+        v = cmul(v, cdf{make_float2(wh, 0.f), make_float2(wl, 0.f)});
+      }
+      v.h = make_float2(v.h.x * inv_n, v.h.y * inv_n);
+      v.l = make_float2(v.l.x * inv_n, v.l.y * inv_n);
+    }
+    return v;
+  };
+  cdf a[16];
+#pragma unroll 1
+  for (int t = 0; t < 8; ++t) {
+    const cdf v = spectrum(i + t * nq);
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (u == t) a[u] = v;  // one copy of the spectrum's code, registers indexed at compile time
+  }
+  const cdf zero{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+  a[8] = i == 0 ? spectrum(n / 2) : zero;
+#pragma unroll
+  for (int t = 9; t < 16; ++t) a[t] = zero;
+  cdf_dft<16>(a);
+  cdf* o = out + (int64_t)j * n + i * 16;
+#pragma unroll
+  for (int t = 0; t < 16; ++t) o[t] = a[t];
+}
+
+// A later radix-R pass (fft.cu's scheme), sign +1.
+template <int R>
+__global__ void __launch_bounds__(128) k_pair_pass(const cdf* __restrict__ in, cdf* __restrict__ out, int64_t n,
+                                                   int64_t Ns, const cdf* __restrict__ roots) {
+  const int64_t nb = n / R;
+  const int64_t i = (int64_t)blockIdx.x * 128 + threadIdx.x;
+  if (i >= nb) return;
+  in += (int64_t)blockIdx.y * n;
+  out += (int64_t)blockIdx.y * n;
+  const int64_t k = i & (Ns - 1);
+  const int64_t step = k * (n / (Ns * R));
+  cdf a[R];
+#pragma unroll
+  for (int t = 0; t < R; ++t) a[t] = in[i + t * nb];
+#pragma unroll
+  for (int t = 1; t < R; ++t) a[t] = cmul(a[t], cconj_pair(roots[t * step]));
+  cdf_dft<R>(a);
+  const int64_t base = (i - k) * R + k;
+#pragma unroll
+  for (int t = 0; t < R; ++t) out[base + t * Ns] = a[t];
+}
+
+// The passes after the first; returns the buffer with the result.
+cdf* pair_passes(cdf* cur, cdf* other, int64_t n, int batch, const cdf* roots, cudaStream_t s) {
+  for (int64_t Ns = 16; Ns < n;) {
+    const int64_t left = n / Ns;
+    auto pass = [&](auto rc) {
+      constexpr int R = decltype(rc)::value;
+      k_pair_pass<R><<<dim3((unsigned)((n / R + 127) / 128), (unsigned)batch), 128, 0, s>>>(cur, other, n, Ns, roots);
+      RF_LAUNCHED();
+      Ns *= R;
+    };
+    if (left >= 16) pass(std::integral_constant<int, 16>{});
+    else if (left == 8) pass(std::integral_constant<int, 8>{});
+    else if (left == 4) pass(std::integral_constant<int, 4>{});
+    else pass(std::integral_constant<int, 2>{});
+    std::swap(cur, other);
+  }
+  return cur;
+}
+
 __device__ __forceinline__ double mag2_rn(double2 v) { return __dadd_rn(__dmul_rn(v.x, v.x), __dmul_rn(v.y, v.y)); }
 
 // The magnitudes are compared as integers (non-negative doubles order as their bits) and formed only
@@ -140,24 +276,36 @@ __device__ __forceinline__ unsigned part_hi(double2 v) {
   return max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu);
 }
 // High word below which both parts of a value with x^2 + y^2 >= m2 cannot lie: of sqrt(m2 / 2) (1 - 2^-19).
-__device__ __forceinline__ unsigned floor_hi(double m2) {
+__device__ __forceinline__ unsigned floor_hi(double m2, double2) {
   return (unsigned)__double2hiint(sqrt(0.5 * m2) * (1.0 - 1.9073486328125e-06));
+}
+// The same for pairs, by the bits of their high parts (2^-18 covers the low parts).
+__device__ __forceinline__ double2 wide(cdf v) {
+  return make_double2((double)v.h.x + (double)v.l.x, (double)v.h.y + (double)v.l.y);
+}
+__device__ __forceinline__ double mag2_rn(cdf v) { return mag2_rn(wide(v)); }
+__device__ __forceinline__ unsigned part_hi(cdf v) {
+  return max(__float_as_uint(v.h.x) & 0x7fffffffu, __float_as_uint(v.h.y) & 0x7fffffffu);
+}
+__device__ __forceinline__ unsigned floor_hi(double m2, cdf) {
+  return __float_as_uint((float)(sqrt(0.5 * m2) * (1.0 - 3.814697265625e-06)));
 }
 
 // max |rho|^2 of a row's part (blockIdx.x of gridDim.x, row blockIdx.y) into amax2 (bits; 0 before).
 // One block per row left most SMs idle: 612 us for 48 rows of 2^19 values.
-__global__ void __launch_bounds__(256) k_row_max2(const double2* __restrict__ rho, int64_t n,
+template <typename V>
+__global__ void __launch_bounds__(256) k_row_max2(const V* __restrict__ rho, int64_t n,
                                                   unsigned long long* __restrict__ amax2) {
-  const double2* r = rho + (int64_t)blockIdx.y * n;
+  const V* r = rho + (int64_t)blockIdx.y * n;
   unsigned long long m = 0;
   unsigned lim = 0;
   for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
-    const double2 v = r[i];
+    const V v = r[i];
     if (part_hi(v) < lim) continue;
     const double a = mag2_rn(v);
     if (a > __longlong_as_double((long long)m)) {  // NaN never counts
       m = (unsigned long long)__double_as_longlong(a);
-      lim = floor_hi(a);
+      lim = floor_hi(a, V{});
     }
   }
 #pragma unroll
@@ -197,16 +345,17 @@ __device__ __forceinline__ void arc_join(ArcPart& b, const ArcPart& c, long long
 // Shortest covering arc of {m : |rho[m]|^2 >= cut2}, first step: a warp summarises `per` consecutive
 // lags, 32 at a time by ballot.  (One block per row with a range per thread read its 2^19 values at a
 // stride: 676 us for 48 rows.)
-__global__ void __launch_bounds__(256) k_arc_parts(const double2* __restrict__ rho, int64_t n, int per, int nparts,
+template <typename V>
+__global__ void __launch_bounds__(256) k_arc_parts(const V* __restrict__ rho, int64_t n, int per, int nparts,
                                                    const double* __restrict__ amax2, double thr, int relative,
                                                    ArcPart* __restrict__ parts) {
   const int j = blockIdx.y;
   const int part = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (part >= nparts) return;
   const int lane = threadIdx.x & 31;
-  const double2* r = rho + (int64_t)j * n;
+  const V* r = rho + (int64_t)j * n;
   const double cut2 = __dmul_rn(__dmul_rn(thr, thr), relative ? amax2[j] : 1.0);
-  const unsigned lim = floor_hi(cut2);
+  const unsigned lim = floor_hi(cut2, V{});
   ArcPart b{-1, -1, {-1, 0}};
   if (!relative || amax2[j] > 0.0) {
     const int64_t lo = (int64_t)part * per, hi = min(n, lo + per);
@@ -214,7 +363,7 @@ __global__ void __launch_bounds__(256) k_arc_parts(const double2* __restrict__ r
       const int64_t m = base + lane;
       bool keep = false;
       if (m < hi) {
-        const double2 v = r[m];
+        const V v = r[m];
         if (part_hi(v) >= lim) keep = mag2_rn(v) >= cut2;
       }
       const unsigned mask = __ballot_sync(0xffffffffu, keep);
@@ -265,8 +414,17 @@ __global__ void __launch_bounds__(32) k_arc_join(const ArcPart* __restrict__ par
   }
 }
 
-template <typename V>
-__global__ void __launch_bounds__(256) k_pack(const double2* __restrict__ rho, int64_t n, const int* __restrict__ m0,
+template <typename R>
+__device__ __forceinline__ R tap_x(double2 v) { return (R)v.x; }
+template <typename R>
+__device__ __forceinline__ R tap_y(double2 v) { return (R)v.y; }
+template <typename R>
+__device__ __forceinline__ R tap_x(cdf v) { return (R)(v.h.x + v.l.x); }
+template <typename R>
+__device__ __forceinline__ R tap_y(cdf v) { return (R)(v.h.y + v.l.y); }
+
+template <typename V, typename W>
+__global__ void __launch_bounds__(256) k_pack(const W* __restrict__ rho, int64_t n, const int* __restrict__ m0,
                                               const int* __restrict__ len, const int64_t* __restrict__ off,
                                               V* __restrict__ taps) {
   using R = typename real_of<V>::type;
@@ -274,21 +432,21 @@ __global__ void __launch_bounds__(256) k_pack(const double2* __restrict__ rho, i
   const int L = len[j];
   const int64_t mask = n - 1;
   for (int64_t l = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; l < L; l += (int64_t)gridDim.x * blockDim.x) {
-    const double2 v = rho[(int64_t)j * n + ((m0[j] + l) & mask)];
-    taps[off[j] + l] = cmake<V>((R)v.x, (R)v.y);
+    const W v = rho[(int64_t)j * n + ((m0[j] + l) & mask)];
+    taps[off[j] + l] = cmake<V>(tap_x<R>(v), tap_y<R>(v));
   }
 }
 
 // Real-kernel form: the real parts only (the imaginary parts are zero after k_real_form).
-template <typename R>
-__global__ void __launch_bounds__(256) k_pack_real(const double2* __restrict__ rho, int64_t n,
+template <typename R, typename W>
+__global__ void __launch_bounds__(256) k_pack_real(const W* __restrict__ rho, int64_t n,
                                                    const int* __restrict__ m0, const int* __restrict__ len,
                                                    const int64_t* __restrict__ off, R* __restrict__ taps) {
   const int j = blockIdx.y;
   const int L = len[j];
   const int64_t mask = n - 1;
   for (int64_t l = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; l < L; l += (int64_t)gridDim.x * blockDim.x)
-    taps[off[j] + l] = (R)rho[(int64_t)j * n + ((m0[j] + l) & mask)].x;
+    taps[off[j] + l] = tap_x<R>(rho[(int64_t)j * n + ((m0[j] + l) & mask)]);
 }
 
 }  // namespace
@@ -397,7 +555,12 @@ rf_kernels* build_impl(rf_ctx* c, const rf_template& ref, const rf_template* nbr
   std::vector<int> hm0(kmax_chunk), hlen(kmax_chunk);
   std::vector<Tf2Bins> dq;
   std::vector<std::vector<int64_t>> off_host;
-  // templates per chunk: three complex128 rows of nb per template, about 1.5 GB in total
+  // FP32 grids: transforms in pairs where the truncation allows (above)
+  auto pairs_at = [&](int64_t nb) {
+    return !f64 && nb >= kPairMinGrid &&
+           ((relative & RF_TRUNC_ANALYTIC) || ((relative & RF_TRUNC_RELATIVE) && thr >= kPairMinThr));
+  };
+  // templates per chunk: three complex128 rows of nb per template (two of pairs), about 1.5 GB in total
   auto chunk_at = [&](int q0) {
     const int64_t nb = kern->grid[order[q0]];
     const int64_t per = 3 * nb * (int64_t)sizeof(double2);
@@ -414,6 +577,12 @@ rf_kernels* build_impl(rf_ctx* c, const rf_template& ref, const rf_template* nbr
   }
   StreamBuf rows(c, rows_bytes, s);
   rows.need();
+  int64_t roots_n = 0;
+  for (int j = 0; j < k; ++j)
+    if (pairs_at(kern->grid[j])) roots_n = std::max(roots_n, kern->grid[j]);
+  StreamBuf roots(c, sizeof(cdf) * (size_t)roots_n, s);
+  if (roots_n) roots.need();
+  int64_t roots_of = 0;
   constexpr int kArcParts = 256;  // warps per row at most
   StreamBuf arcs(c, sizeof(ArcPart) * kArcParts * (size_t)kmax_chunk, s);
   arcs.need();
@@ -430,21 +599,46 @@ rf_kernels* build_impl(rf_ctx* c, const rf_template& ref, const rf_template* nbr
     dq.resize(cnt);  // read by the copy until the chunk's synchronisation below
     for (int q = 0; q < cnt; ++q) dq[q] = tf2_bins_minus(make_tf2_bins(tg[order[q0 + q]], dfb), qr);
     RF_CUDA(cudaMemcpyAsync(d_dq, dq.data(), sizeof(Tf2Bins) * cnt, cudaMemcpyHostToDevice, s));
-    double2* bufK = rows.as<double2>();
-    double2* bufR = bufK + cnt * nb;
-    double2* bufT = bufR + cnt * nb;
-    dim3 g1((unsigned)((nb + 255) / 256), (unsigned)cnt);
-    k_kernel_spectrum<<<g1, 256, 0, s>>>(d_dq, d_dfls + q0, nb, dfb, k0, k1, c->g.f_low, c->g.f_high, c->g.df_high,
-                                         c->pw.as<double>(), c->pw_stride, bufK);
-    RF_LAUNCHED();
-    fft_c2c_f64(bufK, bufR, bufT, nb, cnt, +1, c->tw64.as<double2>(), n, s);
-    if (relative & RF_KERNEL_REAL) {
-      k_real_form<<<(unsigned)std::min<int64_t>(4096, (cnt * nb + 255) / 256), 256, 0, s>>>(bufR, cnt * nb);
-      RF_LAUNCHED();
-    }
-    RF_CUDA(cudaMemsetAsync(d_amax, 0, sizeof(double) * cnt, s));
     const unsigned mx = (unsigned)std::max<int64_t>(1, std::min<int64_t>(nb / 2048, (8LL * c->nsm + cnt - 1) / cnt));
-    k_row_max2<<<dim3(mx, (unsigned)cnt), 256, 0, s>>>(bufR, nb, reinterpret_cast<unsigned long long*>(d_amax));
+    const unsigned rg = (unsigned)std::min<int64_t>(4096, (cnt * nb + 255) / 256);
+    const bool pairs = pairs_at(nb);
+    double2* bufR = nullptr;
+    cdf* bufP = nullptr;
+    RF_CUDA(cudaMemsetAsync(d_amax, 0, sizeof(double) * cnt, s));
+    auto amax_bits = reinterpret_cast<unsigned long long*>(d_amax);
+    if (pairs) {
+      if (roots_of != nb) {
+        k_split_roots<<<(unsigned)((nb + 255) / 256), 256, 0, s>>>(c->tw64.as<double2>(), n / nb, nb, roots.as<cdf>());
+        RF_LAUNCHED();
+        roots_of = nb;
+      }
+      cdf* a = rows.as<cdf>();
+      cdf* b = a + cnt * nb;
+      k_pair_first<<<dim3((unsigned)((nb / 16 + 127) / 128), (unsigned)cnt), 128, 0, s>>>(
+          d_dq, d_dfls + q0, nb, dfb, k0, k1, c->g.f_low, c->g.f_high, c->g.df_high, c->pw.as<double>(), c->pw_stride,
+          roots.as<cdf>(), a);
+      RF_LAUNCHED();
+      bufP = pair_passes(a, b, nb, cnt, roots.as<cdf>(), s);
+      if (real_form) {
+        k_real_form<<<rg, 256, 0, s>>>(bufP, cnt * nb);
+        RF_LAUNCHED();
+      }
+      k_row_max2<cdf><<<dim3(mx, (unsigned)cnt), 256, 0, s>>>(bufP, nb, amax_bits);
+    } else {
+      double2* bufK = rows.as<double2>();
+      bufR = bufK + cnt * nb;
+      double2* bufT = bufR + cnt * nb;
+      dim3 g1((unsigned)((nb + 255) / 256), (unsigned)cnt);
+      k_kernel_spectrum<<<g1, 256, 0, s>>>(d_dq, d_dfls + q0, nb, dfb, k0, k1, c->g.f_low, c->g.f_high, c->g.df_high,
+                                           c->pw.as<double>(), c->pw_stride, bufK);
+      RF_LAUNCHED();
+      fft_c2c_f64(bufK, bufR, bufT, nb, cnt, +1, c->tw64.as<double2>(), n, s);
+      if (real_form) {
+        k_real_form<<<rg, 256, 0, s>>>(bufR, cnt * nb);
+        RF_LAUNCHED();
+      }
+      k_row_max2<double2><<<dim3(mx, (unsigned)cnt), 256, 0, s>>>(bufR, nb, amax_bits);
+    }
     RF_LAUNCHED();
     if (relative & RF_TRUNC_ANALYTIC) {
       k_analytic_span<<<(cnt + 63) / 64, 64, 0, s>>>(pr, d_tgs + q0, d_dfls + q0, d_amax, cnt, thr,
@@ -454,8 +648,13 @@ rf_kernels* build_impl(rf_ctx* c, const rf_template& ref, const rf_template* nbr
     } else {
       const int per = (int)std::max<int64_t>(32, nb / kArcParts);
       const int np = (int)((nb + per - 1) / per);
-      k_arc_parts<<<dim3((unsigned)((np + 7) / 8), (unsigned)cnt), 256, 0, s>>>(
-          bufR, nb, per, np, d_amax, thr, relative & RF_TRUNC_RELATIVE, arcs.as<ArcPart>());
+      const dim3 ga((unsigned)((np + 7) / 8), (unsigned)cnt);
+      if (pairs)
+        k_arc_parts<cdf><<<ga, 256, 0, s>>>(bufP, nb, per, np, d_amax, thr, relative & RF_TRUNC_RELATIVE,
+                                            arcs.as<ArcPart>());
+      else
+        k_arc_parts<double2><<<ga, 256, 0, s>>>(bufR, nb, per, np, d_amax, thr, relative & RF_TRUNC_RELATIVE,
+                                                arcs.as<ArcPart>());
       RF_LAUNCHED();
       k_arc_join<<<cnt, 32, 0, s>>>(arcs.as<ArcPart>(), np, nb, d_m0, d_len);
     }
@@ -483,14 +682,20 @@ rf_kernels* build_impl(rf_ctx* c, const rf_template& ref, const rf_template* nbr
     StreamBuf offd(c, sizeof(int64_t) * (cnt + 1), s);
     RF_CUDA(cudaMemcpyAsync(offd.need().p, off.data(), sizeof(int64_t) * (cnt + 1), cudaMemcpyHostToDevice, s));
     dim3 g2(64, (unsigned)cnt);
-    if (real_form && f64)
-      k_pack_real<double><<<g2, 256, 0, s>>>(bufR, nb, d_m0, d_len, offd.as<int64_t>(), static_cast<double*>(dst));
-    else if (real_form)
-      k_pack_real<float><<<g2, 256, 0, s>>>(bufR, nb, d_m0, d_len, offd.as<int64_t>(), static_cast<float*>(dst));
-    else if (f64)
-      k_pack<double2><<<g2, 256, 0, s>>>(bufR, nb, d_m0, d_len, offd.as<int64_t>(), static_cast<double2*>(dst));
-    else
-      k_pack<float2><<<g2, 256, 0, s>>>(bufR, nb, d_m0, d_len, offd.as<int64_t>(), static_cast<float2*>(dst));
+    const int64_t* od = offd.as<int64_t>();
+    auto pack = [&](auto* src) {
+      using S = std::remove_pointer_t<decltype(src)>;
+      if (real_form && f64)
+        k_pack_real<double, S><<<g2, 256, 0, s>>>(src, nb, d_m0, d_len, od, static_cast<double*>(dst));
+      else if (real_form)
+        k_pack_real<float, S><<<g2, 256, 0, s>>>(src, nb, d_m0, d_len, od, static_cast<float*>(dst));
+      else if (f64)
+        k_pack<double2, S><<<g2, 256, 0, s>>>(src, nb, d_m0, d_len, od, static_cast<double2*>(dst));
+      else
+        k_pack<float2, S><<<g2, 256, 0, s>>>(src, nb, d_m0, d_len, od, static_cast<float2*>(dst));
+    };
+    if (pairs) pack(bufP);
+    else pack(bufR);
     RF_LAUNCHED();
     off_host.push_back(std::move(off));  // read by the copy above
     q0 += cnt;

@@ -42,3 +42,26 @@ def test_arcs(n_build, real):
             m2 = rho.real ** 2 + rho.imag ** 2
             m0, L = _arc(m2 >= thr * thr * m2.max())
             assert (k.lag0[j], k.length[j]) == (m0, L), (n_build, thr, j)
+
+
+@pytest.mark.parametrize("n_build", [4096, 1 << 14, 0, -1])
+@pytest.mark.parametrize("real", [False, True])
+@pytest.mark.parametrize("analytic", [False, True])
+def test_fp32_grids_keep_the_fp64_spans(n_build, real, analytic):
+    """Kernels of an FP32 grid (transforms in FP32 pairs): spans equal to those of the FP64 grid, every
+    tap within one FP32 rounding (2^-24 of it) plus the pairs' error (2^-43 of the largest tap)."""
+    torch = pytest.importorskip("torch")
+    from paper_2511_12894_gb300 import RatioFilter
+    n = 1 << 17
+    grids = [RatioFilter(n, 2048.0, 20.0, 971.0, 7, d) for d in ("f32", "f64")]
+    ip = torch.ones(n // 2 + 1, dtype=torch.float64, device="cuda")
+    ref = workload.Template(1.6, 1.5)
+    rng = np.random.default_rng(3)
+    nb = [ref] + [workload.Template(1.6 + a, 1.5 + b) for a, b in rng.uniform(-0.02, 0.02, (6, 2))]
+    for thr in (1e-2, 3e-5, 1e-6, 1e-7, 1e-9) if not analytic else (1e-4, 1e-6):
+        k32, k64 = (g.build_ratio_kernels(ref, nb, ip, thr, n_build=n_build, real=real, analytic=analytic)
+                    for g in grids)
+        assert np.array_equal(k32.lag0, k64.lag0) and np.array_equal(k32.length, k64.length), thr
+        a, b = k32.taps().to(k64.taps().dtype).cpu().numpy(), k64.taps().cpu().numpy()
+        a, b = a.view(np.float64), b.view(np.float64)
+        assert (np.abs(a - b) <= 2.0 ** -24 * np.abs(b) + 2.0 ** -43 * np.abs(b).max()).all(), thr
