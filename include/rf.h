@@ -125,7 +125,7 @@ uint64_t rf_launch_count(void);
 const char* rf_last_error(void);
 
 /* Create a context for one grid on the current device.  Allocates the FFT twiddle and
- * bin-power tables and workspaces (about 56 n bytes, and up to 100 MB for batches of reference
+ * bin-power tables and workspaces (about 68 n bytes, and up to 100 MB for batches of reference
  * templates).  Caller frees with rf_destroy. */
 rf_status rf_create(const rf_grid* grid, rf_ctx** out);
 

@@ -71,7 +71,9 @@ constexpr int64_t kF4Chunk = int64_t(1) << 25;
 // Tables of powers of the bin index k = 0..n/2 (rows of `stride`): k^(1/3), k^(-5/3), ln(k)/3 and
 // k^(-7/6), 0 at k = 0.  The cube root is corrected by its exact residual, so the first two are good
 // to about half an ulp.
-__global__ void __launch_bounds__(256) k_bin_powers(int64_t nbins, int64_t stride, double* __restrict__ pw) {
+// pw32 (if not null): the first three as FP32 pairs.
+__global__ void __launch_bounds__(256) k_bin_powers(int64_t nbins, int64_t stride, double* __restrict__ pw,
+                                                    float2* __restrict__ pw32) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nbins) return;
   double u = 0.0, u5 = 0.0, lu = 0.0, ua = 0.0;
@@ -95,6 +97,13 @@ __global__ void __launch_bounds__(256) k_bin_powers(int64_t nbins, int64_t strid
   pw[stride + i] = u5;
   pw[2 * stride + i] = lu;
   pw[3 * stride + i] = ua;
+  if (pw32) {
+    const double t[3] = {u, u5, lu};
+    for (int q = 0; q < 3; ++q) {
+      const float h = (float)t[q];
+      pw32[q * stride + i] = make_float2(h, (float)(t[q] - (double)h));
+    }
+  }
 }
 
 // Partial sums of 4 df B(f_k)^2 inv_psd[k] over the bins k0..k1 of the band, one partial per
@@ -142,9 +151,9 @@ struct FiltRefs {
 // Filters F_r[k] = (4 / (n N)) conj(h~_r,k) inv_psd[k], k = 0..n/2, of `cnt` references; 0 outside
 // the bins k0..k1 of the band.  With X the unnormalised DFT of the data, X[k] F_r[k] is the
 // integrand of Eq. 2 (4 df dt = 4 / n).  One thread per bin: the tables and inv_psd are read once
-// for all references.  PREC: phase, amplitude and product in FP64, rounded once (stored filters);
-// else (FP32 grids, filters made and used within one call) the FP64 phase is reduced to a
-// fraction of a turn before the FP32 sine and cosine.
+// for all references.  PREC: phase, amplitude and product in FP64, rounded once (stored filters,
+// FP64 grids); else (filters made and used within one call on an FP32 grid) the FP64 phase is reduced
+// to a fraction of a turn before the FP32 sine and cosine.
 template <typename V, bool PREC>
 __global__ void __launch_bounds__(256) k_ref_filters(const double* __restrict__ ip, const double* __restrict__ pw,
                                                      int64_t stride, const double* __restrict__ sig, FiltRefs refs,
@@ -170,6 +179,32 @@ __global__ void __launch_bounds__(256) k_ref_filters(const double* __restrict__ 
       sincospif(2.0f * (float)t, &s, &c);
       F[r * fstride + k] = cmake<V>((R)a * c, (R)a * s);
     }
+  }
+}
+
+// The same for FP32 grids with the phase in FP32 pairs (templates with t_c = 0).  Three references at
+// n = 2^20: the FP64 phase took 49 us of the FP64 pipe.
+struct FiltPairs {
+  Tf2Pairs q[kFiltRefs];
+};
+__global__ void __launch_bounds__(256) k_ref_filters_pairs(const double* __restrict__ ip,
+                                                           const double* __restrict__ ua,
+                                                           const float2* __restrict__ pw32, int64_t stride,
+                                                           const double* __restrict__ sig, FiltPairs refs, int cnt,
+                                                           int64_t nbins, int64_t k0, int64_t k1,
+                                                           float2* __restrict__ F, int64_t fstride) {
+  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= nbins) return;
+  if (k < k0 || k > k1) {
+    for (int r = 0; r < cnt; ++r) F[r * fstride + k] = make_float2(0.f, 0.f);
+    return;
+  }
+  const float2 u = pw32[k], u5 = pw32[stride + k], lu = pw32[2 * stride + k];
+  const float a = (float)(sig[1] * ua[k] * ip[k]);
+  for (int r = 0; r < cnt; ++r) {
+    float s, c;
+    sincospif(2.0f * tf2_turn(refs.q[r], Pair{u.x, u.y}, Pair{u5.x, u5.y}, Pair{lu.x, lu.y}), &s, &c);
+    F[r * fstride + k] = make_float2(a * c, a * s);
   }
 }
 
@@ -220,7 +255,22 @@ void launch_filters(rf_ctx* c, const double* inv_psd, const double* sig, int cnt
   for (int r0 = 0; r0 < cnt; r0 += kFiltRefs) {
     const int m = std::min(kFiltRefs, cnt - r0);
     FiltRefs fr{};
-    for (int r = 0; r < m; ++r) fr.q[r] = make_tf2_bins(make_tf2(refs[r0 + r], c->g.pn_order), df);
+    bool at_zero = true;
+    for (int r = 0; r < m; ++r) {
+      fr.q[r] = make_tf2_bins(make_tf2(refs[r0 + r], c->g.pn_order), df);
+      at_zero = at_zero && fr.q[r].d == 0.0;
+    }
+    if constexpr (!PREC) {
+      if (at_zero) {
+        FiltPairs fp{};
+        for (int r = 0; r < m; ++r) fp.q[r] = make_tf2_pairs(fr.q[r]);
+        k_ref_filters_pairs<<<(unsigned)((nbins + 255) / 256), 256, 0, s>>>(
+            inv_psd, c->pw.as<double>() + 3 * c->pw_stride, c->pw32.as<float2>(), c->pw_stride, sig, fp, m, nbins, k0,
+            k1, F + (int64_t)r0 * fstride, fstride);
+        RF_LAUNCHED();
+        continue;
+      }
+    }
     k_ref_filters<V, PREC><<<(unsigned)((nbins + 255) / 256), 256, 0, s>>>(
         inv_psd, c->pw.as<double>(), c->pw_stride, sig, fr, m, nbins, k0, k1, F + (int64_t)r0 * fstride, fstride);
     RF_LAUNCHED();
@@ -233,7 +283,10 @@ void mf_create(rf_ctx* c) {
   const int64_t nbins = c->n / 2 + 1;
   c->pw_stride = (nbins + 15) & ~(int64_t)15;
   c->pw.ensure(sizeof(double) * 4 * (size_t)c->pw_stride);
-  k_bin_powers<<<(unsigned)((nbins + 255) / 256), 256>>>(nbins, c->pw_stride, c->pw.as<double>());
+  const bool f32 = c->g.dtype == RF_F32;
+  if (f32) c->pw32.ensure(sizeof(float2) * 3 * (size_t)c->pw_stride);
+  k_bin_powers<<<(unsigned)((nbins + 255) / 256), 256>>>(nbins, c->pw_stride, c->pw.as<double>(),
+                                                         f32 ? c->pw32.as<float2>() : nullptr);
   RF_LAUNCHED();
   RF_CUDA(cudaStreamSynchronize(nullptr));
   // up to 8 references, 2^22 intermediate values in all (above that one reference fills the GPU)

@@ -160,7 +160,8 @@ struct rf_ctx {
   int tw4_lo_bits = 0;
   // Powers of the bin index k = 0..n/2 in FP64, rows of pw_stride: k^(1/3), k^(-5/3), ln(k)/3 and
   // k^(-7/6) (0 at k = 0): the template phase and amplitude on any grid f_k = k df (tf2.cuh).
-  rf::DevBuf pw;
+  // pw32 (FP32 grids): the first three as FP32 pairs.
+  rf::DevBuf pw, pw32;
   int64_t pw_stride = 0;
   // Filters and intermediates of a batch of mf_batch references of rf_mf_reference, sized when the
   // context is made, so that the call never allocates (mf_batch = 1: fa and fb serve).

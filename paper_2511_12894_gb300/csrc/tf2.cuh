@@ -74,6 +74,41 @@ __device__ __forceinline__ double tf2_turn(const Tf2Bins& q, int64_t k, double u
   return t - ((t + big) - big);
 }
 
+// The same phase in FP32 pairs (value h + l, about 46 bits; the scheme of cdf.cuh for real numbers)
+// for filters that are rounded to FP32 in the same kernel: 3e4 turns keep 2e-9 of a turn, below the
+// rounding of the angle to FP32, and the FP32 pipes are 60 times as wide as the FP64 pipe.
+struct Pair {
+  float h, l;
+};
+inline Pair make_pair_of(double x) {
+  const float h = (float)x;
+  return Pair{h, (float)(x - (double)h)};
+}
+struct Tf2Pairs {
+  Pair b0, b2, b3, b4, b7, l5, l6, m6, e;  // no term in k: for t_c = 0
+};
+inline Tf2Pairs make_tf2_pairs(const Tf2Bins& q) {
+  return Tf2Pairs{make_pair_of(q.b0), make_pair_of(q.b2), make_pair_of(q.b3),
+                  make_pair_of(q.b4), make_pair_of(q.b7), make_pair_of(q.l5),
+                  make_pair_of(q.l6), make_pair_of(q.m6), make_pair_of(q.e)};
+}
+__device__ __forceinline__ Pair pair_mul(Pair a, Pair b) {
+  const float p = __fmul_rn(a.h, b.h);
+  return Pair{p, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.h, b.h, -p)))};
+}
+__device__ __forceinline__ Pair pair_add(Pair a, Pair b) {
+  const float s = __fadd_rn(a.h, b.h), t = __fadd_rn(s, -a.h);
+  const float e = __fadd_rn(__fadd_rn(a.h, -__fadd_rn(s, -t)), __fadd_rn(b.h, -t));
+  return Pair{s, __fadd_rn(e, __fadd_rn(a.l, b.l))};
+}
+__device__ __forceinline__ float tf2_turn(const Tf2Pairs& q, Pair u, Pair u5, Pair lu) {
+  const Pair p = pair_add(pair_mul(u, pair_add(pair_mul(u, q.b4), q.b3)), q.b2);
+  const Pair lead = pair_mul(u5, pair_add(pair_mul(pair_mul(u, u), p), q.b0));
+  const Pair high = pair_mul(u, pair_add(pair_mul(q.l6, lu), pair_add(pair_mul(q.b7, u), q.m6)));
+  const Pair t = pair_add(lead, pair_add(high, pair_add(pair_mul(q.l5, lu), q.e)));
+  return __fadd_rn(__fadd_rn(t.h, -rintf(t.h)), t.l);
+}
+
 // Psi(f) in radians, f > 0.
 __device__ __forceinline__ double tf2_phase(const Tf2& p, double f) {
   const double v = cbrt(kPi * p.M * f);
