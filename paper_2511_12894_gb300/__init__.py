@@ -165,10 +165,36 @@ def _templates(ts: Sequence) -> ctypes.Array:
     return arr
 
 
-def _stream(stream=None):
+_raw_stream = None   # (device index) -> cudaStream_t of the current stream, as an integer
+
+
+def _stream(stream=None) -> int:
+    """cudaStream_t of ``stream`` or of the current one.  The raw query costs a tenth of building a
+    torch.cuda.Stream object (3 us), which is a large part of the shortest calls."""
+    if stream is not None:
+        return stream.cuda_stream
+    global _raw_stream
+    if _raw_stream is None:
+        import torch
+        _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or \
+            (lambda device: torch.cuda.current_stream(device).cuda_stream)
+    return _raw_stream(_current_device())
+
+
+def _current_device() -> int:
     import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    return torch.cuda.current_device()
+
+
+_Tensor = None
+
+
+def _is_tensor(t) -> bool:
+    global _Tensor
+    if _Tensor is None:
+        import torch
+        _Tensor = torch.Tensor
+    return isinstance(t, _Tensor)
 
 
 def _need(t, count: int, name: str):
@@ -182,8 +208,7 @@ def _need(t, count: int, name: str):
 def _dev(t, dtype, name, count: int = 0):
     """Contiguous, 16-byte-aligned CUDA tensor of the given dtype with at least ``count``
     elements (copied only if its layout needs it)."""
-    import torch
-    if not isinstance(t, torch.Tensor):
+    if not _is_tensor(t):
         raise TypeError(f"{name} must be a torch tensor")
     _need(t, count, name)
     if not t.is_cuda:
@@ -198,8 +223,7 @@ def _dev(t, dtype, name, count: int = 0):
 def _out(t, dtype, count: int, name: str):
     """A caller's output tensor, written in place (so never copied): CUDA, of the given dtype,
     contiguous, 16-byte aligned and holding at least ``count`` elements."""
-    import torch
-    if not isinstance(t, torch.Tensor):
+    if not _is_tensor(t):
         raise TypeError(f"{name} must be a torch tensor")
     _need(t, count, name)
     if not t.is_cuda:
@@ -231,7 +255,7 @@ class Kernels:
         dt = self.ctx.rdtype if self.real else self.ctx.cdtype
         t = torch.empty(int(self.offset[-1]), dtype=dt, device="cuda")
         if t.numel():
-            _check(_lib.rf_kernels_copy_taps(self.handle, ctypes.c_void_p(t.data_ptr()), _stream()))
+            _check(_lib.rf_kernels_copy_taps(self.handle, t.data_ptr(), _stream()))
         return t
 
     def prepare(self, block: int = 0, part: int = 0, stream=None) -> None:
@@ -348,7 +372,7 @@ class RatioFilter:
         out = _out(out, self.cdtype, nf, "out") if out is not None else \
             torch.empty(nf, dtype=self.cdtype, device="cuda")
         t = _templates([tmpl])
-        _check(_lib.rf_template_fd(self.handle, t, ctypes.c_void_p(out.data_ptr()), _stream(stream)))
+        _check(_lib.rf_template_fd(self.handle, t, out.data_ptr(), _stream(stream)))
         return out
 
     def mf_reference(self, x, inv_psd, refs: Sequence, z_out=None, sigma_out=None, stream=None):
@@ -361,9 +385,9 @@ class RatioFilter:
             torch.empty((nref, self.n), dtype=self.cdtype, device="cuda")
         sg = _out(sigma_out, torch.float64, nref, "sigma_out") if sigma_out is not None else \
             torch.empty(nref, dtype=torch.float64, device="cuda")
-        _check(_lib.rf_mf_reference(self.handle, ctypes.c_void_p(x.data_ptr()), ctypes.c_void_p(ip.data_ptr()),
-                                    nref, _templates(refs), ctypes.c_void_p(z.data_ptr()),
-                                    ctypes.c_void_p(sg.data_ptr()), _stream(stream)))
+        _check(_lib.rf_mf_reference(self.handle, x.data_ptr(), ip.data_ptr(),
+                                    nref, _templates(refs), z.data_ptr(),
+                                    sg.data_ptr(), _stream(stream)))
         return z, sg
 
     def reference_filters(self, inv_psd, refs: Sequence, filt_out=None, sigma_out=None, stream=None):
@@ -376,8 +400,8 @@ class RatioFilter:
             torch.empty((nref, nf), dtype=self.cdtype, device="cuda")
         sg = _out(sigma_out, torch.float64, nref, "sigma_out") if sigma_out is not None else \
             torch.empty(nref, dtype=torch.float64, device="cuda")
-        _check(_lib.rf_reference_filters(self.handle, ctypes.c_void_p(ip.data_ptr()), nref, _templates(refs),
-                                         ctypes.c_void_p(f.data_ptr()), ctypes.c_void_p(sg.data_ptr()),
+        _check(_lib.rf_reference_filters(self.handle, ip.data_ptr(), nref, _templates(refs),
+                                         f.data_ptr(), sg.data_ptr(),
                                          _stream(stream)))
         return f, sg
 
@@ -390,8 +414,8 @@ class RatioFilter:
         nref = f2.shape[0]
         z = _out(z_out, self.cdtype, nref * self.n, "z_out") if z_out is not None else \
             torch.empty((nref, self.n), dtype=self.cdtype, device="cuda")
-        _check(_lib.rf_mf_filtered(self.handle, ctypes.c_void_p(x.data_ptr()), nref, ctypes.c_void_p(f2.data_ptr()),
-                                   ctypes.c_void_p(z.data_ptr()), _stream(stream)))
+        _check(_lib.rf_mf_filtered(self.handle, x.data_ptr(), nref, f2.data_ptr(),
+                                   z.data_ptr(), _stream(stream)))
         return z
 
     def _wrap_kernels(self, h: ctypes.c_void_p) -> Kernels:
@@ -425,7 +449,7 @@ class RatioFilter:
         flags = (RF_TRUNC_RELATIVE if relative else 0) | (RF_TRUNC_ANALYTIC if analytic else 0) | \
             (RF_KERNEL_REAL if real else 0)
         _check(_lib.rf_build_ratio_kernels(self.handle, _templates([ref]), _templates(nbrs), len(nbrs),
-                                           ctypes.c_void_p(ip.data_ptr()), float(threshold), flags,
+                                           ip.data_ptr(), float(threshold), flags,
                                            int(n_build), ctypes.byref(h), _stream(stream)))
         return self._wrap_kernels(h)
 
@@ -454,8 +478,8 @@ class RatioFilter:
         z_ref = _dev(z_ref, self.cdtype, "z_ref", self.n)
         out = _out(out, self.cdtype, kern.k * self.n, "out") if out is not None else \
             torch.empty((kern.k, self.n), dtype=self.cdtype, device="cuda")
-        _check(_lib.rf_reconstruct(self.handle, ctypes.c_void_p(z_ref.data_ptr()), kern.handle, ALGOS[algo],
-                                   PRECS[prec], ctypes.c_void_p(out.data_ptr()), _stream(stream)))
+        _check(_lib.rf_reconstruct(self.handle, z_ref.data_ptr(), kern.handle, ALGOS[algo],
+                                   PRECS[prec], out.data_ptr(), _stream(stream)))
         return out
 
     def device_status(self) -> None:
@@ -497,9 +521,9 @@ class RatioFilter:
             torch.empty((kern.k, nw), dtype=torch.float32, device="cuda")
         ao = _out(arg_out, torch.int32, kern.k * nw, "arg_out") if arg_out is not None else \
             torch.empty((kern.k, nw), dtype=torch.int32, device="cuda")
-        _check(_lib.rf_reconstruct_winmax(self.handle, ctypes.c_void_p(z_ref.data_ptr()), kern.handle, ALGOS[algo],
-                                          PRECS[prec], int(W), ctypes.c_void_p(mo.data_ptr()),
-                                          ctypes.c_void_p(ao.data_ptr()), _stream(stream)))
+        _check(_lib.rf_reconstruct_winmax(self.handle, z_ref.data_ptr(), kern.handle, ALGOS[algo],
+                                          PRECS[prec], int(W), mo.data_ptr(),
+                                          ao.data_ptr(), _stream(stream)))
         return mo, ao
 
     def reconstruct_batched(self, z_refs: Sequence, kerns: Sequence[Kernels], W: int, algo: str = "auto",
@@ -521,7 +545,7 @@ class RatioFilter:
         kp = (ctypes.c_void_p * G)(*[k.handle.value if isinstance(k.handle, ctypes.c_void_p) else k.handle
                                      for k in kerns])
         _check(_lib.rf_reconstruct_batched(self.handle, G, zp, kp, ALGOS[algo], PRECS[prec], int(W),
-                                           ctypes.c_void_p(mo.data_ptr()), ctypes.c_void_p(ao.data_ptr()),
+                                           mo.data_ptr(), ao.data_ptr(),
                                            _stream(stream)))
         return mo, ao
 
@@ -541,7 +565,7 @@ class RatioFilter:
         kp = (ctypes.c_void_p * G)(*[k.handle.value if isinstance(k.handle, ctypes.c_void_p) else k.handle
                                      for k in kerns])
         p = lambda a: ctypes.c_void_p(a.ctypes.data)
-        _check(_lib.rf_stream_winmax(self.handle, p(x), x.size, G, ctypes.c_void_p(fl.data_ptr()), kp, int(W),
+        _check(_lib.rf_stream_winmax(self.handle, p(x), x.size, G, fl.data_ptr(), kp, int(W),
                                      int(guard), p(rm), p(ra), p(nm), p(na), _stream(stream)))
         return rm, ra, nm[:rows], na[:rows]
 
@@ -556,8 +580,8 @@ class RatioFilter:
             torch.empty((z2.shape[0], nw), dtype=torch.float32, device="cuda")
         ao = _out(arg_out, torch.int32, cnt, "arg_out") if arg_out is not None else \
             torch.empty((z2.shape[0], nw), dtype=torch.int32, device="cuda")
-        _check(_lib.rf_winmax(self.handle, ctypes.c_void_p(z2.data_ptr()), z2.shape[0], int(W),
-                              ctypes.c_void_p(mo.data_ptr()), ctypes.c_void_p(ao.data_ptr()), _stream(stream)))
+        _check(_lib.rf_winmax(self.handle, z2.data_ptr(), z2.shape[0], int(W),
+                              mo.data_ptr(), ao.data_ptr(), _stream(stream)))
         return mo, ao
 
 
@@ -577,10 +601,10 @@ def mf_reference_noalloc(grid: rf_grid, x, inv_psd, ref, z_out, sigma_out=None, 
     z_out = _out(z_out, cd, grid.n, "z_out")
     if sigma_out is not None:
         sigma_out = _out(sigma_out, torch.float64, 1, "sigma_out")
-    sp = ctypes.c_void_p(sigma_out.data_ptr()) if sigma_out is not None else None
-    _check(lib.rf_mf_reference_noalloc(ctypes.byref(grid), ctypes.c_void_p(x.data_ptr()),
-                                       ctypes.c_void_p(ip.data_ptr()), _templates([ref]),
-                                       ctypes.c_void_p(z_out.data_ptr()), sp, _stream(stream)))
+    sp = sigma_out.data_ptr() if sigma_out is not None else None
+    _check(lib.rf_mf_reference_noalloc(ctypes.byref(grid), x.data_ptr(),
+                                       ip.data_ptr(), _templates([ref]),
+                                       z_out.data_ptr(), sp, _stream(stream)))
 
 
 __all__ = ["mf_reference_noalloc", "rf_grid", "rf_tune_entry", "RatioFilter", "Kernels", "RFError", "load_library", "launch_count", "EXPORTED", "LIB_PATH"]
