@@ -22,8 +22,9 @@
 // k <= n/2, zero above (the matched-filter integrand, formed on load).
 //
 // FP32 grids of at most 16384 points fit one thread block: block_mf forms the spectrum of the data,
-// the product with a filter and the inverse transform in one launch, a block per reference (each
-// forms the spectrum anew: the copies run at the same time on other SMs).
+// the product with a filter and the inverse transform in one launch, a block (or, from 2^14 to 2^16
+// points and for few references, a cluster of blocks) per reference.
+#include <cstdint>
 #include <type_traits>
 
 #include "blockfft.cuh"
@@ -261,6 +262,96 @@ __global__ void __launch_bounds__(B / 16) k_block_mf(const float* __restrict__ x
   for (int t = 0; t < 16; ++t) out[t * NT] = v[t];
 }
 
+// A whole matched filter on a cluster of eight blocks, one cluster per reference: the four-step data
+// transform, the product and the four-step inverse, with the two exchanges between columns and rows
+// through distributed shared memory.  n = N1 N2; block r of the cluster owns the columns and the
+// output rows [r GC, r GC + GC) of N1 points and the spectrum's rows [r GR, r GR + GR) of N2 points.  The
+// spectrum comes out as X[k1 + N1 k2] in the block that owns k1, which is a column of the inverse
+// transform (input index N1 a + b with b = k1, a = k2), so the product and the inverse's columns need
+// no exchange.  A single block takes 16 us for 2^14 samples (two 16384-point transforms in a row on
+// one SM), the four launches of the two-pass form about as long.
+constexpr int kClusterBlocks = 8;
+
+// Line l of a tile starts at 16-byte offsets 2 l modulo the banks; rows of an exchange buffer of
+// L points are one value apart.
+template <int L> constexpr int cl_line() { return BlockFFTShape<L>::SMEM / 16 * 16 + 2; }
+template <int L> constexpr int cl_row() { return L + 1; }
+template <int N1, int N2> constexpr size_t cl_smem() {
+  const int gc = N2 / kClusterBlocks, gr = N1 / kClusterBlocks;
+  const int work = gc * cl_line<N1>() > gr * cl_line<N2>() ? gc * cl_line<N1>() : gr * cl_line<N2>();
+  return sizeof(float2) * (size_t)(work + gr * cl_row<N2>() + gc * cl_row<N1>());
+}
+
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// v to the value at `p` of this block's shared memory, in block `rank` of the cluster
+__device__ __forceinline__ void st_cluster(float2* p, int rank, float2 v) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
+}
+
+template <int N1, int N2>
+__global__ void __cluster_dims__(kClusterBlocks, 1, 1) __launch_bounds__(N1 * N2 / 16 / kClusterBlocks)
+    k_cluster_mf(const float* __restrict__ x, const float2* __restrict__ F, int64_t fstride,
+                 float2* __restrict__ out, const float2* __restrict__ tb1, const float2* __restrict__ tb2,
+                 const float2* __restrict__ tw) {
+  constexpr int N = N1 * N2, GC = N2 / kClusterBlocks, GR = N1 / kClusterBlocks;
+  constexpr int NT1 = N1 / 16, NT2 = N2 / 16;
+  constexpr int WORK = GC * cl_line<N1>() > GR * cl_line<N2>() ? GC * cl_line<N1>() : GR * cl_line<N2>();
+  float2* work = reinterpret_cast<float2*>(f4_raw);
+  float2* rows = work + WORK;               // GR rows of N2 points (the spectrum's)
+  float2* outs = rows + GR * cl_row<N2>();  // GC rows of N1 points (the output's)
+  const int rank = (int)(blockIdx.x % kClusterBlocks);
+  const int64_t ref = blockIdx.x / kClusterBlocks;
+  const int c = (int)threadIdx.x % GC, lc = (int)threadIdx.x / GC;  // column or output row, index in its line
+  const int g = (int)threadIdx.x % GR, lr = (int)threadIdx.x / GR;  // spectrum row, index in its line
+  float2 v[16];
+  {
+    // data columns b of N1 points, to rows k1
+    const int b = rank * GC + c;
+#pragma unroll
+    for (int t = 0; t < 16; ++t) v[t] = make_float2(__ldg(x + (int64_t)N2 * (lc + t * NT1) + b), 0.f);
+    block_fft<N1, -1>(v, work + c * cl_line<N1>(), tb1, lc);
+#pragma unroll
+    for (int t = 0; t < 16; ++t) {
+      const int k1 = lc + t * NT1;
+      st_cluster(rows + (k1 % GR) * cl_row<N2>() + b, k1 / GR, cmul(v[t], __ldg(tw + b * k1)));
+    }
+  }
+  cluster_barrier();
+  {
+    // spectrum rows k1, the product, and the inverse's columns k1
+    const int k1 = rank * GR + g;
+#pragma unroll
+    for (int t = 0; t < 16; ++t) v[t] = rows[g * cl_row<N2>() + lr + t * NT2];
+    block_fft<N2, -1>(v, work + g * cl_line<N2>(), tb2, lr);
+    const float2* f = F + ref * fstride + k1;
+#pragma unroll
+    for (int t = 0; t < 16; ++t) {
+      const int k = k1 + N1 * (lr + t * NT2);
+      v[t] = k <= N / 2 ? cmul(v[t], __ldg(f + (k - k1))) : make_float2(0.f, 0.f);
+    }
+    __syncthreads();  // the forward transform's last stage has read `work`
+    block_fft<N2, +1>(v, work + g * cl_line<N2>(), tb2, lr);
+#pragma unroll
+    for (int t = 0; t < 16; ++t) {
+      const int q = lr + t * NT2;  // output row
+      st_cluster(outs + (q % GC) * cl_row<N1>() + k1, q / GC, cmulc(v[t], __ldg(tw + k1 * q)));
+    }
+  }
+  cluster_barrier();  // also: `work` has been read by the whole block
+  {
+#pragma unroll
+    for (int t = 0; t < 16; ++t) v[t] = outs[c * cl_row<N1>() + lc + t * NT1];
+    block_fft<N1, +1>(v, work + c * cl_line<N1>(), tb1, lc);
+    float2* o = out + ref * N + rank * GC + c;
+#pragma unroll
+    for (int t = 0; t < 16; ++t) o[(int64_t)N2 * (lc + t * NT1)] = v[t];
+  }
+}
+
 constexpr int kF4MinLog = 15;    // FP32: below, one block does it (block_mf)
 constexpr int kF4MinLog64 = 14;  // N1, N2 >= 128
 constexpr int kF4MaxLog = 24;    // N1, N2 <= 4096
@@ -270,7 +361,7 @@ constexpr int kF4MaxLog = 24;    // N1, N2 <= 4096
 // (8 columns of 2048 points, one block per SM: 640 us against 624 for 6 references of 2^23 samples); shorter
 // lines, of small transforms, in tiles of 4 for more blocks.  FP64: at most 1024 threads.
 template <typename V, int L> constexpr int f4_cols_g() {
-  return sizeof(V) == 8 ? (L == 512 || L == 1024 ? 8 : 4) : (L >= 4096 ? 2 : 4);
+  return sizeof(V) == 8 ? (L == 512 || L == 1024 ? 8 : 4) : (L <= 256 || L >= 4096 ? 2 : 4);
 }
 template <typename V, int L> constexpr int f4_rows_r() { return sizeof(V) == 16 && (L <= 256 || L >= 4096) ? 2 : 4; }
 
@@ -379,7 +470,15 @@ void fft4_inverse_product(const rf_ctx* c, const double2* X, const double2* F, i
   two_passes<double2, kF4Product, +1>(c, X, F, fstride, out, tmp, batch, s);
 }
 
-bool block_mf_supported(const rf_ctx* c) { return c->g.dtype == RF_F32 && c->n >= 512 && c->n <= 16384; }
+// One launch per call: up to 2^14 samples always, 2^14 .. 2^16 on clusters while all of them run at
+// once (each forms the data's spectrum anew; beyond that the two-pass form, which forms it once, and
+// for 2^14 samples one block per reference keep more of the GPU on useful work).
+bool cluster_mf(const rf_ctx* c, int nref) {
+  return c->n >= 16384 && c->n <= 65536 && (int64_t)nref * kClusterBlocks <= c->nsm;
+}
+bool block_mf_supported(const rf_ctx* c, int nref) {
+  return c->g.dtype == RF_F32 && ((c->n >= 512 && c->n <= 16384) || cluster_mf(c, nref));
+}
 
 void block_mf(const rf_ctx* c, const float* x, const float2* F, int64_t fstride, float2* out, int nref,
               cudaStream_t s) {
@@ -391,6 +490,22 @@ void block_mf(const rf_ctx* c, const float* x, const float2* F, int64_t fstride,
                                                        line_tables<float2, B>(c));
     RF_LAUNCHED();
   };
+  auto cluster = [&](auto n1, auto n2) {
+    constexpr int N1 = decltype(n1)::value, N2 = decltype(n2)::value;
+    auto fn = k_cluster_mf<N1, N2>;
+    RF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cl_smem<N1, N2>()));
+    fn<<<(unsigned)(nref * kClusterBlocks), N1 * N2 / 16 / kClusterBlocks, cl_smem<N1, N2>(), s>>>(
+        x, F, fstride, out, line_tables<float2, N1>(c), line_tables<float2, N2>(c), c->tw32.as<float2>());
+    RF_LAUNCHED();
+  };
+  using I128 = std::integral_constant<int, 128>;
+  using I256 = std::integral_constant<int, 256>;
+  if (cluster_mf(c, nref)) {
+    if (c->n == 16384) cluster(I128{}, I128{});
+    else if (c->n == 32768) cluster(I128{}, I256{});
+    else cluster(I256{}, I256{});
+    return;
+  }
   switch (ilog2(c->n)) {
     case 9: run(std::integral_constant<int, 512>{}); break;
     case 10: run(std::integral_constant<int, 1024>{}); break;

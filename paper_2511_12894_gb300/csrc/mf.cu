@@ -125,22 +125,30 @@ __global__ void __launch_bounds__(kRedThreads) k_sigma2_bins(const double* __res
   if (threadIdx.x == 0) part[blockIdx.x] = amp2 * sh[0];
 }
 
-// out[0] = sigma^2, out[1] = the filter scale 4 / (n sqrt(sigma^2)) df^(-7/6); sigma to `nref`
-// places of sigma_out (every template of the unit-amplitude family has the same N).  One warp.
-__global__ void __launch_bounds__(32) k_sigma2_finish(const double* __restrict__ part, int count, double n,
-                                                      double amp, double* __restrict__ out,
-                                                      double* __restrict__ sigma_out, int nref) {
-  double acc = 0.0;
-  for (int i = threadIdx.x; i < count; i += 32) acc += part[i];
+// sigma^2 from the partials, by the first warp of a block in one fixed order (the same value in every
+// block), and from it the filter scale 4 / (n sqrt(sigma^2)) df^(-7/6), for every thread.  A kernel of its
+// own for this took 5.8 us of latency between the partials and the filters.
+struct SigmaArgs {
+  const double* part;
+  int count;
+  double n, amp;      // amp = df^(-7/6)
+  double* sigma_out;  // null, or `nref` places for sigma (every template of the family has the same N)
+  int nref;
+};
+__device__ __forceinline__ double sigma_scale(const SigmaArgs& a) {
+  __shared__ double sh;
+  if (threadIdx.x < 32) {
+    double acc = 0.0;
+    for (int i = threadIdx.x; i < a.count; i += 32) acc += a.part[i];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  const double sg = sqrt(acc);
-  if (threadIdx.x == 0) {
-    out[0] = acc;
-    out[1] = 4.0 / (n * sg) * amp;
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    const double sg = sqrt(acc);
+    if (threadIdx.x == 0) sh = 4.0 / (a.n * sg) * a.amp;
+    if (blockIdx.x == 0 && a.sigma_out)
+      for (int r = threadIdx.x; r < a.nref; r += 32) a.sigma_out[r] = sg;
   }
-  if (sigma_out)
-    for (int r = threadIdx.x; r < nref; r += 32) sigma_out[r] = sg;
+  __syncthreads();
+  return sh;
 }
 
 constexpr int kFiltRefs = 8;  // references of one filter launch (their coefficients are arguments)
@@ -156,10 +164,11 @@ struct FiltRefs {
 // to a fraction of a turn before the FP32 sine and cosine.
 template <typename V, bool PREC>
 __global__ void __launch_bounds__(256) k_ref_filters(const double* __restrict__ ip, const double* __restrict__ pw,
-                                                     int64_t stride, const double* __restrict__ sig, FiltRefs refs,
+                                                     int64_t stride, SigmaArgs sig, FiltRefs refs,
                                                      int cnt, int64_t nbins, int64_t k0, int64_t k1,
                                                      V* __restrict__ F, int64_t fstride) {
   using R = typename real_of<V>::type;
+  const double scale = sigma_scale(sig);
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= nbins) return;
   if (k < k0 || k > k1) {
@@ -167,7 +176,7 @@ __global__ void __launch_bounds__(256) k_ref_filters(const double* __restrict__ 
     return;
   }
   const double u = pw[k], u5 = pw[stride + k], lu = pw[2 * stride + k];
-  const double a = sig[1] * pw[3 * stride + k] * ip[k];
+  const double a = scale * pw[3 * stride + k] * ip[k];
   for (int r = 0; r < cnt; ++r) {
     const double t = tf2_turn(refs.q[r], k, u, u5, lu);
     if constexpr (PREC) {
@@ -190,9 +199,10 @@ struct FiltPairs {
 __global__ void __launch_bounds__(256) k_ref_filters_pairs(const double* __restrict__ ip,
                                                            const double* __restrict__ ua,
                                                            const float2* __restrict__ pw32, int64_t stride,
-                                                           const double* __restrict__ sig, FiltPairs refs, int cnt,
-                                                           int64_t nbins, int64_t k0, int64_t k1,
+                                                           SigmaArgs sig, FiltPairs refs, int cnt, int64_t nbins,
+                                                           int64_t k0, int64_t k1,
                                                            float2* __restrict__ F, int64_t fstride) {
+  const double scale = sigma_scale(sig);
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= nbins) return;
   if (k < k0 || k > k1) {
@@ -200,7 +210,7 @@ __global__ void __launch_bounds__(256) k_ref_filters_pairs(const double* __restr
     return;
   }
   const float2 u = pw32[k], u5 = pw32[stride + k], lu = pw32[2 * stride + k];
-  const float a = (float)(sig[1] * ua[k] * ip[k]);
+  const float a = (float)(scale * ua[k] * ip[k]);
   for (int r = 0; r < cnt; ++r) {
     float s, c;
     sincospif(2.0f * tf2_turn(refs.q[r], Pair{u.x, u.y}, Pair{u5.x, u5.y}, Pair{lu.x, lu.y}), &s, &c);
@@ -227,26 +237,24 @@ __global__ void __launch_bounds__(256) k_template_fd(Tf2Bins q, const double* __
 // df^(-7/6)
 double amp_scale(double df) { return 1.0 / (df * std::cbrt(std::sqrt(df))); }
 
-// sigma^2 and the filter scale into c->red (after the partials), sigma to sigma_out[nref] (or null)
-double* launch_sigma2(rf_ctx* c, const double* inv_psd, double* sigma_out, int nref, cudaStream_t s) {
+// The partial sums of sigma^2; the filters finish them (and write sigma to sigma_out[nref], or null).
+SigmaArgs launch_sigma2(rf_ctx* c, const double* inv_psd, double* sigma_out, int nref, cudaStream_t s) {
   const double df = c->g.fs / (double)c->n;
   int64_t k0, k1;
   band_bins(c->g, &k0, &k1);
   const double amp = amp_scale(df);
   double* part = c->red.as<double>();
-  double* sig = part + kRedBlocks;
   // two blocks per SM at most, so that the one-warp sum of the partials stays short
-  const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(kRedBlocks, 2 * c->nsm), (k1 - k0 + 1) / (2 * kRedThreads)));
+  const int blocks = (int)std::max<int64_t>(
+      1, std::min<int64_t>(std::min(kRedBlocks, 2 * c->nsm), (k1 - k0 + 1) / (2 * kRedThreads)));
   k_sigma2_bins<<<blocks, kRedThreads, 0, s>>>(inv_psd, c->pw.as<double>() + 3 * c->pw_stride, k0, k1,
                                                4.0 * df * amp * amp, part);
   RF_LAUNCHED();
-  k_sigma2_finish<<<1, 32, 0, s>>>(part, blocks, (double)c->n, amp, sig, sigma_out, nref);
-  RF_LAUNCHED();
-  return sig;
+  return SigmaArgs{part, blocks, (double)c->n, amp, sigma_out, nref};
 }
 
 template <typename V, bool PREC>
-void launch_filters(rf_ctx* c, const double* inv_psd, const double* sig, int cnt, const rf_template* refs, V* F,
+void launch_filters(rf_ctx* c, const double* inv_psd, SigmaArgs sig, int cnt, const rf_template* refs, V* F,
                     int64_t fstride, cudaStream_t s) {
   const int64_t nbins = c->n / 2 + 1;
   const double df = c->g.fs / (double)c->n;
@@ -268,12 +276,14 @@ void launch_filters(rf_ctx* c, const double* inv_psd, const double* sig, int cnt
             inv_psd, c->pw.as<double>() + 3 * c->pw_stride, c->pw32.as<float2>(), c->pw_stride, sig, fp, m, nbins, k0,
             k1, F + (int64_t)r0 * fstride, fstride);
         RF_LAUNCHED();
+        sig.sigma_out = nullptr;  // written once
         continue;
       }
     }
     k_ref_filters<V, PREC><<<(unsigned)((nbins + 255) / 256), 256, 0, s>>>(
         inv_psd, c->pw.as<double>(), c->pw_stride, sig, fr, m, nbins, k0, k1, F + (int64_t)r0 * fstride, fstride);
     RF_LAUNCHED();
+    sig.sigma_out = nullptr;  // written once
   }
 }
 
@@ -319,7 +329,7 @@ void inverse_product(rf_ctx* c, const double2* X, const double2* F, int64_t fstr
 
 // Filters of a batch, then one product inverse for the batch.
 template <typename V, typename Inverse>
-void mf_batches(rf_ctx* c, const double* inv_psd, const double* sig, int32_t nref, const rf_template* refs,
+void mf_batches(rf_ctx* c, const double* inv_psd, SigmaArgs sig, int32_t nref, const rf_template* refs,
                 V* z_out, Inverse&& inverse, cudaStream_t s) {
   constexpr bool PREC = sizeof(V) == sizeof(double2);
   const int64_t n = c->n, nbins = n / 2 + 1;
@@ -330,6 +340,7 @@ void mf_batches(rf_ctx* c, const double* inv_psd, const double* sig, int32_t nre
   for (int r0 = 0; r0 < nref; r0 += batch) {
     const int cnt = std::min(batch, nref - r0);
     launch_filters<V, PREC>(c, inv_psd, sig, cnt, refs + r0, F, fstride, s);
+    sig.sigma_out = nullptr;
     inverse(F, fstride, z_out + (int64_t)r0 * n, tmp, cnt);
   }
 }
@@ -338,14 +349,14 @@ void mf_batches(rf_ctx* c, const double* inv_psd, const double* sig, int32_t nre
 
 void mf_reference_impl(rf_ctx* c, const void* x, const double* inv_psd, int32_t nref, const rf_template* refs,
                        void* z_out, double* sigma_out, cudaStream_t s) {
-  const double* sig = launch_sigma2(c, inv_psd, sigma_out, nref, s);
+  const SigmaArgs sig = launch_sigma2(c, inv_psd, sigma_out, nref, s);
   if (c->g.dtype == RF_F64) {
     forward_real(c, static_cast<const double*>(x), c->xf.as<double2>(), c->fb.as<double2>(), s);
     mf_batches(c, inv_psd, sig, nref, refs, static_cast<double2*>(z_out),
                [&](const double2* F, int64_t fs, double2* z, double2* tmp, int cnt) {
                  inverse_product(c, c->xf.as<double2>(), F, fs, z, tmp, cnt, s);
                }, s);
-  } else if (block_mf_supported(c)) {
+  } else if (block_mf_supported(c, nref)) {
     mf_batches(c, inv_psd, sig, nref, refs, static_cast<float2*>(z_out),
                [&](const float2* F, int64_t fs, float2* z, float2*, int cnt) {
                  block_mf(c, static_cast<const float*>(x), F, fs, z, cnt, s);
@@ -362,7 +373,7 @@ void mf_reference_impl(rf_ctx* c, const void* x, const double* inv_psd, int32_t 
 void reference_filters_impl(rf_ctx* c, const double* inv_psd, int32_t nref, const rf_template* refs, void* filt,
                             double* sigma_out, cudaStream_t s) {
   const int64_t nb = c->n / 2 + 1;
-  const double* sig = launch_sigma2(c, inv_psd, sigma_out, nref, s);
+  const SigmaArgs sig = launch_sigma2(c, inv_psd, sigma_out, nref, s);
   if (c->g.dtype == RF_F64)
     launch_filters<double2, true>(c, inv_psd, sig, nref, refs, static_cast<double2*>(filt), nb, s);
   else
@@ -372,7 +383,7 @@ void reference_filters_impl(rf_ctx* c, const double* inv_psd, int32_t nref, cons
 void mf_filtered_impl(rf_ctx* c, const void* x, int32_t nref, const void* filt, void* z_out, cudaStream_t s) {
   const int64_t n = c->n;
   const int64_t nb = n / 2 + 1;
-  if (block_mf_supported(c)) {
+  if (block_mf_supported(c, nref)) {
     block_mf(c, static_cast<const float*>(x), static_cast<const float2*>(filt), nb, static_cast<float2*>(z_out), nref,
              s);
     return;

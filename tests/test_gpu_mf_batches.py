@@ -53,3 +53,26 @@ def test_every_size_against_a_64_bit_transform(dtype, log2n):
     want = torch.fft.ifft(full) * n
     tol = 1e-12 if dtype == "f64" else 2e-6
     assert (z - want).abs().max().item() <= tol * want.abs().max().item()
+
+
+@pytest.mark.parametrize("log2n", [14, 15, 16])
+@pytest.mark.parametrize("nref", [1, 19, 20, 40])
+def test_clusters_and_the_forms_beyond_them(log2n, nref):
+    """Few references run on clusters, more on the other forms: rows agree with a 64-bit transform on
+    both sides of the line."""
+    torch = pytest.importorskip("torch")
+    from paper_2511_12894_gb300 import RatioFilter, launch_count
+    n = 1 << log2n
+    rf = RatioFilter(n, 2048.0, 20.0, 971.0, 7, "f32")
+    g = torch.Generator(device="cuda")
+    g.manual_seed(nref)
+    x = torch.randn(n, device="cuda", generator=g)
+    filt = torch.view_as_complex(torch.randn((nref, n // 2 + 1, 2), device="cuda", generator=g))
+    a = launch_count()
+    z = rf.mf_filtered(x, filt)
+    if nref * 8 <= torch.cuda.get_device_properties(0).multi_processor_count:
+        assert launch_count() - a == 1
+    full = torch.zeros((nref, n), dtype=torch.complex128, device="cuda")
+    full[:, : n // 2 + 1] = torch.fft.rfft(x.double()) * filt.to(torch.complex128)
+    want = torch.fft.ifft(full) * n
+    assert (z - want).abs().max().item() <= 2e-6 * want.abs().max().item()
