@@ -159,14 +159,37 @@ __global__ void __launch_bounds__(256) k_split_roots(const double2* __restrict__
   out[m] = cdf{make_float2(x, y), make_float2((float)(w.x - (double)x), (float)(w.y - (double)y))};
 }
 
-// exp(2 pi i t), t in [-1/2, 1/2]: the nearest 4096th root of unity and the series of the rest, whose
-// angle is below 7.7e-4 (relative errors of FP32 in its square and cube: 2e-14 and less).
-__device__ __forceinline__ cdf expi_turn(double t, const cdf* __restrict__ roots, int64_t root_step) {
-  const double big = 6755399441055744.0;
-  const double r = fma(t, 4096.0, big);
-  const double d = fma(-(r - big), 1.0 / 4096.0, t);
-  const float dh = (float)d, dl = (float)(d - (double)dh);
-  constexpr double two_pi = 6.28318530717958647692528676655900577;
+// exp(i (Psi_j - Psi_ref)) of bin k.  The phase is in 4096ths of a turn: the leading term, of up to
+// 10^6 of them, in FP64, reduced to a whole number and a rest that leaves the FP64 pipe as a
+// fixed-point number (its conversions to FP32 run at that pipe's rate); the others, fifty times smaller, in pairs
+// (2^-46 of them is 10^-12 of a turn).  Then the nearest 4096th root of unity and the series of the rest,
+// whose angle is below 7.7e-4 (relative errors of FP32 in its square and cube: 2e-14 and less).
+struct PairPhase {
+  double b0, d;
+  Tf2Pairs q;
+};
+__device__ __forceinline__ cdf expi_phase(const PairPhase& f, int64_t k, double u5d, Pair u, Pair u5, Pair lu,
+                                          const cdf* __restrict__ roots, int64_t root_step) {
+  double t = u5d * f.b0;
+  if (f.d != 0.0) t = fma((double)k, f.d, t);
+  const double big = 6755399441055744.0;  // 1.5 2^52: the sum's low bits are the nearest whole number's
+  const double r = t + big;
+  const double rest = t - (r - big);
+  constexpr double fix = 1536.0;  // 1.5 2^10: rest in units of 2^-42
+  const long long i = __double_as_longlong(rest + fix) - 0x4098000000000000ll;
+  const Pair p = pair_add(pair_mul(u, pair_add(pair_mul(u, f.q.b4), f.q.b3)), f.q.b2);
+  const Pair low = pair_mul(pair_mul(u5, pair_mul(u, u)), p);
+  const Pair high = pair_mul(u, pair_add(pair_mul(f.q.l6, lu), pair_add(pair_mul(f.q.b7, u), f.q.m6)));
+  const Pair s = pair_add(low, pair_add(high, pair_add(pair_mul(f.q.l5, lu), f.q.e)));
+  const float whole = rintf(s.h);
+  // the rest's two halves are exact in FP32: 22 bits and sign, 20 bits
+  const Pair fx{(float)(int)(i >> 20) * 2.384185791015625e-07f, (float)(int)(i & 0xfffff) * 2.2737367544323206e-13f};
+  Pair d = pair_add(fx, Pair{__fadd_rn(s.h, -whole), s.l});
+  const float m = rintf(d.h);
+  const int idx = __double2loint(r) + (int)whole + (int)m;
+  const float dh = __fadd_rn(__fadd_rn(d.h, -m), d.l);  // and what that sum loses
+  const float dl = __fadd_rn(__fadd_rn(__fadd_rn(d.h, -m), -dh), d.l);
+  constexpr double two_pi = 6.28318530717958647692528676655900577 / 4096.0;
   constexpr float ph = (float)two_pi, pl = (float)(two_pi - (double)ph);
   const float ah = __fmul_rn(dh, ph);
   const float al = __fmaf_rn(dh, ph, -ah) + (dh * pl + dl * ph);
@@ -175,7 +198,7 @@ __device__ __forceinline__ cdf expi_turn(double t, const cdf* __restrict__ roots
   const float ch = __fadd_rn(1.f, c1);
   const cdf e{make_float2(ch, ah),
               make_float2(__fadd_rn(c1, -__fadd_rn(ch, -1.f)), al + ah * q * __fmaf_rn(q, 1.f / 120.f, -1.f / 6.f))};
-  return cmul(e, cconj_pair(roots[(int64_t)(__double2loint(r) & 4095) * root_step]));
+  return cmul(e, cconj_pair(roots[(int64_t)(idx & 4095) * root_step]));
 }
 
 // First radix-16 pass of row blockIdx.y with K~ (as k_kernel_spectrum) formed on load: its bins above
@@ -183,21 +206,34 @@ __device__ __forceinline__ cdf expi_turn(double t, const cdf* __restrict__ roots
 __global__ void __launch_bounds__(128) k_pair_first(const Tf2Bins* __restrict__ dq, const double* __restrict__ dfl,
                                                     int64_t n, double df, int64_t k0, int64_t k1, double f_low,
                                                     double f_high, double df_high, const double* __restrict__ pw,
-                                                    int64_t stride, const cdf* __restrict__ roots,
-                                                    cdf* __restrict__ out) {
+                                                    const float2* __restrict__ pw32, int64_t stride,
+                                                    const cdf* __restrict__ roots, cdf* __restrict__ out) {
   const int64_t nq = n / 16;
   const int64_t i = (int64_t)blockIdx.x * 128 + threadIdx.x;
   if (i >= nq) return;
   const int j = blockIdx.y;
-  const Tf2Bins q = dq[j];
+  const Tf2Bins q = dq[j];  // in 4096ths of a turn
+  auto split = [](double x) {
+    const float h = (float)x;
+    return Pair{h, (float)(x - (double)h)};
+  };
+  const PairPhase f{q.b0, q.d,
+                    Tf2Pairs{Pair{0.f, 0.f}, split(q.b2), split(q.b3), split(q.b4), split(q.b7), split(q.l5),
+                             split(q.l6), split(q.m6), split(q.e)}};
   const float inv_n = 1.f / (float)n;  // n a power of two: exact
   const int64_t root_step = n / 4096;
   auto spectrum = [&](int64_t k) {
     cdf v{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
     const bool in = k >= k0 && k <= k1;
-    const double w = in ? 1.0 : (k > 0 ? window_w((double)k * df, f_low, f_high, dfl[j], df_high) : 0.0);
-    if (w > 0.0) {
-      v = expi_turn(tf2_turn(q, k, pw[k], pw[stride + k], pw[2 * stride + k]), roots, root_step);
+    double w = 1.0;
+    bool any = in;
+    if (!in && k > 0) {
+      w = window_w((double)k * df, f_low, f_high, dfl[j], df_high);
+      any = w > 0.0;
+    }
+    if (any) {
+      const float2 u = pw32[k], u5 = pw32[stride + k], lu = pw32[2 * stride + k];
+      v = expi_phase(f, k, pw[stride + k], Pair{u.x, u.y}, Pair{u5.x, u5.y}, Pair{lu.x, lu.y}, roots, root_step);
       if (!in) {
         const float wh = (float)w, wl = (float)(w - (double)wh);
         v = cmul(v, cdf{make_float2(wh, 0.f), make_float2(wl, 0.f)});
@@ -302,6 +338,7 @@ __global__ void __launch_bounds__(256) k_row_max2(const V* __restrict__ rho, int
   for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
     const V v = r[i];
     if (part_hi(v) < lim) continue;
+    asm volatile("" ::: "memory");  // no FP64 for the values left out
     const double a = mag2_rn(v);
     if (a > __longlong_as_double((long long)m)) {  // NaN never counts
       m = (unsigned long long)__double_as_longlong(a);
@@ -359,22 +396,58 @@ __global__ void __launch_bounds__(256) k_arc_parts(const V* __restrict__ rho, in
   ArcPart b{-1, -1, {-1, 0}};
   if (!relative || amax2[j] > 0.0) {
     const int64_t lo = (int64_t)part * per, hi = min(n, lo + per);
+    // eight groups loaded ahead; FP64 is entered only where a warp has a candidate (the empty asm keeps
+    // the compiler from evaluating it for every value, which took 333 to 700 us)
+    constexpr int U = 8;
+    unsigned masks[U];
     for (int64_t base = lo; base < hi; base += 32) {
-      const int64_t m = base + lane;
-      bool keep = false;
-      if (m < hi) {
-        const V v = r[m];
-        if (part_hi(v) >= lim) keep = mag2_rn(v) >= cut2;
+      const int u = (int)((base - lo) / 32) % U;
+      if (u == 0) {
+        V v[U];
+#pragma unroll
+        for (int g = 0; g < U; ++g) {
+          const int64_t m = base + 32 * g + lane;
+          v[g] = m < hi ? r[m] : V{};
+        }
+        unsigned any = 0;
+#pragma unroll
+        for (int g = 0; g < U; ++g) {
+          masks[g] = __ballot_sync(0xffffffffu, part_hi(v[g]) >= lim && base + 32 * g + lane < hi);
+          any |= masks[g];
+        }
+        if (!any) {
+          base += 32 * (U - 1);
+          continue;
+        }
+#pragma unroll
+        for (int g = 0; g < U; ++g)
+          if (masks[g]) {
+            asm volatile("" ::: "memory");
+            masks[g] = __ballot_sync(0xffffffffu, ((masks[g] >> lane) & 1u) && mag2_rn(v[g]) >= cut2);
+          }
       }
-      const unsigned mask = __ballot_sync(0xffffffffu, keep);
+      unsigned mask = 0;
+#pragma unroll
+      for (int g = 0; g < U; ++g)
+        if (g == u) mask = masks[g];
       if (!mask) continue;
       const int f = __ffs(mask) - 1;
       if (b.last >= 0) arc_take(b.best, base + f - b.last - 1, base + f, n);
       if (b.first < 0) b.first = base + f;
-      // the lags after the first of the group: all of them while no gap is known, else only those
-      // that follow a gap
+      // The lags after the first of the group.  Neighbouring lags are gaps of width 0, which matter only
+      // while no wider gap is known: then the smallest signed lag of them, the first above n/2 or the
+      // first.  (Taking every lag of a dense range in turn made its few warps the launch's tail.)
       unsigned rest = mask & (mask - 1);
-      if (b.best.gap > 0) rest &= ~(mask << 1);
+      if (b.best.gap < 1) {
+        const unsigned z = rest & (mask << 1);
+        if (z) {
+          arc_take(b.best, 0, base + __ffs(z) - 1, n);
+          const int64_t s = n / 2 + 1 - base;  // lags from here on are negative ones
+          const unsigned z2 = s <= 0 ? z : (s < 32 ? z >> s << s : 0u);
+          if (z2) arc_take(b.best, 0, base + __ffs(z2) - 1, n);
+        }
+      }
+      rest &= ~(mask << 1);
       while (rest) {
         const int q = __ffs(rest) - 1;
         rest &= rest - 1;
@@ -597,7 +670,9 @@ rf_kernels* build_impl(rf_ctx* c, const rf_template& ref, const rf_template* nbr
     band_bins(gb, &k0, &k1);
     const Tf2Bins qr = make_tf2_bins(pr, dfb);
     dq.resize(cnt);  // read by the copy until the chunk's synchronisation below
-    for (int q = 0; q < cnt; ++q) dq[q] = tf2_bins_minus(make_tf2_bins(tg[order[q0 + q]], dfb), qr);
+    // (for pairs in 4096ths of a turn, an exact scaling)
+    const double unit = pairs_at(nb) ? 4096.0 : 1.0;
+    for (int q = 0; q < cnt; ++q) dq[q] = tf2_bins_minus(make_tf2_bins(tg[order[q0 + q]], dfb), qr, unit);
     RF_CUDA(cudaMemcpyAsync(d_dq, dq.data(), sizeof(Tf2Bins) * cnt, cudaMemcpyHostToDevice, s));
     const unsigned mx = (unsigned)std::max<int64_t>(1, std::min<int64_t>(nb / 2048, (8LL * c->nsm + cnt - 1) / cnt));
     const unsigned rg = (unsigned)std::min<int64_t>(4096, (cnt * nb + 255) / 256);
@@ -615,8 +690,8 @@ rf_kernels* build_impl(rf_ctx* c, const rf_template& ref, const rf_template* nbr
       cdf* a = rows.as<cdf>();
       cdf* b = a + cnt * nb;
       k_pair_first<<<dim3((unsigned)((nb / 16 + 127) / 128), (unsigned)cnt), 128, 0, s>>>(
-          d_dq, d_dfls + q0, nb, dfb, k0, k1, c->g.f_low, c->g.f_high, c->g.df_high, c->pw.as<double>(), c->pw_stride,
-          roots.as<cdf>(), a);
+          d_dq, d_dfls + q0, nb, dfb, k0, k1, c->g.f_low, c->g.f_high, c->g.df_high, c->pw.as<double>(),
+          c->pw32.as<float2>(), c->pw_stride, roots.as<cdf>(), a);
       RF_LAUNCHED();
       bufP = pair_passes(a, b, nb, cnt, roots.as<cdf>(), s);
       if (real_form) {

@@ -786,7 +786,8 @@ void os_prepare_forms(rf_ctx* c, rf_kernels* kern, int nb, const BucketSpec* spe
     RF_CUDA(cudaMemcpyAsync(gpd.p, gp.data(), sizeof(int) * G, cudaMemcpyHostToDevice, s));
     float2* dst = kern->os_spec.as<float2>() + off[o.idx[0]];
     // FP64 transforms of the partitions, a bounded number of rows at a time
-    const int chunk = (int)std::max<int64_t>(1, std::min<int64_t>(4096, ((int64_t)256 << 20) / (3LL * B * 16)));
+    const int chunk = (int)std::min<int64_t>(
+        G, std::max<int64_t>(1, std::min<int64_t>(4096, ((int64_t)256 << 20) / (3LL * B * 16))));
     rows.ensure((size_t)3 * chunk * B * sizeof(double2));
     double2* in = rows.as<double2>();
     double2* out = in + (int64_t)chunk * B;

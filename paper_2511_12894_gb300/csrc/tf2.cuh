@@ -59,10 +59,13 @@ inline Tf2Bins make_tf2_bins(const Tf2& p, double df) {
   return q;
 }
 
-inline Tf2Bins tf2_bins_minus(const Tf2Bins& a, const Tf2Bins& b) {
-  return Tf2Bins{a.b0 - b.b0, a.b2 - b.b2, a.b3 - b.b3, a.b4 - b.b4, a.b7 - b.b7,
-                 a.l5 - b.l5, a.l6 - b.l6, a.m6 - b.m6, a.d - b.d,   a.e - b.e};
+// a - b, times `unit` (a power of two: the phase in parts of a turn)
+inline Tf2Bins tf2_bins_minus(const Tf2Bins& a, const Tf2Bins& b, double unit) {
+  return Tf2Bins{unit * (a.b0 - b.b0), unit * (a.b2 - b.b2), unit * (a.b3 - b.b3), unit * (a.b4 - b.b4),
+                 unit * (a.b7 - b.b7), unit * (a.l5 - b.l5), unit * (a.l6 - b.l6), unit * (a.m6 - b.m6),
+                 unit * (a.d - b.d),   unit * (a.e - b.e)};
 }
+
 
 // The phase of bin k as a fraction of a turn in [-1/2, 1/2].
 __device__ __forceinline__ double tf2_turn(const Tf2Bins& q, int64_t k, double u, double u5, double lu) {
