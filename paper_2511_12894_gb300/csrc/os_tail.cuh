@@ -39,6 +39,33 @@ template <int CH>
 __device__ __forceinline__ void window_keys(const float (&mv)[CH], int cnt, int i0, int64_t n, int64_t W,
                                             int64_t nw, int fastwin, unsigned long long* __restrict__ kj) {
   const int lane = threadIdx.x & 31;
+  // The usual case, decided for the warp: all of its 32 CH outputs exist and lie in one window.  The
+  // largest value is 12 to 16 maxima per thread, its first index is looked for where it sits, and no
+  // window or bound is compared per output (that was about 8% of the instructions of a 4096-point
+  // block: 125 short kernels at n = 2^20 545 us before).
+  {
+    const int iA = __shfl_sync(0xffffffffu, i0, 0);
+    const int wA = iA / (int)W;
+    const bool one = iA - wA * (int)W + 32 * CH <= (int)W && iA + 32 * CH <= (int)n;
+    if (__all_sync(0xffffffffu, one && cnt == CH)) {
+      float m = -1.f;  // stays if every value is NaN
+#pragma unroll
+      for (int e = 0; e < CH; ++e) m = fmaxf(m, mv[e]);
+      const unsigned hi = m >= 0.f ? __float_as_uint(m) : 0u;
+      const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+      unsigned lo = 0u;
+      if (m >= 0.f && hi == mh) {
+        int first = 0;
+#pragma unroll
+        for (int e = CH - 1; e >= 0; --e)
+          if (mv[e] == m) first = e;
+        lo = 0xffffffffu - (unsigned)(i0 + first);
+      }
+      lo = __reduce_max_sync(0xffffffffu, lo);
+      if (lane == 0 && lo) atomicMax(kj + wA, ((unsigned long long)mh << 32) | lo);
+      return;
+    }
+  }
   // sample index and window of this thread's first output; its outputs i0 + e (wrapping to
   // 0 at n) lie in window w0 below e_b = min(W - r0, n - i0) and in the next window w1 (w0 + 1,
   // or 0 after the wrap) from e_b on: at most two windows when W >= CH, which fastwin implies
