@@ -76,6 +76,18 @@ __device__ __forceinline__ V rot16(V a) {
     return cmake<V>(-a.x, -a.y);
   } else if constexpr (q == 12) {
     return cmake<V>(SIGN * a.y, -SIGN * a.x);
+  } else if constexpr (sizeof(R) == 4 && (q & 3) == 2) {
+    // (c, s) = H (+-1, +-1): two sums and one paired product, three instructions instead of four
+    // (0.3 to 0.5% of the overlap-save calls)
+    constexpr float H = 0.70710678118654752440f;
+    constexpr bool cp = q == 2 || q == 14, sp = (q < 8) == (SIGN > 0);
+    // x c - y s, x s + y c with c = cp ? H : -H, s = sp ? H : -H
+    const float x = (cp ? a.x : -a.x) - (sp ? a.y : -a.y);
+    const float y = (sp ? a.x : -a.x) + (cp ? a.y : -a.y);
+    V r;
+    asm("{.reg .b64 ra, rb, rd;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %4};\n\t"
+        "mul.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;}" : "=f"(r.x), "=f"(r.y) : "f"(x), "f"(y), "f"(H));
+    return r;
   } else {
     // cos(2 pi q / 16), sin(2 pi q / 16)
     constexpr double C1 = 0.92387953251128675613;  // cos(pi/8)
