@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(256) k_ref_filters(const double* __restrict__ 
 }
 
 // The same for FP32 grids with the phase in FP32 pairs (templates with t_c = 0).  Three references at
-// n = 2^20: the FP64 phase took 49 us of the FP64 pipe.
+// n = 2^20: the FP64 phase took 49 us of the FP64 pipe, this 12.5 us (issue 73%).
 struct FiltPairs {
   Tf2Pairs q[kFiltRefs];
 };
@@ -327,6 +327,21 @@ void inverse_product(rf_ctx* c, const double2* X, const double2* F, int64_t fstr
   else ifft_product_f64(X, F, fstride, z, tmp, c->n, cnt, c->tw64.as<double2>(), c->n, s);
 }
 
+// The one-launch form reads the data and the filters in every block, after other blocks may have
+// written their rows, so a caller's output that overlaps an input takes the passes, which transform
+// the data before anything is written.
+bool overlap(const void* a, size_t na, const void* b, size_t nb) {
+  const char* p = static_cast<const char*>(a);
+  const char* q = static_cast<const char*>(b);
+  return p < q + nb && q < p + na;
+}
+bool one_launch(const rf_ctx* c, int nref, const void* x, const void* filt, const void* z) {
+  if (!block_mf_supported(c, nref)) return false;
+  const size_t zb = sizeof(float2) * (size_t)nref * (size_t)c->n;
+  return !overlap(x, sizeof(float) * (size_t)c->n, z, zb) &&
+         !(filt && overlap(filt, sizeof(float2) * (size_t)nref * (size_t)(c->n / 2 + 1), z, zb));
+}
+
 // Filters of a batch, then one product inverse for the batch.
 template <typename V, typename Inverse>
 void mf_batches(rf_ctx* c, const double* inv_psd, SigmaArgs sig, int32_t nref, const rf_template* refs,
@@ -356,7 +371,7 @@ void mf_reference_impl(rf_ctx* c, const void* x, const double* inv_psd, int32_t 
                [&](const double2* F, int64_t fs, double2* z, double2* tmp, int cnt) {
                  inverse_product(c, c->xf.as<double2>(), F, fs, z, tmp, cnt, s);
                }, s);
-  } else if (block_mf_supported(c, nref)) {
+  } else if (one_launch(c, nref, x, nullptr, z_out)) {
     mf_batches(c, inv_psd, sig, nref, refs, static_cast<float2*>(z_out),
                [&](const float2* F, int64_t fs, float2* z, float2*, int cnt) {
                  block_mf(c, static_cast<const float*>(x), F, fs, z, cnt, s);
@@ -383,7 +398,7 @@ void reference_filters_impl(rf_ctx* c, const double* inv_psd, int32_t nref, cons
 void mf_filtered_impl(rf_ctx* c, const void* x, int32_t nref, const void* filt, void* z_out, cudaStream_t s) {
   const int64_t n = c->n;
   const int64_t nb = n / 2 + 1;
-  if (block_mf_supported(c, nref)) {
+  if (one_launch(c, nref, x, filt, z_out)) {
     block_mf(c, static_cast<const float*>(x), static_cast<const float2*>(filt), nb, static_cast<float2*>(z_out), nref,
              s);
     return;

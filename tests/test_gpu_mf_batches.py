@@ -76,3 +76,25 @@ def test_clusters_and_the_forms_beyond_them(log2n, nref):
     full[:, : n // 2 + 1] = torch.fft.rfft(x.double()) * filt.to(torch.complex128)
     want = torch.fft.ifft(full) * n
     assert (z - want).abs().max().item() <= 2e-6 * want.abs().max().item()
+
+
+def test_output_over_the_inputs():
+    """An output that overlaps the data or the filters gives the same rows."""
+    torch = pytest.importorskip("torch")
+    from paper_2511_12894_gb300 import RatioFilter
+    n, nref = 1 << 14, 5
+    rf = RatioFilter(n, 2048.0, 20.0, 971.0, 7, "f32")
+    g = torch.Generator(device="cuda")
+    g.manual_seed(2)
+    x = torch.randn(n, device="cuda", generator=g)
+    filt = torch.view_as_complex(torch.randn((nref, n // 2 + 1, 2), device="cuda", generator=g))
+    want = rf.mf_filtered(x, filt)
+    buf = torch.zeros(nref * n * 2, device="cuda")
+    for at in (0, 2 * n):                             # the data inside the output rows
+        buf[at:at + n] = x
+        z = rf.mf_filtered(buf[at:at + n], filt, z_out=torch.view_as_complex(buf.view(-1, 2)).view(nref, n))
+        assert (z - want).abs().max().item() <= 4e-6 * want.abs().max().item()
+    flat = torch.zeros(nref * n, dtype=torch.complex64, device="cuda")
+    flat[: filt.numel()] = filt.flatten()             # the filters inside the output rows
+    z = rf.mf_filtered(x, flat[: filt.numel()].view(nref, -1), z_out=flat.view(nref, n))
+    assert (z - want).abs().max().item() <= 4e-6 * want.abs().max().item()
