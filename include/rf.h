@@ -22,7 +22,7 @@
  *   RF_F64: real data double, complex data interleaved double2 (complex128);
  *   RF_F32: real data float,  complex data interleaved float2  (complex64).
  *   Template phases, their differences and all normalisation sums are FP64 in
- *   both modes.
+ *   both modes, except where a call says that RF_F32 grids take pairs of FP32 values.
  * Memory.  Unless stated otherwise a pointer argument is caller-owned DEVICE
  *   memory, 16-byte aligned, on the device that was current at rf_create.
  *   Host arrays are marked "host".  Opaque handles own their memory and are
@@ -147,6 +147,7 @@ rf_status rf_template_fd(rf_ctx* ctx, const rf_template* tmpl, void* h_out, rf_s
  *   N^2 = 4 df sum_{f_low<=f_k<=f_high} |h~_k|^2 inv_psd[k]             (Eq. 3, FP64)
  *   z[i] = (4 df / N) sum_{k=0}^{n/2} x~_k conj(h~_k) inv_psd[k] band_k exp(+2 pi i i k / n)
  * with x~_k = dt sum_j x[j] exp(-2 pi i j k / n) computed once for all references.
+ * On RF_F32 grids the phase of templates with tc = 0 is formed in pairs of FP32 values (about 46 bits).
  * x: real[n] (grid dtype); inv_psd: double[n/2+1], 1/S_n(f_k) (values outside the band are
  * ignored: Eq. 4); refs: host array of nref templates; z_out: complex[nref][n] (grid dtype);
  * sigma_out: double[nref] (device, N of each reference).  Async on stream. */
@@ -171,7 +172,9 @@ rf_status rf_reference_filters(rf_ctx* ctx, const double* inv_psd, int32_t nref,
  * in a CUDA graph).  Async on stream. */
 rf_status rf_mf_filtered(rf_ctx* ctx, const void* x, int32_t nref, const void* filt, void* z_out, rf_stream stream);
 
-/* Ratio kernels of k neighbours of one reference (Sec. II.B-II.D).  Per neighbour j, in FP64:
+/* Ratio kernels of k neighbours of one reference (Sec. II.B-II.D).  Per neighbour j, in FP64
+ * (RF_F32 grids: the transform and the small phase terms in pairs of FP32 values, about 46 bits of
+ * the largest magnitude, with RF_TRUNC_ANALYTIC or a relative thr >= 1e-7 on grids of at least 4096):
  *   K~_k = (N_ref/N_j) W(f_k) conj(h~_j(f_k) / h~_ref(f_k))   (Eqs. 5, 7 and window Eq. 9)
  *   rho[m] = (1/n) sum_{k=0}^{n/2} K~_k exp(+2 pi i k m / n),  m = 0..n-1
  * then truncation, chosen by the flags `relative` (RF_TRUNC_RELATIVE | RF_TRUNC_ANALYTIC):
@@ -429,7 +432,8 @@ typedef struct {
  * than 1024 taps.  out (host, may be NULL): up to max_out entries, the winner first; *n_out (host,
  * may be NULL) the number written.  Kernel sets end up prepared for the winner (a bucketed
  * winner, overlap-save or mixed, is then what RF_ALGO_AUTO runs; for another form, the last
- * layout timed).  Allocates; SYNCHRONISES `stream`. */
+ * layout timed).  On RF_F64 grids, where the direct sum is the only candidate, RF_ALGO_AUTO keeps
+ * the rule of rf_reconstruct.  Allocates; SYNCHRONISES `stream`. */
 rf_status rf_autotune(rf_ctx* ctx, int32_t G, const void* const* z_refs, rf_kernels* const* ks, int64_t W,
                       int32_t flags, int32_t max_os, rf_tune_entry* out, int32_t max_out, int32_t* n_out,
                       rf_stream stream);

@@ -12,8 +12,8 @@
 // Ns >= 32) every store of a warp is one contiguous run.  A pass of few butterflies takes small
 // thread blocks, so that it spreads over the SMs: a radix-16 FP64 butterfly is about 230
 // instructions on two FP64 lanes per SM, and the passes of one 2^16-point row took 18.5 us each
-// on 16 blocks of 256 threads (128 blocks of one warp: the FP64 matched filter of 2^16 samples
-// went from 188 to 111 us; FP32 at 2^14 samples from 49 to 45 us).
+// on 16 blocks of 256 threads (128 blocks of one warp took the FP64 matched filter of 2^16 samples
+// from 188 to 111 us, before the four-step form carried it).
 #include <array>
 #include <cmath>
 
