@@ -330,6 +330,14 @@ bool capturing(cudaStream_t s) {
   return st != cudaStreamCaptureStatusNone;
 }
 
+// Allocations of this thread while another thread captures a stream: the capture neither forbids
+// them nor records them.
+struct RelaxedCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedCapture() { (void)cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCapture() { (void)cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 }  // namespace
 
 void os64_create(rf_ctx* c) {
@@ -364,6 +372,8 @@ void os64_create(rf_ctx* c) {
 bool reconstruct_os64(rf_ctx* c, const void* z_ref, rf_kernels* kern, void* z_out, int64_t W, float* max_out,
                       int32_t* argmax_out, cudaStream_t s) {
   if (!c->pool || kern->k == 0) return false;
+  RelaxedCapture relaxed;
+  std::unique_lock<std::mutex> lock(kern->os64_mu);
   int B = kern->os64_B, Q = kern->os64_Q;
   if (B < 0) return false;
   if (!B) {
@@ -389,6 +399,7 @@ bool reconstruct_os64(rf_ctx* c, const void* z_ref, rf_kernels* kern, void* z_ou
       return false;
     }
   }
+  lock.unlock();
   const bool win = max_out != nullptr;
   const int64_t n = c->n;
   const int Lp = B / Q, H = B - Lp;

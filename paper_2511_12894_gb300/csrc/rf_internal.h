@@ -6,6 +6,7 @@
 #include <cstdint>
 #include <cstdio>
 #include <memory>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -260,7 +261,9 @@ struct rf_kernels {
   rf::DevBuf os_off_d;     // int64 [k]: element offset of kernel j's first partition spectrum
   rf::DevBuf os_parts_d;   // int32 [k]
   // FP64 overlap-save (reconstruct_os64.cu): layout (os64_B = 0: not prepared, -1: the direct sum)
-  // and partition spectra, double2.
+  // and partition spectra, double2.  The first AUTO call prepares them under os64_mu: several
+  // contexts may share a kernel set.
+  std::mutex os64_mu;
   int os64_B = 0, os64_Q = 0;
   rf::DevBuf os64_spec, os64_off_d, os64_parts_d;
   // Tensor-core direct form: split-BF16 (or TF32) tap operands per group of gemm_NJ neighbours and

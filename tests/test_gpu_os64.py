@@ -98,3 +98,44 @@ def test_streams_are_independent_and_capture_works(torch):
     torch.cuda.synchronize()
     assert all(torch.equal(a, b) for a, b in zip(o1, want1))
     assert all(torch.equal(a, b) for a, b in zip(o2, want2))
+
+
+def test_first_calls_of_several_threads(torch):
+    """One kernel set, a context per thread: the first calls at once, one of them while another
+    stream is captured."""
+    import threading
+    from paper_2511_12894_gb300 import RatioFilter
+    n, W = 1 << 14, 512
+    rf, z, kern = _case(torch, n, [900, 901, 902, 903])
+    want, wanta = rf.reconstruct_winmax(z, kern, W, "direct")
+    rfs = [RatioFilter(n, 1024.0, 40.0, 459.0, 2, "f64") for _ in range(4)]
+    outs = [(torch.empty_like(want), torch.empty_like(wanta)) for _ in rfs]
+    streams = [torch.cuda.Stream() for _ in rfs]
+    start = threading.Barrier(len(rfs))
+    errors = []
+
+    def work(r, s, o):
+        try:
+            start.wait()
+            r.reconstruct_winmax(z, kern, W, max_out=o[0], arg_out=o[1], stream=s)
+        except Exception as e:
+            errors.append(e)
+
+    buf = torch.zeros(16, device="cuda")
+    threads = [threading.Thread(target=work, args=a) for a in zip(rfs, streams, outs)]
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, capture_error_mode="global"):
+        buf.add_(1.0)
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+        buf.add_(1.0)
+    assert not errors
+    g.replay()
+    torch.cuda.synchronize()
+    assert buf.min().item() == buf.max().item() == 2.0
+    for p, a in outs:
+        assert torch.equal(a, wanta)
+        assert (p - want).abs().max().item() <= 1e-6 * want.max().item()   # FP32 outputs
