@@ -282,8 +282,15 @@ template <int N1, int N2> constexpr size_t cl_smem() {
   return sizeof(float2) * (size_t)(work + gr * cl_row<N2>() + gc * cl_row<N1>());
 }
 
+__device__ __forceinline__ void cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 __device__ __forceinline__ void cluster_barrier() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  cluster_arrive();
+  cluster_wait();
 }
 // v to the value at `p` of this block's shared memory, in block `rank` of the cluster
 __device__ __forceinline__ void st_cluster(float2* p, int rank, float2 v) {
@@ -307,6 +314,10 @@ __global__ void __cluster_dims__(kClusterBlocks, 1, 1) __launch_bounds__(N1 * N2
   const int64_t ref = blockIdx.x / kClusterBlocks;
   const int c = (int)threadIdx.x % GC, lc = (int)threadIdx.x / GC;  // column or output row, index in its line
   const int g = (int)threadIdx.x % GR, lr = (int)threadIdx.x / GR;  // spectrum row, index in its line
+  // A block's shared memory may be accessed by its peers only once it is known to have started: every
+  // block arrives here and waits just before its first store into the others, so that the loads and the
+  // first transform hide the barrier.
+  cluster_arrive();
   float2 v[16];
   {
     // data columns b of N1 points, to rows k1
@@ -314,6 +325,7 @@ __global__ void __cluster_dims__(kClusterBlocks, 1, 1) __launch_bounds__(N1 * N2
 #pragma unroll
     for (int t = 0; t < 16; ++t) v[t] = make_float2(__ldg(x + (int64_t)N2 * (lc + t * NT1) + b), 0.f);
     block_fft<N1, -1>(v, work + c * cl_line<N1>(), tb1, lc);
+    cluster_wait();
 #pragma unroll
     for (int t = 0; t < 16; ++t) {
       const int k1 = lc + t * NT1;
