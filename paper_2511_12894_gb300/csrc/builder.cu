@@ -317,13 +317,16 @@ __device__ __forceinline__ unsigned part_hi(double2 v) {
 __device__ __forceinline__ unsigned floor_hi(double m2, double2) {
   return (unsigned)__double2hiint(sqrt(0.5 * m2) * (1.0 - 1.9073486328125e-06));
 }
-// The same for pairs, by the bits of their high parts (2^-18 covers the low parts).
+// The same for pairs, by the bits of h + l rounded to FP32 (2^-18 covers the rounding).  h alone will
+// not do: the pairs are not renormalised, so after a cancellation l is of the size of the rounding of
+// the terms that cancelled, up to a quarter of a value 1e-7 of the row's largest.
 __device__ __forceinline__ double2 wide(cdf v) {
   return make_double2((double)v.h.x + (double)v.l.x, (double)v.h.y + (double)v.l.y);
 }
 __device__ __forceinline__ double mag2_rn(cdf v) { return mag2_rn(wide(v)); }
 __device__ __forceinline__ unsigned part_hi(cdf v) {
-  return max(__float_as_uint(v.h.x) & 0x7fffffffu, __float_as_uint(v.h.y) & 0x7fffffffu);
+  const float2 s = cadd(v.h, v.l);
+  return max(__float_as_uint(s.x) & 0x7fffffffu, __float_as_uint(s.y) & 0x7fffffffu);
 }
 __device__ __forceinline__ unsigned floor_hi(double m2, cdf) {
   return __float_as_uint((float)(sqrt(0.5 * m2) * (1.0 - 3.814697265625e-06)));

@@ -5,8 +5,8 @@
 // (the exact error of h + h by Knuth's two-sum, the low parts added to it), a product four plus the
 // sum, each done for the real and the imaginary part at once by the paired FP32 instructions, and is
 // five to seven times faster than its FP64 counterpart.  The pairs are not renormalised: l collects
-// the rounding errors of h, a few ulp of h, and the neglected terms are of the order of 2^-46 of the
-// operands.  Divisions of labour: the phase of a template stays FP64; sums of the transform and
+// the rounding errors of h, and the neglected terms are of the order of 2^-46 of the operands.  Both
+// are relative to the operands: where a sum cancels, l can be as large as h.  Divisions of labour: the phase of a template stays FP64; sums of the transform and
 // products with roots of unity are pairs; magnitudes that decide a threshold are formed in FP64 from
 // h + l.
 #pragma once
