@@ -174,7 +174,10 @@ rf_status rf_mf_filtered(rf_ctx* ctx, const void* x, int32_t nref, const void* f
 
 /* Ratio kernels of k neighbours of one reference (Sec. II.B-II.D).  Per neighbour j, in FP64
  * (RF_F32 grids: the transform and the small phase terms in pairs of FP32 values, about 46 bits of
- * the largest magnitude, with RF_TRUNC_ANALYTIC or a relative thr >= 1e-7 on grids of at least 4096):
+ * the largest magnitude, with RF_TRUNC_ANALYTIC or RF_TRUNC_RELATIVE on grids of at least 4096 bins, for the
+ * kernels whose smallest kept taps that leaves as good as their rounding: relative thresholds from
+ * about 4e-6 for neighbours of one bank.  A kernel whose span the pairs' error could change is made again
+ * in FP64, so spans are those of FP64, and each kernel is the same whatever else the call builds):
  *   K~_k = (N_ref/N_j) W(f_k) conj(h~_j(f_k) / h~_ref(f_k))   (Eqs. 5, 7 and window Eq. 9)
  *   rho[m] = (1/n) sum_{k=0}^{n/2} K~_k exp(+2 pi i k m / n),  m = 0..n-1
  * then truncation, chosen by the flags `relative` (RF_TRUNC_RELATIVE | RF_TRUNC_ANALYTIC):

@@ -31,6 +31,31 @@ namespace rf {
 
 namespace {
 
+// ---------------------------------------------------------------- FP32 grids: transforms in pairs
+// The taps of an FP32 grid are rounded to FP32, and the transform that makes them cost 2.9 of the 7 ms
+// of building 48 kernels on 2^19 bins, all of it on the FP64 pipe.  The same radix passes in FP32
+// pairs (cdf.cuh) are bound by HBM: 172 to 184 us per radix-16 pass of those rows (805 MB, 55% of the
+// copy rate), the whole build 1.87 ms.  The leading term of the phase stays FP64.
+//
+// Pairs serve where the result is the FP64 one:
+// * A row's error is bounded by eps times its largest value: 2^-43 for the transform (2^-46.4 measured,
+//   n = 2^14 .. 2^22) and what the phase loses, 2^-53 of its leading term and 2^-46 of the others.
+// * A kernel is made in pairs when eps is at most 2^-23 of the truncation threshold, so that the smallest
+//   kept tap is as good as its rounding to FP32 (thresholds from about 4e-6 for neighbours of one
+//   bank); else, for absolute thresholds on |rho|^2 and for grids below 4096 bins, in FP64.  Each
+//   kernel is judged by itself: what else is built in the call makes no difference.
+// * A kernel whose span depends on a lag within eps of the cut (or, for analytic spans, on the last
+//   bits of the largest value) is made again in FP64 before it is cut.
+constexpr int64_t kPairMinGrid = 4096;
+constexpr double kPairTransformErr = 1.0 / (double)(1ll << 43);
+constexpr double kPairTapErr = 1.0 / (double)(1 << 23);
+
+// A template's phase minus the reference's (for pairs in 4096ths of a turn) and, for pairs, eps.
+struct RowPhase {
+  Tf2Bins q;
+  double eps;
+};
+
 __global__ void k_df_low(Tf2 ref, const Tf2* __restrict__ tg, int count, double f_low, double df_low_max,
                          double* __restrict__ out) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -59,13 +84,16 @@ __global__ void k_grid_extent(Tf2 ref, const Tf2* __restrict__ tg, const double*
 // on both sides of its lag time c_e = -dt(f_e); the kept lags run from floor(min(c_e - d_e) fs)
 // to ceil(max(c_e + d_e) fs), at most the grid.
 // (rfac: |r| = rfac fs |rho|, 2 for the complex kernel, 1 for the real form's taps 2 Re rho.)
+// rp: null, or the rows' phases (kernels in pairs): a span that the error of the row's largest value
+// could change, or taps kept down to a level that it disturbs, are marked by len = -len - 1.
 __global__ void k_analytic_span(Tf2 ref, const Tf2* __restrict__ tg, const double* __restrict__ dfl,
-                                const double* __restrict__ amax2, int count, double thr, int relative, double rfac,
-                                int64_t nb, double fs, double f_low, double f_high, double df_high,
-                                int* __restrict__ m0_out, int* __restrict__ len_out) {
+                                const double* __restrict__ amax2, const RowPhase* __restrict__ rp, int count,
+                                double thr, int relative, double rfac, int64_t nb, double fs, double f_low,
+                                double f_high, double df_high, int* __restrict__ m0_out, int* __restrict__ len_out) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= count) return;
-  const double amp = relative ? thr * rfac * fs * sqrt(amax2[j]) : thr;
+  const double top = rfac * fs * sqrt(amax2[j]);
+  const double amp = relative ? thr * top : thr;
   if (!(amp > 0.0)) {
     m0_out[j] = 0;
     len_out[j] = 0;
@@ -73,28 +101,47 @@ __global__ void k_analytic_span(Tf2 ref, const Tf2* __restrict__ tg, const doubl
   }
   const double fe[4] = {f_low - dfl[j], f_low, f_high, f_high + df_high};
   const double dfe[4] = {dfl[j], dfl[j], df_high, df_high};
-  double lo = INFINITY, hi = -INFINITY;
+  double c[4];
 #pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    const double c = -((tf2_dphase(tg[j], fe[e]) - tf2_dphase(ref, fe[e])) / kTwoPi);
-    const double R = tf2_amp(fe[e]) / tf2_amp(fe[e]);  // B_j / B_ref: one amplitude law
-    const double d = cbrt(R / (4.0 * kPi * dfe[e] * dfe[e] * amp));
-    lo = fmin(lo, c - d);
-    hi = fmax(hi, c + d);
+  for (int e = 0; e < 4; ++e) c[e] = -((tf2_dphase(tg[j], fe[e]) - tf2_dphase(ref, fe[e])) / kTwoPi);
+  auto span = [&](double a, int& m0, int& len) {
+    double lo = INFINITY, hi = -INFINITY;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const double R = tf2_amp(fe[e]) / tf2_amp(fe[e]);  // B_j / B_ref: one amplitude law
+      const double d = cbrt(R / (4.0 * kPi * dfe[e] * dfe[e] * a));
+      lo = fmin(lo, c[e] - d);
+      hi = fmax(hi, c[e] + d);
+    }
+    // a span as long as the grid (a tiny amplitude, or a taper of width 0) keeps the whole
+    // grid from lag 0; decided in double, before any integer conversion
+    const double flo = floor(lo * fs), fhi = ceil(hi * fs);
+    if (!(fhi - flo + 1.0 < (double)nb)) {
+      m0 = 0;
+      len = (int)nb;
+      return;
+    }
+    const long long m_lo = (long long)flo, m_hi = (long long)fhi;
+    long long m = m_lo & (nb - 1);
+    if (m > nb / 2) m -= nb;
+    m0 = (int)m;
+    len = (int)(m_hi - m_lo + 1);
+  };
+  int m0, len;
+  span(amp, m0, len);
+  bool unsure = false;
+  if (rp) {
+    const double eps = rp[j].eps;
+    unsure = !(eps * top <= kPairTapErr * amp);
+    if (relative && !unsure) {
+      int ma, la, mb, lb;
+      span(amp * (1.0 - eps), ma, la);
+      span(amp * (1.0 + eps), mb, lb);
+      unsure = ma != mb || la != lb;
+    }
   }
-  // a span as long as the grid (a tiny amplitude, or a taper of width 0) keeps the whole
-  // grid from lag 0; decided in double, before any integer conversion
-  const double flo = floor(lo * fs), fhi = ceil(hi * fs);
-  if (!(fhi - flo + 1.0 < (double)nb)) {
-    m0_out[j] = 0;
-    len_out[j] = (int)nb;
-    return;
-  }
-  const long long m_lo = (long long)flo, m_hi = (long long)fhi;
-  long long m0 = m_lo & (nb - 1);
-  if (m0 > nb / 2) m0 -= nb;
-  m0_out[j] = (int)m0;
-  len_out[j] = (int)(m_hi - m_lo + 1);
+  m0_out[j] = m0;
+  len_out[j] = unsure ? -len - 1 : len;
 }
 
 // Real-kernel form: rho -> 2 Re rho in place (imaginary parts zero).
@@ -108,7 +155,7 @@ __global__ void k_real_form(cdf* __restrict__ rho, int64_t count) {
     rho[i] = cdf{make_float2(2.f * rho[i].h.x, 0.f), make_float2(2.f * rho[i].l.x, 0.f)};
 }
 
-// One row per template (grid.y): K~ over the full length-n buffer.  dq: the template's phase minus
+// One row per template (grid.y): K~ over the full length-n buffer.  rp: the template's phase minus
 // the reference's (tf2.cuh); [k0, k1]: the bins inside [f_low, f_high], where W = 1.  Bound by the
 // FP64 pipe (two lanes per SM): the phase from the tables of bin powers is about ten multiply-adds
 // a bin.
@@ -117,7 +164,7 @@ __global__ void k_real_form(cdf* __restrict__ rho, int64_t count) {
 // stationary-phase family has the amplitude law A f^-7/6 on the same band, so h~_j / h~_ref =
 // (A_j / A_ref) e^{-i dPsi} and N_j / N_ref = A_j / A_ref: the two amplitude factors cancel exactly
 // for any scales A, and |K~| = W.
-__global__ void __launch_bounds__(256) k_kernel_spectrum(const Tf2Bins* __restrict__ dq,
+__global__ void __launch_bounds__(256) k_kernel_spectrum(const RowPhase* __restrict__ rp,
                                                          const double* __restrict__ dfl, int64_t n, double df,
                                                          int64_t k0, int64_t k1, double f_low, double f_high,
                                                          double df_high, const double* __restrict__ pw,
@@ -132,25 +179,14 @@ __global__ void __launch_bounds__(256) k_kernel_spectrum(const Tf2Bins* __restri
         k >= k0 && k <= k1 ? inv_n : inv_n * window_w((double)k * df, f_low, f_high, dfl[j], df_high);
     if (a > 0.0) {
       double s, c;
-      sincospi(2.0 * tf2_turn(dq[j], k, pw[k], pw[stride + k], pw[2 * stride + k]), &s, &c);
+      sincospi(2.0 * tf2_turn(rp[j].q, k, pw[k], pw[stride + k], pw[2 * stride + k]), &s, &c);
       out = make_double2(a * c, a * s);
     }
   }
   K[(int64_t)j * n + k] = out;
 }
 
-// ---------------------------------------------------------------- FP32 grids: transforms in pairs
-// The taps of an FP32 grid are rounded to FP32, and the transform that makes them cost 2.9 of the 7 ms
-// of building 48 kernels on 2^19 bins, all of it on the FP64 pipe.  The same radix passes in FP32
-// pairs (cdf.cuh) are bound by HBM: 172 to 184 us per radix-16 pass of those rows (805 MB, 55% of the
-// copy rate), the whole build 1.87 ms.  The leading term of the phase stays FP64.  A pair carries
-// about 46 bits of the row's largest value, so the kept span, decided at thr times that value, is
-// the FP64 one wherever thr is
-// far above 2^-46: pairs are used from thr = 1e-7 on (and for analytic spans, which only take the
-// largest value), FP64 below it, for absolute thresholds and for grids below 4096 bins.
-constexpr double kPairMinThr = 1e-7;
-constexpr int64_t kPairMinGrid = 4096;
-
+// ---------------------------------------------------------------- pairs
 // exp(-2 pi i m / nb) as pairs, from the FP64 table of n entries
 __global__ void __launch_bounds__(256) k_split_roots(const double2* __restrict__ tw, int64_t stride, int64_t nb,
                                                      cdf* __restrict__ out) {
@@ -205,7 +241,7 @@ __device__ __forceinline__ cdf expi_phase(const PairPhase& f, int64_t k, double 
 
 // First radix-16 pass of row blockIdx.y with K~ (as k_kernel_spectrum) formed on load: its bins above
 // n/2 are zero, so half of the inputs are never formed and the spectrum never reaches memory.
-__global__ void __launch_bounds__(128) k_pair_first(const Tf2Bins* __restrict__ dq, const double* __restrict__ dfl,
+__global__ void __launch_bounds__(128) k_pair_first(const RowPhase* __restrict__ rp, const double* __restrict__ dfl,
                                                     int64_t n, double df, int64_t k0, int64_t k1, double f_low,
                                                     double f_high, double df_high, const double* __restrict__ pw,
                                                     const float2* __restrict__ pw32, int64_t stride,
@@ -214,7 +250,7 @@ __global__ void __launch_bounds__(128) k_pair_first(const Tf2Bins* __restrict__ 
   const int64_t i = (int64_t)blockIdx.x * 128 + threadIdx.x;
   if (i >= nq) return;
   const int j = blockIdx.y;
-  const Tf2Bins q = dq[j];  // in 4096ths of a turn
+  const Tf2Bins q = rp[j].q;  // in 4096ths of a turn
   auto split = [](double x) {
     const float h = (float)x;
     return Pair{h, (float)(x - (double)h)};
@@ -368,15 +404,17 @@ __device__ __forceinline__ void arc_take(ArcBest& b, long long gap, long long m,
   }
 }
 
-// Kept lags of a contiguous range: first and last (-1: none) and the widest gap between two
-// consecutive ones with the lag after it.
+// Kept lags of a contiguous range: first and last (-1: none), the widest gap between two
+// consecutive ones with the lag after it, and whether some lag's value is too near the cut to say.
 struct ArcPart {
   long long first, last;
   ArcBest best;
+  int unsure;
 };
 
 // b followed by a later range c
 __device__ __forceinline__ void arc_join(ArcPart& b, const ArcPart& c, long long n) {
+  b.unsure |= c.unsure;
   if (c.first < 0) return;
   if (b.last >= 0) arc_take(b.best, c.first - b.last - 1, c.first, n);
   if (c.best.gap >= 0) arc_take(b.best, c.best.gap, c.best.m0, n);
@@ -386,10 +424,12 @@ __device__ __forceinline__ void arc_join(ArcPart& b, const ArcPart& c, long long
 
 // Shortest covering arc of {m : |rho[m]|^2 >= cut2}, first step: a warp summarises `per` consecutive
 // lags, 32 at a time by ballot.  (One block per row with a range per thread read its 2^19 values at a
-// stride: 676 us for 48 rows.)
+// stride: 676 us for 48 rows.)  Pairs: lags whose |rho| is within eps of the row's largest of the cut
+// are reported (rp).  The values are compared as integers, so that this costs no FP64.
 template <typename V>
 __global__ void __launch_bounds__(256) k_arc_parts(const V* __restrict__ rho, int64_t n, int per, int nparts,
-                                                   const double* __restrict__ amax2, double thr, int relative,
+                                                   const double* __restrict__ amax2,
+                                                   const RowPhase* __restrict__ rp, double thr, int relative,
                                                    ArcPart* __restrict__ parts) {
   const int j = blockIdx.y;
   const int part = blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -397,8 +437,15 @@ __global__ void __launch_bounds__(256) k_arc_parts(const V* __restrict__ rho, in
   const int lane = threadIdx.x & 31;
   const V* r = rho + (int64_t)j * n;
   const double cut2 = __dmul_rn(__dmul_rn(thr, thr), relative ? amax2[j] : 1.0);
-  const unsigned lim = floor_hi(cut2, V{});
-  ArcPart b{-1, -1, {-1, 0}};
+  // (|rho| -+ eps max)^2 of cut2, the square of eps in the 2^-10
+  const double band = std::is_same<V, cdf>::value ? (2.0 + 0x1p-10) * rp[j].eps * thr * amax2[j] : 0.0;
+  const unsigned lim = floor_hi(fmax(0.0, cut2 - band), V{});
+  using U64 = unsigned long long;
+  const U64 cut_bits = (U64)__double_as_longlong(cut2), inf_bits = 0x7ff0000000000000ull;
+  const U64 lo_bits = (U64)__double_as_longlong(fmax(0.0, cut2 - band));
+  const U64 band_bits = (U64)__double_as_longlong(cut2 + band) - lo_bits;
+  bool near = false;
+  ArcPart b{-1, -1, {-1, 0}, 0};
   if (!relative || amax2[j] > 0.0) {
     const int64_t lo = (int64_t)part * per, hi = min(n, lo + per);
     // eight groups loaded ahead; FP64 is entered only where a warp has a candidate (the empty asm keeps
@@ -428,7 +475,10 @@ __global__ void __launch_bounds__(256) k_arc_parts(const V* __restrict__ rho, in
         for (int g = 0; g < U; ++g)
           if (masks[g]) {
             asm volatile("" ::: "memory");
-            masks[g] = __ballot_sync(0xffffffffu, ((masks[g] >> lane) & 1u) && mag2_rn(v[g]) >= cut2);
+            const bool cand = (masks[g] >> lane) & 1u;
+            const U64 m2 = cand ? (U64)__double_as_longlong(mag2_rn(v[g])) : ~0ull;
+            masks[g] = __ballot_sync(0xffffffffu, m2 >= cut_bits && m2 <= inf_bits);
+            if (std::is_same<V, cdf>::value) near |= m2 - lo_bits <= band_bits;
           }
       }
       unsigned mask = 0;
@@ -462,33 +512,48 @@ __global__ void __launch_bounds__(256) k_arc_parts(const V* __restrict__ rho, in
       b.last = base + 31 - __clz(mask);
     }
   }
+  if (std::is_same<V, cdf>::value) b.unsure = __any_sync(0xffffffffu, near);
   if (lane == 0) parts[(int64_t)j * nparts + part] = b;
 }
 
-// Second step, a warp per row: the ranges joined in order, then the circle closed.
+// Second step, a warp per row: the ranges joined in order, then the circle closed.  A row with a lag
+// too near the cut has len = -len - 1.
 __global__ void __launch_bounds__(32) k_arc_join(const ArcPart* __restrict__ parts, int nparts, int64_t n,
                                                  int* __restrict__ m0_out, int* __restrict__ len_out) {
   const int j = blockIdx.x, lane = threadIdx.x;
   const int ch = (nparts + 31) / 32;
-  ArcPart b{-1, -1, {-1, 0}};
+  ArcPart b{-1, -1, {-1, 0}, 0};
   for (int q = lane * ch; q < min(nparts, (lane + 1) * ch); ++q) arc_join(b, parts[(int64_t)j * nparts + q], n);
-  ArcPart g{-1, -1, {-1, 0}};
+  ArcPart g{-1, -1, {-1, 0}, 0};
   for (int l = 0; l < 32; ++l) {
     ArcPart c;
     c.first = __shfl_sync(0xffffffffu, b.first, l);
     c.last = __shfl_sync(0xffffffffu, b.last, l);
     c.best.gap = __shfl_sync(0xffffffffu, b.best.gap, l);
     c.best.m0 = __shfl_sync(0xffffffffu, b.best.m0, l);
+    c.unsure = __shfl_sync(0xffffffffu, b.unsure, l);
     arc_join(g, c, n);
   }
   if (lane) return;
-  if (g.first < 0) {
-    m0_out[j] = 0;
-    len_out[j] = 0;
-  } else {
+  int m0 = 0, len = 0;
+  if (g.first >= 0) {
     arc_take(g.best, g.first + n - g.last - 1, g.first, n);
-    m0_out[j] = (int)arc_key(g.best.m0, n);
-    len_out[j] = (int)(n - g.best.gap);
+    m0 = (int)arc_key(g.best.m0, n);
+    len = (int)(n - g.best.gap);
+  }
+  m0_out[j] = m0;
+  len_out[j] = g.unsure ? -len - 1 : len;
+}
+
+// Row at[blockIdx.y] of pairs from row blockIdx.y in FP64.
+__global__ void __launch_bounds__(256) k_rows_to_pairs(const double2* __restrict__ in, const int* __restrict__ at,
+                                                       int64_t n, cdf* __restrict__ out) {
+  in += (int64_t)blockIdx.y * n;
+  out += (int64_t)at[blockIdx.y] * n;
+  for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
+    const double2 v = in[i];
+    const float2 h = make_float2((float)v.x, (float)v.y);
+    out[i] = cdf{h, make_float2((float)(v.x - (double)h.x), (float)(v.y - (double)h.y))};
   }
 }
 
@@ -561,7 +626,7 @@ rf_kernels* build_impl(rf_ctx* c, const rf_template& ref, const rf_template* nbr
   // [phase differences][amax2][m0][len]
   const int64_t kmax_chunk = std::min<int64_t>(k, 4096);
   const size_t meta_bytes = 2 * sizeof(Tf2) * (size_t)k + sizeof(double) * (3 * (size_t)k + 8 + kmax_chunk) +
-                            (sizeof(Tf2Bins) + 2 * sizeof(int)) * (size_t)kmax_chunk + 8192;
+                            (sizeof(RowPhase) + 2 * sizeof(int)) * (size_t)kmax_chunk + 8192;
   StreamBuf meta(c, meta_bytes, s);
   char* mp = meta.need().as<char>();
   auto carve = [&](size_t bytes) {
@@ -574,7 +639,7 @@ rf_kernels* build_impl(rf_ctx* c, const rf_template& ref, const rf_template* nbr
   double* d_ext = reinterpret_cast<double*>(carve(sizeof(double) * k));
   Tf2* d_tgs = reinterpret_cast<Tf2*>(carve(sizeof(Tf2) * k));
   double* d_dfls = reinterpret_cast<double*>(carve(sizeof(double) * k));
-  Tf2Bins* d_dq = reinterpret_cast<Tf2Bins*>(carve(sizeof(Tf2Bins) * kmax_chunk));
+  RowPhase* d_rp = reinterpret_cast<RowPhase*>(carve(sizeof(RowPhase) * kmax_chunk));
   double* d_amax = reinterpret_cast<double*>(carve(sizeof(double) * kmax_chunk));
   int* d_m0 = reinterpret_cast<int*>(carve(sizeof(int) * kmax_chunk));
   int* d_len = reinterpret_cast<int*>(carve(sizeof(int) * kmax_chunk));
@@ -604,10 +669,32 @@ rf_kernels* build_impl(rf_ctx* c, const rf_template& ref, const rf_template* nbr
     for (int j = 0; j < k; ++j) kern->grid[j] = n_build;
   }
   RF_CUDA(cudaStreamSynchronize(s));  // df_low is on the host
-  // neighbours in grid order (stable), chunks of one grid
+  // which kernels are made in pairs (eps > 0; the rule above)
+  const bool rel = relative & RF_TRUNC_RELATIVE, analytic = relative & RF_TRUNC_ANALYTIC;
+  auto phase_of = [&](int j, double unit) {
+    const double dfb = c->g.fs / (double)kern->grid[j];
+    return tf2_bins_minus(make_tf2_bins(tg[j], dfb), make_tf2_bins(pr, dfb), unit);
+  };
+  std::vector<double> eps(k, 0.0);
+  if (!f64 && (rel || analytic))
+    for (int j = 0; j < k; ++j) {
+      const int64_t nb = kern->grid[j];
+      if (nb < kPairMinGrid) continue;
+      const double dfb = c->g.fs / (double)nb;
+      const double ka = std::max(1.0, std::floor((c->g.f_low - kern->df_low[j]) / dfb));
+      const double kb = std::max(ka, std::min(0.5 * (double)nb, std::ceil((c->g.f_high + c->g.df_high) / dfb)));
+      const Tf2Size size = tf2_bins_size(phase_of(j, 1.0), ka, kb);
+      const double e = kPairTransformErr + kTwoPi * (size.lead * 0x1p-53 + size.rest * 0x1p-46);
+      // (an absolute analytic amplitude shows its level only beside the largest value: k_analytic_span;
+      // below 2^-30 of the phase every term also fits the integers of expi_phase)
+      if (e <= (rel ? std::min(kPairTapErr * thr, 0x1p-30) : 0x1p-30)) eps[j] = e;
+    }
+  // neighbours in grid order (stable), FP64 before pairs; chunks of one grid and kind
   std::vector<int> order(k);
   for (int j = 0; j < k; ++j) order[j] = j;
-  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return kern->grid[a] < kern->grid[b]; });
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+    return kern->grid[a] != kern->grid[b] ? kern->grid[a] < kern->grid[b] : (eps[a] > 0.0) < (eps[b] > 0.0);
+  });
   bool identity = true;
   for (int q = 0; q < k && identity; ++q) identity = order[q] == q;
   if (identity) {
@@ -631,20 +718,17 @@ rf_kernels* build_impl(rf_ctx* c, const rf_template& ref, const rf_template* nbr
   std::vector<int> part_of(k);
   std::vector<int64_t> at_in_part(k);
   std::vector<int> hm0(kmax_chunk), hlen(kmax_chunk);
-  std::vector<Tf2Bins> dq;
+  std::vector<RowPhase> rp;
   std::vector<std::vector<int64_t>> off_host;
-  // FP32 grids: transforms in pairs where the truncation allows (above)
-  auto pairs_at = [&](int64_t nb) {
-    return !f64 && nb >= kPairMinGrid &&
-           ((relative & RF_TRUNC_ANALYTIC) || ((relative & RF_TRUNC_RELATIVE) && thr >= kPairMinThr));
-  };
   // templates per chunk: three complex128 rows of nb per template (two of pairs), about 1.5 GB in total
   auto chunk_at = [&](int q0) {
     const int64_t nb = kern->grid[order[q0]];
     const int64_t per = 3 * nb * (int64_t)sizeof(double2);
     const int64_t most = std::min<int64_t>(kmax_chunk, std::max<int64_t>(1, ((int64_t)1536 << 20) / per));
     int cnt = 0;
-    while (q0 + cnt < k && cnt < most && kern->grid[order[q0 + cnt]] == nb) ++cnt;
+    while (q0 + cnt < k && cnt < most && kern->grid[order[q0 + cnt]] == nb &&
+           (eps[order[q0 + cnt]] > 0.0) == (eps[order[q0]] > 0.0))
+      ++cnt;
     return cnt;
   };
   size_t rows_bytes = 0;
@@ -657,7 +741,7 @@ rf_kernels* build_impl(rf_ctx* c, const rf_template& ref, const rf_template* nbr
   rows.need();
   int64_t roots_n = 0;
   for (int j = 0; j < k; ++j)
-    if (pairs_at(kern->grid[j])) roots_n = std::max(roots_n, kern->grid[j]);
+    if (eps[j] > 0.0) roots_n = std::max(roots_n, kern->grid[j]);
   StreamBuf roots(c, sizeof(cdf) * (size_t)roots_n, s);
   if (roots_n) roots.need();
   int64_t roots_of = 0;
@@ -673,19 +757,52 @@ rf_kernels* build_impl(rf_ctx* c, const rf_template& ref, const rf_template* nbr
     gb.n = nb;
     int64_t k0, k1;
     band_bins(gb, &k0, &k1);
-    const Tf2Bins qr = make_tf2_bins(pr, dfb);
-    dq.resize(cnt);  // read by the copy until the chunk's synchronisation below
+    const bool pairs = eps[order[q0]] > 0.0;
+    rp.resize(cnt);  // read by the copy until the chunk's synchronisation below
     // (for pairs in 4096ths of a turn, an exact scaling)
-    const double unit = pairs_at(nb) ? 4096.0 : 1.0;
-    for (int q = 0; q < cnt; ++q) dq[q] = tf2_bins_minus(make_tf2_bins(tg[order[q0 + q]], dfb), qr, unit);
-    RF_CUDA(cudaMemcpyAsync(d_dq, dq.data(), sizeof(Tf2Bins) * cnt, cudaMemcpyHostToDevice, s));
-    const unsigned mx = (unsigned)std::max<int64_t>(1, std::min<int64_t>(nb / 2048, (8LL * c->nsm + cnt - 1) / cnt));
-    const unsigned rg = (unsigned)std::min<int64_t>(4096, (cnt * nb + 255) / 256);
-    const bool pairs = pairs_at(nb);
+    for (int q = 0; q < cnt; ++q)
+      rp[q] = RowPhase{phase_of(order[q0 + q], pairs ? 4096.0 : 1.0), eps[order[q0 + q]]};
+    RF_CUDA(cudaMemcpyAsync(d_rp, rp.data(), sizeof(RowPhase) * cnt, cudaMemcpyHostToDevice, s));
+    // rho of m rows: in FP64 (three rows of workspace each), and in the real form
+    auto real_rows = [&](auto* R, int m) {
+      if (!real_form) return;
+      k_real_form<<<(unsigned)std::min<int64_t>(4096, (m * nb + 255) / 256), 256, 0, s>>>(R, m * nb);
+      RF_LAUNCHED();
+    };
+    auto rows64 = [&](const RowPhase* d_p, const double* d_l, int m, double2* bufK) {
+      double2* bufR = bufK + m * nb;
+      double2* bufT = bufR + m * nb;
+      k_kernel_spectrum<<<dim3((unsigned)((nb + 255) / 256), (unsigned)m), 256, 0, s>>>(
+          d_p, d_l, nb, dfb, k0, k1, c->g.f_low, c->g.f_high, c->g.df_high, c->pw.as<double>(), c->pw_stride, bufK);
+      RF_LAUNCHED();
+      fft_c2c_f64(bufK, bufR, bufT, nb, m, +1, c->tw64.as<double2>(), n, s);
+      real_rows(bufR, m);
+      return bufR;
+    };
+    // the kept spans of m rows: first lags into d_s, lengths into d_n
+    auto spans = [&](auto* R, const Tf2* d_t, const double* d_l, const RowPhase* d_p, int m, double* d_a, int* d_s,
+                     int* d_n) {
+      using V = std::remove_pointer_t<decltype(R)>;
+      RF_CUDA(cudaMemsetAsync(d_a, 0, sizeof(double) * m, s));
+      const unsigned mx = (unsigned)std::max<int64_t>(1, std::min<int64_t>(nb / 2048, (8LL * c->nsm + m - 1) / m));
+      k_row_max2<V><<<dim3(mx, (unsigned)m), 256, 0, s>>>(R, nb, reinterpret_cast<unsigned long long*>(d_a));
+      RF_LAUNCHED();
+      if (analytic) {
+        k_analytic_span<<<(m + 63) / 64, 64, 0, s>>>(pr, d_t, d_l, d_a, std::is_same<V, cdf>::value ? d_p : nullptr,
+                                                     m, thr, rel, real_form ? 1.0 : 2.0, nb, c->g.fs, c->g.f_low,
+                                                     c->g.f_high, c->g.df_high, d_s, d_n);
+      } else {
+        const int per = (int)std::max<int64_t>(32, nb / kArcParts);
+        const int np = (int)((nb + per - 1) / per);
+        k_arc_parts<V><<<dim3((unsigned)((np + 7) / 8), (unsigned)m), 256, 0, s>>>(R, nb, per, np, d_a, d_p, thr, rel,
+                                                                                   arcs.as<ArcPart>());
+        RF_LAUNCHED();
+        k_arc_join<<<m, 32, 0, s>>>(arcs.as<ArcPart>(), np, nb, d_s, d_n);
+      }
+      RF_LAUNCHED();
+    };
     double2* bufR = nullptr;
     cdf* bufP = nullptr;
-    RF_CUDA(cudaMemsetAsync(d_amax, 0, sizeof(double) * cnt, s));
-    auto amax_bits = reinterpret_cast<unsigned long long*>(d_amax);
     if (pairs) {
       if (roots_of != nb) {
         k_split_roots<<<(unsigned)((nb + 255) / 256), 256, 0, s>>>(c->tw64.as<double2>(), n / nb, nb, roots.as<cdf>());
@@ -695,53 +812,64 @@ rf_kernels* build_impl(rf_ctx* c, const rf_template& ref, const rf_template* nbr
       cdf* a = rows.as<cdf>();
       cdf* b = a + cnt * nb;
       k_pair_first<<<dim3((unsigned)((nb / 16 + 127) / 128), (unsigned)cnt), 128, 0, s>>>(
-          d_dq, d_dfls + q0, nb, dfb, k0, k1, c->g.f_low, c->g.f_high, c->g.df_high, c->pw.as<double>(),
+          d_rp, d_dfls + q0, nb, dfb, k0, k1, c->g.f_low, c->g.f_high, c->g.df_high, c->pw.as<double>(),
           c->pw32.as<float2>(), c->pw_stride, roots.as<cdf>(), a);
       RF_LAUNCHED();
       bufP = pair_passes(a, b, nb, cnt, roots.as<cdf>(), s);
-      if (real_form) {
-        k_real_form<<<rg, 256, 0, s>>>(bufP, cnt * nb);
-        RF_LAUNCHED();
-      }
-      k_row_max2<cdf><<<dim3(mx, (unsigned)cnt), 256, 0, s>>>(bufP, nb, amax_bits);
+      real_rows(bufP, cnt);
+      spans(bufP, d_tgs + q0, d_dfls + q0, d_rp, cnt, d_amax, d_m0, d_len);
     } else {
-      double2* bufK = rows.as<double2>();
-      bufR = bufK + cnt * nb;
-      double2* bufT = bufR + cnt * nb;
-      dim3 g1((unsigned)((nb + 255) / 256), (unsigned)cnt);
-      k_kernel_spectrum<<<g1, 256, 0, s>>>(d_dq, d_dfls + q0, nb, dfb, k0, k1, c->g.f_low, c->g.f_high, c->g.df_high,
-                                           c->pw.as<double>(), c->pw_stride, bufK);
-      RF_LAUNCHED();
-      fft_c2c_f64(bufK, bufR, bufT, nb, cnt, +1, c->tw64.as<double2>(), n, s);
-      if (real_form) {
-        k_real_form<<<rg, 256, 0, s>>>(bufR, cnt * nb);
-        RF_LAUNCHED();
-      }
-      k_row_max2<double2><<<dim3(mx, (unsigned)cnt), 256, 0, s>>>(bufR, nb, amax_bits);
+      bufR = rows64(d_rp, d_dfls + q0, cnt, rows.as<double2>());
+      spans(bufR, d_tgs + q0, d_dfls + q0, d_rp, cnt, d_amax, d_m0, d_len);
     }
-    RF_LAUNCHED();
-    if (relative & RF_TRUNC_ANALYTIC) {
-      k_analytic_span<<<(cnt + 63) / 64, 64, 0, s>>>(pr, d_tgs + q0, d_dfls + q0, d_amax, cnt, thr,
-                                                     relative & RF_TRUNC_RELATIVE,
-                                                     (relative & RF_KERNEL_REAL) ? 1.0 : 2.0, nb, c->g.fs,
-                                                     c->g.f_low, c->g.f_high, c->g.df_high, d_m0, d_len);
-    } else {
-      const int per = (int)std::max<int64_t>(32, nb / kArcParts);
-      const int np = (int)((nb + per - 1) / per);
-      const dim3 ga((unsigned)((np + 7) / 8), (unsigned)cnt);
-      if (pairs)
-        k_arc_parts<cdf><<<ga, 256, 0, s>>>(bufP, nb, per, np, d_amax, thr, relative & RF_TRUNC_RELATIVE,
-                                            arcs.as<ArcPart>());
-      else
-        k_arc_parts<double2><<<ga, 256, 0, s>>>(bufR, nb, per, np, d_amax, thr, relative & RF_TRUNC_RELATIVE,
-                                                arcs.as<ArcPart>());
-      RF_LAUNCHED();
-      k_arc_join<<<cnt, 32, 0, s>>>(arcs.as<ArcPart>(), np, nb, d_m0, d_len);
-    }
-    RF_LAUNCHED();
     RF_CUDA(cudaMemcpyAsync(hm0.data(), d_m0, sizeof(int) * cnt, cudaMemcpyDeviceToHost, s));
     RF_CUDA(cudaMemcpyAsync(hlen.data(), d_len, sizeof(int) * cnt, cudaMemcpyDeviceToHost, s));
     RF_CUDA(cudaStreamSynchronize(s));
+    // kernels in pairs whose span their error could change: again in FP64
+    std::vector<int> redo;
+    for (int q = 0; q < cnt; ++q)
+      if (hlen[q] < 0) redo.push_back(q);
+    for (size_t r0 = 0; r0 < redo.size();) {
+      const int64_t per = 3 * nb * (int64_t)sizeof(double2);
+      const int m = (int)std::min<int64_t>((int64_t)(redo.size() - r0),
+                                           std::max<int64_t>(1, ((int64_t)512 << 20) / per));
+      StreamBuf work(c, (size_t)(per * m), s);
+      std::vector<Tf2> ht(m);
+      std::vector<RowPhase> hp(m);
+      std::vector<double> hl(m);
+      std::vector<int> hs(m), hn(m);
+      for (int i = 0; i < m; ++i) {
+        const int j = order[q0 + redo[r0 + i]];
+        ht[i] = tg[j];
+        hp[i] = RowPhase{phase_of(j, 1.0), 0.0};
+        hl[i] = kern->df_low[j];
+      }
+      StreamBuf bt(c, sizeof(Tf2) * m, s), bp(c, sizeof(RowPhase) * m, s), bl(c, 2 * sizeof(double) * m, s),
+          bi(c, 3 * sizeof(int) * m, s);
+      RF_CUDA(cudaMemcpyAsync(bt.need().p, ht.data(), sizeof(Tf2) * m, cudaMemcpyHostToDevice, s));
+      RF_CUDA(cudaMemcpyAsync(bp.need().p, hp.data(), sizeof(RowPhase) * m, cudaMemcpyHostToDevice, s));
+      RF_CUDA(cudaMemcpyAsync(bl.need().p, hl.data(), sizeof(double) * m, cudaMemcpyHostToDevice, s));
+      RF_CUDA(cudaMemcpyAsync(bi.need().p, &redo[r0], sizeof(int) * m, cudaMemcpyHostToDevice, s));
+      double2* R = rows64(bp.as<RowPhase>(), bl.as<double>(), m, work.need().as<double2>());
+      spans(R, bt.as<Tf2>(), bl.as<double>(), bp.as<RowPhase>(), m, bl.as<double>() + m, bi.as<int>() + m,
+            bi.as<int>() + 2 * m);
+      k_rows_to_pairs<<<dim3((unsigned)std::min<int64_t>(1024, (nb + 255) / 256), (unsigned)m), 256, 0, s>>>(
+          R, bi.as<int>(), nb, bufP);
+      RF_LAUNCHED();
+      RF_CUDA(cudaMemcpyAsync(hs.data(), bi.as<int>() + m, sizeof(int) * m, cudaMemcpyDeviceToHost, s));
+      RF_CUDA(cudaMemcpyAsync(hn.data(), bi.as<int>() + 2 * m, sizeof(int) * m, cudaMemcpyDeviceToHost, s));
+      RF_CUDA(cudaStreamSynchronize(s));
+      for (int i = 0; i < m; ++i) {
+        hm0[redo[r0 + i]] = hs[i];
+        hlen[redo[r0 + i]] = hn[i];
+      }
+      r0 += m;
+    }
+    if (!redo.empty()) {
+      RF_CUDA(cudaMemcpyAsync(d_m0, hm0.data(), sizeof(int) * cnt, cudaMemcpyHostToDevice, s));
+      RF_CUDA(cudaMemcpyAsync(d_len, hlen.data(), sizeof(int) * cnt, cudaMemcpyHostToDevice, s));
+      RF_CUDA(cudaStreamSynchronize(s));
+    }
     std::vector<int64_t> off(cnt + 1, 0);
     for (int q = 0; q < cnt; ++q) {
       const int j = order[q0 + q];

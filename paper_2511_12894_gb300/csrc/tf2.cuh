@@ -59,13 +59,26 @@ inline Tf2Bins make_tf2_bins(const Tf2& p, double df) {
   return q;
 }
 
-// a - b, times `unit` (a power of two: the phase in parts of a turn)
+// a - b, times `unit` (a power of two: the phase in parts of a turn); whole turns of the constant
+// term go (exactly), so that a large phi_c costs the other terms no bits
 inline Tf2Bins tf2_bins_minus(const Tf2Bins& a, const Tf2Bins& b, double unit) {
+  const double e = a.e - b.e;
   return Tf2Bins{unit * (a.b0 - b.b0), unit * (a.b2 - b.b2), unit * (a.b3 - b.b3), unit * (a.b4 - b.b4),
                  unit * (a.b7 - b.b7), unit * (a.l5 - b.l5), unit * (a.l6 - b.l6), unit * (a.m6 - b.m6),
-                 unit * (a.d - b.d),   unit * (a.e - b.e)};
+                 unit * (a.d - b.d),   unit * (e - std::rint(e))};
 }
 
+// Bounds over the bins ka..kb >= 1 of the leading terms (u^-5 and k) and of the sum of the others.
+struct Tf2Size {
+  double lead, rest;
+};
+inline Tf2Size tf2_bins_size(const Tf2Bins& q, double ka, double kb) {
+  const double ua = std::cbrt(ka), ub = std::cbrt(kb), l = std::log(kb) / 3.0;
+  return Tf2Size{std::fabs(q.b0) / (ka * ua * ua) + std::fabs(q.d) * kb,
+                 std::fabs(q.b2) / ka + std::fabs(q.b3) / (ua * ua) + std::fabs(q.b4) / ua +
+                     std::fabs(q.b7) * ub * ub + std::fabs(q.l5) * l + std::fabs(q.l6) * ub * l +
+                     std::fabs(q.m6) * ub + std::fabs(q.e)};
+}
 
 // The phase of bin k as a fraction of a turn in [-1/2, 1/2].
 __device__ __forceinline__ double tf2_turn(const Tf2Bins& q, int64_t k, double u, double u5, double lu) {
