@@ -147,7 +147,8 @@ rf_status rf_template_fd(rf_ctx* ctx, const rf_template* tmpl, void* h_out, rf_s
  *   N^2 = 4 df sum_{f_low<=f_k<=f_high} |h~_k|^2 inv_psd[k]             (Eq. 3, FP64)
  *   z[i] = (4 df / N) sum_{k=0}^{n/2} x~_k conj(h~_k) inv_psd[k] band_k exp(+2 pi i i k / n)
  * with x~_k = dt sum_j x[j] exp(-2 pi i j k / n) computed once for all references.
- * On RF_F32 grids the phase of templates with tc = 0 is formed in pairs of FP32 values (about 46 bits).
+ * On RF_F32 grids the phase of templates with tc = 0 that stays below 2^18 turns in the band is formed in
+ * pairs of FP32 values (about 46 bits), the others' in FP64; each row is the same whatever else is in refs.
  * x: real[n] (grid dtype); inv_psd: double[n/2+1], 1/S_n(f_k) (values outside the band are
  * ignored: Eq. 4); refs: host array of nref templates; z_out: complex[nref][n] (grid dtype);
  * sigma_out: double[nref] (device, N of each reference).  Async on stream. */

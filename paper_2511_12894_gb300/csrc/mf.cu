@@ -191,8 +191,12 @@ __global__ void __launch_bounds__(256) k_ref_filters(const double* __restrict__ 
   }
 }
 
-// The same for FP32 grids with the phase in FP32 pairs (templates with t_c = 0).  Three references at
-// n = 2^20: the FP64 phase took 49 us of the FP64 pipe, this 12.5 us (issue 73%).
+// The same for FP32 grids with the phase in FP32 pairs, for templates with t_c = 0 whose phase stays
+// below kPairTurns in the band.  Three references at n = 2^20: the FP64 phase took 49 us of the FP64
+// pipe, this 12.5 us.  A pair keeps about 2^-46 of the phase; 2^18 turns of it (two bodies of 0.3 solar
+// masses from 5 Hz, 1.0 from 2.4 Hz) leave 2^-28 of a turn, an eighth of the rounding of the angle to
+// FP32 that follows in either form.  Bodies of 0.01 solar masses, 7e7 turns from 5 Hz, lost 1e-5 rad.
+constexpr double kPairTurns = 262144.0;
 struct FiltPairs {
   Tf2Pairs q[kFiltRefs];
 };
@@ -260,28 +264,34 @@ void launch_filters(rf_ctx* c, const double* inv_psd, SigmaArgs sig, int cnt, co
   const double df = c->g.fs / (double)c->n;
   int64_t k0, k1;
   band_bins(c->g, &k0, &k1);
-  for (int r0 = 0; r0 < cnt; r0 += kFiltRefs) {
-    const int m = std::min(kFiltRefs, cnt - r0);
-    FiltRefs fr{};
-    bool at_zero = true;
-    for (int r = 0; r < m; ++r) {
-      fr.q[r] = make_tf2_bins(make_tf2(refs[r0 + r], c->g.pn_order), df);
-      at_zero = at_zero && fr.q[r].d == 0.0;
+  // Each reference in the form its own phase asks for, whatever else is in the call: launches of runs of
+  // one kind (places beside the coefficients would mix kinds in a launch: 71 -> 73 us for three references at 2^20).
+  const unsigned grid = (unsigned)((nbins + 255) / 256);
+  FiltRefs fr;
+  FiltPairs fp;
+  for (int r0 = 0, m; r0 < cnt; r0 += m) {
+    bool pairs = false;
+    for (m = 0; m < kFiltRefs && r0 + m < cnt; ++m) {
+      const Tf2Bins q = make_tf2_bins(make_tf2(refs[r0 + m], c->g.pn_order), df);
+      const Tf2Size size = tf2_bins_size(q, (double)k0, (double)std::max(k0, k1));
+      const bool p = !PREC && q.d == 0.0 && size.lead + size.rest <= kPairTurns;
+      if (m > 0 && p != pairs) break;
+      pairs = p;
+      if (p) fp.q[m] = make_tf2_pairs(q);
+      else fr.q[m] = q;
     }
+    V* Fr = F + (int64_t)r0 * fstride;
+    bool done = false;
     if constexpr (!PREC) {
-      if (at_zero) {
-        FiltPairs fp{};
-        for (int r = 0; r < m; ++r) fp.q[r] = make_tf2_pairs(fr.q[r]);
-        k_ref_filters_pairs<<<(unsigned)((nbins + 255) / 256), 256, 0, s>>>(
-            inv_psd, c->pw.as<double>() + 3 * c->pw_stride, c->pw32.as<float2>(), c->pw_stride, sig, fp, m, nbins, k0,
-            k1, F + (int64_t)r0 * fstride, fstride);
-        RF_LAUNCHED();
-        sig.sigma_out = nullptr;  // written once
-        continue;
+      if (pairs) {
+        k_ref_filters_pairs<<<grid, 256, 0, s>>>(inv_psd, c->pw.as<double>() + 3 * c->pw_stride, c->pw32.as<float2>(),
+                                                 c->pw_stride, sig, fp, m, nbins, k0, k1, Fr, fstride);
+        done = true;
       }
     }
-    k_ref_filters<V, PREC><<<(unsigned)((nbins + 255) / 256), 256, 0, s>>>(
-        inv_psd, c->pw.as<double>(), c->pw_stride, sig, fr, m, nbins, k0, k1, F + (int64_t)r0 * fstride, fstride);
+    if (!done)
+      k_ref_filters<V, PREC><<<grid, 256, 0, s>>>(inv_psd, c->pw.as<double>(), c->pw_stride, sig, fr, m, nbins, k0, k1,
+                                                  Fr, fstride);
     RF_LAUNCHED();
     sig.sigma_out = nullptr;  // written once
   }

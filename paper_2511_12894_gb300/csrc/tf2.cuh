@@ -56,11 +56,12 @@ inline Tf2Bins make_tf2_bins(const Tf2& p, double df) {
   q.m6 = s * c * (p.a[6] + p.a6log * std::log(4.0 * c));
   q.d = df * p.tc;
   q.e = s * (p.a[5] + p.a5log * std::log(c * kSqrt6)) - p.phic / kTwoPi - 0.125;
+  q.e -= std::rint(q.e);  // whole turns, exactly: a large phi_c costs the other terms no bits
   return q;
 }
 
-// a - b, times `unit` (a power of two: the phase in parts of a turn); whole turns of the constant
-// term go (exactly), so that a large phi_c costs the other terms no bits
+// a - b, times `unit` (a power of two: the phase in parts of a turn), whole turns of the constant
+// term taken off
 inline Tf2Bins tf2_bins_minus(const Tf2Bins& a, const Tf2Bins& b, double unit) {
   const double e = a.e - b.e;
   return Tf2Bins{unit * (a.b0 - b.b0), unit * (a.b2 - b.b2), unit * (a.b3 - b.b3), unit * (a.b4 - b.b4),
@@ -91,7 +92,7 @@ __device__ __forceinline__ double tf2_turn(const Tf2Bins& q, int64_t k, double u
 }
 
 // The same phase in FP32 pairs (value h + l, about 46 bits; the scheme of cdf.cuh for real numbers)
-// for filters that are rounded to FP32 in the same kernel: 3e4 turns keep 2e-9 of a turn, below the
+// for filters that are rounded to FP32 in the same kernel: 3e4 turns keep 5e-10 of a turn, below the
 // rounding of the angle to FP32, and the FP32 pipes are 60 times as wide as the FP64 pipe.
 struct Pair {
   float h, l;
