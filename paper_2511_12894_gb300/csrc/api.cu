@@ -148,7 +148,7 @@ rf_status rf_create(const rf_grid* grid, rf_ctx** out) {
     for (int64_t m = 0; m < n; ++m) tw32[m] = make_float2((float)tw[m].x, (float)tw[m].y);
     c->tw32.ensure(sizeof(float2) * n);
     RF_CUDA(cudaMemcpy(c->tw32.p, tw32.data(), sizeof(float2) * n, cudaMemcpyHostToDevice));
-    if (g.dtype == RF_F32 && fft4_supported(n, false)) {
+    if (g.dtype == RF_F32 && fft4_forward_supported(n, false)) {
       // four-step FFT twiddles: the low table, then every 2^lo-th entry
       const int lo = fft4_lo_bits(n);
       std::vector<float2> t4((size_t)((int64_t(1) << lo) + (n >> lo)));

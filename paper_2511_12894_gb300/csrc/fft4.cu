@@ -367,6 +367,11 @@ __global__ void __cluster_dims__(kClusterBlocks, 1, 1) __launch_bounds__(N1 * N2
 constexpr int kF4MinLog = 15;    // FP32: below, one block does it (block_mf)
 constexpr int kF4MinLog64 = 14;  // N1, N2 >= 128
 constexpr int kF4MaxLog = 24;    // N1, N2 <= 4096
+// FP64: beyond these the radix-16 passes of fft.cu, which waste less of the FP64 pipe once a launch fills
+// it, are faster.  Data transform, four-step against radix: 363 / 416 us at 2^21, 767 / 672 at 2^22; inverse
+// of one reference 39 / about 80 us at 2^18 (each of 100: 32 / 30), 83 / 76 at 2^19, 175 / 157 at 2^20.
+constexpr int kF4MaxForward64 = 21;
+constexpr int kF4MaxInverse64 = 18;
 
 // Tile widths: G columns of N1 points, R rows of N2 points.  FP32: lines of 512 and 1024 points in
 // tiles of 8 columns, longer ones in tiles of 4, so that two blocks share an SM up to 2048 points
@@ -440,24 +445,35 @@ void split(int64_t n, int& n1log, int& n2log) {
 template <typename V, int MODE, int SIGN>
 void two_passes(const rf_ctx* c, const void* in, const V* F, int64_t fstride, V* out, V* tmp, int batch,
                 cudaStream_t s) {
-  RF_REQUIRE(fft4_supported(c->n, sizeof(V) == 16), "fft4: n=%lld is not supported", (long long)c->n);
+  constexpr bool f64 = sizeof(V) == 16;
+  RF_REQUIRE(SIGN < 0 ? fft4_forward_supported(c->n, f64) : fft4_inverse_supported(c->n, f64),
+             "fft4: n=%lld is not supported", (long long)c->n);
   RF_REQUIRE(sizeof(V) == 16 || c->tw4.p != nullptr, "fft4: twiddle tables missing");
   RF_REQUIRE(batch >= 1 && batch <= 65535, "fft4: batch %d out of range", batch);
   RF_REQUIRE(in != out && in != tmp && out != tmp, "fft4: buffers must be distinct");
   int n1log, n2log;
   split(c->n, n1log, n2log);
+  constexpr int longest = 1 << (((f64 ? (SIGN < 0 ? kF4MaxForward64 : kF4MaxInverse64) : kF4MaxLog) + 1) / 2);
   dispatch_line(n1log, [&](auto l) {
-    launch_cols<V, decltype(l)::value, MODE, SIGN>(in, F, fstride, tmp, n2log, batch, c, s);
+    if constexpr (decltype(l)::value <= longest)
+      launch_cols<V, decltype(l)::value, MODE, SIGN>(in, F, fstride, tmp, n2log, batch, c, s);
   });
-  dispatch_line(n2log, [&](auto l) { launch_rows<V, decltype(l)::value, SIGN>(tmp, out, n1log, batch, c, s); });
+  dispatch_line(n2log, [&](auto l) {
+    if constexpr (decltype(l)::value <= longest)
+      launch_rows<V, decltype(l)::value, SIGN>(tmp, out, n1log, batch, c, s);
+  });
 }
 
 }  // namespace
 
-bool fft4_supported(int64_t n, bool f64) {
-  if (n <= 0 || (n & (n - 1)) != 0) return false;
-  const int b = ilog2(n);
-  return b >= (f64 ? kF4MinLog64 : kF4MinLog) && b <= kF4MaxLog;
+namespace {
+bool in_logs(int64_t n, int lo, int hi) { return n >= (int64_t)1 << lo && n <= (int64_t)1 << hi && (n & (n - 1)) == 0; }
+}  // namespace
+bool fft4_forward_supported(int64_t n, bool f64) {
+  return in_logs(n, f64 ? kF4MinLog64 : kF4MinLog, f64 ? kF4MaxForward64 : kF4MaxLog);
+}
+bool fft4_inverse_supported(int64_t n, bool f64) {
+  return in_logs(n, f64 ? kF4MinLog64 : kF4MinLog, f64 ? kF4MaxInverse64 : kF4MaxLog);
 }
 
 int fft4_lo_bits(int64_t n) { return (ilog2(n) + 1) / 2; }

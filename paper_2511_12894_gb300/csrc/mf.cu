@@ -322,21 +322,21 @@ namespace {
 
 // The context's transforms: two-pass four-step where n allows, else radix passes.
 void forward_real(rf_ctx* c, const float* x, float2* X, float2* tmp, cudaStream_t s) {
-  if (fft4_supported(c->n, false)) fft4_forward_real(c, x, X, tmp, s);
+  if (fft4_forward_supported(c->n, false)) fft4_forward_real(c, x, X, tmp, s);
   else fft_r2c_f32(x, X, tmp, c->n, c->tw32.as<float2>(), c->n, s);
 }
 void forward_real(rf_ctx* c, const double* x, double2* X, double2* tmp, cudaStream_t s) {
-  if (fft4_supported(c->n, true)) fft4_forward_real(c, x, X, tmp, s);
+  if (fft4_forward_supported(c->n, true)) fft4_forward_real(c, x, X, tmp, s);
   else fft_r2c_f64(x, X, tmp, c->n, c->tw64.as<double2>(), c->n, s);
 }
 void inverse_product(rf_ctx* c, const float2* X, const float2* F, int64_t fstride, float2* z, float2* tmp, int cnt,
                      cudaStream_t s) {
-  if (fft4_supported(c->n, false)) fft4_inverse_product(c, X, F, fstride, z, tmp, cnt, s);
+  if (fft4_inverse_supported(c->n, false)) fft4_inverse_product(c, X, F, fstride, z, tmp, cnt, s);
   else ifft_product_f32(X, F, fstride, z, tmp, c->n, cnt, c->tw32.as<float2>(), c->n, s);
 }
 void inverse_product(rf_ctx* c, const double2* X, const double2* F, int64_t fstride, double2* z, double2* tmp, int cnt,
                      cudaStream_t s) {
-  if (fft4_supported(c->n, true)) fft4_inverse_product(c, X, F, fstride, z, tmp, cnt, s);
+  if (fft4_inverse_supported(c->n, true)) fft4_inverse_product(c, X, F, fstride, z, tmp, cnt, s);
   else ifft_product_f64(X, F, fstride, z, tmp, c->n, cnt, c->tw64.as<double2>(), c->n, s);
 }
 
@@ -420,8 +420,8 @@ void mf_filtered_impl(rf_ctx* c, const void* x, int32_t nref, const void* filt, 
     using V = decltype(vtag);
     using T = typename real_of<V>::type;
     // references per launch, bounded by the temporary buffer
-    const int64_t most = fft4_supported(n, sizeof(T) == 8) ? std::max<int64_t>(1, kF4Chunk / n)
-                                                           : std::min<int64_t>(65535, ((int64_t)1 << 27) / n);
+    const int64_t most = fft4_inverse_supported(n, sizeof(T) == 8) ? std::max<int64_t>(1, kF4Chunk / n)
+                                                                   : std::min<int64_t>(65535, ((int64_t)1 << 27) / n);
     const int chunk = (int)std::max<int64_t>(1, std::min<int64_t>(nref, most));
     c->mf_tmp.ensure(sizeof(V) * (size_t)chunk * n);
     forward_real(c, static_cast<const T*>(x), c->xf.as<V>(), c->mf_tmp.as<V>(), s);

@@ -334,7 +334,8 @@ void fft_c2c_f32(const float2* in, float2* out, float2* tmp, int64_t n, int batc
 // 2^14 points a whole matched filter per thread block.  Forward of real data (natural order out) and
 // the inverse of the one-sided product X[k] F_r[k] (k <= n/2, zero above; row r of F at r fstride).
 // tmp holds batch n complex values.
-bool fft4_supported(int64_t n, bool f64);
+bool fft4_forward_supported(int64_t n, bool f64);
+bool fft4_inverse_supported(int64_t n, bool f64);
 int fft4_lo_bits(int64_t n);
 void fft4_forward_real(const rf_ctx* c, const float* x, float2* out, float2* tmp, cudaStream_t s);
 void fft4_forward_real(const rf_ctx* c, const double* x, double2* out, double2* tmp, cudaStream_t s);
@@ -343,7 +344,8 @@ void fft4_inverse_product(const rf_ctx* c, const float2* X, const float2* F, int
 void fft4_inverse_product(const rf_ctx* c, const double2* X, const double2* F, int64_t fstride, double2* out,
                           double2* tmp, int batch, cudaStream_t s);
 // FP32, n = 512 .. 16384, and to 65536 for few references: the spectrum of x and the inverse transforms
-// of its products with `nref` filters (rows of fstride >= n/2 + 1) in one launch.
+// of its products with `nref` filters (rows of fstride >= n/2 + 1) in one launch; `out` is apart from
+// x and F (blocks read both after others have written).
 bool block_mf_supported(const rf_ctx* c, int nref);
 void block_mf(const rf_ctx* c, const float* x, const float2* F, int64_t fstride, float2* out, int nref,
               cudaStream_t s);
