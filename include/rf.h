@@ -148,7 +148,9 @@ rf_status rf_template_fd(rf_ctx* ctx, const rf_template* tmpl, void* h_out, rf_s
  *   z[i] = (4 df / N) sum_{k=0}^{n/2} x~_k conj(h~_k) inv_psd[k] band_k exp(+2 pi i i k / n)
  * with x~_k = dt sum_j x[j] exp(-2 pi i j k / n) computed once for all references.
  * On RF_F32 grids the phase of templates with tc = 0 that stays below 2^18 turns in the band is formed in
- * pairs of FP32 values (about 46 bits), the others' in FP64; each row is the same whatever else is in refs.
+ * pairs of FP32 values (about 46 bits), the others' in FP64; each row is the same whatever else is in refs
+ * (RF_F32 grids of 2^14 to 2^16 samples: among calls of at most SMs / 8 references, and among larger
+ * ones; between the two, rows differ by rounding, below 1e-6 of max|z|).  x may lie inside z_out.
  * x: real[n] (grid dtype); inv_psd: double[n/2+1], 1/S_n(f_k) (values outside the band are
  * ignored: Eq. 4); refs: host array of nref templates; z_out: complex[nref][n] (grid dtype);
  * sigma_out: double[nref] (device, N of each reference).  Async on stream. */

@@ -341,18 +341,17 @@ void inverse_product(rf_ctx* c, const double2* X, const double2* F, int64_t fstr
 }
 
 // The one-launch form reads the data and the filters in every block, after other blocks may have
-// written their rows, so a caller's output that overlaps an input takes the passes, which transform
-// the data before anything is written.
+// written their rows: inputs that the caller's output overlaps are copied first.
 bool overlap(const void* a, size_t na, const void* b, size_t nb) {
   const char* p = static_cast<const char*>(a);
   const char* q = static_cast<const char*>(b);
   return p < q + nb && q < p + na;
 }
-bool one_launch(const rf_ctx* c, int nref, const void* x, const void* filt, const void* z) {
-  if (!block_mf_supported(c, nref)) return false;
-  const size_t zb = sizeof(float2) * (size_t)nref * (size_t)c->n;
-  return !overlap(x, sizeof(float) * (size_t)c->n, z, zb) &&
-         !(filt && overlap(filt, sizeof(float2) * (size_t)nref * (size_t)(c->n / 2 + 1), z, zb));
+const float* data_apart(rf_ctx* c, int nref, const void* x, const void* z, cudaStream_t s) {
+  const size_t xb = sizeof(float) * (size_t)c->n;
+  if (!overlap(x, xb, z, sizeof(float2) * (size_t)nref * (size_t)c->n)) return static_cast<const float*>(x);
+  RF_CUDA(cudaMemcpyAsync(c->xf.p, x, xb, cudaMemcpyDeviceToDevice, s));
+  return c->xf.as<float>();
 }
 
 // Filters of a batch, then one product inverse for the batch.
@@ -384,11 +383,10 @@ void mf_reference_impl(rf_ctx* c, const void* x, const double* inv_psd, int32_t 
                [&](const double2* F, int64_t fs, double2* z, double2* tmp, int cnt) {
                  inverse_product(c, c->xf.as<double2>(), F, fs, z, tmp, cnt, s);
                }, s);
-  } else if (one_launch(c, nref, x, nullptr, z_out)) {
+  } else if (block_mf_supported(c, nref)) {
+    const float* xa = data_apart(c, nref, x, z_out, s);
     mf_batches(c, inv_psd, sig, nref, refs, static_cast<float2*>(z_out),
-               [&](const float2* F, int64_t fs, float2* z, float2*, int cnt) {
-                 block_mf(c, static_cast<const float*>(x), F, fs, z, cnt, s);
-               }, s);
+               [&](const float2* F, int64_t fs, float2* z, float2*, int cnt) { block_mf(c, xa, F, fs, z, cnt, s); }, s);
   } else {
     forward_real(c, static_cast<const float*>(x), c->xf.as<float2>(), c->fb.as<float2>(), s);
     mf_batches(c, inv_psd, sig, nref, refs, static_cast<float2*>(z_out),
@@ -411,9 +409,16 @@ void reference_filters_impl(rf_ctx* c, const double* inv_psd, int32_t nref, cons
 void mf_filtered_impl(rf_ctx* c, const void* x, int32_t nref, const void* filt, void* z_out, cudaStream_t s) {
   const int64_t n = c->n;
   const int64_t nb = n / 2 + 1;
-  if (one_launch(c, nref, x, filt, z_out)) {
-    block_mf(c, static_cast<const float*>(x), static_cast<const float2*>(filt), nb, static_cast<float2*>(z_out), nref,
-             s);
+  if (block_mf_supported(c, nref)) {
+    const float* xa = data_apart(c, nref, x, z_out, s);
+    const float2* F = static_cast<const float2*>(filt);
+    const size_t fb = sizeof(float2) * (size_t)nref * (size_t)nb;
+    if (overlap(filt, fb, z_out, sizeof(float2) * (size_t)nref * (size_t)n)) {
+      c->mf_tmp.ensure(fb);
+      RF_CUDA(cudaMemcpyAsync(c->mf_tmp.p, filt, fb, cudaMemcpyDeviceToDevice, s));
+      F = c->mf_tmp.as<float2>();
+    }
+    block_mf(c, xa, F, nb, static_cast<float2*>(z_out), nref, s);
     return;
   }
   auto run = [&](auto vtag) {
@@ -421,7 +426,7 @@ void mf_filtered_impl(rf_ctx* c, const void* x, int32_t nref, const void* filt, 
     using T = typename real_of<V>::type;
     // references per launch, bounded by the temporary buffer
     const int64_t most = fft4_inverse_supported(n, sizeof(T) == 8) ? std::max<int64_t>(1, kF4Chunk / n)
-                                                                   : std::min<int64_t>(65535, ((int64_t)1 << 27) / n);
+                                                           : std::min<int64_t>(65535, ((int64_t)1 << 27) / n);
     const int chunk = (int)std::max<int64_t>(1, std::min<int64_t>(nref, most));
     c->mf_tmp.ensure(sizeof(V) * (size_t)chunk * n);
     forward_real(c, static_cast<const T*>(x), c->xf.as<V>(), c->mf_tmp.as<V>(), s);

@@ -344,8 +344,8 @@ void fft4_inverse_product(const rf_ctx* c, const float2* X, const float2* F, int
 void fft4_inverse_product(const rf_ctx* c, const double2* X, const double2* F, int64_t fstride, double2* out,
                           double2* tmp, int batch, cudaStream_t s);
 // FP32, n = 512 .. 16384, and to 65536 for few references: the spectrum of x and the inverse transforms
-// of its products with `nref` filters (rows of fstride >= n/2 + 1) in one launch; `out` is apart from
-// x and F (blocks read both after others have written).
+// of its products with `nref` filters (rows of fstride >= n/2 + 1) in one launch; `out` is apart from x
+// and F, which every block reads after others have written.
 bool block_mf_supported(const rf_ctx* c, int nref);
 void block_mf(const rf_ctx* c, const float* x, const float2* F, int64_t fstride, float2* out, int nref,
               cudaStream_t s);

@@ -52,3 +52,46 @@ def test_phase_of_light_bodies(m):
              for r in (r32, r64)]
         worst = max(worst, np.abs(np.angle(z[0] * np.conj(z[1]))).max())
     assert worst <= 4 * np.pi * 2.0 ** -24, worst
+
+
+@pytest.mark.parametrize("log2n,nref", [(9, 3), (13, 5), (14, 5), (14, 25), (16, 3)])
+def test_output_over_the_inputs_keeps_the_bits(log2n, nref):
+    """Rows of an output that overlaps the data or the filters are those of a separate output."""
+    torch = pytest.importorskip("torch")
+    n = 1 << log2n
+    rf, x, ip = _inputs(torch, n)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(nref)
+    filt = torch.view_as_complex(torch.randn((nref, n // 2 + 1, 2), device="cuda", generator=g))
+    want = rf.mf_filtered(x, filt)
+    buf = torch.zeros(nref * n * 2, device="cuda")
+    out = torch.view_as_complex(buf.view(-1, 2)).view(nref, n)
+    for at in (0, n, 2 * n):
+        buf[at:at + n] = x
+        assert torch.equal(rf.mf_filtered(buf[at:at + n], filt, z_out=out), want)
+    flat = torch.zeros(nref * n, dtype=torch.complex64, device="cuda")
+    flat[: filt.numel()] = filt.flatten()
+    assert torch.equal(rf.mf_filtered(x, flat[: filt.numel()].view(nref, -1), z_out=flat.view(nref, n)), want)
+    refs = _mixed(nref, 6)
+    want, _ = rf.mf_reference(x, ip, refs)
+    buf[n:2 * n] = x
+    assert torch.equal(rf.mf_reference(buf[n:2 * n], ip, refs, z_out=out)[0], want)
+
+
+@pytest.mark.parametrize("log2n", [14, 15, 16])
+def test_rows_within_each_form(log2n):
+    """2^14 to 2^16 samples: calls of few references agree bit for bit, and so do calls of many; between
+    the two forms rows differ by rounding."""
+    torch = pytest.importorskip("torch")
+    n = 1 << log2n
+    few = torch.cuda.get_device_properties(0).multi_processor_count // 8
+    rf, x, _ = _inputs(torch, n)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(log2n)
+    filt = torch.view_as_complex(torch.randn((2 * few + 3, n // 2 + 1, 2), device="cuda", generator=g))
+    call = lambda count: rf.mf_filtered(x, filt[:count].contiguous())
+    many, more = call(few + 1), call(2 * few + 3)
+    assert torch.equal(many, more[: few + 1])
+    one, full = call(1), call(few)
+    assert torch.equal(one[0], full[0]) and torch.equal(call(few // 2), full[: few // 2])
+    assert (full - many[:few]).abs().max().item() <= 1e-6 * many.abs().max().item()
