@@ -168,11 +168,14 @@ rf_status rf_reference_filters(rf_ctx* ctx, const double* inv_psd, int32_t nref,
 
 /* Reference matched filter from stored filters: X = DFT(x) once (unnormalised, Eq. 1), then
  * for each reference z_r[i] = sum_{k=0}^{n/2} X[k] filt[r][k] exp(+2 pi i i k / n), which is
- * z_ref of rf_mf_reference (Eqs. 2, 6).  The product is formed inside the first pass of the
- * inverse transform.  x: real[n]; filt: complex[nref][n/2+1]; z_out: complex[nref][n] (grid
- * dtype).  The first call allocates a temporary of up to min(nref, 2^27 / n) x n complex
- * values (later calls with as many references reuse it, so a warmed-up call can be captured
- * in a CUDA graph).  Async on stream. */
+ * z_ref of rf_mf_reference (Eqs. 2, 6).  x: real[n]; filt: complex[nref][n/2+1]; z_out:
+ * complex[nref][n] (grid dtype); x or filt may lie inside z_out.  RF_F32 grids of 2^9 to 2^13 samples,
+ * of 2^14, and for at most SMs / 8 references of 2^15 and 2^16, run in one launch without a temporary (unless
+ * filt lies inside z_out: a copy of the filters).  The others take a temporary of min(nref, R) x n complex
+ * values, rounded up to a power of two, R = 2^25 / n (RF_F32, and RF_F64 from 2^14 to 2^18 samples) or 2^27 / n, at
+ * most 65535.  It grows on the first call that needs more, and what a captured graph uses is kept: a call can be
+ * captured once the same call (references, and whether filt lies inside z_out) has run.  Rows of a call do not
+ * depend on the other filters (RF_F32 grids of 2^14 to 2^16 samples: see rf_mf_reference).  Async on stream. */
 rf_status rf_mf_filtered(rf_ctx* ctx, const void* x, int32_t nref, const void* filt, void* z_out, rf_stream stream);
 
 /* Ratio kernels of k neighbours of one reference (Sec. II.B-II.D).  Per neighbour j, in FP64

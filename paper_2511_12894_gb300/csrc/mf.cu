@@ -414,9 +414,9 @@ void mf_filtered_impl(rf_ctx* c, const void* x, int32_t nref, const void* filt, 
     const float2* F = static_cast<const float2*>(filt);
     const size_t fb = sizeof(float2) * (size_t)nref * (size_t)nb;
     if (overlap(filt, fb, z_out, sizeof(float2) * (size_t)nref * (size_t)n)) {
-      c->mf_tmp.ensure(fb);
-      RF_CUDA(cudaMemcpyAsync(c->mf_tmp.p, filt, fb, cudaMemcpyDeviceToDevice, s));
-      F = c->mf_tmp.as<float2>();
+      void* copy = c->mf_tmp.ensure(fb);
+      RF_CUDA(cudaMemcpyAsync(copy, filt, fb, cudaMemcpyDeviceToDevice, s));
+      F = static_cast<const float2*>(copy);
     }
     block_mf(c, xa, F, nb, static_cast<float2*>(z_out), nref, s);
     return;
@@ -428,12 +428,12 @@ void mf_filtered_impl(rf_ctx* c, const void* x, int32_t nref, const void* filt, 
     const int64_t most = fft4_inverse_supported(n, sizeof(T) == 8) ? std::max<int64_t>(1, kF4Chunk / n)
                                                            : std::min<int64_t>(65535, ((int64_t)1 << 27) / n);
     const int chunk = (int)std::max<int64_t>(1, std::min<int64_t>(nref, most));
-    c->mf_tmp.ensure(sizeof(V) * (size_t)chunk * n);
-    forward_real(c, static_cast<const T*>(x), c->xf.as<V>(), c->mf_tmp.as<V>(), s);
+    V* tmp = static_cast<V*>(c->mf_tmp.ensure(sizeof(V) * (size_t)chunk * n));
+    forward_real(c, static_cast<const T*>(x), c->xf.as<V>(), tmp, s);
     for (int r0 = 0; r0 < nref; r0 += chunk) {
       const int cnt = std::min(chunk, nref - r0);
       inverse_product(c, c->xf.as<V>(), static_cast<const V*>(filt) + (int64_t)r0 * nb, nb,
-                      static_cast<V*>(z_out) + (int64_t)r0 * n, c->mf_tmp.as<V>(), cnt, s);
+                      static_cast<V*>(z_out) + (int64_t)r0 * n, tmp, cnt, s);
     }
   };
   if (c->g.dtype == RF_F64) run(double2{});

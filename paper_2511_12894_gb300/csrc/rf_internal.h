@@ -67,6 +67,22 @@ struct DevBuf {
   T* as() const { return static_cast<T*>(p); }
 };
 
+// A device buffer that grows by powers of two and keeps what it outgrew: a graph captured with an earlier
+// buffer stays valid while the owner lives, and all of them together are below twice the largest.
+struct KeptBuf {
+  DevBuf at[64];
+  int log = -1;
+  void* ensure(size_t b) {
+    int l = 8;
+    while (((size_t)1 << l) < b) ++l;
+    if (l > log) {
+      at[l].ensure((size_t)1 << l);
+      log = l;
+    }
+    return at[log].p;
+  }
+};
+
 // Pinned host memory, grown on demand (contents are not kept).
 struct PinBuf {
   void* p = nullptr;
@@ -174,7 +190,7 @@ struct rf_ctx {
   rf::DevBuf red;      // FP64 reduction scratch
   rf::DevBuf scratch;  // growable: packed window keys, OS block spectra, builder chunks
   rf::DevBuf scratch2;
-  rf::DevBuf mf_tmp;   // inverse-transform temporaries of the stored-filter matched filter
+  rf::KeptBuf mf_tmp;  // inverse-transform temporaries of the stored-filter matched filter
   rf::DevBuf status;   // int: device-side error status (RF_ETIMEOUT from bounded waits), 0 if none
   size_t reserved = 0;
   int64_t max_chunk = 0;  // builder templates per chunk
