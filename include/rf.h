@@ -376,9 +376,10 @@ void rf_kernels_free(rf_kernels* kern);
  * RF_F64 grids, whichever is modelled cheaper of the direct sum and a double-precision overlap-save
  * (the first such call prepares the kernel set and SYNCHRONISES `stream`; while a set is not prepared
  * a call under stream capture runs the direct sum; the workspace comes in stream order from a pool of
- * the context).  In the overlap-save forms a non-finite sample of z_ref reaches every output of the
- * blocks that hold it.  The context's workspace grows on first use ((B / Lp) n
- * complex64 for OS; see rf_reserve).  Async on stream, except that an OS call on a kernel set that was not
+ * the context; a captured call holds it as allocation nodes of the graph).  In the FP32 overlap-save
+ * forms a non-finite sample of z_ref reaches every output of the blocks that hold it; the FP64 one sums
+ * the blocks whose samples are not finite, or range over more than about 2^10, directly.  The
+ * context's workspace grows on first use ((B / Lp) n complex64 for OS; see rf_reserve).  Async on stream, except that an OS call on a kernel set that was not
  * prepared prepares it first (see rf_kernels_prepare). */
 rf_status rf_reconstruct(rf_ctx* ctx, const void* z_ref, const rf_kernels* kern, int32_t algo,
                          int32_t prec, void* z_out, rf_stream stream);

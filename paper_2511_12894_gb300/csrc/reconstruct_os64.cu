@@ -7,8 +7,14 @@
 // here in FP64 throughout.  Bound by the FP64 pipe (about 1.6 multiply-adds per clock and SM,
 // measured): a block costs about 3.4 log2(B) + 4 P + 5 FP64 instructions per point, the direct sum
 // 4 L per output.  16 neighbours of 930 taps at n = 2^16 with window peaks: 7157 us by the direct
-// sum, 155 us here (the first call, which prepares the spectra, 398 us).  Non-finite samples of z_ref
-// reach every output of the blocks that hold them, as in the FP32 form.
+// sum, 155 us here (the first call, which prepares the spectra, 398 us).
+//
+// A transform mixes all samples of its block: one that is not finite would reach every output of the
+// block, and the rounding of a loud stretch the quiet ones beside it, where the direct sum keeps both to the
+// kernel's own samples.  Each segment therefore leaves the magnitudes of its loudest sample and of its quietest
+// run of 32 samples, and a block whose segments span more than 2^10 between the two, or come near the
+// end of the FP64 range, forms its outputs as direct sums instead: 2^10 roundings are the 1e-12 that FP64
+// results are held to, and series of a matched filter stay within 2^5.
 //
 // Window peaks compare |z|^2 in FP64.  A block leaves the best of each of its pieces (its run of
 // outputs cut at window boundaries and at the wrap to sample 0) in a list, and a second kernel
@@ -54,18 +60,47 @@ __device__ __forceinline__ Piece warp_piece(Piece b) {
 // Most pieces of a run of H outputs: the window boundaries inside it and the wrap.
 __host__ __device__ constexpr int64_t piece_slots(int64_t H, int64_t W) { return (H - 1) / W + 3; }
 
+// High words of the magnitudes max(|x|, |y|) of a segment: its largest, and the smallest of the
+// largest of runs of 32 samples (NaN is above infinity).
+struct Range64 {
+  unsigned hi, lo;
+};
+// Whether a block of these segments is left to the direct sum.
+__device__ __forceinline__ bool too_wide(Range64 r) {
+  constexpr unsigned top = (1023u + 960u) << 20;  // 2^960: no sum of a block or product overflows below it
+  return r.hi >= top || (r.hi >> 20) > (r.lo >> 20) + 10u;
+}
+
 // Segment spectra: block q transforms z_ref[(q Lp + t) mod n], t < B.
 template <int B>
 __global__ void __launch_bounds__(B / 16) k_os64_segments(const double2* __restrict__ z_ref, int64_t n, int Lp,
-                                                          const double2* __restrict__ tw, double2* __restrict__ Zs) {
+                                                          const double2* __restrict__ tw, double2* __restrict__ Zs,
+                                                          Range64* __restrict__ ranges) {
   constexpr int NT = B / 16;
   extern __shared__ __align__(16) double2 sm64[];
+  __shared__ Range64 wr[NT / 32];
   const int64_t q = blockIdx.x;
   const int tid = threadIdx.x;
   double2 v[16];
 #pragma unroll
   for (int t = 0; t < 16; ++t) v[t] = z_ref[(q * Lp + tid + t * NT) & (n - 1)];
-  block_fft<B, -1>(v, sm64, tw);
+  Range64 r{0u, ~0u};
+#pragma unroll
+  for (int t = 0; t < 16; ++t) {  // a warp's samples of one t are a run of 32
+    const unsigned h = __reduce_max_sync(0xffffffffu, max((unsigned)__double2hiint(v[t].x) & 0x7fffffffu,
+                                                          (unsigned)__double2hiint(v[t].y) & 0x7fffffffu));
+    r.hi = max(r.hi, h);
+    r.lo = min(r.lo, h);
+  }
+  if ((tid & 31) == 0) wr[tid >> 5] = r;
+  block_fft<B, -1>(v, sm64, tw);  // its barriers come between that and this
+  if (tid == 0) {
+    for (int w = 1; w < NT / 32; ++w) {
+      r.hi = max(r.hi, wr[w].hi);
+      r.lo = min(r.lo, wr[w].lo);
+    }
+    ranges[q] = r;
+  }
 #pragma unroll
   for (int t = 0; t < 16; ++t) Zs[q * B + tid + t * NT] = v[t];
 }
@@ -102,6 +137,41 @@ __global__ void __launch_bounds__(B / 16) k_os64_partitions(const void* __restri
   }
 }
 
+// The kernels and the series themselves, for blocks formed as direct sums.
+struct Direct64 {
+  const double2* z;
+  const void* taps;  // double2, or double (real)
+  const int64_t* off;
+  const int* len;
+  int real;
+};
+
+// sum_l c_j[l] z[(o - l) mod n], in partial sums of 128 terms
+__device__ __noinline__ double2 direct64(const Direct64& d, int j, int64_t o, int64_t mask) {
+  const int L = d.len[j];
+  const double* cr = static_cast<const double*>(d.taps) + d.off[j] * (d.real ? 1 : 2);
+  double2 sum = make_double2(0.0, 0.0);
+  for (int l0 = 0; l0 < L; l0 += 128) {
+    double2 p = make_double2(0.0, 0.0);
+    const int l1 = min(L, l0 + 128);
+    for (int l = l0; l < l1; ++l) {
+      const double2 z = __ldg(d.z + ((o - l) & mask));
+      if (d.real) {
+        const double c = __ldg(cr + l);
+        p.x = fma(c, z.x, p.x);
+        p.y = fma(c, z.y, p.y);
+      } else {
+        const double a = __ldg(cr + 2 * (int64_t)l), b = __ldg(cr + 2 * (int64_t)l + 1);
+        p.x = fma(a, z.x, fma(-b, z.y, p.x));
+        p.y = fma(a, z.y, fma(b, z.x, p.y));
+      }
+    }
+    sum.x += p.x;
+    sum.y += p.y;
+  }
+  return sum;
+}
+
 // Output block blockIdx.x of neighbour j0 + blockIdx.y: the partition products, the inverse
 // transform, then the series row or the pieces of the window peaks.
 template <int B, int Q, bool WINMAX>
@@ -110,6 +180,7 @@ __global__ void __launch_bounds__(B / 16, 8192 / B) k_os64(const double2* __rest
                                                            const int64_t* __restrict__ spec_off,
                                                            const int* __restrict__ parts,
                                                            const int* __restrict__ lag0, int j0,
+                                                           const Range64* __restrict__ ranges, Direct64 dir,
                                                            const double2* __restrict__ tw, int64_t n, int NQ,
                                                            double2* __restrict__ z_out, Piece* __restrict__ pieces,
                                                            int64_t W, int64_t slots) {
@@ -124,7 +195,11 @@ __global__ void __launch_bounds__(B / 16, 8192 / B) k_os64(const double2* __rest
 #pragma unroll
   for (int t = 0; t < 16; ++t) v[t] = make_double2(0.0, 0.0);
   int sp = s * (Q - 1) - 1;
+  Range64 range{0u, ~0u};
   for (int p = 0; p < P; ++p, --sp) {
+    const Range64 r = ranges[sp & (NQ - 1)];
+    range.hi = max(range.hi, r.hi);
+    range.lo = min(range.lo, r.lo);
     const double2* z = Zs + (int64_t)(sp & (NQ - 1)) * B + tid;  // NQ a power of two
     const double2* c = C + (int64_t)p * B;
 #pragma unroll
@@ -139,6 +214,16 @@ __global__ void __launch_bounds__(B / 16, 8192 / B) k_os64(const double2* __rest
   const int64_t o0 = (int64_t)s * H;  // pre-relabel index of block position LP
   const int64_t base = (o0 + lag0[j]) & mask;
   const int cnt = (int)min((int64_t)H, n - o0);
+  if (too_wide(range)) {
+#pragma unroll 1
+    for (int t = 16 / Q; t < 16; ++t) {
+      const int e = tid + t * NT - LP;
+      const double2 y = e < cnt ? direct64(dir, j, o0 + e, mask) : make_double2(0.0, 0.0);
+#pragma unroll
+      for (int u = 16 / Q; u < 16; ++u)
+        if (u == t) v[u] = y;  // registers indexed at compile time
+    }
+  }
   if constexpr (!WINMAX) {
 #pragma unroll
     for (int t = 16 / Q; t < 16; ++t) {
@@ -406,18 +491,22 @@ bool reconstruct_os64(rf_ctx* c, const void* z_ref, rf_kernels* kern, void* z_ou
   const int NQ = (int)(n / Lp), NB = (int)((n + H - 1) / H);
   const int64_t nw = win ? (n + W - 1) / W : 0, slots = win ? piece_slots(H, W) : 0;
   const size_t zs_bytes = sizeof(double2) * (size_t)NQ * B;
-  const size_t need = zs_bytes + sizeof(Piece) * (size_t)kern->k * NB * (size_t)slots;
+  const size_t range_bytes = (sizeof(Range64) * (size_t)NQ + 15) & ~(size_t)15;
+  const size_t need = zs_bytes + range_bytes + sizeof(Piece) * (size_t)kern->k * NB * (size_t)slots;
   if (need > kWork64Max) return false;
   StreamBuf work(c, need, s);
   if (!work.p) return false;
   double2* Zs = static_cast<double2*>(work.p);
-  Piece* pieces = reinterpret_cast<Piece*>(static_cast<char*>(work.p) + zs_bytes);
+  Range64* ranges = reinterpret_cast<Range64*>(static_cast<char*>(work.p) + zs_bytes);
+  Piece* pieces = reinterpret_cast<Piece*>(static_cast<char*>(work.p) + zs_bytes + range_bytes);
+  const Direct64 dir{static_cast<const double2*>(z_ref), kern->taps.p, kern->off_d.as<int64_t>(),
+                     kern->len_d.as<int>(), kern->real ? 1 : 0};
   const double2* tw = c->twb64.as<double2>() + c->twb64_off[table64(B)];
   dispatch64(B, Q, [&](auto bc, auto qc) {
     constexpr int BB = decltype(bc)::value, QQ = decltype(qc)::value;
     auto seg = k_os64_segments<BB>;
     RF_CUDA(cudaFuncSetAttribute(seg, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem64<BB>(0)));
-    seg<<<NQ, BB / 16, smem64<BB>(0), s>>>(static_cast<const double2*>(z_ref), n, Lp, tw, Zs);
+    seg<<<NQ, BB / 16, smem64<BB>(0), s>>>(static_cast<const double2*>(z_ref), n, Lp, tw, Zs, ranges);
     RF_LAUNCHED();
     auto run = [&](auto fn, size_t smem) {
       RF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -425,7 +514,7 @@ bool reconstruct_os64(rf_ctx* c, const void* z_ref, rf_kernels* kern, void* z_ou
         const int cnt = std::min(65535, kern->k - j0);
         fn<<<dim3((unsigned)NB, (unsigned)cnt), BB / 16, smem, s>>>(
             Zs, kern->os64_spec.as<double2>(), kern->os64_off_d.as<int64_t>(), kern->os64_parts_d.as<int>(),
-            kern->lag0_d.as<int>(), j0, tw, n, NQ, static_cast<double2*>(z_out), pieces, W, slots);
+            kern->lag0_d.as<int>(), j0, ranges, dir, tw, n, NQ, static_cast<double2*>(z_out), pieces, W, slots);
         RF_LAUNCHED();
       }
     };
