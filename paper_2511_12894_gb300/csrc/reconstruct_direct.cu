@@ -219,55 +219,66 @@ void launch_direct(rf_ctx* c, const rf_kernels* kern, const V* z_ref, V* z_out, 
   }
 }
 
-// Window peaks of series already in memory: CS blocks per (window, series), one cluster.  Block c
-// reads the c-th part of the window with 16-byte loads and the cluster's first block takes the
-// best of the parts through distributed shared memory, so no workspace is needed (calls on
-// several streams stay independent).  Bound by HBM.  One block per window left most SMs idle when
-// windows are long: 6 series of 2^23 samples in 2^20-sample windows took 464 us on 48 blocks of
-// 256 threads (24 series of 2^20 in 2^17-sample windows: 65 us).
-template <typename V, int NT>
-__global__ void __launch_bounds__(NT) k_winmax_series(const V* __restrict__ z, int64_t n, int64_t W, int64_t nw,
-                                                      int CS, float* __restrict__ max_out,
-                                                      int* __restrict__ arg_out) {
-  using R = typename real_of<V>::type;
-  constexpr int E = 16 / (int)sizeof(V);  // samples per 16-byte load
-  const int64_t w = blockIdx.x / (unsigned)CS;
-  const int part = (int)(blockIdx.x % (unsigned)CS);
-  const int64_t row = blockIdx.y;
-  const V* zr = z + row * n;
-  const int64_t wlo = w * W, whi = min(n, wlo + W);
-  const int64_t per = ((whi - wlo + CS - 1) / CS + E - 1) / E * E;
-  const int64_t lo = min(whi, wlo + part * per), hi = min(whi, lo + per);
-  R bv = (R)-1;
-  long long bi = 0;
-  auto take = [&](V a, int64_t i) {
-    const R v = a.x * a.x + a.y * a.y;
-    if (v > bv) {
-      bv = v;
-      bi = i;
-    }
-  };
-  if constexpr (E == 1) {
-    int64_t i = lo + threadIdx.x;
+// Window peaks of series already in memory.  |z|^2 is compared as an integer (non-negative floating-point
+// numbers order as their bits; -1: none, NaN never counts): the FP64 pipe, two lanes per SM, has the
+// magnitudes to form, and comparisons on it as well (a block of 512 threads, each going through the
+// warps' results) made FP64 windows of 1024 samples take 186 us for 4 series of 2^20, 2893 for 64 (256
+// threads: 73 and 1097; now 23 and 247, 4.35 TB/s).
+template <typename V> struct PeakKey { using type = int; };
+template <> struct PeakKey<double2> { using type = long long; };
+__device__ __forceinline__ int peak_key(float2 a) { return __float_as_int(a.x * a.x + a.y * a.y); }
+__device__ __forceinline__ long long peak_key(double2 a) { return __double_as_longlong(a.x * a.x + a.y * a.y); }
+template <typename K>
+__device__ __forceinline__ float peak_value(K k) {
+  if constexpr (sizeof(K) == 4) return k < 0 ? -1.f : __int_as_float(k);
+  else return k < 0 ? -1.f : (float)__longlong_as_double(k);
+}
+template <typename K>
+struct Peak {
+  K k;
+  int i;
+};
+template <typename K>
+__device__ __forceinline__ void peak_take(Peak<K>& b, K k, int i) {  // samples in increasing order
+  constexpr K inf = sizeof(K) == 4 ? (K)0x7f800000 : (K)0x7ff0000000000000ll;
+  if (k > b.k && k <= inf) b = Peak<K>{k, i};
+}
+template <typename K>
+__device__ __forceinline__ void peak_join(Peak<K>& b, Peak<K> o) {
+  if (o.k > b.k || (o.k == b.k && o.i < b.i)) b = o;
+}
+template <typename K>
+__device__ __forceinline__ Peak<K> peak_warp(Peak<K> b) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    peak_join(b, Peak<K>{__shfl_xor_sync(0xffffffffu, b.k, o), __shfl_xor_sync(0xffffffffu, b.i, o)});
+  return b;
+}
+
+// The peak of samples [lo, hi) of a row by threads tid < NT, 16-byte loads, four in flight each; every thread
+// meets its samples in increasing order.
+template <typename V, int NT, typename K>
+__device__ __forceinline__ void peak_scan(Peak<K>& b, const V* __restrict__ zr, int lo, int hi, int tid) {
+  if constexpr (sizeof(V) == 16) {
+    int i = lo + tid;
     for (; i + 3 * NT < hi; i += 4 * NT) {
       V a[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) a[u] = __ldg(zr + i + u * NT);
 #pragma unroll
-      for (int u = 0; u < 4; ++u) take(a[u], i + u * NT);
+      for (int u = 0; u < 4; ++u) peak_take(b, peak_key(a[u]), i + u * NT);
     }
-    for (; i < hi; i += NT) take(zr[i], i);
+    for (; i < hi; i += NT) peak_take(b, peak_key(zr[i]), i);
   } else {
-    // rows start 16-byte aligned (n even): pairs [2p, 2p + 1] inside [lo, hi), and up to one
-    // sample at each end; every thread meets its samples in increasing order
-    const int64_t p0 = (lo + 1) / 2, p1 = hi / 2;
-    if (threadIdx.x == 0 && (lo & 1) && lo < hi) take(zr[lo], lo);
+    // rows start 16-byte aligned (n even): pairs [2p, 2p + 1] inside [lo, hi), and up to one sample at each end
+    const int p0 = (lo + 1) / 2, p1 = hi / 2;
+    if (tid == 0 && (lo & 1) && lo < hi) peak_take(b, peak_key(zr[lo]), lo);
     const float4* z4 = reinterpret_cast<const float4*>(zr);
-    auto pair = [&](float4 q, int64_t p) {
-      take(cmake<V>(q.x, q.y), 2 * p);
-      take(cmake<V>(q.z, q.w), 2 * p + 1);
+    auto pair = [&](float4 q, int p) {
+      peak_take(b, peak_key(make_float2(q.x, q.y)), 2 * p);
+      peak_take(b, peak_key(make_float2(q.z, q.w)), 2 * p + 1);
     };
-    int64_t p = p0 + threadIdx.x;
+    int p = p0 + tid;
     for (; p + 3 * NT < p1; p += 4 * NT) {
       float4 a[4];
 #pragma unroll
@@ -276,33 +287,87 @@ __global__ void __launch_bounds__(NT) k_winmax_series(const V* __restrict__ z, i
       for (int u = 0; u < 4; ++u) pair(a[u], p + u * NT);
     }
     for (; p < p1; p += NT) pair(__ldg(z4 + p), p);
-    if (threadIdx.x == 0 && (hi & 1) && hi - 1 >= 2 * p0 && lo < hi) take(zr[hi - 1], hi - 1);
+    if (tid == 0 && (hi & 1) && hi - 1 >= 2 * p0 && lo < hi) peak_take(b, peak_key(zr[hi - 1]), hi - 1);
   }
-  Best<R> b = block_best<R, NT>(bv, bi);
+}
+
+// Windows that a warp takes.  Up to 2048 samples it costs no more than a block (64 series of 2^20 in
+// FP32: 77.5 us at 1024, 79 at 2048); at 4096 too few loads are in flight (87.8 against 77.8; 16 series of
+// 2^16 in FP64 23.2 against 17.7).
+constexpr int64_t kShortWindow = 1024;
+
+// Short windows: a warp each.  (A block each spent its time on starting and reducing: 16-sample windows of
+// 4 series of 2^20 took 550 us in FP32, 10262 in FP64; now 42 and 54.)
+template <typename V>
+__global__ void __launch_bounds__(256) k_winmax_short(const V* __restrict__ z, int64_t n, int W, int nw,
+                                                      float* __restrict__ max_out, int* __restrict__ arg_out) {
+  using K = typename PeakKey<V>::type;
+  const int w = blockIdx.x * 8 + (int)(threadIdx.x >> 5);
+  const int64_t row = blockIdx.y;
+  if (w >= nw) return;
+  const int lane = threadIdx.x & 31;
+  const int lo = w * W, hi = min((int)n, lo + W);
+  Peak<K> b{-1, 0};
+  peak_scan<V, 32>(b, z + row * n, lo, hi, lane);
+  b = peak_warp(b);
+  if (lane == 0) {
+    max_out[row * nw + w] = peak_value(b.k);
+    arg_out[row * nw + w] = b.i;
+  }
+}
+
+// Longer windows: CS blocks per (window, series), one cluster.  Block c
+// reads the c-th part of the window and the cluster's first block takes the
+// best of the parts through distributed shared memory, so no workspace is needed (calls on
+// several streams stay independent).  Bound by HBM.  One block per window left most SMs idle when
+// windows are long: 6 series of 2^23 samples in 2^20-sample windows took 464 us on 48 blocks of
+// 256 threads (24 series of 2^20 in 2^17-sample windows: 65 us).
+template <typename V, int NT>
+__global__ void __launch_bounds__(NT) k_winmax_series(const V* __restrict__ z, int64_t n, int64_t W, int nw,
+                                                      int CS, float* __restrict__ max_out,
+                                                      int* __restrict__ arg_out) {
+  using K = typename PeakKey<V>::type;
+  constexpr int E = 16 / (int)sizeof(V);  // samples per 16-byte load
+  const int w = (int)(blockIdx.x / (unsigned)CS);
+  const int part = (int)(blockIdx.x % (unsigned)CS);
+  const int64_t row = blockIdx.y;
+  const int wlo = (int)(w * W), whi = (int)min(n, wlo + W);
+  const int per = ((whi - wlo + CS - 1) / CS + E - 1) / E * E;
+  const int lo = min(whi, wlo + part * per), hi = min(whi, lo + per);
+  Peak<K> b{-1, 0};
+  peak_scan<V, NT>(b, z + row * n, lo, hi, (int)threadIdx.x);
+  __shared__ Peak<K> wb[NT / 32];
+  __shared__ Peak<K> best;
+  b = peak_warp(b);
+  if ((threadIdx.x & 31) == 0) wb[threadIdx.x >> 5] = b;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    b = threadIdx.x < NT / 32 ? wb[threadIdx.x] : Peak<K>{-1, 0x7fffffff};
+    b = peak_warp(b);
+  }
   if (CS > 1) {
-    __shared__ Best<R> best;
     if (threadIdx.x == 0) best = b;
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     if (part == 0 && threadIdx.x == 0) {
       const uint32_t own = (uint32_t)__cvta_generic_to_shared(&best);
       for (int c = 1; c < CS; ++c) {
         uint32_t at;
-        Best<R> o;
+        Peak<K> o;
         asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(own), "r"(c));
-        if constexpr (sizeof(R) == 8)
-          asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(o.v) : "r"(at) : "memory");
+        if constexpr (sizeof(K) == 8)
+          asm volatile("ld.shared::cluster.s64 %0, [%1];" : "=l"(o.k) : "r"(at) : "memory");
         else
-          asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(o.v) : "r"(at) : "memory");
-        asm volatile("ld.shared::cluster.s64 %0, [%1];" : "=l"(o.i) : "r"(at + (uint32_t)offsetof(Best<R>, i)) : "memory");
-        if (better(o.v, o.i, b.v, b.i)) b = o;
+          asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(o.k) : "r"(at) : "memory");
+        asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(o.i) : "r"(at + (uint32_t)offsetof(Peak<K>, i)) : "memory");
+        peak_join(b, o);
       }
     }
     // the other blocks' shared memory stays until it has been read
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
   }
   if (part == 0 && threadIdx.x == 0) {
-    max_out[row * nw + w] = (float)b.v;
-    arg_out[row * nw + w] = (int)b.i;
+    max_out[row * nw + w] = peak_value(b.k);
+    arg_out[row * nw + w] = b.i;
   }
 }
 
@@ -325,9 +390,23 @@ void launch_winmax_series(rf_ctx* c, const void* z, int32_t count, int64_t W, in
   at.val.clusterDim.z = 1;
   cfg.attrs = &at;
   cfg.numAttrs = CS > 1 ? 1 : 0;
-  RF_CUDA(cudaLaunchKernelEx(&cfg, k_winmax_series<V, NT>, static_cast<const V*>(z), c->n, W, nw, CS, max_out,
+  RF_CUDA(cudaLaunchKernelEx(&cfg, k_winmax_series<V, NT>, static_cast<const V*>(z), c->n, W, (int)nw, CS, max_out,
                              (int*)argmax_out));
   RF_LAUNCHED();
+}
+
+template <typename V>
+void winmax_rows(rf_ctx* c, const void* z, int32_t count, int64_t W, int64_t nw, float* max_out, int32_t* argmax_out,
+                 cudaStream_t s) {
+  if (W <= kShortWindow) {
+    k_winmax_short<V><<<dim3((unsigned)((nw + 7) / 8), (unsigned)count), 256, 0, s>>>(
+        static_cast<const V*>(z), c->n, (int)W, (int)nw, max_out, (int*)argmax_out);
+    RF_LAUNCHED();
+  } else if (W >= 8192) {  // enough samples for 512 threads with four 16-byte loads each in flight
+    launch_winmax_series<V, 512>(c, z, count, W, nw, max_out, argmax_out, s);
+  } else {
+    launch_winmax_series<V, 256>(c, z, count, W, nw, max_out, argmax_out, s);
+  }
 }
 
 }  // namespace
@@ -361,12 +440,8 @@ void winmax_series(rf_ctx* c, const void* z, int32_t count, int64_t W, float* ma
   const int64_t n = c->n;
   const int64_t nw = (n + W - 1) / W;
   RF_REQUIRE(nw <= 0x7fffffff && count <= 65535, "winmax: too many windows or series");
-  if (c->g.dtype == RF_F64)
-    launch_winmax_series<double2, 512>(c, z, count, W, nw, max_out, argmax_out, s);
-  else if (W >= 8192)  // enough samples for 512 threads with four 16-byte loads each in flight
-    launch_winmax_series<float2, 512>(c, z, count, W, nw, max_out, argmax_out, s);
-  else
-    launch_winmax_series<float2, 256>(c, z, count, W, nw, max_out, argmax_out, s);
+  if (c->g.dtype == RF_F64) winmax_rows<double2>(c, z, count, W, nw, max_out, argmax_out, s);
+  else winmax_rows<float2>(c, z, count, W, nw, max_out, argmax_out, s);
 }
 
 }  // namespace rf

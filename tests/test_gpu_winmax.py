@@ -38,3 +38,27 @@ def test_nan_never_wins():
     z[0, W + 40000] = float("nan")
     P, A = rf.winmax(z, W)
     assert P[0].tolist() == [-1.0, 4.0] and A[0].tolist() == [0, W + 77]
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("W", [1, 2, 31, 32, 33, 64, 257, 1000, 1023, 1024, 1025, 2049])
+def test_short_windows(dtype, W):
+    """A warp per window up to 1024 samples, a block beyond: odd starts, ragged last windows, ties, windows
+    of NaN and infinity."""
+    torch = pytest.importorskip("torch")
+    from paper_2511_12894_gb300 import RatioFilter
+    n, count = 1 << 14, 2
+    rf = RatioFilter(n, 2048.0, 20.0, 971.0, 7, dtype)
+    rng = np.random.default_rng(W)
+    z = rng.integers(-3, 4, (count, n)) + 1j * rng.integers(-3, 4, (count, n))
+    z[0, rng.integers(0, n, 300)] = np.nan
+    z[1, : 3 * W] = np.nan
+    z[1, rng.integers(3 * W, n, 9)] = np.inf
+    P, A = rf.winmax(torch.tensor(z, dtype=rf.cdtype, device="cuda"), W)
+    nw = -(-n // W)
+    with np.errstate(invalid="ignore"):
+        m = np.abs(z.real) ** 2 + np.abs(z.imag) ** 2
+    m = np.pad(np.where(np.isnan(m), -1.0, m), ((0, 0), (0, nw * W - n)), constant_values=-2.0).reshape(count, nw, W)
+    best = m.max(-1)
+    assert np.array_equal(P.cpu().numpy(), best.astype(np.float32))
+    assert np.array_equal(A.cpu().numpy(), np.where(best < 0, 0, m.argmax(-1) + W * np.arange(nw)))
