@@ -452,39 +452,43 @@ void os64_create(rf_ctx* c) {
   RF_CUDA(cudaMemcpy(c->twb64.p, tw.data(), sizeof(double2) * tw.size(), cudaMemcpyHostToDevice));
 }
 
-// False where the direct sum should run instead: it is modelled cheaper, the kernel set cannot be
-// prepared now (stream capture) or memory for the spectra is short.
-bool reconstruct_os64(rf_ctx* c, const void* z_ref, rf_kernels* kern, void* z_out, int64_t W, float* max_out,
-                      int32_t* argmax_out, cudaStream_t s) {
+// Prepares a kernel set where the transform form is modelled cheaper.  os64_B is settled (-1: the direct
+// sum) by the model and the bound on the spectra alone; a set that met a shortage of memory or a stream
+// under capture stays open, and the next call tries again.
+bool os64_prepare(rf_ctx* c, rf_kernels* kern, cudaStream_t s) {
   if (!c->pool || kern->k == 0) return false;
   RelaxedCapture relaxed;
-  std::unique_lock<std::mutex> lock(kern->os64_mu);
-  int B = kern->os64_B, Q = kern->os64_Q;
-  if (B < 0) return false;
-  if (!B) {
-    choose64(c, kern, &B, &Q);
-    if (!B) {
-      kern->os64_B = -1;
-      return false;
-    }
+  std::lock_guard<std::mutex> lock(kern->os64_mu);
+  if (kern->os64_B) return kern->os64_B > 0;
+  int B, Q;
+  choose64(c, kern, &B, &Q);
+  if (B) {
     int64_t rows = 0;
     for (const int L : kern->len) rows += std::max(1, (L + B / Q - 1) / (B / Q));
-    if (rows > INT_MAX / 2 || sizeof(double2) * (size_t)rows * B > kWork64Max) {
-      kern->os64_B = -1;
-      return false;
-    }
-    if (capturing(s)) return false;
-    try {
-      prepare64(c, kern, B, Q, s);
-    } catch (const Fail& e) {
-      if (e.st != RF_ENOMEM) throw;
-      clear_error();
-      kern->os64_spec.release();
-      kern->os64_B = -1;
-      return false;
-    }
+    if (rows > INT_MAX / 2 || sizeof(double2) * (size_t)rows * B > kWork64Max) B = 0;
   }
-  lock.unlock();
+  if (!B) {
+    kern->os64_B = -1;
+    return false;
+  }
+  if (capturing(s)) return false;
+  try {
+    prepare64(c, kern, B, Q, s);
+  } catch (const Fail& e) {
+    if (e.st != RF_ENOMEM) throw;
+    clear_error();
+    kern->os64_spec.release();
+    return false;
+  }
+  return true;
+}
+
+// False where the direct sum should run instead: the set is not prepared or memory for the call is short.
+bool reconstruct_os64(rf_ctx* c, const void* z_ref, rf_kernels* kern, void* z_out, int64_t W, float* max_out,
+                      int32_t* argmax_out, cudaStream_t s) {
+  if (!os64_prepare(c, kern, s)) return false;
+  RelaxedCapture relaxed;
+  const int B = kern->os64_B, Q = kern->os64_Q;  // they no longer change
   const bool win = max_out != nullptr;
   const int64_t n = c->n;
   const int Lp = B / Q, H = B - Lp;
