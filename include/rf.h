@@ -266,7 +266,10 @@ rf_status rf_kernels_info(const rf_kernels* kern, int32_t* k, const int32_t** le
  * (sum_j ceil(L_j / Lp) x B complex64; for a real-form set the Hermitian half, bins 0..B/2 in
  * rows of B/2 + 8, and block sizes up to 16384).  Each output block transform then keeps B - Lp
  * outputs.  The first overlap-save reconstruction prepares with the modelled choice if this
- * was not called.  Allocates; SYNCHRONISES `stream`.  RF_EINVAL for other sizes. */
+ * was not called.  On RF_F64 grids block and part are 0 (else RF_EUNSUPPORTED) and the set is prepared for
+ * the double-precision form that RF_ALGO_AUTO then runs, as its first call would do: partition spectra of up to
+ * 8 GB (beyond that, or where the direct sum is modelled cheaper, or while memory is short, nothing is prepared and
+ * AUTO runs the direct sum).  Allocates; SYNCHRONISES `stream`.  RF_EINVAL for other sizes. */
 rf_status rf_kernels_prepare(rf_ctx* ctx, rf_kernels* kern, int32_t block, int32_t part, rf_stream stream);
 
 /* Overlap-save layout a kernel set is prepared for: block size and partition length of its

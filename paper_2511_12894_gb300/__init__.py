@@ -260,7 +260,7 @@ class Kernels:
 
     def prepare(self, block: int = 0, part: int = 0, stream=None) -> None:
         """Overlap-save preparation with block size ``block`` and partition length ``part``
-        (0: defaults); synchronises."""
+        (0: defaults, the only ones on FP64 grids); synchronises."""
         _check(_lib.rf_kernels_prepare(self.ctx.handle, self.handle, int(block), int(part), _stream(stream)))
 
     def prepare_buckets(self, cuts: Sequence[int], blocks: Sequence[int], parts: Sequence[int], stream=None) -> None:

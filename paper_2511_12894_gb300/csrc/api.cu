@@ -331,6 +331,10 @@ rf_status rf_kernels_prepare(rf_ctx* ctx, rf_kernels* kern, int32_t block, int32
     check_ctx(ctx);
     RF_REQUIRE(kern != nullptr, "kern is NULL");
     RF_REQUIRE(kern->n == ctx->n && kern->dtype == ctx->g.dtype, "kernels were made for another grid");
+    if (ctx->g.dtype == RF_F64 && block == 0 && part == 0) {  // what AUTO prepares on its first call
+      os64_prepare(ctx, kern, (cudaStream_t)stream);
+      return;
+    }
     if (ctx->g.dtype != RF_F32 || ctx->n < 512) {
       set_error("overlap-save needs an RF_F32 grid with n >= 512");
       throw Fail{RF_EUNSUPPORTED};

@@ -401,9 +401,10 @@ rf_kernels* import_impl(rf_ctx* c, int32_t k, const int32_t* lag0, const int32_t
 // ---------------------------------------------------------------- reconstruct
 void reconstruct_direct(rf_ctx* c, const void* z_ref, const rf_kernels* kern, void* z_out,
                         int64_t W, float* max_out, int32_t* argmax_out, cudaStream_t s);
-// FP64 overlap-save (reconstruct_os64.cu): tables and pool of an RF_F64 context; a reconstruction,
-// false when the direct sum is to run instead
+// FP64 overlap-save (reconstruct_os64.cu): tables of an RF_F64 context; the preparation of a set and a
+// reconstruction, both false when the direct sum is to run instead
 void os64_create(rf_ctx* c);
+bool os64_prepare(rf_ctx* c, rf_kernels* kern, cudaStream_t s);
 bool reconstruct_os64(rf_ctx* c, const void* z_ref, rf_kernels* kern, void* z_out, int64_t W, float* max_out,
                       int32_t* argmax_out, cudaStream_t s);
 void winmax_series(rf_ctx* c, const void* z, int32_t count, int64_t W, float* max_out,

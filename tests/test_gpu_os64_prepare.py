@@ -43,3 +43,28 @@ def test_a_shortage_of_memory_passes():
     call()
     assert _launches(call) == 3
     assert torch.equal(ao, arg) and torch.allclose(mo, want, rtol=1e-6, atol=0.0)
+
+
+def test_prepared_ahead_of_the_first_call():
+    """A set prepared by the caller: its first AUTO call neither prepares nor synchronises, so it can be captured in
+    the overlap-save form; other layouts are refused as before."""
+    torch = pytest.importorskip("torch")
+    from paper_2511_12894_gb300 import RFError
+    n, W = 1 << 14, 512
+    rf, z, kern = _set(torch, n, [900, 901, 902, 903])
+    with pytest.raises(RFError):
+        kern.prepare(4096, 1024)
+    kern.prepare()
+    want, arg = rf.reconstruct_winmax(z, kern, W, "direct")
+    mo, ao = torch.empty_like(want), torch.empty_like(arg)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        used = _launches(lambda: rf.reconstruct_winmax(z, kern, W, max_out=mo, arg_out=ao))
+    assert used == 3
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(ao, arg) and torch.allclose(mo, want, rtol=1e-6, atol=0.0)
+    rf2, z2, short = _set(torch, n, [1, 2, 3])
+    short.prepare()                                   # the direct sum is cheaper: nothing to prepare
+    assert _launches(lambda: rf2.reconstruct(z2, short)) == 1
