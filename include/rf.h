@@ -445,9 +445,8 @@ typedef struct {
  * than 1024 taps.  out (host, may be NULL): up to max_out entries, the winner first; *n_out (host,
  * may be NULL) the number written.  Kernel sets end up prepared for the winner (a bucketed
  * winner, overlap-save or mixed, is then what RF_ALGO_AUTO runs; for another form, the last
- * layout timed).  On RF_F64 grids the candidates are the direct sum and, where some set's choice of
- * RF_ALGO_AUTO is the double-precision overlap-save, that choice (algo RF_ALGO_AUTO, with the block size and
- * partition length of the first such set).  Allocates; SYNCHRONISES `stream`. */
+ * layout timed).  On RF_F64 grids, where the direct sum is the only candidate, RF_ALGO_AUTO keeps
+ * the rule of rf_reconstruct.  Allocates; SYNCHRONISES `stream`. */
 rf_status rf_autotune(rf_ctx* ctx, int32_t G, const void* const* z_refs, rf_kernels* const* ks, int64_t W,
                       int32_t flags, int32_t max_os, rf_tune_entry* out, int32_t max_out, int32_t* n_out,
                       rf_stream stream);

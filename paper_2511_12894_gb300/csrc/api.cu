@@ -5,7 +5,6 @@
 #include <cstring>
 #include <memory>
 #include <new>
-#include <vector>
 
 #include "rf_internal.h"
 
@@ -600,13 +599,11 @@ rf_status rf_reconstruct_batched(rf_ctx* ctx, int32_t G, const void* const* z_re
     int64_t rows = 0;
     int a = RF_ALGO_AUTO;
     int32_t pa = prec;
-    std::vector<int> forms(G);  // FP64 sets run one by one, each in its own
     for (int g = 0; g < G; ++g) {
       RF_REQUIRE(ks[g] != nullptr, "ks[%d] is NULL", g);
       int32_t pg = prec;
       const int ag = check_recon(ctx, z_refs[g], ks[g], algo, pg);
-      forms[g] = ag;
-      RF_REQUIRE(g == 0 || ctx->g.dtype == RF_F64 || (ag == a && pg == pa),
+      RF_REQUIRE(g == 0 || (ag == a && pg == pa),
                  "the groups resolve to different forms (tune them together with rf_autotune)");
       a = ag;
       pa = pg;
@@ -624,11 +621,11 @@ rf_status rf_reconstruct_batched(rf_ctx* ctx, int32_t G, const void* const* z_re
     int64_t row = 0;
     for (int g = 0; g < G; ++g) {
       if (ks[g]->k) {
-        if (forms[g] == RF_ALGO_GEMM)
+        if (a == RF_ALGO_GEMM)
           reconstruct_gemm(ctx, z_refs[g], ks[g], prec, nullptr, W, max_out + row * nw, argmax_out + row * nw,
                            (cudaStream_t)stream);
         else
-          run_direct(forms[g], ctx, z_refs[g], ks[g], nullptr, W, max_out + row * nw, argmax_out + row * nw,
+          run_direct(a, ctx, z_refs[g], ks[g], nullptr, W, max_out + row * nw, argmax_out + row * nw,
                      (cudaStream_t)stream);
       }
       row += ks[g]->k;

@@ -5,8 +5,7 @@
 // tensor-core form at the cheapest split precision that meets the FP32-equivalent accuracy
 // (bf16x6) in both of its tile layouts when the kernels are short enough for it to compete,
 // mixed forms (the tensor-core form for the shortest kernels, the fastest overlap-save layout for
-// the rest, within one call), and the direct sum for short kernels; on FP64 grids the direct sum and the
-// form AUTO takes by itself.  Each candidate runs the fused window-peak
+// the rest, within one call), and the direct sum for short kernels.  Each candidate runs the fused window-peak
 // form once to warm up and then three times between CUDA events; the fastest wins and is
 // recorded in every kernel set, so that RF_ALGO_AUTO follows it.
 #include <algorithm>
@@ -70,13 +69,6 @@ void autotune_impl(rf_ctx* c, int32_t G, const void* const* z_refs, rf_kernels* 
     cands.push_back(Cand{RF_ALGO_GEMM, gemm_wide_nj(RF_PREC_BF16X6), 1, RF_PREC_BF16X6, 0.0});
   }
   if (!f32 || max_len <= 1024) cands.push_back(Cand{RF_ALGO_DIRECT, 0, 0, RF_PREC_NATIVE, 0.0});
-  // FP64 grids: what AUTO runs by itself where it is not the direct sum for every set
-  if (!f32)
-    for (int g = 0; g < G; ++g)
-      if (os64_prepare(c, ks[g], s)) {
-        cands.push_back(Cand{RF_ALGO_AUTO, ks[g]->os64_B, ks[g]->os64_B / ks[g]->os64_Q, RF_PREC_NATIVE, 0.0});
-        break;
-      }
   RF_REQUIRE(!cands.empty(), "no reconstruction form to tune");
   const int64_t nw = (c->n + W - 1) / W;
   DevBuf pk, ak;
@@ -99,8 +91,7 @@ void autotune_impl(rf_ctx* c, int32_t G, const void* const* z_refs, rf_kernels* 
         if (cd.algo == RF_ALGO_OS || cd.algo == RF_ALGO_OS_BINS || cd.cut)
           reconstruct_os(c, z_refs[g], k, nullptr, W, mo, ao, s);
         else if (cd.algo == RF_ALGO_GEMM) reconstruct_gemm(c, z_refs[g], k, cd.prec, nullptr, W, mo, ao, s);
-        else if (cd.algo != RF_ALGO_AUTO || !reconstruct_os64(c, z_refs[g], k, nullptr, W, mo, ao, s))
-          reconstruct_direct(c, z_refs[g], k, nullptr, W, mo, ao, s);
+        else reconstruct_direct(c, z_refs[g], k, nullptr, W, mo, ao, s);
       }
       row += k->k;
     }
@@ -238,7 +229,8 @@ void autotune_impl(rf_ctx* c, int32_t G, const void* const* z_refs, rf_kernels* 
   for (int g = 0; g < G; ++g) {
     // bucketed preparations (overlap-save, two-phase or mixed) run through the overlap-save entry
     const bool bucketed = w.cut || w.algo == RF_ALGO_OS_BINS;
-    ks[g]->tuned_algo = bucketed ? RF_ALGO_OS : w.algo;
+    // (on FP64 grids the direct sum is the only form timed, and AUTO keeps its own rule)
+    ks[g]->tuned_algo = bucketed ? RF_ALGO_OS : (f32 ? w.algo : RF_ALGO_AUTO);
     ks[g]->tuned_prec = bucketed ? RF_PREC_NATIVE : w.prec;
   }
   RF_CUDA(cudaStreamSynchronize(s));

@@ -68,21 +68,3 @@ def test_prepared_ahead_of_the_first_call():
     rf2, z2, short = _set(torch, n, [1, 2, 3])
     short.prepare()                                   # the direct sum is cheaper: nothing to prepare
     assert _launches(lambda: rf2.reconstruct(z2, short)) == 1
-
-
-def test_autotune_times_what_auto_runs():
-    """The winner of the autotuner is the form AUTO runs afterwards, and tuned and untuned sets share a batch."""
-    torch = pytest.importorskip("torch")
-    n, W = 1 << 14, 512
-    for lens, algo, used in (([900, 901, 902], "auto", 3), ([2, 3, 4], "direct", 1)):
-        rf, z, kern = _set(torch, n, lens)
-        table = rf.autotune([z], [kern], W)
-        assert table[0]["algo"] == algo and {t["algo"] for t in table} >= {"direct", algo}
-        if algo == "auto":
-            assert table[0]["block"] in (1024, 2048, 4096) and table[0]["ms"] < table[1]["ms"]
-        assert _launches(lambda: rf.reconstruct_winmax(z, kern, W)) == used
-        other = rf.kernels_import(np.zeros(2, np.int32), [700, 800], np.ones(1500, np.complex128))
-        P, A = rf.reconstruct_batched([z, z], [kern, other], W)
-        for k, rows in ((kern, slice(0, 3)), (other, slice(3, 5))):
-            Pd, Ad = rf.reconstruct_winmax(z, k, W, "direct")
-            assert torch.equal(A[rows], Ad) and torch.allclose(P[rows], Pd, rtol=1e-6, atol=0.0)
