@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <cstdio>
 #include <memory>
@@ -67,19 +68,18 @@ struct DevBuf {
   T* as() const { return static_cast<T*>(p); }
 };
 
-// A device buffer that grows by powers of two and keeps what it outgrew: a graph captured with an earlier
-// buffer stays valid while the owner lives, and all of them together are below twice the largest.
+// A device buffer that keeps what it outgrew: a graph captured with an earlier buffer stays valid while
+// the owner lives.  It at least doubles when it grows, so what it keeps is below its size.
 struct KeptBuf {
   DevBuf at[64];
-  int log = -1;
+  int used = 0;
   void* ensure(size_t b) {
-    int l = 8;
-    while (((size_t)1 << l) < b) ++l;
-    if (l > log) {
-      at[l].ensure((size_t)1 << l);
-      log = l;
+    const size_t have = used ? at[used - 1].bytes : 0;
+    if (!used || b > have) {
+      at[used].ensure(std::max(b, 2 * have));
+      ++used;
     }
-    return at[log].p;
+    return at[used - 1].p;
   }
 };
 
