@@ -125,8 +125,10 @@ uint64_t rf_launch_count(void);
 const char* rf_last_error(void);
 
 /* Create a context for one grid on the current device.  Allocates the FFT twiddle and
- * bin-power tables and workspaces (about 68 n bytes, and up to 100 MB for batches of reference
- * templates).  Caller frees with rf_destroy. */
+ * bin-power tables and workspaces: 76 n bytes for RF_F32, 88 n bytes for RF_F64, and for batches of
+ * reference templates up to 50 MB (RF_F32) or 100 MB (RF_F64).  Between calls the context also keeps what
+ * its calls have grown: their workspaces, and up to 2 GB of stream-ordered temporaries of kernel building and of
+ * the double-precision overlap-save.  Caller frees all of it with rf_destroy. */
 rf_status rf_create(const rf_grid* grid, rf_ctx** out);
 
 /* Release a context and everything it owns.  Waits for the device.  NULL is a no-op. */
