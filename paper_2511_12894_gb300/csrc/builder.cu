@@ -251,13 +251,8 @@ __global__ void __launch_bounds__(128) k_pair_first(const RowPhase* __restrict__
   if (i >= nq) return;
   const int j = blockIdx.y;
   const Tf2Bins q = rp[j].q;  // in 4096ths of a turn
-  auto split = [](double x) {
-    const float h = (float)x;
-    return Pair{h, (float)(x - (double)h)};
-  };
   const PairPhase f{q.b0, q.d,
-                    Tf2Pairs{Pair{0.f, 0.f}, split(q.b2), split(q.b3), split(q.b4), split(q.b7), split(q.l5),
-                             split(q.l6), split(q.m6), split(q.e)}};
+                    make_tf2_pairs(q)};
   const float inv_n = 1.f / (float)n;  // n a power of two: exact
   const int64_t root_step = n / 4096;
   auto spectrum = [&](int64_t k) {

@@ -12,8 +12,7 @@
 // Ns >= 32) every store of a warp is one contiguous run.  A pass of few butterflies takes small
 // thread blocks, so that it spreads over the SMs: a radix-16 FP64 butterfly is about 230
 // instructions on two FP64 lanes per SM, and the passes of one 2^16-point row took 18.5 us each
-// on 16 blocks of 256 threads (128 blocks of one warp took the FP64 matched filter of 2^16 samples
-// from 188 to 111 us, before the four-step form carried it).
+// on 16 blocks of 256 threads (one FP64 reference of 2^13 samples: 128 us in blocks of 256, 68 now).
 #include <array>
 #include <cmath>
 
@@ -73,10 +72,11 @@ __global__ void __launch_bounds__(256) k_stockham_first_mul(const V* __restrict_
 }
 
 // Threads per block for `work` butterflies: 256, halved down to one warp while there are fewer
-// blocks than two per SM of a 152-SM part.
+// blocks than two per SM (152 of them on GB300, the one part this is built for; rf_mf_reference_noalloc runs
+// the passes without a context to ask).
 int pass_threads(int64_t work) {
   int nt = 256;
-  while (nt > 32 && work / nt < 304) nt /= 2;
+  while (nt > 32 && work / nt < 2 * 152) nt /= 2;
   return nt;
 }
 

@@ -97,14 +97,14 @@ __device__ __forceinline__ double tf2_turn(const Tf2Bins& q, int64_t k, double u
 struct Pair {
   float h, l;
 };
-inline Pair make_pair_of(double x) {
+__host__ __device__ __forceinline__ Pair make_pair_of(double x) {
   const float h = (float)x;
   return Pair{h, (float)(x - (double)h)};
 }
 struct Tf2Pairs {
   Pair b0, b2, b3, b4, b7, l5, l6, m6, e;  // no term in k: for t_c = 0
 };
-inline Tf2Pairs make_tf2_pairs(const Tf2Bins& q) {
+__host__ __device__ __forceinline__ Tf2Pairs make_tf2_pairs(const Tf2Bins& q) {
   return Tf2Pairs{make_pair_of(q.b0), make_pair_of(q.b2), make_pair_of(q.b3),
                   make_pair_of(q.b4), make_pair_of(q.b7), make_pair_of(q.l5),
                   make_pair_of(q.l6), make_pair_of(q.m6), make_pair_of(q.e)};
