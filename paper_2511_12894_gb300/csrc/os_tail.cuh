@@ -32,6 +32,15 @@ __device__ __forceinline__ unsigned long long warp_max_key(unsigned long long k)
 }
 
 
+// Whether the magnitudes of a block have a region of shared memory beside the transform's.  Blocks of 1024
+// and 2048 points with seven eighths of outputs share the transform's: 16 and 8 of them on an SM with the
+// larger regions leave the L1 cache too small to hold the loads of many partitions in flight (40 kernels of
+// 3000 taps at n = 2^18 in blocks of 1024: 258 us with regions of their own, 233 without; 2048: 154, 148).
+template <int B, int Q>
+constexpr bool os_own_magnitudes() {
+  return !(Q == 8 && (B == 1024 || B == 2048));
+}
+
 // Window peaks of this thread's CH consecutive outputs mv[0..cnt) whose first sample index is
 // i0 (later ones step by one and wrap to 0 at n), merged into the packed keys kj[window].
 // Warp-wide: every lane of the warp calls it (lanes without outputs pass cnt = 0).
@@ -159,11 +168,13 @@ __device__ __forceinline__ void os_block_tail(float2 (&v)[16], int s, int64_t m0
     }
     __syncthreads();  // the next block's FFT overwrites the shared memory read above
   } else {
-    // |y|^2 into its own region, so that no barrier is needed before these writes (the last stage
-    // of slower warps still reads the transform's region); the barrier after them also frees the
-    // transform's region for the next block, whose own barriers come before the region of the
-    // magnitudes is written again
-    float* mag = reinterpret_cast<float*>(sm + S::SMEM);
+    // |y|^2 into its own region (but see os_own_magnitudes), so that no barrier is needed before these
+    // writes (the last stage of slower warps still reads the transform's region); the barrier after them
+    // also frees the transform's region for the next block, whose own barriers come before the region of
+    // the magnitudes is written again
+    constexpr bool own = os_own_magnitudes<B, Q>();
+    float* mag = reinterpret_cast<float*>(sm + (own ? S::SMEM : 0));
+    if (!own) __syncthreads();
 #pragma unroll
     for (int t = 16 / Q; t < 16; ++t) mag[tid + t * NT - LP] = v[t].x * v[t].x + v[t].y * v[t].y;
     __syncthreads();
@@ -181,6 +192,7 @@ __device__ __forceinline__ void os_block_tail(float2 (&v)[16], int s, int64_t m0
     // outputs of this thread that exist (all but possibly in the last block)
     const int64_t avail = lim - qbase;
     const int cnt = avail <= 0 ? 0 : (avail >= CH ? CH : (int)avail);
+    if (!own) __syncthreads();  // read before the next block's transform writes there
     window_keys<CH>(mv, cnt, (int)((base + qbase) & mask), n, W, nw, fastwin, kj);
   }
 }
@@ -188,7 +200,8 @@ __device__ __forceinline__ void os_block_tail(float2 (&v)[16], int s, int64_t m0
 // Shared memory of a CTA that runs os_block_tail: the transform's region, then the magnitudes.
 template <int B, int Q, bool WINMAX>
 constexpr size_t os_tail_smem() {
-  return sizeof(float2) * BlockFFTShape<B>::SMEM + (WINMAX ? sizeof(float) * (B - B / Q) : 0);
+  return sizeof(float2) * BlockFFTShape<B>::SMEM +
+         (WINMAX && os_own_magnitudes<B, Q>() ? sizeof(float) * (B - B / Q) : 0);
 }
 
 // ------------------------------------------------------- 32768-point blocks on CTA pairs
