@@ -315,6 +315,15 @@ def scipy_baseline(cfg, x, filt_row, kern, n_nbrs=8, budget_s=20.0):
 
 # --------------------------------------------------------------------------- ncu traffic
 
+def mf_transform(dtype: str, n: int, refs: int, sms: int) -> str:
+    """The form in which the library runs stored-filter matched filters of this size."""
+    if dtype == "f32" and (1 << 9 <= n <= 1 << 14 or (n <= 1 << 16 and refs * 8 <= sms)) and n >= 1 << 9:
+        return "one launch per call"
+    if n >= (1 << 15 if dtype == "f32" else 1 << 14) and n <= (1 << 24 if dtype == "f32" else 1 << 18):
+        return "four-step, two passes"
+    return "four-step data transform, radix-16 inverses" if 1 << 18 < n <= 1 << 21 else "radix-16 passes"
+
+
 def ncu_traffic(kernel: str, layout: str = None):
     """DRAM bytes per launch of `kernel` from the committed ncu capture, or None when the
     kernel's sources (or its layout) changed since that capture, or no capture exists."""
@@ -684,8 +693,7 @@ def main():
     mf_info = {"references": G, "kernel_ms": mf_avg_ms, "us_per_reference": mf_avg_ms * 1e3 / G,
                "alg_bytes": mf_bytes, "achieved_gbs": mf_bytes / (mf_avg_ms / 1e3) / 1e9,
                "frac_of_hbm": mf_bytes / (mf_avg_ms / 1e3) / 1e9 / hbm_peak,
-               "transform": ("four-step, two passes" if cfg.dtype == "f32" and (1 << 18) <= n <= (1 << 24)
-                             else "radix-16 passes"),
+               "transform": mf_transform(cfg.dtype, n, G, props.multi_processor_count),
                "bytes_note": "data in once; per reference its filter in and z_ref out (the minimum)"
                              if args.mf == "filtered" else "data in once; per reference z_ref out"}
 
