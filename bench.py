@@ -693,7 +693,7 @@ def main():
     mf_info = {"references": G, "kernel_ms": mf_avg_ms, "us_per_reference": mf_avg_ms * 1e3 / G,
                "alg_bytes": mf_bytes, "achieved_gbs": mf_bytes / (mf_avg_ms / 1e3) / 1e9,
                "frac_of_hbm": mf_bytes / (mf_avg_ms / 1e3) / 1e9 / hbm_peak,
-               "transform": mf_transform(cfg.dtype, n, G, props.multi_processor_count),
+               "transform": mf_transform(cfg.dtype, n, G, torch.cuda.get_device_properties(dev).multi_processor_count),
                "bytes_note": "data in once; per reference its filter in and z_ref out (the minimum)"
                              if args.mf == "filtered" else "data in once; per reference z_ref out"}
 
