@@ -34,8 +34,8 @@ namespace {
 // ---------------------------------------------------------------- FP32 grids: transforms in pairs
 // The taps of an FP32 grid are rounded to FP32, and the transform that makes them cost 2.9 of the 7 ms
 // of building 48 kernels on 2^19 bins, all of it on the FP64 pipe.  The same radix passes in FP32
-// pairs (cdf.cuh) are bound by HBM: 172 to 184 us per radix-16 pass of those rows (805 MB, 55% of the
-// copy rate), the whole build 1.87 ms.  The leading term of the phase stays FP64.
+// pairs (cdf.cuh) are bound by HBM: 171 us per radix-16 pass of those rows (754 MB, 65% of the
+// copy rate; the first one, which forms the spectrum, 452 us, by the FP64 pipe), the whole build 1.83 ms.  The leading term of the phase stays FP64.
 //
 // Pairs serve where the result is the FP64 one:
 // * A row's error is bounded by eps times its largest value: 2^-43 for the transform (2^-46.4 measured,
