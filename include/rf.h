@@ -174,7 +174,7 @@ rf_status rf_reference_filters(rf_ctx* ctx, const double* inv_psd, int32_t nref,
  * complex[nref][n] (grid dtype); x or filt may lie inside z_out.  RF_F32 grids of 2^9 to 2^13 samples,
  * of 2^14, and for at most SMs / 8 references of 2^15 and 2^16, run in one launch without a temporary (unless
  * filt lies inside z_out: a copy of the filters).  The others take a temporary of min(nref, R) x n complex
- * values, R = 2^25 / n (RF_F32, and RF_F64 from 2^14 to 2^18 samples) or 2^27 / n, at most 65535.  It grows, at
+ * values, R = 2^25 / n (RF_F32 from 2^15 samples on, RF_F64 from 2^14 to 2^18) or 2^27 / n, at most 65535.  It grows, at
  * least twofold, on the first call that needs more, and what it outgrew stays for captured graphs: a call can be
  * captured once the same call (references, and whether filt lies inside z_out) has run.  Rows of a call do not
  * depend on the other filters (RF_F32 grids of 2^14 to 2^16 samples: see rf_mf_reference).  Async on stream. */

@@ -378,9 +378,9 @@ constexpr int kF4MaxInverse64 = 18;
 // (8 columns of 2048 points, one block per SM: 640 us against 624 for 6 references of 2^23 samples); shorter
 // lines, of small transforms, in tiles of 4 for more blocks.  FP64: at most 1024 threads.
 template <typename V, int L> constexpr int f4_cols_g() {
-  return sizeof(V) == 8 ? (L == 512 || L == 1024 ? 8 : 4) : (L <= 256 || L >= 4096 ? 2 : 4);
+  return sizeof(V) == 8 ? (L == 512 || L == 1024 ? 8 : 4) : (L <= 256 ? 2 : 4);
 }
-template <typename V, int L> constexpr int f4_rows_r() { return sizeof(V) == 16 && (L <= 256 || L >= 4096) ? 2 : 4; }
+template <typename V, int L> constexpr int f4_rows_r() { return sizeof(V) == 16 && L <= 256 ? 2 : 4; }
 
 template <typename V, int L>
 const V* line_tables(const rf_ctx* c) {
